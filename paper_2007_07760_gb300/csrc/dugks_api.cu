@@ -13,6 +13,7 @@
 #include <mutex>
 #include <atomic>
 #include <string>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -26,7 +27,7 @@ using namespace dugks::host;
 
 struct dugks_ctx {
     dugks_params p{};
-    int dev = 0;
+    int dev = 0, sms = 0;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     int pitch = 0;
@@ -46,6 +47,8 @@ struct dugks_ctx {
     int tile_w = TILE_X, tile_h = TILE_Y, tiles_x = 0, ntiles = 0;
     // TMA-staged two-stage path (orders 2, 3)
     bool fast = false;
+    bool march = false;         // fast, as a row march (two-stage, orders 2-3, phi a plane of its own)
+    MarchPlan plan{};
     int variant = 0;
     CUtensorMap tmX[2], tmPhi[4];
     double coef_h = -1.0;
@@ -141,8 +144,18 @@ bool encode_map(CUtensorMap *m, void *base, size_t es, bool half, const dugks_ct
     return encode_plane_map(m, base, es, half, c->pitch, c->p.ny, c->plane, nplanes, bw, bh);
 }
 
+// whether the fast path of this context is the row march
+bool marches(const dugks_ctx *c) { return c->p.stages == 2 && c->p.order <= 3 && c->p.precision != DUGKS_FP64; }
+
 template <typename T, typename ST>
 bool setup_fast(dugks_ctx *c) {
+    if (marches(c)) {
+        c->march = true;
+        c->plan = march_plan(c->variant, c->p.nx, c->p.ny, c->p.precision == DUGKS_FP16F, c->sms);
+        c->tile_w = 32 * c->plan.cols - 4;
+        c->tile_h = c->plan.rows;
+        return true;
+    }
     const FastGeom g = Launch<T, ST>::fast_geom(c->variant, c->p.order, c->p.stages);
     const bool half = Store<T, ST>::deviation;
     for (int s = 0; s < 2; s++)
@@ -153,6 +166,14 @@ bool setup_fast(dugks_ctx *c) {
     c->tile_h = g.tile_h;
     return true;
 }
+
+// the march needs no tensor maps; the TMA-staged kernels need the driver's encoder
+bool fast_capable(const dugks_ctx *c) {
+    return c->p.stages != 1 && (c->p.stages == 2 || c->p.precision != DUGKS_FP16F) && (marches(c) || encode_fn() != nullptr);
+}
+
+// strips of the row march start one column before the grid
+int strips(const dugks_ctx *c) { return c->fast && c->march ? c->plan.strips : (c->p.nx + c->tile_w - 1) / c->tile_w; }
 
 template <typename T, typename ST>
 int run_init(dugks_ctx *c) {
@@ -256,15 +277,22 @@ int step_t2(dugks_ctx *c, double *dbg = nullptr) {
                                       vortex_factors<T>(c, t, t - dt, t + h), c->tmX[c->cur], c->tmPhi[iPo],
                                       c->tmPhi[iPc], c->p.flux, KIND_T2, c->stream);
     } else if (c->fast) {
+        // orders 2 and 3: the row march where phi is a plane of its own, else the TMA-staged kernel
+        using Coefs = typename std::conditional<Store<T, ST>::phi_plane, MarchCoefs<T>, FaceCoefs<T>>::type;
         if (c->coef_h != h) {
-            FaceCoefs<T> cf = make_face_coefs<T>(c->p.order, c->p.flux, h);
-            c->coefs.assign(reinterpret_cast<unsigned char *>(&cf), reinterpret_cast<unsigned char *>(&cf) + sizeof cf);
+            Coefs cf;
+            if constexpr (Store<T, ST>::phi_plane) cf = make_march_coefs<T>(c->p.order, h);
+            else cf = make_face_coefs<T>(c->p.order, c->p.flux, h);
+            c->coefs.assign(reinterpret_cast<const unsigned char *>(&cf), reinterpret_cast<const unsigned char *>(&cf) + sizeof cf);
             c->coef_h = h;
         }
-        const FaceCoefs<T> &cf = *reinterpret_cast<const FaceCoefs<T> *>(c->coefs.data());
+        const Coefs &cf = *reinterpret_cast<const Coefs *>(c->coefs.data());
         const FastExtra<T> fx = vortex_factors<T>(c, t, t - dt, t + h);
-        e = Launch<T, ST>::step_fast(q, cf, fx, c->tmX[c->cur], c->tmPhi[iPo], c->tmPhi[iPc], c->p.order,
-                                     c->p.flux, c->variant, c->stream);
+        if constexpr (Store<T, ST>::phi_plane)
+            e = Launch<T, ST>::step_march(q, cf, fx, c->p.flux, c->plan.cols, c->plan.early, c->stream);
+        else
+            e = Launch<T, ST>::step_fast(q, cf, fx, c->tmX[c->cur], c->tmPhi[iPo], c->tmPhi[iPc], c->p.order,
+                                         c->p.flux, c->variant, c->stream);
     } else {
         if (c->p.order == 5) return fail(c, DUGKS_EINVAL, "order 5 needs the TMA-staged kernels");
         e = Launch<T, ST>::step(q, c->p.order, c->p.flux, KIND_T2, c->stream);
@@ -619,7 +647,8 @@ int dugks_create(const dugks_params *p, const double *phi0_host, void *cuda_stre
     // the TMA-staged kernels serve every order and both schemes (three-stage: full
     // storage; orders 4-5 and the three-stage scheme: one tile shape each)
     // (the DVM has one kernel of its own)
-    c->fast = p->stages != 1 && (p->stages == 2 || p->precision != DUGKS_FP16F) && encode_fn() != nullptr;
+    cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->dev);
+    c->fast = fast_capable(c);
     if (c->fast && (p->stages == 3 || p->order >= 4)) {
         c->variant = 2;
     } else if (c->fast) {
@@ -653,7 +682,7 @@ int dugks_create(const dugks_params *p, const double *phi0_host, void *cuda_stre
             c->tile_h = TILE_Y;
         }
     }
-    c->tiles_x = (p->nx + c->tile_w - 1) / c->tile_w;
+    c->tiles_x = strips(c);
     c->ntiles = c->tiles_x * ((p->ny + c->tile_h - 1) / c->tile_h);
     if (ok) ok = dev_malloc(&c->partial, (size_t)c->ntiles * sizeof(double)) == cudaSuccess;
     if (!ok) {
@@ -871,9 +900,7 @@ int dugks_selftest_fail_allocs(int32_t skip, int32_t count) {
 
 int dugks_set_variant(dugks_ctx *c, int variant) {
     if (!c || variant < -1 || variant >= FAST_VARIANTS) return DUGKS_EINVAL;
-    const bool fast_capable =
-        c->p.stages != 1 && (c->p.stages == 2 || c->p.precision != DUGKS_FP16F) && encode_fn() != nullptr;
-    if (!fast_capable) return DUGKS_OK;
+    if (!fast_capable(c)) return DUGKS_OK;
     // order 4 and the three-stage kernels have one tile shape
     if ((c->p.stages == 3 || c->p.order >= 4) && variant >= 0) variant = 2;
     // order 5 exists on the TMA-staged path only
@@ -893,7 +920,7 @@ int dugks_set_variant(dugks_ctx *c, int variant) {
                                                        : setup_fast<float, __half>(c);
         if (!ok) return fail(c, DUGKS_ECUDA, "tensor map encoding failed");
     }
-    c->tiles_x = (c->p.nx + c->tile_w - 1) / c->tile_w;
+    c->tiles_x = strips(c);
     const int ntiles = c->tiles_x * ((c->p.ny + c->tile_h - 1) / c->tile_h);
     if (ntiles > c->ntiles) {
         cudaFree(c->partial);

@@ -798,6 +798,72 @@ struct BatchUniform {
     int *status;
 };
 
+// The parameters of a grid's current step; returns the phi plane roles (iPc, iPo).
+template <typename T, typename ST>
+__device__ __forceinline__ int2 batch_step_params(const BatchUniform<T> &u, const BatchGrid<T> *G, StepParams<T> &p,
+                                                  FastExtra<T> &fe) {
+    constexpr bool PHIP = Store<T, ST>::phi_plane;
+    const long long step = G->step;
+    p.nx = G->nx;
+    p.ny = G->ny;
+    p.pitch = G->pitch;
+    p.plane = G->plane;
+    p.status = u.status;
+    p.tiles_x = G->tiles_x;
+    p.tile_w = u.tile_w;
+    p.tile_h = u.tile_h;
+    p.acc = nullptr;
+    p.out2 = nullptr;
+    p.mass_partial = nullptr;
+    p.ufield = p.vfield = nullptr;
+    p.a = T(1) - u.b;
+    p.b = u.b;
+    p.h = u.h;
+    p.c1 = u.c1;
+    p.c2 = u.c2;
+    p.c3 = u.c3;
+    p.al1 = T(1) - u.be1;
+    p.be1 = u.be1;
+    p.ga1 = u.ga1;
+    p.al2 = p.be2 = p.ga2 = T(0);
+    p.tau = u.tau;
+    p.theta_c = u.theta_c;
+    p.phiA = u.phiA;
+    p.phiB = u.phiB;
+    p.inv_dtD = u.inv_dt;
+    p.useD = (u.dtphiu && step > 0) ? 1 : 0;
+    p.seed = (uint32_t)step;
+    p.vel_kind = G->vel_kind;
+    p.vp0 = (T)G->vp[0];
+    p.vp1 = (T)G->vp[1];
+    p.vp2 = (T)G->vp[2];
+    p.t = G->tl[0];
+    p.t_old = G->tl[1];
+    p.t_face = G->tl[2];
+    p.qscale = u.qscale;
+    p.qinv = u.qinv;
+    fe.vc_t = G->vc[0];
+    fe.vc_told = G->vc[1];
+    fe.vc_tface = G->vc[2];
+    const int cur = (int)(step & 1);
+    p.X = G->X[cur];
+    p.out1 = G->X[1 - cur];
+    int iPc = 0, iPo, iOut;
+    if constexpr (PHIP) {   // roles rotate with period 3 (see the context API)
+        iPc = (3 - (int)(step % 3)) % 3;
+        iPo = (iPc + 1) % 3;
+        iOut = (iPc + 2) % 3;
+        p.phi_cur = G->phi[iPc];
+    } else {
+        iPo = cur;
+        iOut = 1 - cur;
+        p.phi_cur = nullptr;
+    }
+    p.phi_old = G->phi[iPo];
+    p.phi_out = G->phi[iOut];
+    return make_int2(iPc, iPo);
+}
+
 template <typename T, typename ST, int ORDER, int FLUX, int NW, int MR>
 __global__ void __launch_bounds__(NW * 32, (FastTile<T, ST, NW, MR>::min_blocks))
 batch_fast_kernel(const __grid_constant__ BatchUniform<T> u, const __grid_constant__ FaceCoefs<T> cf,
@@ -815,64 +881,9 @@ batch_fast_kernel(const __grid_constant__ BatchUniform<T> u, const __grid_consta
         const long long step = G->step;
         if (step >= G->target) continue;   // frozen grid (uniform for the CTA)
         StepParams<T> p;
-        p.nx = G->nx;
-        p.ny = G->ny;
-        p.pitch = G->pitch;
-        p.plane = G->plane;
-        p.status = u.status;
-        p.tiles_x = G->tiles_x;
-        p.tile_w = u.tile_w;
-        p.tile_h = u.tile_h;
-        p.acc = nullptr;
-        p.out2 = nullptr;
-        p.mass_partial = nullptr;
-        p.ufield = p.vfield = nullptr;
-        p.a = T(1) - u.b;
-        p.b = u.b;
-        p.h = u.h;
-        p.c1 = u.c1;
-        p.c2 = u.c2;
-        p.c3 = u.c3;
-        p.al1 = T(1) - u.be1;
-        p.be1 = u.be1;
-        p.ga1 = u.ga1;
-        p.al2 = p.be2 = p.ga2 = T(0);
-        p.tau = u.tau;
-        p.theta_c = u.theta_c;
-        p.phiA = u.phiA;
-        p.phiB = u.phiB;
-        p.inv_dtD = u.inv_dt;
-        p.useD = (u.dtphiu && step > 0) ? 1 : 0;
-        p.seed = (uint32_t)step;
-        p.vel_kind = G->vel_kind;
-        p.vp0 = (T)G->vp[0];
-        p.vp1 = (T)G->vp[1];
-        p.vp2 = (T)G->vp[2];
-        p.t = G->tl[0];
-        p.t_old = G->tl[1];
-        p.t_face = G->tl[2];
-        p.qscale = u.qscale;
-        p.qinv = u.qinv;
         FastExtra<T> fe;
-        fe.vc_t = G->vc[0];
-        fe.vc_told = G->vc[1];
-        fe.vc_tface = G->vc[2];
-        const int cur = (int)(step & 1);
-        p.X = G->X[cur];
-        p.out1 = G->X[1 - cur];
-        int iPc = 0, iPo, iOut;
-        if constexpr (PHIP) {   // roles rotate with period 3 (see the context API)
-            iPc = (3 - (int)(step % 3)) % 3;
-            iPo = (iPc + 1) % 3;
-            iOut = (iPc + 2) % 3;
-            p.phi_cur = G->phi[iPc];
-        } else {
-            iPo = cur;
-            iOut = 1 - cur;
-            p.phi_cur = nullptr;
-        }
-        p.phi_old = G->phi[iPo];
-        p.phi_out = G->phi[iOut];
+        const int2 roles = batch_step_params<T, ST>(u, G, p, fe);
+        const int cur = (int)(step & 1), iPc = roles.x, iPo = roles.y;
         if (threadIdx.x == 0 && w.x != fenced) {
             // tensor maps written to global memory by the host: order them for the TMA
             // unit (once per grid: the descriptors do not change during a launch)

@@ -5,6 +5,7 @@
 
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -156,6 +157,74 @@ inline FaceCoefs<T, R> make_face_coefs_r(int order, int flux, double h) {
 template <typename T>
 inline FaceCoefs<T> make_face_coefs(int order, int flux, double h) {
     return make_face_coefs_r<T, 1>(order, flux, h);
+}
+
+// Expansion coefficients of the row march (orders 2 and 3; the fields are described at
+// MarchCoefs). The terms of order 2 and above in the displacement are those of order 3.
+template <typename T>
+inline MarchCoefs<T> make_march_coefs(int order, double h) {
+    MarchCoefs<T> m;
+    const double c = 0.5 - h, q = order >= 3 ? 1.0 : 0.0;
+    auto row = [&](double x, double y, int b, T *w) {   // C, R + L, R - L
+        const double l = taylor_w(order, x, y, -1, b), r = taylor_w(order, x, y, 1, b);
+        w[0] = (T)taylor_w(order, x, y, 0, b);
+        w[1] = (T)(0.5 * (r + l));
+        w[2] = (T)(0.5 * (r - l));
+    };
+    for (int b = -1; b <= 1; b++) {
+        row(c, -h, b, m.dx[b + 1]);
+        row(-h, c, b, m.dy[b + 1]);
+    }
+    m.px = (T)(c / 12.0);
+    m.pe = (T)(q * c * c / 12.0);
+    m.nu = (T)((0.5 * c + q * 0.5 * c * c) / 6.0);
+    m.nd = (T)((-0.5 * c + q * 0.5 * c * c) / 6.0);
+    m.nm = (T)(-q * c * c / 6.0);
+    m.ge = (T)(q / 96.0);
+    m.gp = (T)(q * h * h / 24.0);
+    m.gd = (T)(h / 24.0);
+    m.b2 = (T)(q * h / 16.0);
+    m.h = (T)h;
+    m.cp = (T)(0.5 - h);
+    m.cm = (T)(-0.5 - h);
+    m.hk = (T)(h / 24.0);
+    return m;
+}
+
+// Lane width (columns a lane), segment rows and launch mode of the row march.
+// A segment of s rows reads s + 4, so long segments do less work, and short ones give more
+// warps. The cost below is a fit to the measured steps (FP32, vortex, 64^2 to 4096^2, s from 1
+// to 64, both widths; within 15%): a row takes `unit` microseconds in a full wave of W = 1;
+// several waves overlap but for 0.43 of one; a little over one wave costs nearly two; and
+// a partial wave is bound by the latency of a row, which grows with n, the warps a scheduler.
+// Measured: 64^2 5.3 us (1 column, s = 1) against 7.8 us with pairs; 256^2 9.0 (1, 2) against
+// 11.4; 1024^2 39.0 (2, 16) against 40.8; 4096^2 356 (2, 48) against 392. Segments over
+// 64 rows lose again (4096^2, 241 rows in one wave: 478 us): the rows in flight then lie all over
+// the planes, more pages than the TLB holds.
+struct MarchPlan { int cols, strips, rows, early; };
+inline MarchPlan march_plan(int variant, int nx, int ny, bool half, int sms) {
+    static constexpr int fixed[6] = {16, 8, 0, 32, 0, 64};   // variants 2 and 4: by the rule
+    MarchPlan m{};
+    double best = 1e300;
+    const int forced = variant >= 0 && variant < 6 ? fixed[variant] : 0;
+    for (int cols = half ? 2 : 1; cols <= 2; cols++) {
+        const int strips = cols == 2 ? MarchTile<float2, float>::strips(nx) : MarchTile<float, float>::strips(nx);
+        const double slots = (cols == 2 ? 8.0 : 12.0) * sms, unit = cols == 2 ? 1.42 : 1.05;
+        for (int want = forced ? forced : 1; want <= (forced ? forced : 64); want++) {
+            const int segs = (ny + want - 1) / want, rows = (ny + segs - 1) / segs;   // segments of equal length
+            const double w = (double)strips * segs, W = w / slots, n = std::max(w / (4.0 * sms), 1.0);
+            const double f = W > 1.5 ? W + 0.43 : W > 1.0 ? 1.9 : cols == 2 ? 1.0 + 0.37 * (n - 1.0) : 0.89 + 0.3 * (n - 1.0);
+            const double cost = unit * (rows + 5) * f;
+            if (cost < best) {
+                best = cost;
+                // Early scheduling of the next kernel hides its launch and velocity factors
+                // (512^2: 15.5 against 16.5 us). On a chip half full it costs instead, because the
+                // waiting warps fill some SMs and leave others idle (256^2, 860 warps: 10.2 against 9.1).
+                m = MarchPlan{cols, strips, rows, W > 0.6 || W < 0.15};
+            }
+        }
+    }
+    return m;
 }
 
 // ---- TMA tensor maps -----------------------------------------------------------

@@ -1,0 +1,9 @@
+// row-march step kernels of the two-stage scheme (orders 2 and 3), single grid and batch; state half deviations, arithmetic float.
+// (One translation unit per precision and kernel family, so they compile in parallel.)
+#include "dugks_launch.cuh"
+
+namespace dugks {
+template cudaError_t Launch<float,__half>::step_march(const StepParams<float> &, const MarchCoefs<float> &, const FastExtra<float> &, int, int, int, cudaStream_t);
+template cudaError_t Launch<float,__half>::batch_march(const BatchUniform<float> &, const MarchCoefs<float> &, const BatchGrid<float> *, const int4 *, int, int, double *, int, int, cudaStream_t);
+template int Launch<float,__half>::march_ctas_per_sm(int, int);
+}  // namespace dugks

@@ -8,6 +8,7 @@
 
 #include "dugks_fast.cuh"
 #include "dugks_kernels.cuh"
+#include "dugks_march.cuh"
 
 namespace dugks {
 
@@ -42,6 +43,14 @@ struct Launch {
                                   const int4 *items, int nitems, double *partials, int order, int flux, int variant,
                                   int ctas, cudaStream_t s);
     static int batch_ctas_per_sm(int order, int flux, int variant);
+    // the row march (two-stage, orders 2 and 3, phi a plane of its own): one strip segment
+    // of p.tile_h rows per CTA
+    static cudaError_t step_march(const StepParams<T> &p, const MarchCoefs<T> &cf, const FastExtra<T> &fe, int flux,
+                                  int cols, int early, cudaStream_t s);
+    static cudaError_t batch_march(const BatchUniform<T> &u, const MarchCoefs<T> &cf, const BatchGrid<T> *grids,
+                                   const int4 *items, int nitems, int max_rows, double *partials, int flux, int ctas,
+                                   cudaStream_t s);
+    static int march_ctas_per_sm(int flux, int rows);
     static cudaError_t step_fast(const StepParams<T> &p, const FaceCoefs<T> &cf, const FastExtra<T> &fe, const CUtensorMap &tmX,
                                  const CUtensorMap &tmPo, const CUtensorMap &tmPc, int order, int flux,
                                  int variant, cudaStream_t s);

@@ -74,7 +74,7 @@ cudaError_t Launch<T, ST>::init(const StepParams<T> &p, const T *phi0, T frac_dt
 
 template <typename T, typename ST>
 cudaError_t Launch<T, ST>::mass_partial(const StepParams<T> &p, cudaStream_t s) {
-    dim3 grid((p.nx + p.tile_w - 1) / p.tile_w, (p.ny + p.tile_h - 1) / p.tile_h);
+    dim3 grid(p.tiles_x, (p.ny + p.tile_h - 1) / p.tile_h);
     mass_partial_kernel<T, ST><<<grid, 256, 0, s>>>(p);
     return cudaGetLastError();
 }
@@ -243,6 +243,65 @@ cudaError_t Launch<T, ST>::step_fast4(const StepParams<T> &p, const FaceCoefs<T,
                              : launch_fast4_t<T, ST, 1, KIND_T3B>(p, cf, fe, tmX, tmPo, tmPc, s);
     }
     return cudaErrorInvalidValue;
+}
+
+template <typename V, typename ST, int FLUX, bool FIELD>
+static cudaError_t launch_march_t(const StepParams<typename Lane<V>::T> &p, const MarchCoefs<typename Lane<V>::T> &cf,
+                                  const FastExtra<typename Lane<V>::T> &fe, int early, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(p.tiles_x, (p.ny + p.tile_h - 1) / p.tile_h);
+    cfg.blockDim = dim3(32);
+    cfg.dynamicSmemBytes = MarchTile<V, ST>::smem_bytes(p.tile_h);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, step_march_kernel<V, ST, FLUX, FIELD>, p, cf, fe, early);
+}
+
+template <typename V, typename ST>
+static cudaError_t launch_march_v(const StepParams<typename Lane<V>::T> &p, const MarchCoefs<typename Lane<V>::T> &cf,
+                                  const FastExtra<typename Lane<V>::T> &fe, int flux, int early, cudaStream_t s) {
+    if (p.vel_kind == VEL_FIELD)
+        return flux == 0 ? launch_march_t<V, ST, 0, true>(p, cf, fe, early, s)
+                         : launch_march_t<V, ST, 1, true>(p, cf, fe, early, s);
+    return flux == 0 ? launch_march_t<V, ST, 0, false>(p, cf, fe, early, s)
+                     : launch_march_t<V, ST, 1, false>(p, cf, fe, early, s);
+}
+
+template <typename T, typename ST>
+cudaError_t Launch<T, ST>::step_march(const StepParams<T> &p, const MarchCoefs<T> &cf, const FastExtra<T> &fe, int flux,
+                                      int cols, int early, cudaStream_t s) {
+    if constexpr (!Store<T, ST>::deviation)
+        if (cols == 1) return launch_march_v<T, ST>(p, cf, fe, flux, early, s);
+    return launch_march_v<float2, ST>(p, cf, fe, flux, early, s);
+}
+
+template <typename T, typename ST>
+cudaError_t Launch<T, ST>::batch_march(const BatchUniform<T> &u, const MarchCoefs<T> &cf, const BatchGrid<T> *grids,
+                                       const int4 *items, int nitems, int max_rows, double *partials, int flux,
+                                       int ctas, cudaStream_t s) {
+    if (nitems <= 0) return cudaSuccess;
+    const int smem = MarchTile<float2, ST>::smem_bytes(max_rows), n = ctas < nitems ? ctas : nitems;
+    if (flux == 0) batch_march_kernel<float2, ST, 0><<<n, 32, smem, s>>>(u, cf, grids, items, nitems, partials);
+    else batch_march_kernel<float2, ST, 1><<<n, 32, smem, s>>>(u, cf, grids, items, nitems, partials);
+    return cudaGetLastError();
+}
+
+template <typename T, typename ST>
+int Launch<T, ST>::march_ctas_per_sm(int flux, int rows) {
+    int n = 0;
+    const int smem = MarchTile<float2, ST>::smem_bytes(rows);
+    const cudaError_t e =
+        flux == 0 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_march_kernel<float2, ST, 0>, 32, smem)
+                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_march_kernel<float2, ST, 1>, 32, smem);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        n = 1;
+    }
+    return n > 0 ? n : 1;
 }
 
 template <typename T, typename ST>

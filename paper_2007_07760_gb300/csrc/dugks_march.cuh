@@ -1,0 +1,807 @@
+// dugks_march.cuh -- the two-stage DUGKS step for stencils of radius 1 (orders 2
+// and 3) as a row march (sm_103a): FP32 and FP16 storage.
+//
+// Same method as step_kernel (dugks_kernels.cuh; equation numbers are the paper's).
+// One warp, which is one CTA, owns a strip of 60 columns and a segment of rows and
+// walks up the rows with everything the step needs of the rows below in registers:
+//  * a lane holds two adjacent columns, and all arithmetic is on that pair (packed
+//    FP32: one instruction, two columns). The left and right neighbours of a pair
+//    are one shuffle each for two cells; no shared-memory exchange and no barrier.
+//  * the face values of Eqs. (24)-(26) are evaluated as expansions about each cell:
+//    cell c gives its own contribution to its east, west, north and south faces, so
+//    a face needs the 3 x 3 cells around one cell instead of 3 x 4 around a face.
+//    An expansion is a sum over the three rows of row terms, so when row j arrives
+//    it completes the expansions of row j - 1, adds the middle terms of row j and
+//    starts row j + 1: each row of bar f^+ is formed and shuffled once.
+//  * the directions normal to a face (the ties of Eq. (26)) enter only the face
+//    moment phi_b, never the difference of a single bar f_k; their sums over the
+//    three directions are taken before the stencil.
+//  * rows arrive through a ring of per-lane cp.async copies two rows ahead.
+// What bounds it: FP32 issue. Rows of a segment are read and expanded with two
+// extra rows on each side, so the segment length trades that overhead against the
+// number of warps in flight (march_rows in dugks_internal.h has the rule).
+#pragma once
+
+#include <type_traits>
+
+#include "dugks_fast.cuh"
+
+namespace dugks {
+
+// Expansion coefficients of one reconstruction time h (host: make_march_coefs).
+// Upwind, with c = 1/2 - h:
+//   dx[b + 1][.]  row b of the expansion at (c, -h), the east face of xi = (1, 1): weights of
+//                 C, R + L and R - L; dy: of the one at (-h, c), the north face. Mirrored for
+//                 the other diagonals
+//   px, pe           row term px (R - L) + pe (L - 2 C + R) of the expansion at (c, 0)
+//   nu, nm, nd       weights of L + 4 C + R of the rows above, at and below at (0, c)
+//   ge, gp, gd, b2   ties: see the row terms G, Q and B in the kernel
+// Central: h and cp = 1/2 - h, cm = -1/2 - h, hk = h / 24.
+template <typename T>
+struct MarchCoefs {
+    T dx[3][3], dy[3][3];
+    T px, pe, nu, nm, nd, ge, gp, gd, b2;
+    T h, cp, cm, hk;
+};
+
+// ---- a lane's columns of one row: a pair (float2, packed arithmetic) or one value -----
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 vfma(float a, float2 b, float2 c) { return __ffma2_rn(make_float2(a, a), b, c); }
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 vadd(float2 a, float b) { return __fadd2_rn(a, make_float2(b, b)); }
+__device__ __forceinline__ float2 vneg(float2 a) { return make_float2(-a.x, -a.y); }   // (an operand modifier)
+__device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __fadd2_rn(a, vneg(b)); }
+__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 vmul(float a, float2 b) { return __fmul2_rn(make_float2(a, a), b); }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float vneg(float a) { return -a; }
+__device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+
+// Neighbouring columns: one shuffle a value or pair each way, and sums and differences
+// taken per column (a pair built of a shuffled and an own value would cost the moves that
+// line it up). Undefined at the warp's edges.
+constexpr unsigned ALL = 0xffffffffu;
+template <typename V>
+struct Sides { V s, d; };   // right + left, right - left
+__device__ __forceinline__ Sides<float2> vsides(float2 c) {
+    const float l = __shfl_up_sync(ALL, c.y, 1), r = __shfl_down_sync(ALL, c.x, 1);
+    return {make_float2(__fadd_rn(c.y, l), __fadd_rn(r, c.x)), make_float2(__fsub_rn(c.y, l), __fsub_rn(r, c.x))};
+}
+__device__ __forceinline__ float2 vless_left(float2 c) {    // c - left
+    return make_float2(__fsub_rn(c.x, __shfl_up_sync(ALL, c.y, 1)), __fsub_rn(c.y, c.x));
+}
+__device__ __forceinline__ float2 vless_right(float2 c) {   // c - right
+    return make_float2(__fsub_rn(c.x, c.y), __fsub_rn(c.y, __shfl_down_sync(ALL, c.x, 1)));
+}
+__device__ __forceinline__ float2 vplus_right(float2 a, float2 c) {   // a + right of c
+    return make_float2(__fadd_rn(a.x, c.y), __fadd_rn(a.y, __shfl_down_sync(ALL, c.x, 1)));
+}
+__device__ __forceinline__ Sides<float> vsides(float c) {
+    const float l = __shfl_up_sync(ALL, c, 1), r = __shfl_down_sync(ALL, c, 1);
+    return {vadd(r, l), vsub(r, l)};
+}
+__device__ __forceinline__ float vless_left(float c) { return vsub(c, __shfl_up_sync(ALL, c, 1)); }
+__device__ __forceinline__ float vless_right(float c) { return vsub(c, __shfl_down_sync(ALL, c, 1)); }
+__device__ __forceinline__ float vplus_right(float a, float c) { return vadd(a, __shfl_down_sync(ALL, c, 1)); }
+
+// columns of a lane: count, value of each, a pair of values
+template <typename V>
+struct Lane {
+    using T = V;
+    static constexpr int N = 1;
+    __device__ static __forceinline__ V make(T a, T) { return a; }
+    __device__ static __forceinline__ T first(V v) { return v; }
+    __device__ static __forceinline__ T second(V v) { return v; }
+};
+template <>
+struct Lane<float2> {
+    using T = float;
+    static constexpr int N = 2;
+    __device__ static __forceinline__ float2 make(float a, float b) { return make_float2(a, b); }
+    __device__ static __forceinline__ float first(float2 v) { return v.x; }
+    __device__ static __forceinline__ float second(float2 v) { return v.y; }
+};
+
+// 1 / sqrt(g) for g well inside the normal range
+__device__ __forceinline__ float rsqrt_n(float g) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(g));
+    return r;
+}
+// 1 / sqrt(g), and 0 for g <= lim
+__device__ __forceinline__ float vnorm(float g, float lim) { return g > lim ? rsqrt_n(g) : 0.0f; }
+__device__ __forceinline__ float2 vnorm(float2 g, float lim) { return make_float2(vnorm(g.x, lim), vnorm(g.y, lim)); }
+
+// a + b rounded stochastically (add_sr): the neighbour n of the rounded sum s on the side of
+// the remainder e is taken with probability |e| / |n - s|; f: a uniform number in [1, 2)
+// of 23 bits, half a bit of which is added
+__device__ __forceinline__ float sr_next(float v, float r) {   // one step away from or toward zero
+    return __int_as_float(__float_as_int(v) + (((__float_as_int(v) ^ __float_as_int(r)) >> 31) | 1));
+}
+__device__ __forceinline__ float sr_uniform(uint32_t bits) { return __uint_as_float((bits >> 9) | 0x3f800000u); }
+__device__ __forceinline__ float vadd_sr(float a, float b, uint32_t cell, uint32_t seed) {
+    const float s = vadd(a, b), bb = vsub(s, a), e = vadd(vsub(a, vsub(s, bb)), vsub(b, bb));
+    const float n = sr_next(s, e), t = vmul(vadd(sr_uniform(mix32(cell ^ seed)), -0.99999994f), vsub(n, s));
+    return fabsf(t) < fabsf(e) ? n : s;
+}
+__device__ __forceinline__ float2 vadd_sr(float2 a, float2 b, uint32_t cell, uint32_t seed) {
+    const float2 s = vadd(a, b), bb = vsub(s, a), e = vadd(vsub(a, vsub(s, bb)), vsub(b, bb));
+    const float2 n = make_float2(sr_next(s.x, e.x), sr_next(s.y, e.y));
+    const float2 f = make_float2(sr_uniform(mix32(cell ^ seed)), sr_uniform(mix32((cell + 1u) ^ seed)));
+    const float2 t = vmul(vadd(f, -0.99999994f), vsub(n, s));
+    return make_float2(fabsf(t.x) < fabsf(e.x) ? n.x : s.x, fabsf(t.y) < fabsf(e.y) ? n.y : s.y);
+}
+
+// ---- per-lane asynchronous copies ------------------------------------------------
+template <int BYTES>
+__device__ __forceinline__ void cp_async(uint32_t dst, const void *src) {
+    static_assert(BYTES == 4 || BYTES == 8, "copy size");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst), "l"(src), "n"(BYTES) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// sin and cos of pi x
+__device__ __forceinline__ void sincospi_(float x, float &s, float &c) { sincospif(x, &s, &c); }
+
+template <typename T>
+struct alignas(16) Row4 { T x, y, z, w; };
+
+// Geometry of a warp: 32 lanes x N columns; bar f^+ is valid on all of them, the expansions
+// on all but the outer ones, and the cells but two columns from each edge are written: 60
+// columns of 64, or 28 of 32. A strip of pairs starts at an odd column, x = 60 bx - 3 (lanes
+// 1 to 30 are written, columns 60 bx - 1 to 60 bx + 58): with the ghost border of 5 a pair
+// then lies on an 8-byte boundary of the plane (4 bytes in FP16 storage).
+template <typename V, typename ST>
+struct MarchTile {
+    using T = typename Lane<V>::T;
+    static constexpr int N = Lane<V>::N;
+    static constexpr int TX = 32 * N - 4;                  // columns written
+    static constexpr int HX = N == 2 ? 3 : 2;              // columns before the strip's tile
+    static constexpr int LO = N == 2 ? 1 : 2, HI = N == 2 ? 30 : 29;   // lanes that write
+    static constexpr int DEPTH = 3;                        // rows in the ring
+    static constexpr int XB = N * (int)sizeof(ST);         // bytes of a lane's columns of the state
+    static constexpr int PB = N * (int)sizeof(T);          // ... of phi
+    static constexpr int oPo = 9 * 32 * XB;                // phi of the older level
+    static constexpr int oP = oPo + 32 * PB;               // phi, one row ahead: columns -1 .. 32 N
+    static constexpr int P0 = N;                           // index of column 0 there (aligned pairs)
+    static constexpr int slot = (oP + (32 * N + P0 + N) * (int)sizeof(T) + 15) / 16 * 16;
+    static constexpr int oRow = DEPTH * slot;              // velocity factors of the segment's rows
+    static constexpr int rows_extra = 4;                   // rows a segment reads past its own
+    static constexpr int strips(int nx) { return (nx + (N == 2 ? 1 : 0) + TX - 1) / TX; }
+    static constexpr int smem_bytes(int rows) { return oRow + (rows + rows_extra) * (int)sizeof(Row4<T>); }
+};
+static_assert(GHOST >= 5, "strips read 3 columns and rows past the grid");
+
+// What a new row j gives: the flux differences Dbar_k of row j - 1 (k = 1 .. 8) without
+// the part of row j's own cells, that part (late: Dbar_k - late_k is complete; upwind: of
+// the south faces, k = 6, 7, 8; central: of the diagonals), the sum of the late parts, and
+// the contributions of row j - 1 to the face moments phi_b of its four faces.
+template <typename V>
+struct RowOut {
+    V D1, D2, D3, D4, D5, D6, D7, D8;
+    V l2, l4, l6, l7, l8, ls;
+    V PE, PW, PN, PS;
+};
+
+using PlusOne = std::integral_constant<int, 1>;
+using MinusOne = std::integral_constant<int, -1>;
+
+// The expansions of the rows in flight.
+template <typename V, int FLUX>
+struct March;
+
+// Upwind faces (Eq. (26)). D_x, e, m below: (R - L) / 2, L - 2 C + R and (L + 4 C + R) / 6 of
+// a row; the lattice-moment stencils are their products in the two directions, e.g.
+// d/dx = (1 4 1)/6 (over rows) of D_x.
+template <typename V>
+struct March<V, 0> {
+    using T = typename Lane<V>::T;
+    // pending expansions: "a" of row j - 1 (waits for row j), "b" of row j (has row j - 1)
+    V e2a, e2b, e8a, e8b, w4a, w4b, w6a, w6b, n2a, n2b, n4a, n4b, s6a, s6b, s8a, s8b;
+    V z1, q1, z5, q5, z3, m3p, z7, m7p, zA, vAp, zB, vBp, zN, gNp, qN1, qN2;
+    V t3p, n2p, n4p;   // north-face values of row j - 2
+
+    __device__ __forceinline__ void clear(V z) {
+        e2a = e2b = e8a = e8b = w4a = w4b = w6a = w6b = n2a = n2b = n4a = n4b = s6a = s6b = s8a = s8b = z;
+        z1 = q1 = z5 = q5 = z3 = m3p = z7 = m7p = zA = vAp = zB = vBp = zN = gNp = qN1 = qN2 = z;
+        t3p = n2p = n4p = z;
+    }
+
+    __device__ __forceinline__ void advance(const MarchCoefs<T> &cf, V F0, V F1, V F2, V F3, V F4, V F5, V F6, V F7,
+                                            V F8, RowOut<V> &o) {
+        // a diagonal direction (SX, SY): the expansions towards its two faces (row b of the
+        // canonical stencil is row SY b here, and R - L changes sign with SX)
+        auto diag = [&](V C, auto sx, auto sy, V &xa, V &xb, V &ya, V &yb, V &ox, V &oy) {
+            constexpr int SX = decltype(sx)::value, SY = decltype(sy)::value;
+            constexpr T sx1 = T(SX);
+            const Sides<V> q = vsides(C);
+            const V s = q.s, d = q.d;
+            ox = vfma(sx1 * cf.dx[1 + SY][2], d, vfma(cf.dx[1 + SY][1], s, vfma(cf.dx[1 + SY][0], C, xa)));
+            xa = vfma(sx1 * cf.dx[1][2], d, vfma(cf.dx[1][1], s, vfma(cf.dx[1][0], C, xb)));
+            xb = vfma(sx1 * cf.dx[1 - SY][2], d, vfma(cf.dx[1 - SY][1], s, vmul(cf.dx[1 - SY][0], C)));
+            oy = vfma(sx1 * cf.dy[1 + SY][2], d, vfma(cf.dy[1 + SY][1], s, vfma(cf.dy[1 + SY][0], C, ya)));
+            ya = vfma(sx1 * cf.dy[1][2], d, vfma(cf.dy[1][1], s, vfma(cf.dy[1][0], C, yb)));
+            yb = vfma(sx1 * cf.dy[1 - SY][2], d, vfma(cf.dy[1 - SY][1], s, vmul(cf.dy[1 - SY][0], C)));
+        };
+        V E2, E8, W4, W6, N2, N4;
+        diag(F2, PlusOne{}, PlusOne{}, e2a, e2b, n2a, n2b, E2, N2);
+        diag(F8, PlusOne{}, MinusOne{}, e8a, e8b, s8a, s8b, E8, o.l8);
+        diag(F4, MinusOne{}, PlusOne{}, w4a, w4b, n4a, n4b, W4, N4);
+        diag(F6, MinusOne{}, MinusOne{}, w6a, w6b, s6a, s6b, W6, o.l6);
+        // directions along an axis, and the ties
+        const Sides<V> q0 = vsides(F0), q1s = vsides(F1), q5s = vsides(F5), q3 = vsides(F3), q7 = vsides(F7);
+        const V s0 = q0.s, d0 = q0.d, s1 = q1s.s, d1 = q1s.d, s5 = q5s.s, d5 = q5s.d;
+        const V s3 = q3.s, d3 = q3.d, s7 = q7.s, d7 = q7.d;
+        // east face of k = 1, west face of k = 5
+        const V e1 = vfma(T(-2), F1, s1), e5 = vfma(T(-2), F5, s5);
+        V q = vfma(cf.px, d1, vmul(cf.pe, e1));
+        const V T1 = vadd(z1, q);
+        z1 = vadd(vfma(T(4), q, F1), q1);
+        q1 = q;
+        q = vfma(-cf.px, d5, vmul(cf.pe, e5));
+        const V T5 = vadd(z5, q);
+        z5 = vadd(vfma(T(4), q, F5), q5);
+        q5 = q;
+        // north face of k = 3, south face of k = 7
+        const V m3 = vfma(T(4), F3, s3), m7 = vfma(T(4), F7, s7);
+        const V T3 = vfma(cf.nu, m3, z3);
+        z3 = vfma(cf.nd, m3p, vfma(cf.nm, m3, F3));
+        m3p = m3;
+        o.l7 = vfma(cf.nd, m7, z7);
+        z7 = vfma(cf.nu, m7p, vfma(cf.nm, m7, F7));
+        m7p = m7;
+        // k = 0, 3, 7 at the east and west faces (weight 1/2 each): A even and B odd in x
+        V A, B;
+        {
+            const V S = vadd(F0, vadd(F3, F7)), sS = vadd(s0, vadd(s3, s7));
+            const V dS = vadd(d0, vadd(d3, d7)), dD = vsub(d7, d3);
+            const V mP = vadd(m3, m7), mD = vsub(m7, m3);
+            const V G = vfma(cf.ge, vfma(T(-2), S, sS), vmul(cf.gp, mP));
+            A = vadd(zA, vfma(cf.gd, mD, G));
+            zA = vadd(vfma(T(0.5), S, vfma(T(4), G, vmul(T(-6) * cf.gp, mP))), vAp);
+            vAp = vfma(-cf.gd, mD, G);
+            const V u = vmul(T(1.0 / 48.0), dS);
+            B = vadd(zB, vfma(cf.b2, dD, u));
+            zB = vfma(T(4), u, vBp);
+            vBp = vfma(-cf.b2, dD, u);
+        }
+        o.PE = vadd(vadd(T1, vadd(E2, E8)), vadd(A, B));
+        o.PW = vadd(vadd(T5, vadd(W4, W6)), vsub(A, B));
+        // k = 0, 1, 5 at the north and south faces
+        {
+            const V S = vadd(F0, vadd(F1, F5)), mS = vfma(T(4), S, vadd(s0, vadd(s1, s5)));
+            const V dD = vsub(d5, d1), eP = vadd(e1, e5);
+            const V G = vfma(cf.gd, dD, vfma(cf.gp, eP, vmul(cf.ge, mS)));
+            A = vadd(zN, G);
+            zN = vadd(vfma(T(0.5), S, vfma(T(4), G, vmul(T(-6) * cf.ge, mS))), gNp);
+            gNp = G;
+            const V Q = vfma(T(1.0 / 48.0), mS, vmul(cf.b2, dD));
+            B = vsub(Q, qN2);
+            qN2 = qN1;
+            qN1 = Q;
+        }
+        o.ls = vadd(o.l7, vadd(o.l6, o.l8));
+        o.PN = vadd(vadd(T3, vadd(N2, N4)), vadd(A, B));
+        o.PS = vadd(o.ls, vsub(A, B));
+        // Dbar_k = xi_x (f_E(c) - f_E(c - E)) + xi_y (f_N(c) - f_N(c - N))
+        o.D1 = vless_left(T1);
+        o.D5 = vless_right(T5);
+        o.D2 = vadd(vless_left(E2), vsub(N2, n2p));
+        o.D4 = vadd(vless_right(W4), vsub(N4, n4p));
+        o.D3 = vsub(T3, t3p);
+        o.D6 = vadd(vless_right(W6), o.l6);
+        o.D7 = o.l7;
+        o.D8 = vadd(vless_left(E8), o.l8);
+        n2p = N2;
+        n4p = N4;
+        t3p = T3;
+    }
+};
+
+// Central faces (Eq. (25)): f_E = (F_c + F_E) / 2 - h [xi_x (F_E - F_c) + xi_y (gy_c + gy_E) / 2] and
+// likewise north. Their differences over a cell are, per direction,
+//   xi_x (R - L) / 2 - h xi_x^2 (L - 2 C + R), the same over rows, and for a diagonal
+//   - h xi_x xi_y / 2 [gy(c + E) - gy(c - E) + gx(c + N) - gx(c - N)],
+// and their sums over k need the gradients of sum_k xi_y F_k and sum_k xi_x F_k only.
+template <typename V>
+struct March<V, 1> {
+    using T = typename Lane<V>::T;
+    struct Diag {
+        V z, c1, m1, m2, zg, d1, gp;   // pending sum and C, m of rows j - 1, j - 2, gx pending, d, 12 gx of row j - 2
+    } a2, a4, a6, a8;
+    V q1, q5, z3, c3, z7, c7;          // row j - 1 (k = 1, 5); pending sums and C of row j - 1 (k = 3, 7)
+    V M0p, Mxp, Myp, my1, my2, zx, dx1;
+
+    __device__ __forceinline__ void clear(V z) {
+        a2 = a4 = a6 = a8 = Diag{z, z, z, z, z, z, z};
+        q1 = q5 = z3 = c3 = z7 = c7 = M0p = Mxp = Myp = my1 = my2 = zx = dx1 = z;
+    }
+
+    __device__ __forceinline__ void advance(const MarchCoefs<T> &cf, V F0, V F1, V F2, V F3, V F4, V F5, V F6, V F7,
+                                            V F8, RowOut<V> &o) {
+        const T h = cf.h, hk = cf.hk, cp = cf.cp, cm = cf.cm;
+        auto diag = [&](Diag &g, V C, auto sx, auto sy, V &D, V &late) {
+            constexpr int SX = decltype(sx)::value, SY = decltype(sy)::value;
+            const Sides<V> q = vsides(C);
+            const V s = q.s, d = q.d;
+            const V m = vfma(T(4), C, s);
+            const V gy = vsub(m, g.m2);            // 12 gy of row j - 1
+            const V gx = vadd(g.zg, d);            // 12 gx of row j - 1
+            const V dg = vsides(gy).d;
+            const T k = T(SX * SY) * hk;
+            D = vfma(-k, vsub(dg, g.gp), vfma(SY > 0 ? cp : cm, C, g.z));
+            late = vmul(k, gx);
+            g.z = vfma(SY > 0 ? cm : cp, g.c1, vfma(T(0.5 * SX), d, vfma(-h, s, vmul(T(4) * h, C))));
+            g.c1 = C;
+            g.m2 = g.m1;
+            g.m1 = m;
+            g.zg = vfma(T(4), d, g.d1);
+            g.d1 = d;
+            g.gp = gx;
+        };
+        diag(a2, F2, PlusOne{}, PlusOne{}, o.D2, o.l2);
+        diag(a4, F4, MinusOne{}, PlusOne{}, o.D4, o.l4);
+        diag(a6, F6, MinusOne{}, MinusOne{}, o.D6, o.l6);
+        diag(a8, F8, PlusOne{}, MinusOne{}, o.D8, o.l8);
+        o.l7 = V{};
+        o.ls = vadd(vadd(o.l2, o.l4), vadd(o.l6, o.l8));
+        o.D1 = q1;
+        o.D5 = q5;
+        const Sides<V> h1 = vsides(F1), h5 = vsides(F5);
+        q1 = vfma(T(0.5), h1.d, vfma(-h, h1.s, vmul(T(2) * h, F1)));
+        q5 = vfma(T(-0.5), h5.d, vfma(-h, h5.s, vmul(T(2) * h, F5)));
+        o.D3 = vfma(cp, F3, z3);
+        z3 = vfma(cm, c3, vmul(T(2) * h, F3));
+        c3 = F3;
+        o.D7 = vfma(cm, F7, z7);
+        z7 = vfma(cp, c7, vmul(T(2) * h, F7));
+        c7 = F7;
+        const V e = vadd(F2, F8), w = vadd(F4, F6), n = vadd(F2, F4), u = vadd(F6, F8);
+        const V M0 = vadd(vadd(F0, vadd(F1, F5)), vadd(vadd(F3, F7), vadd(e, w)));
+        const V Mx = vadd(vsub(F1, F5), vsub(e, w)), My = vadd(vsub(F3, F7), vsub(n, u));
+        const V my = vfma(T(4), My, vsides(My).s);
+        const V dx = vsides(Mx).d;
+        const V bx = vfma(T(0.5), M0p, vmul(-hk, vsub(my, my2))), by = vfma(T(0.5), M0p, vmul(-hk, vadd(zx, dx)));
+        o.PE = vfma(h, Mxp, bx);
+        o.PW = vfma(-h, Mxp, bx);
+        o.PN = vfma(h, Myp, by);
+        o.PS = vfma(-h, Myp, by);
+        my2 = my1;
+        my1 = my;
+        zx = vfma(T(4), dx, dx1);
+        dx1 = dx;
+        M0p = M0;
+        Mxp = Mx;
+        Myp = My;
+    }
+};
+
+// One strip (rows y0 .. y0 + rows - 1) of one grid. FIELD: the velocity is given at cell
+// centres (p.ufield, p.vfield).
+template <typename V, typename ST, int FLUX, bool FIELD>
+__device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T> &p,
+                                            const MarchCoefs<typename Lane<V>::T> &cf,
+                                            const FastExtra<typename Lane<V>::T> &fe, int bx, int y0, int rows,
+                                            double *mass_out, unsigned char *smem) {
+    using T = typename Lane<V>::T;
+    using LN = Lane<V>;
+    using MT = MarchTile<V, ST>;
+    constexpr bool DEV = Store<T, ST>::deviation;
+    static_assert(Store<T, ST>::phi_plane, "phi is a plane of its own");
+    static_assert(!DEV || LN::N == 2, "half-precision values travel as pairs");
+    constexpr int XB = MT::XB, PB = MT::PB, DEPTH = MT::DEPTH, N = LN::N;
+    const int lane = threadIdx.x & 31;
+    const int nx = p.nx, ny = p.ny;
+    const int x = MT::TX * bx - MT::HX + N * lane;   // the lane's first column
+    // element offset of the lane's columns in a row; lanes past the ghost border read padding
+    const int col = min(x + GHOST, p.pitch - N);
+    const bool wr = lane >= MT::LO && lane <= MT::HI;
+    const bool ok0 = wr && x >= 0 && x < nx, ok1 = N == 2 && wr && x + 1 >= 0 && x + 1 < nx;
+    const int npk = rows + MT::rows_extra;
+
+    // ---- velocity: every prescribed kind but the cell field is a product of a column
+    // and a row factor, u = cu(x) ru(y), v = cv(x) rv(y) (times the reversal factor)
+    Row4<T> *sRow = reinterpret_cast<Row4<T> *>(smem + MT::oRow);
+    const bool reversing = p.vel_kind == VEL_VORTEX || p.vel_kind == VEL_DEFORM;
+    const T vct = reversing ? fe.vc_t : T(1), vco = reversing ? fe.vc_told : T(1), vcf = reversing ? fe.vc_tface : T(1);
+    const T gc2 = p.ga1 * p.c2, hg3 = T(0.5) * p.ga1 * p.c3;
+    const T f3 = T(3) * gc2;               // (face velocities carry 3 gamma c2)
+    V cu{}, cv{}, cuE{}, cvE{};            // column factors at the centres and east faces
+    if constexpr (!FIELD) {
+        // one sine and cosine serve both factors at an abscissa (ordinate) s:
+        // vortex sin^2(pi s / L), sin(2 pi s / L); deformation sin, cos(4 pi s / L)
+        auto waves = [&](T s, T &a, T &b) {
+            T sn, cs;
+            sincospi_((p.vel_kind == VEL_DEFORM ? T(4) * s : s) / p.vp0, sn, cs);
+            const bool def = p.vel_kind == VEL_DEFORM;
+            a = def ? sn : sn * sn;
+            b = def ? cs : T(2) * sn * cs;
+        };
+        auto col_factor = [&](T s, T &a, T &b) {
+            if (reversing) {
+                waves(s, a, b);
+                a *= -p.vp1;
+                b *= p.vel_kind == VEL_DEFORM ? -p.vp1 : p.vp1;
+            } else {
+                a = p.vel_kind == VEL_UNIFORM ? p.vp0 : T(1);
+                b = p.vel_kind == VEL_UNIFORM ? p.vp1 : p.vp2 * (s - p.vp0);
+            }
+        };
+        const T g0 = T(wrap_small(x, nx)), g1 = T(wrap_small(x + 1, nx)), ff = vcf * f3;
+        T a0, b0, a1 = T(0), b1 = T(0);
+        col_factor(g0 + T(0.5), a0, b0);
+        if (N == 2) col_factor(g1 + T(0.5), a1, b1);
+        cu = LN::make(a0, a1);
+        cv = LN::make(b0, b1);
+        col_factor(g0 + T(1), a0, b0);
+        if (N == 2) col_factor(g1 + T(1), a1, b1);
+        cuE = LN::make(a0 * ff, a1 * ff);
+        cvE = LN::make(b0 * ff, b1 * ff);
+        for (int i = lane; i < npk; i += 32) {
+            const T g = T(wrap_small(y0 - 2 + i, ny));
+            Row4<T> r;
+            if (reversing) {   // (vortex: u takes sin(2 pi y / L), v sin^2(pi y / L))
+                T a, b;
+                waves(g + T(0.5), a, b);
+                r.x = p.vel_kind == VEL_DEFORM ? a : b;
+                r.y = p.vel_kind == VEL_DEFORM ? b : a;
+                waves(g + T(1), a, b);
+                r.z = p.vel_kind == VEL_DEFORM ? a : b;
+                r.w = p.vel_kind == VEL_DEFORM ? b : a;
+            } else {
+                r.x = p.vel_kind == VEL_UNIFORM ? T(1) : -p.vp2 * (g + T(0.5) - p.vp1);
+                r.z = p.vel_kind == VEL_UNIFORM ? T(1) : -p.vp2 * (g + T(1) - p.vp1);
+                r.y = r.w = T(1);
+            }
+            r.z *= ff;
+            r.w *= ff;
+            sRow[i] = r;
+        }
+    }
+    pdl_wait();   // the previous kernel's output (launched with programmatic serialization)
+
+    // ---- copies: packet i holds the state and phi_old of row y0 - 2 + i and phi of the row above
+    const uint32_t ring = smem_u32(smem);
+    const size_t row0 = (size_t)(y0 - 2 + GHOST) * p.pitch;
+    const ST *gX = static_cast<const ST *>(p.X) + row0 + col;
+    const T *gPo = p.phi_old + row0 + col;
+    const T *gP = p.phi_cur + row0 + p.pitch + col;
+    // lane 0 also fetches the column before the strip, lane 31 the one after it
+    const int hcol = lane == 0 ? max(x + GHOST - 1, 0) : min(x + N + GHOST, p.pitch - 1);
+    const T *gH = p.phi_cur + row0 + p.pitch + hcol;
+    const bool halo = lane == 0 || lane == 31;
+    const uint32_t hdst = MT::oP + (lane == 0 ? MT::P0 - 1 : MT::P0 + 32 * N) * (int)sizeof(T);
+    const size_t plane = p.plane;
+    int fetched = 0;
+    uint32_t fslot = 0;   // byte offset of the slot the next packet goes to
+    auto fetch = [&]() {
+        if (fetched < npk) {
+            const uint32_t s = ring + fslot;
+#pragma unroll
+            for (int k = 0; k < 9; k++) cp_async<XB>(s + k * 32 * XB + lane * XB, gX + k * plane);
+            cp_async<PB>(s + MT::oPo + lane * PB, gPo);
+            cp_async<PB>(s + MT::oP + (MT::P0 + N * lane) * (int)sizeof(T), gP);
+            if (halo) cp_async<(int)sizeof(T)>(s + hdst, gH);
+            gX += p.pitch;
+            gPo += p.pitch;
+            gP += p.pitch;
+            gH += p.pitch;
+            fetched++;
+            fslot = fslot + MT::slot == DEPTH * MT::slot ? 0 : fslot + MT::slot;
+        }
+        cp_commit();   // (an empty group at the end keeps the count of groups in step)
+    };
+#pragma unroll
+    for (int i = 0; i < DEPTH - 1; i++) fetch();
+
+    // FIELD: the cell field is read from its planes a row at a time (rows j, j - 1, j - 2)
+    const T *gU = nullptr, *gW = nullptr;
+    V fu0{}, fv0{}, fu1{}, fv1{}, fu2{}, fv2{};
+    if constexpr (FIELD) {
+        gU = p.ufield + row0 + col;
+        gW = p.vfield + row0 + col;
+    }
+    // V = theta n + 3 d(phi u)/dt: the second term is u_spatial (phi vD + phi_old vDo)
+    const T vD = p.useD ? T(3) * p.inv_dtD * vct : T(0), vDo = p.useD ? T(-3) * p.inv_dtD * vco : T(0);
+    const T v3 = T(3) * vct;
+
+    // ---- rows below the first packet: phi of rows y0 - 3 and y0 - 2
+    V pc1, pc2{}, pc3{};           // phi of rows j, j - 1, j - 2
+    V pd1, pm1, pm0, pz;           // gradient rows: R - L, L + 4 C + R; 4 d(j) + d(j - 1)
+    {
+        const T *q = p.phi_cur + row0 - p.pitch + col;
+        const int lo = x + GHOST - 1 < 0 ? 0 : -1, hi = col + N < p.pitch ? N : N - 1;
+        const V a = *reinterpret_cast<const V *>(q), b = *reinterpret_cast<const V *>(q + p.pitch);
+        auto row = [&](V c, T l, T r, V &d, V &m) {
+            if constexpr (N == 2) {
+                d = LN::make(LN::second(c) - l, r - LN::first(c));
+                m = vfma(T(4), c, LN::make(LN::second(c) + l, r + LN::first(c)));
+            } else {
+                d = r - l;
+                m = vfma(T(4), c, r + l);
+            }
+        };
+        V d0;
+        row(a, q[lo], q[hi], d0, pm0);
+        row(b, q[p.pitch + lo], q[p.pitch + hi], pd1, pm1);
+        pz = vfma(T(4), pd1, d0);
+        pc1 = b;
+    }
+    const T gmc = p.ga1 * (T(1) - p.c2);
+    March<V, FLUX> mx;
+    mx.clear(V{});
+    // rows in flight: X + be (g - X) of row j - 1; the same less the flux of row j - 2
+    V b1{}, b2{}, b3{}, b4{}, b5{}, b6{}, b7{}, b8{};
+    V r1{}, r2{}, r3{}, r4{}, r5{}, r6{}, r7{}, r8{};
+    V sDp{}, phEp{}, pNp{};            // row j - 2: flux sum, phi_b east, own part of phi_b north
+    V v0x{}, v0y{}, v1x{}, v1y{};      // V of rows j - 1, j - 2
+    V f0p{}, f1p{}, f2p{};             // north-face moments of row j - 3
+    double msum = 0.0;
+    uint32_t cslot = 0;
+    const uint32_t seed = mix32(p.seed);
+    // lanes whose columns have images in the ghost border left or right of the grid
+    const bool xedge = x < GHOST || x + N - 1 >= nx - GHOST;
+
+    __syncwarp();
+#pragma unroll 2
+    for (int it = 0; it < npk; it++) {
+        cp_wait<DEPTH - 2>();
+        __syncwarp();
+        fetch();
+        const unsigned char *sl = smem + cslot;
+        cslot = cslot + MT::slot == DEPTH * MT::slot ? 0 : cslot + MT::slot;
+
+        // ---- phi of the row above, gradient and cell quantities of row j ------------
+        const T *sP = reinterpret_cast<const T *>(sl + MT::oP) + MT::P0 + N * lane;
+        const V pc0 = *reinterpret_cast<const V *>(sP);
+        const T pl = sP[-1], pr = sP[N];
+        V pd0, pmn;
+        if constexpr (N == 2) {
+            pd0 = LN::make(__fsub_rn(LN::second(pc0), pl), __fsub_rn(pr, LN::first(pc0)));
+            pmn = vfma(T(4), pc0, LN::make(__fadd_rn(LN::second(pc0), pl), __fadd_rn(pr, LN::first(pc0))));
+        } else {
+            pd0 = vsub(pr, pl);
+            pmn = vfma(T(4), pc0, vadd(pr, pl));
+        }
+        const V gx = vadd(pz, pd0), gy = vsub(pmn, pm0);   // 12 grad phi
+        pz = vfma(T(4), pd0, pd1);
+        pd1 = pd0;
+        pm0 = pm1;
+        pm1 = pmn;
+        const V ph = pc1;
+        V Vx, Vy, Px, Py;
+        {
+            // n = grad phi / |grad phi|; 0 where |grad phi|^2 <= 1e-24 (Eq. (2))
+            V inv = vnorm(vfma(gx, gx, vmul(gy, gy)), T(144e-24));
+            inv = vmul(inv, vmul(vmul(p.theta_c, vadd(ph, -p.phiA)), vadd(ph, -p.phiB)));   // theta of Eq. (4)
+            const V po = *reinterpret_cast<const V *>(sl + MT::oPo + lane * PB);
+            const V w = vfma(vD, ph, vmul(vDo, po));
+            V us, vs;
+            if constexpr (FIELD) {
+                fu2 = fu1; fv2 = fv1; fu1 = fu0; fv1 = fv0;
+                fu0 = *reinterpret_cast<const V *>(gU);
+                fv0 = *reinterpret_cast<const V *>(gW);
+                gU += p.pitch;
+                gW += p.pitch;
+                us = fu0;
+                vs = fv0;
+            } else {
+                const Row4<T> rf = sRow[it];
+                us = vmul(rf.x, cu);
+                vs = vmul(rf.y, cv);
+            }
+            Vx = vfma(gx, inv, vmul(us, w));             // Eq. (14b)
+            Vy = vfma(gy, inv, vmul(vs, w));
+            const V p3 = vmul(v3, ph);
+            Px = vfma(us, p3, vmul(p.tau, Vx));          // g_k = w_k (phi + xi_k . P)
+            Py = vfma(vs, p3, vmul(p.tau, Vy));
+        }
+
+        // ---- bar f^+_k = X + b (g - X) and X + be (g - X) of row j -------------------
+        V F0, F1, F2, F3, F4, F5, F6, F7, F8;
+        V nb1, nb2, nb3, nb4, nb5, nb6, nb7, nb8;
+        {
+            auto cell = [&](int k, V g, V &F) -> V {     // returns X + be (g - X)
+                const T wk = wq<T>(k);
+                const unsigned char *q = sl + k * 32 * XB + lane * XB;
+                V X, t;
+                if constexpr (DEV) {
+                    X = vfma(p.qinv, __half22float2(*reinterpret_cast<const __half2 *>(q)), ph);
+                    t = vmul(wk, vsub(g, X));
+                    X = vmul(wk, X);
+                } else {
+                    X = *reinterpret_cast<const V *>(q);
+                    t = vfma(wk, g, vneg(X));
+                }
+                F = vfma(p.b, t, X);
+                return vfma(p.be1, t, X);
+            };
+            const V gp = vadd(ph, Px), gm = vsub(ph, Px);
+            cell(0, ph, F0);
+            nb1 = cell(1, gp, F1);
+            nb2 = cell(2, vadd(gp, Py), F2);
+            nb3 = cell(3, vadd(ph, Py), F3);
+            nb4 = cell(4, vadd(gm, Py), F4);
+            nb5 = cell(5, gm, F5);
+            nb6 = cell(6, vsub(gm, Py), F6);
+            nb7 = cell(7, vsub(ph, Py), F7);
+            nb8 = cell(8, vsub(gp, Py), F8);
+        }
+
+        // ---- expansions: row j completes row j - 1 -----------------------------------
+        RowOut<V> ro;
+        mx.advance(cf, F0, F1, F2, F3, F4, F5, F6, F7, F8, ro);
+
+        // ---- row j - 2 is complete: faces, flux and store ----------------------------
+        // (computed in the first rows too, where nothing is stored: one straight block)
+        const V phN = vadd(pNp, ro.PS), phE = phEp;
+        // face moments: phi_b and (3 gamma c2 phi_b u_b + gamma c3 V_b) at the east and north faces
+        V uE, vE, uN, vN;
+        if constexpr (FIELD) {
+            const T hf = T(0.5) * f3;
+            uE = vmul(hf, vplus_right(fu2, fu2));
+            vE = vmul(hf, vplus_right(fv2, fv2));
+            uN = vmul(hf, vadd(fu2, fu1));
+            vN = vmul(hf, vadd(fv2, fv1));
+        } else {
+            const Row4<T> rf = sRow[max(it - 2, 0)];
+            uE = vmul(rf.x, cuE);
+            vE = vmul(rf.y, cvE);
+            uN = vmul(rf.z, cu);
+            vN = vmul(rf.w, cv);
+        }
+        const V x1 = vfma(phE, uE, vmul(hg3, vplus_right(v1x, v1x)));
+        const V x2 = vfma(phE, vE, vmul(hg3, vplus_right(v1y, v1y)));
+        const V y1 = vfma(phN, uN, vmul(hg3, vadd(v1x, v0x)));
+        const V y2 = vfma(phN, vN, vmul(hg3, vadd(v1y, v0y)));
+        const V A1 = vmul(gc2, vless_left(phE)), A2 = vmul(gc2, vsub(phN, f0p));
+        const V B1 = vless_left(x1), B2 = vadd(vless_left(x2), vsub(y1, f1p)), B3 = vsub(y2, f2p);
+        f0p = phN;
+        f1p = y1;
+        f2p = y2;
+        const int y = y0 + it - 4;
+        const V S13 = vadd(B1, B3);
+        // new phi = phi + gamma sum_k L_k (sum_k w_k xi_k = 0, sum_k w_k xi_a xi_b = delta_ab / 3)
+        const V dph = vfma(T(-1.0 / 3.0), S13, vmul(-gmc, vsub(sDp, ro.ls)));
+        const V phn = vadd_sr(pc3, dph, (uint32_t)y * (uint32_t)nx + (uint32_t)x, seed);
+        V o[9];
+        {
+            // gamma w_k (c2 Phi_k + c3 Psi_k) = w_k (xi_x A1 + xi_y A2 + xi_x^2 B1 + xi_x xi_y B2 + xi_y^2 B3)
+            const T w1 = wq<T>(1), w2 = wq<T>(2);
+            // (the late parts of Dbar)
+            const V p7 = FLUX == 0 ? vfma(gmc, ro.l7, r7) : r7;
+            const V p6 = vfma(gmc, ro.l6, r6), p8 = vfma(gmc, ro.l8, r8);
+            const V p2 = FLUX == 0 ? r2 : vfma(gmc, ro.l2, r2), p4 = FLUX == 0 ? r4 : vfma(gmc, ro.l4, r4);
+            o[1] = vfma(-w1, vadd(B1, A1), r1);
+            o[5] = vfma(-w1, vsub(B1, A1), r5);
+            o[3] = vfma(-w1, vadd(B3, A2), r3);
+            o[7] = vfma(-w1, vsub(B3, A2), p7);
+            const V sp = vadd(S13, B2), sm = vsub(S13, B2), ap = vadd(A1, A2), am = vsub(A1, A2);
+            o[2] = vfma(-w2, vadd(sp, ap), p2);
+            o[6] = vfma(-w2, vsub(sp, ap), p6);
+            o[8] = vfma(-w2, vadd(sm, am), p8);
+            o[4] = vfma(-w2, vsub(sm, am), p4);
+            // rest component: the new phi is exactly phn (up to this subtraction)
+            o[0] = vsub(phn, vadd(vadd(vadd(o[1], o[2]), vadd(o[3], o[4])), vadd(vadd(o[5], o[6]), vadd(o[7], o[8]))));
+        }
+        // ---- row j - 1: X + be (g - X) - gamma (1 - c2) Dbar ---------------------------
+        r1 = vfma(-gmc, ro.D1, b1);
+        r2 = vfma(-gmc, ro.D2, b2);
+        r3 = vfma(-gmc, ro.D3, b3);
+        r4 = vfma(-gmc, ro.D4, b4);
+        r5 = vfma(-gmc, ro.D5, b5);
+        r6 = vfma(-gmc, ro.D6, b6);
+        r7 = vfma(-gmc, ro.D7, b7);
+        r8 = vfma(-gmc, ro.D8, b8);
+        sDp = vadd(vadd(vadd(ro.D1, ro.D2), vadd(ro.D3, ro.D4)), vadd(vadd(ro.D5, ro.D6), vadd(ro.D7, ro.D8)));
+        phEp = vplus_right(ro.PE, ro.PW);
+        pNp = ro.PN;
+        b1 = nb1; b2 = nb2; b3 = nb3; b4 = nb4; b5 = nb5; b6 = nb6; b7 = nb7; b8 = nb8;
+        v1x = v0x; v1y = v0y;
+        v0x = Vx; v0y = Vy;
+        pc3 = pc2; pc2 = pc1; pc1 = pc0;
+
+        // ---- store row j - 2 -----------------------------------------------------------
+        const bool st0 = ok0 && it >= 4, st1 = ok1 && it >= 4;
+        using OV = typename std::conditional<DEV, __half2, V>::type;
+        OV ov[9];
+        if constexpr (DEV) {
+#pragma unroll
+            for (int k = 0; k < 9; k++)
+                ov[k] = __float22half2_rn(vmul(p.qscale / wq<T>(k), vfma(-wq<T>(k), phn, o[k])));
+        } else {
+#pragma unroll
+            for (int k = 0; k < 9; k++) ov[k] = o[k];
+        }
+        ST *O = static_cast<ST *>(p.out1);
+        // one column of this lane at element offset g
+        auto put0 = [&](long long g) {
+#pragma unroll
+            for (int k = 0; k < 9; k++) {
+                if constexpr (N == 2) O[(long long)(k * plane) + g] = ov[k].x;
+                else O[(long long)(k * plane) + g] = ov[k];
+            }
+            p.phi_out[g] = LN::first(phn);
+        };
+        auto put1 = [&](long long g) {
+            if constexpr (N == 2) {
+#pragma unroll
+                for (int k = 0; k < 9; k++) O[(long long)(k * plane) + g + 1] = ov[k].y;
+                p.phi_out[g + 1] = LN::second(phn);
+            }
+        };
+        const size_t g = (size_t)(y + GHOST) * p.pitch + (size_t)(x + GHOST);
+        if (st0 && (N == 1 || st1)) {
+#pragma unroll
+            for (int k = 0; k < 9; k++) *reinterpret_cast<OV *>(O + k * plane + g) = ov[k];
+            *reinterpret_cast<V *>(p.phi_out + g) = phn;
+        } else if (st0) {
+            put0(g);
+        } else if (st1) {
+            put1(g);
+        }
+        if (st0) msum += (double)LN::first(phn);
+        if (st1) msum += (double)LN::second(phn);
+        // periodic images in the ghost border
+        if ((st0 || st1) && (xedge || y < GHOST || y >= ny - GHOST)) {
+#pragma unroll 1
+            for (int im = 0; im < 9; im++) {
+                const int ay = im / 3 - 1, ax = im - 3 * (im / 3) - 1;
+                const int yy = y + ay * ny, xx = x + ax * nx;
+                if (im == 4 || yy < -GHOST || yy >= ny + GHOST) continue;
+                const long long gi = (long long)(yy + GHOST) * p.pitch + (xx + GHOST);
+                if (st0 && xx >= -GHOST && xx < nx + GHOST) put0(gi);
+                if (st1 && xx + 1 >= -GHOST && xx + 1 < nx + GHOST) put1(gi);
+            }
+        }
+    }
+    cp_wait<0>();
+    if (mass_out != nullptr) {
+        for (int o = 16; o > 0; o >>= 1) msum += __shfl_down_sync(ALL, msum, o);
+        if (lane == 0) *mass_out = msum;
+    }
+}
+
+// One grid: blockIdx.x = strip, blockIdx.y = segment of p.tile_h rows. EARLY: dependents may
+// be scheduled at once (a grid that leaves room for them on the chip: their velocity factors
+// are ready when this grid ends).
+template <typename V, typename ST, int FLUX, bool FIELD>
+__global__ void __launch_bounds__(32, (sizeof(V) == 4 ? 12 : 8))
+step_march_kernel(const __grid_constant__ StepParams<typename Lane<V>::T> p,
+                  const __grid_constant__ MarchCoefs<typename Lane<V>::T> cf,
+                  const __grid_constant__ FastExtra<typename Lane<V>::T> fe, const int early) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    if (early) pdl_trigger();
+    const int y0 = blockIdx.y * p.tile_h;
+    march_strip<V, ST, FLUX, FIELD>(p, cf, fe, blockIdx.x, y0, min(p.tile_h, p.ny - y0),
+                                    p.mass_partial ? p.mass_partial + blockIdx.y * p.tiles_x + blockIdx.x : nullptr,
+                                    smem);
+    if (!early) pdl_trigger();
+}
+
+// Many grids: CTAs stride over the work list (grid, strip, first row, rows).
+template <typename V, typename ST, int FLUX>
+__global__ void __launch_bounds__(32, 8)
+batch_march_kernel(const __grid_constant__ BatchUniform<typename Lane<V>::T> u,
+                   const __grid_constant__ MarchCoefs<typename Lane<V>::T> cf,
+                   const BatchGrid<typename Lane<V>::T> *__restrict__ grids, const int4 *__restrict__ items, int nitems,
+                   double *__restrict__ partials) {
+    using T = typename Lane<V>::T;
+    extern __shared__ __align__(128) unsigned char smem[];
+    for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
+        const int4 w = items[it];
+        const BatchGrid<T> *G = grids + w.x;
+        if (G->step >= G->target) continue;   // frozen grid
+        StepParams<T> p;
+        FastExtra<T> fe;
+        batch_step_params<T, ST>(u, G, p, fe);
+        march_strip<V, ST, FLUX, false>(p, cf, fe, w.y, w.z, w.w, partials + it, smem);
+        __syncwarp();   // the next strip's copies overwrite the ring
+    }
+}
+
+}  // namespace dugks
