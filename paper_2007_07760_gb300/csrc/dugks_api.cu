@@ -13,7 +13,6 @@
 #include <mutex>
 #include <atomic>
 #include <string>
-#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -47,7 +46,7 @@ struct dugks_ctx {
     int tile_w = TILE_X, tile_h = TILE_Y, tiles_x = 0, ntiles = 0;
     // TMA-staged two-stage path (orders 2, 3)
     bool fast = false;
-    bool march = false;         // fast, as a row march (two-stage, orders 2-3, phi a plane of its own)
+    bool march = false;         // fast, as a row march (two-stage, orders 2 and 3)
     MarchPlan plan{};
     int variant = 0;
     CUtensorMap tmX[2], tmPhi[4];
@@ -145,14 +144,14 @@ bool encode_map(CUtensorMap *m, void *base, size_t es, bool half, const dugks_ct
 }
 
 // whether the fast path of this context is the row march
-bool marches(const dugks_ctx *c) { return c->p.stages == 2 && c->p.order <= 3 && c->p.precision != DUGKS_FP64; }
+bool marches(const dugks_ctx *c) { return c->p.stages == 2 && c->p.order <= 3; }
 
 template <typename T, typename ST>
 bool setup_fast(dugks_ctx *c) {
     if (marches(c)) {
         c->march = true;
-        c->plan = march_plan(c->variant, c->p.nx, c->p.ny, c->p.precision == DUGKS_FP16F, c->sms);
-        c->tile_w = 32 * c->plan.cols - 4;
+        c->plan = march_plan(c->variant, c->p.nx, c->p.ny, c->p.precision, c->sms);
+        c->tile_w = c->plan.width;
         c->tile_h = c->plan.rows;
         return true;
     }
@@ -277,22 +276,16 @@ int step_t2(dugks_ctx *c, double *dbg = nullptr) {
                                       vortex_factors<T>(c, t, t - dt, t + h), c->tmX[c->cur], c->tmPhi[iPo],
                                       c->tmPhi[iPc], c->p.flux, KIND_T2, c->stream);
     } else if (c->fast) {
-        // orders 2 and 3: the row march where phi is a plane of its own, else the TMA-staged kernel
-        using Coefs = typename std::conditional<Store<T, ST>::phi_plane, MarchCoefs<T>, FaceCoefs<T>>::type;
+        // orders 2 and 3: the row march
         if (c->coef_h != h) {
-            Coefs cf;
-            if constexpr (Store<T, ST>::phi_plane) cf = make_march_coefs<T>(c->p.order, h);
-            else cf = make_face_coefs<T>(c->p.order, c->p.flux, h);
-            c->coefs.assign(reinterpret_cast<const unsigned char *>(&cf), reinterpret_cast<const unsigned char *>(&cf) + sizeof cf);
+            const MarchCoefs<T> cf = make_march_coefs<T>(c->p.order, h);
+            c->coefs.assign(reinterpret_cast<const unsigned char *>(&cf),
+                            reinterpret_cast<const unsigned char *>(&cf) + sizeof cf);
             c->coef_h = h;
         }
-        const Coefs &cf = *reinterpret_cast<const Coefs *>(c->coefs.data());
-        const FastExtra<T> fx = vortex_factors<T>(c, t, t - dt, t + h);
-        if constexpr (Store<T, ST>::phi_plane)
-            e = Launch<T, ST>::step_march(q, cf, fx, c->p.flux, c->plan.cols, c->plan.early, c->stream);
-        else
-            e = Launch<T, ST>::step_fast(q, cf, fx, c->tmX[c->cur], c->tmPhi[iPo], c->tmPhi[iPc], c->p.order,
-                                         c->p.flux, c->variant, c->stream);
+        e = Launch<T, ST>::step_march(q, *reinterpret_cast<const MarchCoefs<T> *>(c->coefs.data()),
+                                      vortex_factors<T>(c, t, t - dt, t + h), c->p.flux, c->plan.cols, c->plan.early,
+                                      c->stream);
     } else {
         if (c->p.order == 5) return fail(c, DUGKS_EINVAL, "order 5 needs the TMA-staged kernels");
         e = Launch<T, ST>::step(q, c->p.order, c->p.flux, KIND_T2, c->stream);

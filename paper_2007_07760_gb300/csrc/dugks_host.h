@@ -165,11 +165,11 @@ template <typename T>
 inline MarchCoefs<T> make_march_coefs(int order, double h) {
     MarchCoefs<T> m;
     const double c = 0.5 - h, q = order >= 3 ? 1.0 : 0.0;
-    auto row = [&](double x, double y, int b, T *w) {   // C, R + L, R - L
+    auto row = [&](double x, double y, int b, T *w) {   // C, R + L, R - L; FP64: C, L, R
         const double l = taylor_w(order, x, y, -1, b), r = taylor_w(order, x, y, 1, b);
         w[0] = (T)taylor_w(order, x, y, 0, b);
-        w[1] = (T)(0.5 * (r + l));
-        w[2] = (T)(0.5 * (r - l));
+        w[1] = (T)(sizeof(T) == 8 ? l : 0.5 * (r + l));
+        w[2] = (T)(sizeof(T) == 8 ? r : 0.5 * (r - l));
     };
     for (int b = -1; b <= 1; b++) {
         row(c, -h, b, m.dx[b + 1]);
@@ -201,26 +201,38 @@ inline MarchCoefs<T> make_march_coefs(int order, double h) {
 // 11.4; 1024^2 39.0 (2, 16) against 40.8; 4096^2 356 (2, 48) against 392. Segments over
 // 64 rows lose again (4096^2, 241 rows in one wave: 478 us): the rows in flight then lie all over
 // the planes, more pages than the TLB holds.
-struct MarchPlan { int cols, strips, rows, early; };
-inline MarchPlan march_plan(int variant, int nx, int ny, bool half, int sms) {
+// FP64: the FP64 unit of each scheduler issues a warp instruction in 64 cycles whatever the
+// number of active lanes, so a step costs the rows of the busiest scheduler: the warps it gets
+// times s + 2.5 rows (the rows at a segment's ends leave out what they do not need).
+struct MarchPlan { int cols, width, strips, rows, early; };
+inline MarchPlan march_plan(int variant, int nx, int ny, int precision, int sms) {
     static constexpr int fixed[6] = {16, 8, 0, 32, 0, 64};   // variants 2 and 4: by the rule
     MarchPlan m{};
     double best = 1e300;
     const int forced = variant >= 0 && variant < 6 ? fixed[variant] : 0;
-    for (int cols = half ? 2 : 1; cols <= 2; cols++) {
-        const int strips = cols == 2 ? MarchTile<float2, float>::strips(nx) : MarchTile<float, float>::strips(nx);
+    const bool f64 = precision == DUGKS_FP64;
+    for (int cols = precision == DUGKS_FP16F ? 2 : 1; cols <= (f64 ? 1 : 2); cols++) {
+        int strips = cols == 2 ? MarchTile<float2, float>::strips(nx) : MarchTile<float, float>::strips(nx);
+        const int width = cols == 2 ? MarchTile<float2, float>::TX : (nx + strips - 1) / strips;
+        if (cols == 1) strips = (nx + width - 1) / width;
         const double slots = (cols == 2 ? 8.0 : 12.0) * sms, unit = cols == 2 ? 1.42 : 1.05;
         for (int want = forced ? forced : 1; want <= (forced ? forced : 64); want++) {
             const int segs = (ny + want - 1) / want, rows = (ny + segs - 1) / segs;   // segments of equal length
-            const double w = (double)strips * segs, W = w / slots, n = std::max(w / (4.0 * sms), 1.0);
-            const double f = W > 1.5 ? W + 0.43 : W > 1.0 ? 1.9 : cols == 2 ? 1.0 + 0.37 * (n - 1.0) : 0.89 + 0.3 * (n - 1.0);
-            const double cost = unit * (rows + 5) * f;
+            const double w = (double)strips * segs, W = w / slots, n = w / (4.0 * sms);
+            double cost;
+            if (f64) {
+                cost = (n > 3.0 ? n + 0.5 : std::ceil(n)) * (rows + 2.5);
+            } else {
+                const double p = std::max(n, 1.0) - 1.0;
+                cost = unit * (rows + 5) * (W > 1.5 ? W + 0.43 : W > 1.0 ? 1.9 : cols == 2 ? 1.0 + 0.37 * p : 0.89 + 0.3 * p);
+            }
             if (cost < best) {
                 best = cost;
                 // Early scheduling of the next kernel hides its launch and velocity factors
                 // (512^2: 15.5 against 16.5 us). On a chip half full it costs instead, because the
-                // waiting warps fill some SMs and leave others idle (256^2, 860 warps: 10.2 against 9.1).
-                m = MarchPlan{cols, strips, rows, W > 0.6 || W < 0.15};
+                // waiting warps fill some SMs and leave others idle (256^2, 860 warps: 10.2 against
+                // 9.1), and in FP64, where a scheduler with two warps takes twice as long.
+                m = MarchPlan{cols, width, strips, rows, !f64 && (W > 0.6 || W < 0.15)};
             }
         }
     }

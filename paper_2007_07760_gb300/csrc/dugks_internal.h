@@ -51,9 +51,6 @@ struct Launch {
                                    const int4 *items, int nitems, int max_rows, double *partials, int flux, int ctas,
                                    cudaStream_t s);
     static int march_ctas_per_sm(int flux, int rows);
-    static cudaError_t step_fast(const StepParams<T> &p, const FaceCoefs<T> &cf, const FastExtra<T> &fe, const CUtensorMap &tmX,
-                                 const CUtensorMap &tmPo, const CUtensorMap &tmPc, int order, int flux,
-                                 int variant, cudaStream_t s);
     // order 4 (radius-2 stencils) on the TMA-staged path, tile 8 warps x 2 rows: the
     // two-stage step (KIND_T2) or a kernel of the three-stage step (full storage only)
     static cudaError_t step_fast4(const StepParams<T> &p, const FaceCoefs<T, 2> &cf, const FastExtra<T> &fe,

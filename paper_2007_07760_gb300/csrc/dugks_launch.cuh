@@ -113,54 +113,6 @@ FastGeom Launch<T, ST>::fast_geom(int variant, int order, int stages) {
     }
 }
 
-template <typename T, typename ST, int ORDER, int FLUX, int NW, int MR>
-static cudaError_t launch_fast_t(const StepParams<T> &p, const FaceCoefs<T> &cf, const FastExtra<T> &fe, const CUtensorMap &tmX,
-                                 const CUtensorMap &tmPo, const CUtensorMap &tmPc, cudaStream_t s) {
-    using FT = FastTile<T, ST, NW, MR>;
-    auto kern = step_fast_kernel<T, ST, ORDER, FLUX, NW, MR>;
-    static std::atomic<uint64_t> configured{0};
-    if (cudaError_t e = smem_attr_once(kern, (int)FT::smem_bytes, configured); e != cudaSuccess) return e;
-    // programmatic dependent launch: scheduled while the previous kernel drains
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((p.nx + FT::TX - 1) / FT::TX, (p.ny + FT::TY - 1) / FT::TY);
-    cfg.blockDim = dim3(FT::NT);
-    cfg.dynamicSmemBytes = FT::smem_bytes;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, p, cf, fe, tmX, tmPo, tmPc);
-}
-
-template <typename T, typename ST, int ORDER, int FLUX>
-static cudaError_t launch_fast_v(const StepParams<T> &p, const FaceCoefs<T> &cf, const FastExtra<T> &fe,
-                                 const CUtensorMap &tmX, const CUtensorMap &tmPo, const CUtensorMap &tmPc, int variant,
-                                 cudaStream_t s) {
-    switch (variant) {
-    case 1: return launch_fast_t<T, ST, ORDER, FLUX, 16, 1>(p, cf, fe, tmX, tmPo, tmPc, s);
-    case 2: return launch_fast_t<T, ST, ORDER, FLUX, 8, 2>(p, cf, fe, tmX, tmPo, tmPc, s);
-    case 3: return launch_fast_t<T, ST, ORDER, FLUX, 12, 3>(p, cf, fe, tmX, tmPo, tmPc, s);
-    case 4: return launch_fast_t<T, ST, ORDER, FLUX, 8, 3>(p, cf, fe, tmX, tmPo, tmPc, s);
-    case 5: return launch_fast_t<T, ST, ORDER, FLUX, 10, 4>(p, cf, fe, tmX, tmPo, tmPc, s);
-    default: return launch_fast_t<T, ST, ORDER, FLUX, 8, fast_mr<T>()>(p, cf, fe, tmX, tmPo, tmPc, s);
-    }
-}
-
-template <typename T, typename ST>
-cudaError_t Launch<T, ST>::step_fast(const StepParams<T> &p, const FaceCoefs<T> &cf, const FastExtra<T> &fe, const CUtensorMap &tmX,
-                                     const CUtensorMap &tmPo, const CUtensorMap &tmPc, int order, int flux,
-                                     int variant, cudaStream_t s) {
-    if (order == 2)
-        return flux == 0 ? launch_fast_v<T, ST, 2, 0>(p, cf, fe, tmX, tmPo, tmPc, variant, s)
-                         : launch_fast_v<T, ST, 2, 1>(p, cf, fe, tmX, tmPo, tmPc, variant, s);
-    if (order == 3)
-        return flux == 0 ? launch_fast_v<T, ST, 3, 0>(p, cf, fe, tmX, tmPo, tmPc, variant, s)
-                         : launch_fast_v<T, ST, 3, 1>(p, cf, fe, tmX, tmPo, tmPc, variant, s);
-    return cudaErrorInvalidValue;
-}
-
 template <typename T, int ORDER, int FLUX, int KIND>
 static cudaError_t launch_fast3_t(const StepParams<T> &p, const FaceCoefs<T> &cf, const FastExtra<T> &fe,
                                   const CUtensorMap &tmX, const CUtensorMap &tmPo, const CUtensorMap &tmPc,
@@ -276,7 +228,8 @@ cudaError_t Launch<T, ST>::step_march(const StepParams<T> &p, const MarchCoefs<T
                                       int cols, int early, cudaStream_t s) {
     if constexpr (!Store<T, ST>::deviation)
         if (cols == 1) return launch_march_v<T, ST>(p, cf, fe, flux, early, s);
-    return launch_march_v<float2, ST>(p, cf, fe, flux, early, s);
+    if constexpr (sizeof(T) == 4) return launch_march_v<float2, ST>(p, cf, fe, flux, early, s);
+    return cudaErrorInvalidValue;
 }
 
 template <typename T, typename ST>

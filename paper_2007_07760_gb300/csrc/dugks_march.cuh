@@ -31,7 +31,8 @@ namespace dugks {
 // Expansion coefficients of one reconstruction time h (host: make_march_coefs).
 // Upwind, with c = 1/2 - h:
 //   dx[b + 1][.]  row b of the expansion at (c, -h), the east face of xi = (1, 1): weights of
-//                 C, R + L and R - L; dy: of the one at (-h, c), the north face. Mirrored for
+//                 C, R + L and R - L (FP64: of C, L and R, which saves the sums where every
+//                 operation counts); dy: of the one at (-h, c), the north face. Mirrored for
 //                 the other diagonals
 //   px, pe           row term px (R - L) + pe (L - 2 C + R) of the expansion at (c, 0)
 //   nu, nm, nd       weights of L + 4 C + R of the rows above, at and below at (0, c)
@@ -58,6 +59,11 @@ __device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b)
 __device__ __forceinline__ float vneg(float a) { return -a; }
 __device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double vfma(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ double vadd(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double vneg(double a) { return -a; }
+__device__ __forceinline__ double vsub(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double vmul(double a, double b) { return __dmul_rn(a, b); }
 
 // Neighbouring columns: one shuffle a value or pair each way, and sums and differences
 // taken per column (a pair built of a shuffled and an own value would cost the moves that
@@ -78,13 +84,17 @@ __device__ __forceinline__ float2 vless_right(float2 c) {   // c - right
 __device__ __forceinline__ float2 vplus_right(float2 a, float2 c) {   // a + right of c
     return make_float2(__fadd_rn(a.x, c.y), __fadd_rn(a.y, __shfl_down_sync(ALL, c.x, 1)));
 }
-__device__ __forceinline__ Sides<float> vsides(float c) {
-    const float l = __shfl_up_sync(ALL, c, 1), r = __shfl_down_sync(ALL, c, 1);
+template <typename V>
+__device__ __forceinline__ Sides<V> vsides(V c) {
+    const V l = __shfl_up_sync(ALL, c, 1), r = __shfl_down_sync(ALL, c, 1);
     return {vadd(r, l), vsub(r, l)};
 }
-__device__ __forceinline__ float vless_left(float c) { return vsub(c, __shfl_up_sync(ALL, c, 1)); }
-__device__ __forceinline__ float vless_right(float c) { return vsub(c, __shfl_down_sync(ALL, c, 1)); }
-__device__ __forceinline__ float vplus_right(float a, float c) { return vadd(a, __shfl_down_sync(ALL, c, 1)); }
+template <typename V>
+__device__ __forceinline__ V vless_left(V c) { return vsub(c, __shfl_up_sync(ALL, c, 1)); }
+template <typename V>
+__device__ __forceinline__ V vless_right(V c) { return vsub(c, __shfl_down_sync(ALL, c, 1)); }
+template <typename V>
+__device__ __forceinline__ V vplus_right(V a, V c) { return vadd(a, __shfl_down_sync(ALL, c, 1)); }
 
 // columns of a lane: count, value of each, a pair of values
 template <typename V>
@@ -112,6 +122,7 @@ __device__ __forceinline__ float rsqrt_n(float g) {
 }
 // 1 / sqrt(g), and 0 for g <= lim
 __device__ __forceinline__ float vnorm(float g, float lim) { return g > lim ? rsqrt_n(g) : 0.0f; }
+__device__ __forceinline__ double vnorm(double g, double lim) { return g > lim ? rsqrt(g) : 0.0; }
 __device__ __forceinline__ float2 vnorm(float2 g, float lim) { return make_float2(vnorm(g.x, lim), vnorm(g.y, lim)); }
 
 // a + b rounded stochastically (add_sr): the neighbour n of the rounded sum s on the side of
@@ -146,6 +157,7 @@ __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0
 
 // sin and cos of pi x
 __device__ __forceinline__ void sincospi_(float x, float &s, float &c) { sincospif(x, &s, &c); }
+__device__ __forceinline__ void sincospi_(double x, double &s, double &c) { sincospi(x, &s, &c); }
 
 template <typename T>
 struct alignas(16) Row4 { T x, y, z, w; };
@@ -159,16 +171,17 @@ template <typename V, typename ST>
 struct MarchTile {
     using T = typename Lane<V>::T;
     static constexpr int N = Lane<V>::N;
-    static constexpr int TX = 32 * N - 4;                  // columns written
-    static constexpr int HX = N == 2 ? 3 : 2;              // columns before the strip's tile
-    static constexpr int LO = N == 2 ? 1 : 2, HI = N == 2 ? 30 : 29;   // lanes that write
-    static constexpr int DEPTH = 3;                        // rows in the ring
+    static constexpr int TX = 32 * N - 4;                  // columns written (at most)
+    // phi a plane of its own, or the sum of the state (FP64)
+    static constexpr bool PHIP = Store<T, ST>::phi_plane;
+    static constexpr int DEPTH = PHIP ? 3 : 4;             // rows in the ring
     static constexpr int XB = N * (int)sizeof(ST);         // bytes of a lane's columns of the state
     static constexpr int PB = N * (int)sizeof(T);          // ... of phi
     static constexpr int oPo = 9 * 32 * XB;                // phi of the older level
     static constexpr int oP = oPo + 32 * PB;               // phi, one row ahead: columns -1 .. 32 N
     static constexpr int P0 = N;                           // index of column 0 there (aligned pairs)
-    static constexpr int slot = (oP + (32 * N + P0 + N) * (int)sizeof(T) + 15) / 16 * 16;
+    // (without phi planes: the state of the columns before and after the strip, 2 x 9 values)
+    static constexpr int slot = (oP + (PHIP ? 32 * N + P0 + N : 18) * (int)sizeof(T) + 15) / 16 * 16;
     static constexpr int oRow = DEPTH * slot;              // velocity factors of the segment's rows
     static constexpr int rows_extra = 4;                   // rows a segment reads past its own
     static constexpr int strips(int nx) { return (nx + (N == 2 ? 1 : 0) + TX - 1) / TX; }
@@ -190,6 +203,11 @@ struct RowOut {
 using PlusOne = std::integral_constant<int, 1>;
 using MinusOne = std::integral_constant<int, -1>;
 
+// What a row j has to give (uniform over the warp): finished values of row j - 1, its flux
+// differences, the middle terms of row j, the first terms of row j + 1. Only the first and
+// last rows of a segment lack one.
+struct Need { bool out, flux, mid, low; };
+
 // The expansions of the rows in flight.
 template <typename V, int FLUX>
 struct March;
@@ -201,101 +219,131 @@ template <typename V>
 struct March<V, 0> {
     using T = typename Lane<V>::T;
     // pending expansions: "a" of row j - 1 (waits for row j), "b" of row j (has row j - 1)
-    V e2a, e2b, e8a, e8b, w4a, w4b, w6a, w6b, n2a, n2b, n4a, n4b, s6a, s6b, s8a, s8b;
+    struct Diag { V xa, xb, ya, yb; } g2, g4, g6, g8;
     V z1, q1, z5, q5, z3, m3p, z7, m7p, zA, vAp, zB, vBp, zN, gNp, qN1, qN2;
     V t3p, n2p, n4p;   // north-face values of row j - 2
 
     __device__ __forceinline__ void clear(V z) {
-        e2a = e2b = e8a = e8b = w4a = w4b = w6a = w6b = n2a = n2b = n4a = n4b = s6a = s6b = s8a = s8b = z;
+        g2 = g4 = g6 = g8 = Diag{z, z, z, z};
         z1 = q1 = z5 = q5 = z3 = m3p = z7 = m7p = zA = vAp = zB = vBp = zN = gNp = qN1 = qN2 = z;
         t3p = n2p = n4p = z;
     }
 
-    __device__ __forceinline__ void advance(const MarchCoefs<T> &cf, V F0, V F1, V F2, V F3, V F4, V F5, V F6, V F7,
-                                            V F8, RowOut<V> &o) {
-        // a diagonal direction (SX, SY): the expansions towards its two faces (row b of the
-        // canonical stencil is row SY b here, and R - L changes sign with SX)
-        auto diag = [&](V C, auto sx, auto sy, V &xa, V &xb, V &ya, V &yb, V &ox, V &oy) {
-            constexpr int SX = decltype(sx)::value, SY = decltype(sy)::value;
-            constexpr T sx1 = T(SX);
+    // a diagonal's row in the basis of its weights: C, R + L, R - L, or C, L, R
+    struct Row { V c, u, v; };
+    __device__ static __forceinline__ Row row(V C) {
+        if constexpr (sizeof(T) == 8) {
+            return Row{C, __shfl_up_sync(ALL, C, 1), __shfl_down_sync(ALL, C, 1)};
+        } else {
             const Sides<V> q = vsides(C);
-            const V s = q.s, d = q.d;
-            ox = vfma(sx1 * cf.dx[1 + SY][2], d, vfma(cf.dx[1 + SY][1], s, vfma(cf.dx[1 + SY][0], C, xa)));
-            xa = vfma(sx1 * cf.dx[1][2], d, vfma(cf.dx[1][1], s, vfma(cf.dx[1][0], C, xb)));
-            xb = vfma(sx1 * cf.dx[1 - SY][2], d, vfma(cf.dx[1 - SY][1], s, vmul(cf.dx[1 - SY][0], C)));
-            oy = vfma(sx1 * cf.dy[1 + SY][2], d, vfma(cf.dy[1 + SY][1], s, vfma(cf.dy[1 + SY][0], C, ya)));
-            ya = vfma(sx1 * cf.dy[1][2], d, vfma(cf.dy[1][1], s, vfma(cf.dy[1][0], C, yb)));
-            yb = vfma(sx1 * cf.dy[1 - SY][2], d, vfma(cf.dy[1 - SY][1], s, vmul(cf.dy[1 - SY][0], C)));
-        };
-        V E2, E8, W4, W6, N2, N4;
-        diag(F2, PlusOne{}, PlusOne{}, e2a, e2b, n2a, n2b, E2, N2);
-        diag(F8, PlusOne{}, MinusOne{}, e8a, e8b, s8a, s8b, E8, o.l8);
-        diag(F4, MinusOne{}, PlusOne{}, w4a, w4b, n4a, n4b, W4, N4);
-        diag(F6, MinusOne{}, MinusOne{}, w6a, w6b, s6a, s6b, W6, o.l6);
-        // directions along an axis, and the ties
-        const Sides<V> q0 = vsides(F0), q1s = vsides(F1), q5s = vsides(F5), q3 = vsides(F3), q7 = vsides(F7);
-        const V s0 = q0.s, d0 = q0.d, s1 = q1s.s, d1 = q1s.d, s5 = q5s.s, d5 = q5s.d;
-        const V s3 = q3.s, d3 = q3.d, s7 = q7.s, d7 = q7.d;
+            return Row{C, q.s, q.d};
+        }
+    }
+    template <int SX>
+    __device__ static __forceinline__ V dot(const T (&w)[3], const Row &r, V acc) {
+        if constexpr (sizeof(T) == 8) return vfma(w[SX > 0 ? 2 : 1], r.v, vfma(w[SX > 0 ? 1 : 2], r.u, vfma(w[0], r.c, acc)));
+        else return vfma(T(SX) * w[2], r.v, vfma(w[1], r.u, vfma(w[0], r.c, acc)));
+    }
+    template <int SX>
+    __device__ static __forceinline__ V dot(const T (&w)[3], const Row &r) {
+        if constexpr (sizeof(T) == 8) return vfma(w[SX > 0 ? 2 : 1], r.v, vfma(w[SX > 0 ? 1 : 2], r.u, vmul(w[0], r.c)));
+        else return vfma(T(SX) * w[2], r.v, vfma(w[1], r.u, vmul(w[0], r.c)));
+    }
+    // a diagonal direction (SX, SY): row b of the canonical stencil is row SY b here, and R - L
+    // changes sign with SX
+    template <int SX, int SY>
+    __device__ static __forceinline__ void faces(const MarchCoefs<T> &cf, const Row &r, const Diag &g, V &ox, V &oy) {
+        ox = dot<SX>(cf.dx[1 + SY], r, g.xa);
+        oy = dot<SX>(cf.dy[1 + SY], r, g.ya);
+    }
+    // a row of a diagonal: the finished values at its two faces, and the pending sums
+    template <int SX, int SY>
+    __device__ static __forceinline__ void diagonal(const MarchCoefs<T> &cf, V C, Diag &g, V &ox, V &oy, Need n) {
+        const Row r = row(C);
+        if (n.out) faces<SX, SY>(cf, r, g, ox, oy);
+        if (n.mid) {
+            g.xa = dot<SX>(cf.dx[1], r, g.xb);
+            g.ya = dot<SX>(cf.dy[1], r, g.yb);
+        }
+        if (n.low) {
+            g.xb = dot<SX>(cf.dx[1 - SY], r);
+            g.yb = dot<SX>(cf.dy[1 - SY], r);
+        }
+    }
+
+    __device__ __forceinline__ void advance(const MarchCoefs<T> &cf, V F0, V F1, V F2, V F3, V F4, V F5, V F6, V F7,
+                                            V F8, RowOut<V> &o, Need n) {
+        V E2{}, E8{}, W4{}, W6{}, N2{}, N4{};
+        diagonal<1, 1>(cf, F2, g2, E2, N2, n);
+        diagonal<1, -1>(cf, F8, g8, E8, o.l8, n);
+        diagonal<-1, 1>(cf, F4, g4, W4, N4, n);
+        diagonal<-1, -1>(cf, F6, g6, W6, o.l6, n);
+        const Sides<V> i0 = vsides(F0), i1 = vsides(F1), i5 = vsides(F5), i3 = vsides(F3), i7 = vsides(F7);
         // east face of k = 1, west face of k = 5
-        const V e1 = vfma(T(-2), F1, s1), e5 = vfma(T(-2), F5, s5);
-        V q = vfma(cf.px, d1, vmul(cf.pe, e1));
+        const V e1 = vfma(T(-2), F1, i1.s), e5 = vfma(T(-2), F5, i5.s);
+        V q = vfma(cf.px, i1.d, vmul(cf.pe, e1));
         const V T1 = vadd(z1, q);
-        z1 = vadd(vfma(T(4), q, F1), q1);
+        if (n.mid) z1 = vadd(vfma(T(4), q, F1), q1);
         q1 = q;
-        q = vfma(-cf.px, d5, vmul(cf.pe, e5));
+        q = vfma(-cf.px, i5.d, vmul(cf.pe, e5));
         const V T5 = vadd(z5, q);
-        z5 = vadd(vfma(T(4), q, F5), q5);
+        if (n.mid) z5 = vadd(vfma(T(4), q, F5), q5);
         q5 = q;
         // north face of k = 3, south face of k = 7
-        const V m3 = vfma(T(4), F3, s3), m7 = vfma(T(4), F7, s7);
+        const V m3 = vfma(T(4), F3, i3.s), m7 = vfma(T(4), F7, i7.s);
         const V T3 = vfma(cf.nu, m3, z3);
-        z3 = vfma(cf.nd, m3p, vfma(cf.nm, m3, F3));
+        if (n.mid) z3 = vfma(cf.nd, m3p, vfma(cf.nm, m3, F3));
         m3p = m3;
         o.l7 = vfma(cf.nd, m7, z7);
-        z7 = vfma(cf.nu, m7p, vfma(cf.nm, m7, F7));
+        if (n.mid) z7 = vfma(cf.nu, m7p, vfma(cf.nm, m7, F7));
         m7p = m7;
         // k = 0, 3, 7 at the east and west faces (weight 1/2 each): A even and B odd in x
         V A, B;
         {
-            const V S = vadd(F0, vadd(F3, F7)), sS = vadd(s0, vadd(s3, s7));
-            const V dS = vadd(d0, vadd(d3, d7)), dD = vsub(d7, d3);
+            const V S = vadd(F0, vadd(F3, F7)), sS = vadd(i0.s, vadd(i3.s, i7.s));
+            const V dS = vadd(i0.d, vadd(i3.d, i7.d)), dD = vsub(i7.d, i3.d);
             const V mP = vadd(m3, m7), mD = vsub(m7, m3);
             const V G = vfma(cf.ge, vfma(T(-2), S, sS), vmul(cf.gp, mP));
             A = vadd(zA, vfma(cf.gd, mD, G));
-            zA = vadd(vfma(T(0.5), S, vfma(T(4), G, vmul(T(-6) * cf.gp, mP))), vAp);
-            vAp = vfma(-cf.gd, mD, G);
+            if (n.mid) zA = vadd(vfma(T(0.5), S, vfma(T(4), G, vmul(T(-6) * cf.gp, mP))), vAp);
+            if (n.low) vAp = vfma(-cf.gd, mD, G);
             const V u = vmul(T(1.0 / 48.0), dS);
             B = vadd(zB, vfma(cf.b2, dD, u));
-            zB = vfma(T(4), u, vBp);
-            vBp = vfma(-cf.b2, dD, u);
+            if (n.mid) zB = vfma(T(4), u, vBp);
+            if (n.low) vBp = vfma(-cf.b2, dD, u);
         }
-        o.PE = vadd(vadd(T1, vadd(E2, E8)), vadd(A, B));
-        o.PW = vadd(vadd(T5, vadd(W4, W6)), vsub(A, B));
+        if (n.flux) {
+            o.PE = vadd(vadd(T1, vadd(E2, E8)), vadd(A, B));
+            o.PW = vadd(vadd(T5, vadd(W4, W6)), vsub(A, B));
+        }
         // k = 0, 1, 5 at the north and south faces
         {
-            const V S = vadd(F0, vadd(F1, F5)), mS = vfma(T(4), S, vadd(s0, vadd(s1, s5)));
-            const V dD = vsub(d5, d1), eP = vadd(e1, e5);
+            const V S = vadd(F0, vadd(F1, F5)), mS = vfma(T(4), S, vadd(i0.s, vadd(i1.s, i5.s)));
+            const V dD = vsub(i5.d, i1.d), eP = vadd(e1, e5);
             const V G = vfma(cf.gd, dD, vfma(cf.gp, eP, vmul(cf.ge, mS)));
             A = vadd(zN, G);
-            zN = vadd(vfma(T(0.5), S, vfma(T(4), G, vmul(T(-6) * cf.ge, mS))), gNp);
+            if (n.mid) zN = vadd(vfma(T(0.5), S, vfma(T(4), G, vmul(T(-6) * cf.ge, mS))), gNp);
             gNp = G;
             const V Q = vfma(T(1.0 / 48.0), mS, vmul(cf.b2, dD));
             B = vsub(Q, qN2);
             qN2 = qN1;
             qN1 = Q;
         }
+        if (!n.out) return;
         o.ls = vadd(o.l7, vadd(o.l6, o.l8));
         o.PN = vadd(vadd(T3, vadd(N2, N4)), vadd(A, B));
         o.PS = vadd(o.ls, vsub(A, B));
-        // Dbar_k = xi_x (f_E(c) - f_E(c - E)) + xi_y (f_N(c) - f_N(c - N))
-        o.D1 = vless_left(T1);
-        o.D5 = vless_right(T5);
-        o.D2 = vadd(vless_left(E2), vsub(N2, n2p));
-        o.D4 = vadd(vless_right(W4), vsub(N4, n4p));
-        o.D3 = vsub(T3, t3p);
-        o.D6 = vadd(vless_right(W6), o.l6);
-        o.D7 = o.l7;
-        o.D8 = vadd(vless_left(E8), o.l8);
+        if (n.flux) {
+            // Dbar_k = xi_x (f_E(c) - f_E(c - E)) + xi_y (f_N(c) - f_N(c - N))
+            o.D1 = vless_left(T1);
+            o.D5 = vless_right(T5);
+            o.D2 = vadd(vless_left(E2), vsub(N2, n2p));
+            o.D4 = vadd(vless_right(W4), vsub(N4, n4p));
+            o.D3 = vsub(T3, t3p);
+            o.D6 = vadd(vless_right(W6), o.l6);
+            o.D7 = o.l7;
+            o.D8 = vadd(vless_left(E8), o.l8);
+        }
         n2p = N2;
         n4p = N4;
         t3p = T3;
@@ -322,7 +370,7 @@ struct March<V, 1> {
     }
 
     __device__ __forceinline__ void advance(const MarchCoefs<T> &cf, V F0, V F1, V F2, V F3, V F4, V F5, V F6, V F7,
-                                            V F8, RowOut<V> &o) {
+                                            V F8, RowOut<V> &o, Need) {
         const T h = cf.h, hk = cf.hk, cp = cf.cp, cm = cf.cm;
         auto diag = [&](Diag &g, V C, auto sx, auto sy, V &D, V &late) {
             constexpr int SX = decltype(sx)::value, SY = decltype(sy)::value;
@@ -391,15 +439,22 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
     using LN = Lane<V>;
     using MT = MarchTile<V, ST>;
     constexpr bool DEV = Store<T, ST>::deviation;
-    static_assert(Store<T, ST>::phi_plane, "phi is a plane of its own");
+    constexpr bool PHIP = MT::PHIP;
+    // FP64 arithmetic is the scarce resource there: rows that complete nothing skip it
+    constexpr bool SKIP = sizeof(T) == 8;
     static_assert(!DEV || LN::N == 2, "half-precision values travel as pairs");
     constexpr int XB = MT::XB, PB = MT::PB, DEPTH = MT::DEPTH, N = LN::N;
     const int lane = threadIdx.x & 31;
     const int nx = p.nx, ny = p.ny;
-    const int x = MT::TX * bx - MT::HX + N * lane;   // the lane's first column
+    // the strip's width and the columns before it. FP64 strips of at most 26 columns leave out
+    // the outermost lanes, whose phi needs a sum over the column past the strip
+    const int tx = N == 2 ? MT::TX : p.tile_w;
+    const bool wide = PHIP || tx > 26;
+    const int hx = N == 2 || !wide ? 3 : 2;
+    const int x = tx * bx - hx + N * lane;   // the lane's first column
     // element offset of the lane's columns in a row; lanes past the ghost border read padding
     const int col = min(x + GHOST, p.pitch - N);
-    const bool wr = lane >= MT::LO && lane <= MT::HI;
+    const bool wr = N == 2 ? lane >= 1 && lane <= 30 : lane >= hx && lane < hx + tx;
     const bool ok0 = wr && x >= 0 && x < nx, ok1 = N == 2 && wr && x + 1 >= 0 && x + 1 < nx;
     const int npk = rows + MT::rows_extra;
 
@@ -465,27 +520,34 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
     pdl_wait();   // the previous kernel's output (launched with programmatic serialization)
 
     // ---- copies: packet i holds the state and phi_old of row y0 - 2 + i and phi of the row above
+    // (without phi planes phi of the row above is summed from the next packet)
     const uint32_t ring = smem_u32(smem);
     const size_t row0 = (size_t)(y0 - 2 + GHOST) * p.pitch;
     const ST *gX = static_cast<const ST *>(p.X) + row0 + col;
     const T *gPo = p.phi_old + row0 + col;
-    const T *gP = p.phi_cur + row0 + p.pitch + col;
+    const T *gP = PHIP ? p.phi_cur + row0 + p.pitch + col : nullptr;
     // lane 0 also fetches the column before the strip, lane 31 the one after it
     const int hcol = lane == 0 ? max(x + GHOST - 1, 0) : min(x + N + GHOST, p.pitch - 1);
-    const T *gH = p.phi_cur + row0 + p.pitch + hcol;
-    const bool halo = lane == 0 || lane == 31;
-    const uint32_t hdst = MT::oP + (lane == 0 ? MT::P0 - 1 : MT::P0 + 32 * N) * (int)sizeof(T);
+    const T *gH = PHIP ? p.phi_cur + row0 + p.pitch + hcol : static_cast<const T *>(p.X) + row0 + hcol;
+    const bool halo = wide && (lane == 0 || lane == 31);
+    const uint32_t hdst = MT::oP + (PHIP ? lane == 0 ? MT::P0 - 1 : MT::P0 + 32 * N : lane == 0 ? 0 : 9) * (int)sizeof(T);
+    const int packets = PHIP ? npk : npk + 1;
     const size_t plane = p.plane;
     int fetched = 0;
     uint32_t fslot = 0;   // byte offset of the slot the next packet goes to
     auto fetch = [&]() {
-        if (fetched < npk) {
+        if (fetched < packets) {
             const uint32_t s = ring + fslot;
 #pragma unroll
             for (int k = 0; k < 9; k++) cp_async<XB>(s + k * 32 * XB + lane * XB, gX + k * plane);
             cp_async<PB>(s + MT::oPo + lane * PB, gPo);
-            cp_async<PB>(s + MT::oP + (MT::P0 + N * lane) * (int)sizeof(T), gP);
-            if (halo) cp_async<(int)sizeof(T)>(s + hdst, gH);
+            if constexpr (PHIP) {
+                cp_async<PB>(s + MT::oP + (MT::P0 + N * lane) * (int)sizeof(T), gP);
+                if (halo) cp_async<(int)sizeof(T)>(s + hdst, gH);
+            } else if (halo) {
+#pragma unroll
+                for (int k = 0; k < 9; k++) cp_async<(int)sizeof(T)>(s + hdst + k * (int)sizeof(T), gH + k * plane);
+            }
             gX += p.pitch;
             gPo += p.pitch;
             gP += p.pitch;
@@ -513,9 +575,6 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
     V pc1, pc2{}, pc3{};           // phi of rows j, j - 1, j - 2
     V pd1, pm1, pm0, pz;           // gradient rows: R - L, L + 4 C + R; 4 d(j) + d(j - 1)
     {
-        const T *q = p.phi_cur + row0 - p.pitch + col;
-        const int lo = x + GHOST - 1 < 0 ? 0 : -1, hi = col + N < p.pitch ? N : N - 1;
-        const V a = *reinterpret_cast<const V *>(q), b = *reinterpret_cast<const V *>(q + p.pitch);
         auto row = [&](V c, T l, T r, V &d, V &m) {
             if constexpr (N == 2) {
                 d = LN::make(LN::second(c) - l, r - LN::first(c));
@@ -525,9 +584,41 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
                 m = vfma(T(4), c, r + l);
             }
         };
-        V d0;
-        row(a, q[lo], q[hi], d0, pm0);
-        row(b, q[p.pitch + lo], q[p.pitch + hi], pd1, pm1);
+        V d0, a, b;
+        T al, ar, bl, br;
+        if constexpr (PHIP) {
+            const T *q = p.phi_cur + row0 - p.pitch + col;
+            const int lo = x + GHOST - 1 < 0 ? 0 : -1, hi = col + N < p.pitch ? N : N - 1;
+            a = *reinterpret_cast<const V *>(q);
+            b = *reinterpret_cast<const V *>(q + p.pitch);
+            al = q[lo];
+            ar = q[hi];
+            bl = q[p.pitch + lo];
+            br = q[p.pitch + hi];
+        } else {   // sum_k X_k, the outer lanes also of the columns past the strip
+            auto sum = [&](const T *q) {
+                T t = T(0);
+#pragma unroll
+                for (int k = 0; k < 9; k++) t += q[k * plane];
+                return t;
+            };
+            const T *q = static_cast<const T *>(p.X) + row0 - p.pitch;
+            a = sum(q + col);
+            b = sum(q + p.pitch + col);
+            T ha = T(0), hb = T(0);
+            if (halo) {
+                ha = sum(q + hcol);
+                hb = sum(q + p.pitch + hcol);
+            }
+            al = __shfl_up_sync(ALL, a, 1);
+            ar = __shfl_down_sync(ALL, a, 1);
+            bl = __shfl_up_sync(ALL, b, 1);
+            br = __shfl_down_sync(ALL, b, 1);
+            if (lane == 0) al = ha, bl = hb;
+            if (lane == 31) ar = ha, br = hb;
+        }
+        row(a, al, ar, d0, pm0);
+        row(b, bl, br, pd1, pm1);
         pz = vfma(T(4), pd1, d0);
         pc1 = b;
     }
@@ -542,23 +633,44 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
     V f0p{}, f1p{}, f2p{};             // north-face moments of row j - 3
     double msum = 0.0;
     uint32_t cslot = 0;
-    const uint32_t seed = mix32(p.seed);
+    const uint32_t seed = PHIP ? mix32(p.seed) : 0u;
     // lanes whose columns have images in the ghost border left or right of the grid
     const bool xedge = x < GHOST || x + N - 1 >= nx - GHOST;
 
     __syncwarp();
-#pragma unroll 2
+    constexpr int UNROLL = sizeof(T) == 8 ? 1 : 2;   // (FP64: the arithmetic hides the moves that two rows would save)
+#pragma unroll UNROLL
     for (int it = 0; it < npk; it++) {
-        cp_wait<DEPTH - 2>();
+        cp_wait<1>();
         __syncwarp();
         fetch();
         const unsigned char *sl = smem + cslot;
         cslot = cslot + MT::slot == DEPTH * MT::slot ? 0 : cslot + MT::slot;
 
         // ---- phi of the row above, gradient and cell quantities of row j ------------
-        const T *sP = reinterpret_cast<const T *>(sl + MT::oP) + MT::P0 + N * lane;
-        const V pc0 = *reinterpret_cast<const V *>(sP);
-        const T pl = sP[-1], pr = sP[N];
+        V pc0;
+        T pl, pr;
+        if constexpr (PHIP) {
+            const T *sP = reinterpret_cast<const T *>(sl + MT::oP) + MT::P0 + N * lane;
+            pc0 = *reinterpret_cast<const V *>(sP);
+            pl = sP[-1];
+            pr = sP[N];
+        } else {
+            const unsigned char *sn = smem + cslot;   // the next packet
+            pc0 = V{};
+#pragma unroll
+            for (int k = 0; k < 9; k++) pc0 = vadd(pc0, *reinterpret_cast<const V *>(sn + k * 32 * XB + lane * XB));
+            T h = T(0);
+            if (halo) {
+                const T *q = reinterpret_cast<const T *>(sn + hdst);
+#pragma unroll
+                for (int k = 0; k < 9; k++) h = vadd(h, q[k]);
+            }
+            pl = __shfl_up_sync(ALL, pc0, 1);
+            pr = __shfl_down_sync(ALL, pc0, 1);
+            if (lane == 0) pl = h;
+            if (lane == 31) pr = h;
+        }
         V pd0, pmn;
         if constexpr (N == 2) {
             pd0 = LN::make(__fsub_rn(LN::second(pc0), pl), __fsub_rn(pr, LN::first(pc0)));
@@ -618,6 +730,7 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
                     t = vfma(wk, g, vneg(X));
                 }
                 F = vfma(p.b, t, X);
+                if (SKIP && (it < 2 || it > npk - 3)) return V{};
                 return vfma(p.be1, t, X);
             };
             const V gp = vadd(ph, Px), gm = vsub(ph, Px);
@@ -634,61 +747,76 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
 
         // ---- expansions: row j completes row j - 1 -----------------------------------
         RowOut<V> ro;
-        mx.advance(cf, F0, F1, F2, F3, F4, F5, F6, F7, F8, ro);
+        mx.advance(cf, F0, F1, F2, F3, F4, F5, F6, F7, F8, ro,
+                   SKIP ? Need{it >= 2, it >= 3 && it <= npk - 2, it >= 1 && it <= npk - 2, it <= npk - 3}
+                        : Need{true, true, true, true});
 
         // ---- row j - 2 is complete: faces, flux and store ----------------------------
-        // (computed in the first rows too, where nothing is stored: one straight block)
+        // (FP32: computed in the first rows too, where nothing is stored: one straight block)
+        V phn{};
+        V o[9];
+        const int y = y0 + it - 4;
+        if (!SKIP || it >= 3) {
         const V phN = vadd(pNp, ro.PS), phE = phEp;
         // face moments: phi_b and (3 gamma c2 phi_b u_b + gamma c3 V_b) at the east and north faces
-        V uE, vE, uN, vN;
+        const T hf = T(0.5) * f3;
+        Row4<T> rf{};
+        V uN, vN;
         if constexpr (FIELD) {
-            const T hf = T(0.5) * f3;
-            uE = vmul(hf, vplus_right(fu2, fu2));
-            vE = vmul(hf, vplus_right(fv2, fv2));
             uN = vmul(hf, vadd(fu2, fu1));
             vN = vmul(hf, vadd(fv2, fv1));
         } else {
-            const Row4<T> rf = sRow[max(it - 2, 0)];
-            uE = vmul(rf.x, cuE);
-            vE = vmul(rf.y, cvE);
+            rf = sRow[max(it - 2, 0)];
             uN = vmul(rf.z, cu);
             vN = vmul(rf.w, cv);
         }
-        const V x1 = vfma(phE, uE, vmul(hg3, vplus_right(v1x, v1x)));
-        const V x2 = vfma(phE, vE, vmul(hg3, vplus_right(v1y, v1y)));
         const V y1 = vfma(phN, uN, vmul(hg3, vadd(v1x, v0x)));
         const V y2 = vfma(phN, vN, vmul(hg3, vadd(v1y, v0y)));
-        const V A1 = vmul(gc2, vless_left(phE)), A2 = vmul(gc2, vsub(phN, f0p));
-        const V B1 = vless_left(x1), B2 = vadd(vless_left(x2), vsub(y1, f1p)), B3 = vsub(y2, f2p);
+        if (!SKIP || it >= 4) {
+            V uE, vE;
+            if constexpr (FIELD) {
+                uE = vmul(hf, vplus_right(fu2, fu2));
+                vE = vmul(hf, vplus_right(fv2, fv2));
+            } else {
+                uE = vmul(rf.x, cuE);
+                vE = vmul(rf.y, cvE);
+            }
+            const V x1 = vfma(phE, uE, vmul(hg3, vplus_right(v1x, v1x)));
+            const V x2 = vfma(phE, vE, vmul(hg3, vplus_right(v1y, v1y)));
+            const V A1 = vmul(gc2, vless_left(phE)), A2 = vmul(gc2, vsub(phN, f0p));
+            const V B1 = vless_left(x1), B2 = vadd(vless_left(x2), vsub(y1, f1p)), B3 = vsub(y2, f2p);
+            const V S13 = vadd(B1, B3);
+            // new phi = phi + gamma sum_k L_k (sum_k w_k xi_k = 0, sum_k w_k xi_a xi_b = delta_ab / 3)
+            const V dph = vfma(T(-1.0 / 3.0), S13, vmul(-gmc, vsub(sDp, ro.ls)));
+            if constexpr (PHIP) phn = vadd_sr(pc3, dph, (uint32_t)y * (uint32_t)nx + (uint32_t)x, seed);
+            else phn = vadd(pc3, dph);
+            {
+                // gamma w_k (c2 Phi_k + c3 Psi_k) = w_k (xi_x A1 + xi_y A2 + xi_x^2 B1 + xi_x xi_y B2 + xi_y^2 B3)
+                const T w1 = wq<T>(1), w2 = wq<T>(2);
+                // (the late parts of Dbar)
+                const V p7 = FLUX == 0 ? vfma(gmc, ro.l7, r7) : r7;
+                const V p6 = vfma(gmc, ro.l6, r6), p8 = vfma(gmc, ro.l8, r8);
+                const V p2 = FLUX == 0 ? r2 : vfma(gmc, ro.l2, r2), p4 = FLUX == 0 ? r4 : vfma(gmc, ro.l4, r4);
+                o[1] = vfma(-w1, vadd(B1, A1), r1);
+                o[5] = vfma(-w1, vsub(B1, A1), r5);
+                o[3] = vfma(-w1, vadd(B3, A2), r3);
+                o[7] = vfma(-w1, vsub(B3, A2), p7);
+                const V sp = vadd(S13, B2), sm = vsub(S13, B2), ap = vadd(A1, A2), am = vsub(A1, A2);
+                o[2] = vfma(-w2, vadd(sp, ap), p2);
+                o[6] = vfma(-w2, vsub(sp, ap), p6);
+                o[8] = vfma(-w2, vadd(sm, am), p8);
+                o[4] = vfma(-w2, vsub(sm, am), p4);
+                // rest component: the new phi is exactly phn (up to this subtraction)
+                o[0] = vsub(phn, vadd(vadd(vadd(o[1], o[2]), vadd(o[3], o[4])), vadd(vadd(o[5], o[6]), vadd(o[7], o[8]))));
+            }
+        }
         f0p = phN;
         f1p = y1;
         f2p = y2;
-        const int y = y0 + it - 4;
-        const V S13 = vadd(B1, B3);
-        // new phi = phi + gamma sum_k L_k (sum_k w_k xi_k = 0, sum_k w_k xi_a xi_b = delta_ab / 3)
-        const V dph = vfma(T(-1.0 / 3.0), S13, vmul(-gmc, vsub(sDp, ro.ls)));
-        const V phn = vadd_sr(pc3, dph, (uint32_t)y * (uint32_t)nx + (uint32_t)x, seed);
-        V o[9];
-        {
-            // gamma w_k (c2 Phi_k + c3 Psi_k) = w_k (xi_x A1 + xi_y A2 + xi_x^2 B1 + xi_x xi_y B2 + xi_y^2 B3)
-            const T w1 = wq<T>(1), w2 = wq<T>(2);
-            // (the late parts of Dbar)
-            const V p7 = FLUX == 0 ? vfma(gmc, ro.l7, r7) : r7;
-            const V p6 = vfma(gmc, ro.l6, r6), p8 = vfma(gmc, ro.l8, r8);
-            const V p2 = FLUX == 0 ? r2 : vfma(gmc, ro.l2, r2), p4 = FLUX == 0 ? r4 : vfma(gmc, ro.l4, r4);
-            o[1] = vfma(-w1, vadd(B1, A1), r1);
-            o[5] = vfma(-w1, vsub(B1, A1), r5);
-            o[3] = vfma(-w1, vadd(B3, A2), r3);
-            o[7] = vfma(-w1, vsub(B3, A2), p7);
-            const V sp = vadd(S13, B2), sm = vsub(S13, B2), ap = vadd(A1, A2), am = vsub(A1, A2);
-            o[2] = vfma(-w2, vadd(sp, ap), p2);
-            o[6] = vfma(-w2, vsub(sp, ap), p6);
-            o[8] = vfma(-w2, vadd(sm, am), p8);
-            o[4] = vfma(-w2, vsub(sm, am), p4);
-            // rest component: the new phi is exactly phn (up to this subtraction)
-            o[0] = vsub(phn, vadd(vadd(vadd(o[1], o[2]), vadd(o[3], o[4])), vadd(vadd(o[5], o[6]), vadd(o[7], o[8]))));
         }
+        const V pho = PHIP ? phn : pc3;   // (without phi planes: phi of X, the next step's older level)
         // ---- row j - 1: X + be (g - X) - gamma (1 - c2) Dbar ---------------------------
+        if (!SKIP || (it >= 3 && it <= npk - 2)) {
         r1 = vfma(-gmc, ro.D1, b1);
         r2 = vfma(-gmc, ro.D2, b2);
         r3 = vfma(-gmc, ro.D3, b3);
@@ -699,6 +827,7 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
         r8 = vfma(-gmc, ro.D8, b8);
         sDp = vadd(vadd(vadd(ro.D1, ro.D2), vadd(ro.D3, ro.D4)), vadd(vadd(ro.D5, ro.D6), vadd(ro.D7, ro.D8)));
         phEp = vplus_right(ro.PE, ro.PW);
+        }
         pNp = ro.PN;
         b1 = nb1; b2 = nb2; b3 = nb3; b4 = nb4; b5 = nb5; b6 = nb6; b7 = nb7; b8 = nb8;
         v1x = v0x; v1y = v0y;
@@ -725,20 +854,20 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
                 if constexpr (N == 2) O[(long long)(k * plane) + g] = ov[k].x;
                 else O[(long long)(k * plane) + g] = ov[k];
             }
-            p.phi_out[g] = LN::first(phn);
+            p.phi_out[g] = LN::first(pho);
         };
         auto put1 = [&](long long g) {
             if constexpr (N == 2) {
 #pragma unroll
                 for (int k = 0; k < 9; k++) O[(long long)(k * plane) + g + 1] = ov[k].y;
-                p.phi_out[g + 1] = LN::second(phn);
+                p.phi_out[g + 1] = LN::second(pho);
             }
         };
         const size_t g = (size_t)(y + GHOST) * p.pitch + (size_t)(x + GHOST);
         if (st0 && (N == 1 || st1)) {
 #pragma unroll
             for (int k = 0; k < 9; k++) *reinterpret_cast<OV *>(O + k * plane + g) = ov[k];
-            *reinterpret_cast<V *>(p.phi_out + g) = phn;
+            *reinterpret_cast<V *>(p.phi_out + g) = pho;
         } else if (st0) {
             put0(g);
         } else if (st1) {
