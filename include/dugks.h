@@ -118,7 +118,7 @@ int dugks_set_velocity(dugks_ctx *c, int kind, const double *params, const doubl
  * and bar f^+, the isotropic gradients of Eq. (2) and of the reconstruction,
  * bar f at x_b - xi h by Eqs. (24)-(26), the face phi, equilibrium, source
  * and original f of Eqs. (27)-(28), and the meso-flux update of Eq. (21), and
- * also writes per-tile FP64 mass partials. Three-stage (Eqs. (29)-(34)): two
+ * also writes FP64 mass partials (per tile or strip segment). Three-stage (Eqs. (29)-(34)): two
  * kernels per step (steps (i)-(ii) and (iii)-(iv) of Sec. II.B.2). DVM
  * (stages = 1): one kernel per step, streaming (Eqs. (11a), (12)), phi of
  * Eq. (13), cell quantities at t + dt and the collision of Eq. (11b), with the
@@ -179,15 +179,14 @@ int dugks_selftest_fail_allocs(int32_t skip, int32_t count);
 /* Text of the last error; never NULL (empty when there was none). */
 const char *dugks_last_error(const dugks_ctx *c);
 
-/* Tile variant of the TMA-staged two-stage kernel (orders 2, 3), warps per CTA x
- * rows of cells per thread: 0 = 8 x 4 (FP64: 8 x 2), 1 = 16 x 1, 2 = 8 x 2,
- * 3 = 12 x 3, 4 = 8 x 3, 5 = 10 x 4 (a tile is 31 cells wide and warps x rows - 1
- * cells high). The default is 2 below 512 x 512 cells and 4 from there up; -1
- * selects the generic fused kernel (one thread per cell and stage, no TMA), the
- * plain comparison path. A tuning choice only: results agree to rounding.
- * Returns DUGKS_EINVAL for any other number. Order 4 and the three-stage
- * scheme have one TMA-staged tile shape each (orders 4-5, two-stage: 10 x 3, FP64
- * 8 x 2; three-stage: 8 x 2): any variant >= 0 selects it.
+/* Segment length of the two-stage kernel of orders 2 and 3 (rows of a strip that one
+ * warp walks up): 0 = 16, 1 = 8, 3 = 32, 5 = 64 rows; 2 and 4 = chosen by a rule on
+ * the grid's size, which is the default (2 below 512 x 512 cells, 4 from there up);
+ * -1 selects the generic fused kernel (one thread per cell and stage), the plain
+ * comparison path. A tuning choice only: results agree to rounding. Returns
+ * DUGKS_EINVAL for any other number. Orders 4 and 5 and the three-stage scheme have
+ * one TMA-staged tile shape each (warps per CTA x rows of cells per thread: orders
+ * 4-5, two-stage: 10 x 3, FP64 8 x 2; three-stage: 8 x 2): any variant >= 0 selects it.
  * dugks_get_variant returns -1 when the context uses the generic kernel. */
 int dugks_set_variant(dugks_ctx *c, int variant);
 int dugks_get_variant(const dugks_ctx *c);
@@ -208,9 +207,8 @@ void dugks_destroy(dugks_ctx *c);
 
 /* ---- many grids per launch ------------------------------------------------
  * A batch advances many independent periodic grids of different sizes with one
- * launch per step: a work list of 31-cell-wide tiles of all grids is processed
- * by a grid-stride set of CTAs (the TMA-staged two-stage kernel), followed by a
- * per-grid FP64 mass and step-counter update. Each grid keeps its own step
+ * launch per step (the two-stage kernel over a work list of the strip segments of
+ * all grids), and a step-counter update per group of steps. Each grid keeps its own step
  * counter on the device, so grids may join (dugks_batch_add) and leave
  * (dugks_batch_remove) between calls of dugks_batch_step, and a sequence of
  * steps is replayed as a CUDA graph. Every grid's result is bitwise the same
@@ -222,8 +220,8 @@ void dugks_destroy(dugks_ctx *c);
  * data moves through pinned staging buffers, and whatever the stream may still
  * read is released only after it has passed. A server can therefore admit and
  * finish grids while earlier steps are still running; several batches on
- * streams of different priority share the GPU tile by tile when their kernels
- * run one CTA per tile (dugks_batch_set_ctas). The calls described as waiting
+ * streams of different priority share the GPU segment by segment when their kernels
+ * run one CTA per segment (dugks_batch_set_ctas). The calls described as waiting
  * (read_phi, mass, status, set_variant, destroy) synchronise the stream. A
  * batch is not thread-safe: one host thread drives it. */
 typedef struct dugks_batch dugks_batch;
@@ -274,10 +272,12 @@ int dugks_batch_collect(dugks_batch *b, int32_t grid_id, double *out_host, int w
 int dugks_batch_fence(dugks_batch *b, uint64_t *ticket);
 int dugks_batch_reached(dugks_batch *b, uint64_t ticket, int32_t *done);
 
-/* CTAs of the step kernel: 0 (default) as many as are resident on the GPU, each
- * striding over the work list; a negative value one CTA per tile, so that a
- * kernel of a higher-priority stream takes SMs as soon as tiles finish; a
- * positive value at most that many. DUGKS_EINVAL for a null batch. */
+/* CTAs of the step kernel: 0 (default) chosen by the library (as many as are resident
+ * on the GPU, each striding over the work list, for lists of up to one and a half
+ * times that many segments and in FP64; else one CTA per segment); a negative value one
+ * CTA per segment, so that a kernel of a higher-priority stream takes SMs as soon as
+ * segments finish; a positive value at most that many. No result depends on it.
+ * DUGKS_EINVAL for a null batch. */
 int dugks_batch_set_ctas(dugks_batch *b, int32_t ctas);
 
 /* Enqueues nsteps steps of every grid that has not reached its target. */
@@ -289,12 +289,11 @@ int64_t dugks_batch_step_index(const dugks_batch *b, int32_t grid_id);
 /* Waits and copies phi (ny * nx doubles) of one grid to the host. */
 int dugks_batch_read_phi(dugks_batch *b, int32_t grid_id, double *out_host);
 
-/* Waits and returns one grid's mass (FP64, fixed-order sum). */
+/* Waits and returns one grid's mass (FP64, fixed-order sum over phi of its state). */
 int dugks_batch_mass(dugks_batch *b, int32_t grid_id, double *out);
 
-/* Tile variant of the batch kernel (0..5 as for dugks_set_variant; default 5 in
- * FP32, 4 otherwise);
- * waits for the stream and rebuilds the grid descriptors. */
+/* Segment length of the batch kernel (0..5 as for dugks_set_variant; default 4, by the
+ * rule, for all its grids together); waits for the stream and rebuilds the work list. */
 int dugks_batch_set_variant(dugks_batch *b, int variant);
 
 /* Cells of all grids that are still advancing. */

@@ -10,10 +10,8 @@ CSRC = os.path.join(HERE, "csrc")
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "libdugks.so")
 SOURCES = ["dugks_api.cu", "dugks_noalloc.cu", "dugks_batch.cu"] + [
-    f"dugks_inst_{p}_{k}.cu" for p in ("f64", "f32", "f16") for k in ("gen", "fast", "batch")] + [
-    "dugks_inst_f64_t3.cu", "dugks_inst_f32_t3.cu", "dugks_inst_f64_o4.cu", "dugks_inst_f32_o4.cu",
-    "dugks_inst_f16_o4.cu", "dugks_inst_f32_march.cu", "dugks_inst_f16_march.cu", "dugks_inst_f64_march.cu",
-    "dugks_inst_dvm.cu"]
+    f"dugks_inst_{p}_{k}.cu" for p in ("f64", "f32", "f16") for k in ("gen", "march", "o4")] + [
+    "dugks_inst_f64_t3.cu", "dugks_inst_f32_t3.cu", "dugks_inst_dvm.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 

@@ -1,4 +1,4 @@
-"""Autotuner of the fast kernel's tile variant (warps per CTA x rows per thread).
+"""Autotuner of the two-stage kernel's variant (the rows of a segment that a warp walks up).
 
 Times each variant on the caller's own solver or batch and caches the winner
 per (kind, precision, order, flux, size bucket) in a JSON file under the
@@ -49,8 +49,8 @@ def _store(d: dict):
         pass
 
 
-# bumped whenever a variant number changes its tile shape (older cache entries are ignored)
-TABLE = 2
+# bumped whenever a variant number changes its meaning (older cache entries are ignored)
+TABLE = 3
 
 
 def key(kind: str, params, cells: int) -> str:

@@ -150,12 +150,13 @@ template <typename T, typename ST>
 bool setup_fast(dugks_ctx *c) {
     if (marches(c)) {
         c->march = true;
-        c->plan = march_plan(c->variant, c->p.nx, c->p.ny, c->p.precision, c->sms);
-        c->tile_w = c->plan.width;
-        c->tile_h = c->plan.rows;
+        const int2 size = make_int2(c->p.nx, c->p.ny);
+        c->plan = march_plan(c->variant, &size, 1, c->p.precision, c->sms);
+        c->tile_w = march_width(c->plan.cols, size.x);
+        c->tile_h = march_segment_rows(c->plan.rows, size.y);
         return true;
     }
-    const FastGeom g = Launch<T, ST>::fast_geom(c->variant, c->p.order, c->p.stages);
+    const FastGeom g = Launch<T, ST>::fast_geom(c->p.order, c->p.stages);
     const bool half = Store<T, ST>::deviation;
     for (int s = 0; s < 2; s++)
         if (!encode_map(&c->tmX[s], c->X[s], sizeof(ST), half, c, 9, g.box_w, g.box_h)) return false;
@@ -172,7 +173,7 @@ bool fast_capable(const dugks_ctx *c) {
 }
 
 // strips of the row march start one column before the grid
-int strips(const dugks_ctx *c) { return c->fast && c->march ? c->plan.strips : (c->p.nx + c->tile_w - 1) / c->tile_w; }
+int strips(const dugks_ctx *c) { return c->fast && c->march ? march_strips(c->plan.cols, c->p.nx) : (c->p.nx + c->tile_w - 1) / c->tile_w; }
 
 template <typename T, typename ST>
 int run_init(dugks_ctx *c) {
@@ -645,8 +646,6 @@ int dugks_create(const dugks_params *p, const double *phi0_host, void *cuda_stre
     if (c->fast && (p->stages == 3 || p->order >= 4)) {
         c->variant = 2;
     } else if (c->fast) {
-        // measured (FP32, L2 flushed between steps): 8 warps x 2 rows per thread fastest
-        // on grids that fill about one wave of tiles (256^2), 8 x 3 from 1024^2 up
         c->variant = (int64_t)p->nx * p->ny >= 512 * 512 ? 4 : 2;
         // tuning override: DUGKS_FAST_VARIANT = 0..FAST_VARIANTS-1
         if (const char *ev = std::getenv("DUGKS_FAST_VARIANT")) {

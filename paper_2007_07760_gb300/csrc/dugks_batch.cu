@@ -1,8 +1,8 @@
 // dugks_batch.cu -- many independent grids per launch (declared in include/dugks.h).
 //
-// Host side of the batch: per-grid device memory and descriptors (BatchGrid,
-// with TMA tensor maps), the work list of tiles, the per-step launches and
-// their CUDA-graph replay. The arithmetic is the fast kernel's, unchanged.
+// Host side of the batch: per-grid device memory and descriptors (BatchGrid), the
+// work list of strip segments, the launches of a group of steps and their CUDA-graph
+// replay. The arithmetic is the row march's, unchanged.
 //
 // Nothing on the path of a running batch waits for the device: grid memory comes
 // from a stream-ordered pool of the batch's own and goes back to it in stream
@@ -34,21 +34,18 @@ namespace {
 struct Slot {
     bool used = false;
     bool retiring = false;   // read-out enqueued (dugks_batch_retire), result not yet collected
-    int nx = 0, ny = 0, pitch = 0, tiles_x = 0, tiles_y = 0;
+    int nx = 0, ny = 0, pitch = 0;
     size_t plane = 0;
     void *X[2] = {nullptr, nullptr};
     void *phi[3] = {nullptr, nullptr, nullptr};
     int64_t step = 0, target = -1;
     int vel_kind = DUGKS_VEL_UNIFORM;
     double vel[3] = {0, 0, 0};
-    bool mass_known = false;
     uint64_t ticket = 0;            // fence after the read-out
     void *pinned = nullptr;         // host buffer the read-out lands in
     size_t pinned_bytes = 0;
-    std::vector<unsigned char> desc;   // encoded descriptor (tensor maps); empty: encode at the next rebuild
 };
 
-constexpr int GRAPH_STEPS = 8;
 // pinned host buffers kept for reuse beyond this are given back
 constexpr size_t PINNED_KEEP = (size_t)1 << 30;
 
@@ -56,15 +53,16 @@ constexpr size_t PINNED_KEEP = (size_t)1 << 30;
 
 struct dugks_batch {
     dugks_params p{};
-    int dev = 0;
+    int dev = 0, sms = 0;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     size_t tsize = 4, ssize = 4;
     int nphi = 2;
-    // 8 warps x 3 rows per thread; FP32: 10 x 4 (measured fastest on mixed batches)
-    int variant = 4;
+    int variant = 4;    // segment length: by the rule of march_plan
+    MarchPlan plan{};
+    int rows = 0;       // the longest segment of the work list
     int ctas = 0;
-    int ctas_req = 0;   // 0: resident CTAs (grid-stride); < 0: one CTA per tile; > 0: at most that many
+    int ctas_req = 0;   // 0: resident CTAs (grid-stride); < 0: one CTA per segment; > 0: at most that many
     std::vector<Slot> slots;
     cudaMemPool_t pool = nullptr;   // grid memory, descriptors and the work list
     // device side
@@ -72,8 +70,6 @@ struct dugks_batch {
     int grids_cap = 0;
     int4 *d_items = nullptr;
     int items_cap = 0, nitems = 0;
-    double *d_partials = nullptr;
-    double *d_mass = nullptr;
     int *d_status = nullptr;
     void *d_tmp = nullptr;       // phi read-out / generic mass partials of the waiting calls
     size_t tmp_bytes = 0;
@@ -246,31 +242,29 @@ size_t plane_of(int nx, int ny, int *pitch_out) {
     return (size_t)(ny + 2 * GHOST) * pitch;
 }
 
-template <typename T, typename ST>
-FastGeom geom(const dugks_batch *b) { return Launch<T, ST>::fast_geom(b->variant); }
-
-FastGeom batch_geom(const dugks_batch *b) {
-    switch (b->p.precision) {
-    case DUGKS_FP64: return geom<double, double>(b);
-    case DUGKS_FP32: return geom<float, float>(b);
-    default: return geom<float, __half>(b);
-    }
-}
-
 int resident_ctas(dugks_batch *b) {
-    int sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->dev);
     int per = 1;
     switch (b->p.precision) {
-    case DUGKS_FP64: per = Launch<double, double>::batch_ctas_per_sm(b->p.order, b->p.flux, b->variant); break;
-    case DUGKS_FP32: per = Launch<float, float>::batch_ctas_per_sm(b->p.order, b->p.flux, b->variant); break;
-    default: per = Launch<float, __half>::batch_ctas_per_sm(b->p.order, b->p.flux, b->variant); break;
+    case DUGKS_FP64: per = Launch<double, double>::batch_ctas_per_sm(b->p.flux, b->plan.cols, b->rows); break;
+    case DUGKS_FP32: per = Launch<float, float>::batch_ctas_per_sm(b->p.flux, b->plan.cols, b->rows); break;
+    default: per = Launch<float, __half>::batch_ctas_per_sm(b->p.flux, b->plan.cols, b->rows); break;
     }
-    return std::max(1, sms) * std::max(1, per);
+    return std::max(1, b->sms) * std::max(1, per);
+}
+
+// By default resident CTAs striding over a list that is little longer (32 grids of 64^2 to
+// 512^2: 79.5 us a step against 82.8), else one CTA a segment, which the hardware hands out as
+// others finish (512 such grids: 897 us against 1353). In FP64 a warp that joins a busy scheduler
+// halves its rate, so the resident set is kept (32 grids: 1966 us against 2389).
+void choose_ctas(dugks_batch *b) {
+    b->ctas = b->ctas_req < 0 ? INT_MAX : b->ctas_req;
+    if (b->ctas_req != 0) return;
+    b->ctas = resident_ctas(b);
+    if (!fp64(b) && 2 * (int64_t)b->nitems > 3 * (int64_t)b->ctas) b->ctas = INT_MAX;
 }
 
 template <typename T>
-void fill_uniform(dugks_batch *b, const FastGeom &g) {
+void fill_uniform(dugks_batch *b) {
     BatchUniform<T> u;
     std::memset(&u, 0, sizeof u);
     const double dt = b->p.cfl, tau = 3.0 * b->p.M, h = 0.5 * dt;
@@ -291,12 +285,11 @@ void fill_uniform(dugks_batch *b, const FastGeom &g) {
     u.qinv = (T)(1.0 / 256.0);
     u.dt = dt;
     u.dtphiu = b->p.dtphiu;
-    u.tile_w = g.tile_w;
-    u.tile_h = g.tile_h;
     u.status = b->d_status;
     b->uniform.assign(reinterpret_cast<unsigned char *>(&u), reinterpret_cast<unsigned char *>(&u) + sizeof u);
-    FaceCoefs<T> cf = make_face_coefs<T>(b->p.order, b->p.flux, h);
-    b->coefs.assign(reinterpret_cast<unsigned char *>(&cf), reinterpret_cast<unsigned char *>(&cf) + sizeof cf);
+    const MarchCoefs<T> cf = make_march_coefs<T>(b->p.order, h);
+    b->coefs.assign(reinterpret_cast<const unsigned char *>(&cf),
+                    reinterpret_cast<const unsigned char *>(&cf) + sizeof cf);
 }
 
 // the current graph is destroyed once the stream has passed its launches
@@ -315,47 +308,39 @@ void drop_graph(dugks_batch *b) {
 // Descriptors and work list of all grids, uploaded in stream order from pinned
 // staging (the steps already queued keep the old ones). Grids that reached their
 // target, or are retiring, keep a frozen descriptor and contribute no tiles.
-template <typename T, typename ST>
+template <typename T>
 int rebuild_t(dugks_batch *b) {
     drop_graph(b);
-    const FastGeom g = Launch<T, ST>::fast_geom(b->variant);
     const int n = (int)b->slots.size();
     if (n > b->grids_cap) {
         const int cap = std::max(16, n * 2);
         void *grids = nullptr;
-        double *mass = nullptr;
-        if (pool_alloc(b, &grids, (size_t)cap * sizeof(BatchGrid<T>)) != cudaSuccess ||
-            pool_alloc(b, &mass, (size_t)cap * sizeof(double)) != cudaSuccess) {
-            pool_free(b, grids);
+        if (pool_alloc(b, &grids, (size_t)cap * sizeof(BatchGrid<T>)) != cudaSuccess)
             return bfail(b, DUGKS_ENOMEM, "batch descriptors");
-        }
-        cudaMemsetAsync(mass, 0, (size_t)cap * sizeof(double), b->stream);
-        if (b->d_mass)
-            cudaMemcpyAsync(mass, b->d_mass, (size_t)b->grids_cap * sizeof(double), cudaMemcpyDeviceToDevice,
-                            b->stream);
         pool_free(b, b->d_grids);
-        pool_free(b, b->d_mass);
         b->d_grids = grids;
-        b->d_mass = mass;
         b->grids_cap = cap;
     }
     auto live = [](const Slot &s) { return s.used && !s.retiring && (s.target < 0 || s.step < s.target); };
-    int nitems = 0;
+    std::vector<int2> sizes;
     for (const Slot &s : b->slots)
-        if (live(s)) nitems += s.tiles_x * s.tiles_y;
+        if (live(s)) sizes.push_back(make_int2(s.nx, s.ny));
+    b->plan = march_plan(b->variant, sizes.data(), (int)sizes.size(), b->p.precision, b->sms);
+    int nitems = 0;
+    b->rows = 1;
+    for (const int2 &q : sizes) {
+        nitems += march_strips(b->plan.cols, q.x) * march_segments(b->plan.rows, q.y);
+        b->rows = std::max(b->rows, march_segment_rows(b->plan.rows, q.y));
+    }
+    b->nitems = nitems;
+    choose_ctas(b);
     if (nitems > b->items_cap) {
         pool_free(b, b->d_items);
-        pool_free(b, b->d_partials);
         b->d_items = nullptr;
-        b->d_partials = nullptr;
         b->items_cap = 0;
         const int cap = nitems * 2;
-        if (pool_alloc(b, &b->d_items, (size_t)cap * sizeof(int4)) != cudaSuccess ||
-            pool_alloc(b, &b->d_partials, (size_t)cap * sizeof(double)) != cudaSuccess) {
-            pool_free(b, b->d_items);
-            b->d_items = nullptr;
+        if (pool_alloc(b, &b->d_items, (size_t)cap * sizeof(int4)) != cudaSuccess)
             return bfail(b, DUGKS_ENOMEM, "batch work list");
-        }
         b->items_cap = cap;
     }
     const size_t gbytes = (size_t)std::max(n, 1) * sizeof(BatchGrid<T>);
@@ -369,66 +354,34 @@ int rebuild_t(dugks_batch *b) {
     }
     BatchGrid<T> *G = static_cast<BatchGrid<T> *>(hg);
     int4 *I = static_cast<int4 *>(hi);
-    const bool half = Store<T, ST>::deviation;
     int k = 0;
     for (int i = 0; i < n; i++) {
-        Slot &s = b->slots[i];
+        const Slot &s = b->slots[i];
         BatchGrid<T> &d = G[i];
-        if (!s.used || s.retiring) {
-            std::memset(&d, 0, sizeof d);
-            d.step = 0;
-            d.target = 0;   // frozen
-            continue;
-        }
-        if (s.desc.size() != sizeof(BatchGrid<T>)) {   // tensor maps, pointers and shape: once per grid
-            BatchGrid<T> e;
-            std::memset(&e, 0, sizeof e);
-            for (int q = 0; q < 2; q++) {
-                e.X[q] = s.X[q];
-                if (!encode_plane_map(&e.tmX[q], s.X[q], b->ssize, half, s.pitch, s.ny, s.plane, 9, g.box_w,
-                                      g.box_h)) {
-                    pinned_put(b, hg, hgs);
-                    pinned_put(b, hi, his);
-                    return bfail(b, DUGKS_ECUDA, "tensor map encoding failed");
-                }
-            }
-            for (int q = 0; q < b->nphi; q++) {
-                e.phi[q] = static_cast<T *>(s.phi[q]);
-                if (!encode_plane_map(&e.tmPhi[q], s.phi[q], sizeof(T), false, s.pitch, s.ny, s.plane, 1, g.box_wt,
-                                      g.box_h)) {
-                    pinned_put(b, hg, hgs);
-                    pinned_put(b, hi, his);
-                    return bfail(b, DUGKS_ECUDA, "tensor map encoding failed");
-                }
-            }
-            if (b->nphi == 2) e.tmPhi[2] = e.tmPhi[0];
-            e.plane = s.plane;
-            e.nx = s.nx;
-            e.ny = s.ny;
-            e.pitch = s.pitch;
-            e.tiles_x = s.tiles_x;
-            e.vel_kind = s.vel_kind;
-            for (int q = 0; q < 3; q++) e.vp[q] = s.vel[q];
-            s.desc.assign(reinterpret_cast<unsigned char *>(&e), reinterpret_cast<unsigned char *>(&e) + sizeof e);
-        }
-        std::memcpy(&d, s.desc.data(), sizeof d);
+        std::memset(&d, 0, sizeof d);   // step 0, target 0: frozen
+        if (!s.used || s.retiring) continue;
+        for (int q = 0; q < 2; q++) d.X[q] = s.X[q];
+        for (int q = 0; q < b->nphi; q++) d.phi[q] = static_cast<T *>(s.phi[q]);
+        d.plane = s.plane;
+        d.nx = s.nx;
+        d.ny = s.ny;
+        d.pitch = s.pitch;
+        d.tile_w = march_width(b->plan.cols, s.nx);
+        d.vel_kind = s.vel_kind;
+        for (int q = 0; q < 3; q++) d.vp[q] = s.vel[q];
         d.step = s.step;
         d.target = s.target < 0 ? (long long)1 << 62 : s.target;
-        d.item0 = k;
-        d.nitems = 0;
-        if (live(s)) {
-            d.nitems = s.tiles_x * s.tiles_y;
-            for (int by = 0; by < s.tiles_y; by++)
-                for (int bx = 0; bx < s.tiles_x; bx++) I[k++] = make_int4(i, bx, by, 0);
-        }
+        if (!live(s)) continue;
+        const int strips = march_strips(b->plan.cols, s.nx), rows = march_segment_rows(b->plan.rows, s.ny);
+        for (int y = 0; y < s.ny; y += rows)
+            for (int x = 0; x < strips; x++) I[k++] = make_int4(i, x, y, std::min(rows, s.ny - y));
     }
-    b->nitems = nitems;
     cudaError_t e = cudaSuccess;
     if (n > 0) e = cudaMemcpyAsync(b->d_grids, hg, (size_t)n * sizeof(BatchGrid<T>), cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess && nitems > 0)
         e = cudaMemcpyAsync(b->d_items, hi, (size_t)nitems * sizeof(int4), cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess)
-        e = launch_batch_factors<T>(static_cast<BatchGrid<T> *>(b->d_grids), n, b->p.cfl, b->stream);
+        e = launch_batch_advance<T>(static_cast<BatchGrid<T> *>(b->d_grids), n, 0, b->p.cfl, b->stream);
     uint64_t t = 0;
     const int fr = e == cudaSuccess ? fence(b, &t) : DUGKS_ECUDA;
     if (fr == DUGKS_OK) {
@@ -445,30 +398,27 @@ int rebuild_t(dugks_batch *b) {
     return DUGKS_OK;
 }
 
-int rebuild(dugks_batch *b) {
-    switch (b->p.precision) {
-    case DUGKS_FP64: return rebuild_t<double, double>(b);
-    case DUGKS_FP32: return rebuild_t<float, float>(b);
-    default: return rebuild_t<float, __half>(b);
-    }
-}
+int rebuild(dugks_batch *b) { return fp64(b) ? rebuild_t<double>(b) : rebuild_t<float>(b); }
 
+// `n` steps (at most GRAPH_STEPS) and the step counters
 template <typename T, typename ST>
-cudaError_t launch_one_step(dugks_batch *b) {
+cudaError_t launch_steps(dugks_batch *b, int n) {
     const BatchUniform<T> &u = *reinterpret_cast<const BatchUniform<T> *>(b->uniform.data());
-    const FaceCoefs<T> &cf = *reinterpret_cast<const FaceCoefs<T> *>(b->coefs.data());
+    const MarchCoefs<T> &cf = *reinterpret_cast<const MarchCoefs<T> *>(b->coefs.data());
     BatchGrid<T> *G = static_cast<BatchGrid<T> *>(b->d_grids);
-    cudaError_t e = Launch<T, ST>::batch_step(u, cf, G, b->d_items, b->nitems, b->d_partials, b->p.order, b->p.flux,
-                                              b->variant, b->ctas, b->stream);
-    if (e != cudaSuccess) return e;
-    return launch_batch_advance<T>(G, (int)b->slots.size(), b->d_partials, b->d_mass, b->d_status, u.dt, b->stream);
+    for (int i = 0; i < n; i++)
+        if (cudaError_t e = Launch<T, ST>::batch_step(u, cf, G, b->d_items, b->nitems, b->rows, i, b->p.flux,
+                                                      b->plan.cols, b->ctas, b->stream);
+            e != cudaSuccess)
+            return e;
+    return launch_batch_advance<T>(G, (int)b->slots.size(), n, u.dt, b->stream);
 }
 
-cudaError_t one_step(dugks_batch *b) {
+cudaError_t steps(dugks_batch *b, int n) {
     switch (b->p.precision) {
-    case DUGKS_FP64: return launch_one_step<double, double>(b);
-    case DUGKS_FP32: return launch_one_step<float, float>(b);
-    default: return launch_one_step<float, __half>(b);
+    case DUGKS_FP64: return launch_steps<double, double>(b, n);
+    case DUGKS_FP32: return launch_steps<float, float>(b, n);
+    default: return launch_steps<float, __half>(b, n);
     }
 }
 
@@ -564,7 +514,6 @@ int dugks_batch_create(const dugks_params *common, void *cuda_stream, dugks_batc
         cudaGetLastError();
         return DUGKS_ECUDA;
     }
-    if (!encode_fn()) return DUGKS_ECUDA;
     dugks_batch *b = new dugks_batch();
     b->p = *common;
     cudaGetDevice(&b->dev);
@@ -579,7 +528,7 @@ int dugks_batch_create(const dugks_params *common, void *cuda_stream, dugks_batc
     b->tsize = fp64(b) ? 8 : 4;
     b->ssize = common->precision == DUGKS_FP64 ? 8 : common->precision == DUGKS_FP32 ? 4 : 2;
     b->nphi = common->precision == DUGKS_FP64 ? 2 : 3;   // FP32 and FP16F: phi is a plane of its own
-    if (common->precision == DUGKS_FP32) b->variant = 5;
+    cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, b->dev);
     if (const char *ev = std::getenv("DUGKS_FAST_VARIANT")) {
         const int v = std::atoi(ev);
         if (v >= 0 && v < FAST_VARIANTS) b->variant = v;
@@ -604,9 +553,8 @@ int dugks_batch_create(const dugks_params *common, void *cuda_stream, dugks_batc
         return DUGKS_ENOMEM;
     }
     cudaMemset(b->d_status, 0, sizeof(int));
-    b->ctas = resident_ctas(b);
-    if (fp64(b)) fill_uniform<double>(b, batch_geom(b));
-    else fill_uniform<float>(b, batch_geom(b));
+    if (fp64(b)) fill_uniform<double>(b);
+    else fill_uniform<float>(b);
     *out = b;
     return DUGKS_OK;
 }
@@ -639,9 +587,6 @@ int dugks_batch_add(dugks_batch *b, int32_t nx, int32_t ny, const double *phi0_h
     s.nx = nx;
     s.ny = ny;
     s.plane = plane_of(nx, ny, &s.pitch);
-    const FastGeom g = batch_geom(b);
-    s.tiles_x = (nx + g.tile_w - 1) / g.tile_w;
-    s.tiles_y = (ny + g.tile_h - 1) / g.tile_h;
     s.vel_kind = vel_kind;
     const int nv = vel_kind == DUGKS_VEL_UNIFORM ? 2 : 3;
     for (int k = 0; k < nv; k++) s.vel[k] = vel_params[k];
@@ -779,7 +724,7 @@ int dugks_batch_set_ctas(dugks_batch *b, int32_t ctas) {
     if (!b) return DUGKS_EINVAL;
     cudaSetDevice(b->dev);
     b->ctas_req = ctas;
-    b->ctas = ctas == 0 ? resident_ctas(b) : ctas < 0 ? INT_MAX : ctas;
+    if (!b->dirty) choose_ctas(b);   // (else with the work list)
     drop_graph(b);   // the next replay is captured with the new grid size
     return DUGKS_OK;
 }
@@ -797,11 +742,12 @@ int dugks_batch_step(dugks_batch *b, int64_t nsteps) {
     int64_t left = nsteps;
     cudaError_t e = cudaSuccess;
     while (left > 0 && e == cudaSuccess) {
-        if (left >= GRAPH_STEPS) {
-            if (!b->graph) {   // capture GRAPH_STEPS steps once; replayed while the work list is unchanged
+        const int m = (int)std::min<int64_t>(left, GRAPH_STEPS);
+        if (m == GRAPH_STEPS) {
+            if (!b->graph) {   // capture a group once; replayed while the work list is unchanged
                 cudaGraph_t g = nullptr;
                 e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
-                for (int i = 0; i < GRAPH_STEPS && e == cudaSuccess; i++) e = one_step(b);
+                if (e == cudaSuccess) e = steps(b, m);
                 cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
                 if (e == cudaSuccess) e = e2;
                 if (e == cudaSuccess) e = cudaGraphInstantiate(&b->graph, g, 0);
@@ -809,19 +755,14 @@ int dugks_batch_step(dugks_batch *b, int64_t nsteps) {
                 if (e != cudaSuccess) break;
             }
             e = cudaGraphLaunch(b->graph, b->stream);
-            left -= GRAPH_STEPS;
-            for (auto &s : b->slots)
-                if (s.used) s.step = s.target < 0 ? s.step + GRAPH_STEPS : std::min(s.target, s.step + GRAPH_STEPS);
         } else {
-            e = one_step(b);
-            left -= 1;
-            for (auto &s : b->slots)
-                if (s.used && (s.target < 0 || s.step < s.target)) s.step += 1;
+            e = steps(b, m);
         }
+        left -= m;
+        for (auto &s : b->slots)
+            if (s.used) s.step = s.target < 0 ? s.step + m : std::min(s.target, s.step + m);
     }
     if (e != cudaSuccess) return bcuda(b, e, "batch step");
-    for (auto &s : b->slots)
-        if (s.used && s.step > 0) s.mass_known = true;
     return DUGKS_OK;
 }
 
@@ -876,32 +817,28 @@ int dugks_batch_mass(dugks_batch *b, int32_t grid_id, double *out) {
     cudaSetDevice(b->dev);
     const Slot &s = b->slots[grid_id];
     cudaError_t e;
-    if (s.mass_known && b->d_mass) {
-        e = cudaMemcpyAsync(out, b->d_mass + grid_id, sizeof(double), cudaMemcpyDeviceToHost, b->stream);
-    } else {
-        // before the first step: reduce the initial state with the generic tiling
-        const int tiles = ((s.nx + TILE_X - 1) / TILE_X) * ((s.ny + TILE_Y - 1) / TILE_Y);
-        const size_t need = (size_t)tiles * sizeof(double) + sizeof(double);
-        if (need > b->tmp_bytes) {
-            cudaStreamSynchronize(b->stream);
-            if (b->d_tmp) cudaFree(b->d_tmp);
-            b->d_tmp = nullptr;
-            b->tmp_bytes = 0;
-            if (dev_malloc(&b->d_tmp, need) != cudaSuccess) {
-                cudaGetLastError();
-                return bfail(b, DUGKS_ENOMEM, "mass buffer");
-            }
-            b->tmp_bytes = need;
+    // from phi of the state, in a tiling that does not depend on the work list
+    const int tiles = ((s.nx + TILE_X - 1) / TILE_X) * ((s.ny + TILE_Y - 1) / TILE_Y);
+    const size_t need = (size_t)tiles * sizeof(double) + sizeof(double);
+    if (need > b->tmp_bytes) {
+        cudaStreamSynchronize(b->stream);
+        if (b->d_tmp) cudaFree(b->d_tmp);
+        b->d_tmp = nullptr;
+        b->tmp_bytes = 0;
+        if (dev_malloc(&b->d_tmp, need) != cudaSuccess) {
+            cudaGetLastError();
+            return bfail(b, DUGKS_ENOMEM, "mass buffer");
         }
-        double *part = static_cast<double *>(b->d_tmp), *res = part + tiles;
-        switch (b->p.precision) {
-        case DUGKS_FP64: { auto q = slot_view<double, double>(b, s); q.mass_partial = part; e = Launch<double, double>::mass_partial(q, b->stream); break; }
-        case DUGKS_FP32: { auto q = slot_view<float, float>(b, s); q.mass_partial = part; e = Launch<float, float>::mass_partial(q, b->stream); break; }
-        default: { auto q = slot_view<float, __half>(b, s); q.mass_partial = part; e = Launch<float, __half>::mass_partial(q, b->stream); break; }
-        }
-        if (e == cudaSuccess) e = launch_mass_final(part, tiles, res, b->d_status, b->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(out, res, sizeof(double), cudaMemcpyDeviceToHost, b->stream);
+        b->tmp_bytes = need;
     }
+    double *part = static_cast<double *>(b->d_tmp), *res = part + tiles;
+    switch (b->p.precision) {
+    case DUGKS_FP64: { auto q = slot_view<double, double>(b, s); q.mass_partial = part; e = Launch<double, double>::mass_partial(q, b->stream); break; }
+    case DUGKS_FP32: { auto q = slot_view<float, float>(b, s); q.mass_partial = part; e = Launch<float, float>::mass_partial(q, b->stream); break; }
+    default: { auto q = slot_view<float, __half>(b, s); q.mass_partial = part; e = Launch<float, __half>::mass_partial(q, b->stream); break; }
+    }
+    if (e == cudaSuccess) e = launch_mass_final(part, tiles, res, b->d_status, b->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(out, res, sizeof(double), cudaMemcpyDeviceToHost, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return bcuda(b, e, "batch mass");
     if (!std::isfinite(*out)) return bfail(b, DUGKS_ENONFINITE, "the field holds NaN or Inf");
@@ -914,16 +851,6 @@ int dugks_batch_set_variant(dugks_batch *b, int variant) {
     cudaError_t e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return bcuda(b, e, "batch synchronize");
     b->variant = variant;
-    b->ctas = b->ctas_req == 0 ? resident_ctas(b) : b->ctas_req < 0 ? INT_MAX : b->ctas_req;
-    const FastGeom g = batch_geom(b);
-    if (fp64(b)) fill_uniform<double>(b, g);
-    else fill_uniform<float>(b, g);
-    for (auto &s : b->slots)
-        if (s.used) {
-            s.tiles_x = (s.nx + g.tile_w - 1) / g.tile_w;
-            s.tiles_y = (s.ny + g.tile_h - 1) / g.tile_h;
-            s.desc.clear();   // tensor-map boxes follow the tile shape
-        }
     b->dirty = true;
     return DUGKS_OK;
 }
@@ -952,7 +879,7 @@ void dugks_batch_destroy(dugks_batch *b) {
     for (auto &g : b->graphs_later) cudaGraphExecDestroy(g.second);
     if (b->pool) {
         for (auto &s : b->slots) free_slot(b, s);
-        for (void *q : {b->d_grids, (void *)b->d_items, (void *)b->d_partials, (void *)b->d_mass}) pool_free(b, q);
+        for (void *q : {b->d_grids, (void *)b->d_items}) pool_free(b, q);
         cudaStreamSynchronize(b->stream);
     }
     for (void *q : {(void *)b->d_status, b->d_tmp})

@@ -1,5 +1,6 @@
-// dugks_fast.cuh -- the DUGKS step staged by TMA (sm_103a): the two-stage step
-// and the two kernels of the three-stage step, stencil orders 2 to 4.
+// dugks_fast.cuh -- the DUGKS step staged by TMA (sm_103a): the two-stage step of
+// orders 4 and 5 and the two kernels of the three-stage step, orders 2 to 4 (the
+// two-stage step of orders 2 and 3 is the row march, dugks_march.cuh).
 //
 // Same arithmetic as step_kernel (dugks_kernels.cuh), organised for throughput:
 //  * the tile's 9 distribution planes plus a halo of 1 + 2R cells (stencil radius
@@ -749,181 +750,6 @@ step_fast_kernel(const __grid_constant__ StepParams<T> p,
     // trigger at entry would place its waiting CTAs while this grid still runs,
     // unevenly when the grid is a single wave)
     pdl_trigger();
-}
-
-// ---- many grids per launch ----------------------------------------------------
-// Per-grid descriptor of a batch, in device memory. The tensor maps are read by
-// TMA from global memory. `step` counts the grid's steps; it selects the
-// ping-pong state set and the phi plane roles, and it is advanced by
-// batch_advance_kernel, so a captured sequence of launches stays valid while
-// grids join and leave (their step counters differ).
-template <typename T>
-struct alignas(64) BatchGrid {
-    CUtensorMap tmX[2];      // state sets 0, 1
-    CUtensorMap tmPhi[3];    // phi planes
-    void *X[2];
-    T *phi[3];
-    long long step, target;  // steps taken; the grid is frozen once step == target
-    size_t plane;
-    int nx, ny, pitch, tiles_x;
-    int item0, nitems;       // its tiles in the work list
-    int vel_kind, pad_;
-    double vp[3];            // velocity parameters (FP64; rounded per precision in the kernel)
-    T tl[3];                 // time levels of the current step: t, t - dt, t + dt/2
-    T vc[3];                 // single vortex: cos(pi t / T) at those levels
-};
-
-// Time levels of a grid's current step and, for the single vortex, its reversal
-// factors, in FP64 (FP64 is slow on this chip: evaluated once per grid and step,
-// by the advance kernel and after each upload of the descriptors, never per tile).
-template <typename T>
-__device__ inline void batch_time_factors(BatchGrid<T> *G, double dt) {
-    const double t = (double)G->step * dt;
-    G->tl[0] = (T)t;
-    G->tl[1] = (T)(t - dt);
-    G->tl[2] = (T)(t + 0.5 * dt);
-    if (G->vel_kind != VEL_VORTEX) return;
-    const double Tp = G->vp[2];
-    G->vc[0] = (T)cospi(t / Tp);
-    G->vc[1] = (T)cospi((t - dt) / Tp);
-    G->vc[2] = (T)cospi((t + 0.5 * dt) / Tp);
-}
-
-// Parameters common to every grid of a batch (same W, M, cfl, order, flux, precision).
-template <typename T>
-struct BatchUniform {
-    T b, h, c1, c2, c3, be1, ga1, tau, theta_c, phiA, phiB, inv_dt, qscale, qinv;
-    double dt;
-    int dtphiu, tile_w, tile_h;
-    int *status;
-};
-
-// The parameters of a grid's current step; returns the phi plane roles (iPc, iPo).
-template <typename T, typename ST>
-__device__ __forceinline__ int2 batch_step_params(const BatchUniform<T> &u, const BatchGrid<T> *G, StepParams<T> &p,
-                                                  FastExtra<T> &fe) {
-    constexpr bool PHIP = Store<T, ST>::phi_plane;
-    const long long step = G->step;
-    p.nx = G->nx;
-    p.ny = G->ny;
-    p.pitch = G->pitch;
-    p.plane = G->plane;
-    p.status = u.status;
-    p.tiles_x = G->tiles_x;
-    p.tile_w = u.tile_w;
-    p.tile_h = u.tile_h;
-    p.acc = nullptr;
-    p.out2 = nullptr;
-    p.mass_partial = nullptr;
-    p.ufield = p.vfield = nullptr;
-    p.a = T(1) - u.b;
-    p.b = u.b;
-    p.h = u.h;
-    p.c1 = u.c1;
-    p.c2 = u.c2;
-    p.c3 = u.c3;
-    p.al1 = T(1) - u.be1;
-    p.be1 = u.be1;
-    p.ga1 = u.ga1;
-    p.al2 = p.be2 = p.ga2 = T(0);
-    p.tau = u.tau;
-    p.theta_c = u.theta_c;
-    p.phiA = u.phiA;
-    p.phiB = u.phiB;
-    p.inv_dtD = u.inv_dt;
-    p.useD = (u.dtphiu && step > 0) ? 1 : 0;
-    p.seed = (uint32_t)step;
-    p.vel_kind = G->vel_kind;
-    p.vp0 = (T)G->vp[0];
-    p.vp1 = (T)G->vp[1];
-    p.vp2 = (T)G->vp[2];
-    p.t = G->tl[0];
-    p.t_old = G->tl[1];
-    p.t_face = G->tl[2];
-    p.qscale = u.qscale;
-    p.qinv = u.qinv;
-    fe.vc_t = G->vc[0];
-    fe.vc_told = G->vc[1];
-    fe.vc_tface = G->vc[2];
-    const int cur = (int)(step & 1);
-    p.X = G->X[cur];
-    p.out1 = G->X[1 - cur];
-    int iPc = 0, iPo, iOut;
-    if constexpr (PHIP) {   // roles rotate with period 3 (see the context API)
-        iPc = (3 - (int)(step % 3)) % 3;
-        iPo = (iPc + 1) % 3;
-        iOut = (iPc + 2) % 3;
-        p.phi_cur = G->phi[iPc];
-    } else {
-        iPo = cur;
-        iOut = 1 - cur;
-        p.phi_cur = nullptr;
-    }
-    p.phi_old = G->phi[iPo];
-    p.phi_out = G->phi[iOut];
-    return make_int2(iPc, iPo);
-}
-
-template <typename T, typename ST, int ORDER, int FLUX, int NW, int MR>
-__global__ void __launch_bounds__(NW * 32, (FastTile<T, ST, NW, MR>::min_blocks))
-batch_fast_kernel(const __grid_constant__ BatchUniform<T> u, const __grid_constant__ FaceCoefs<T> cf,
-                  const BatchGrid<T> *__restrict__ grids, const int4 *__restrict__ items, int nitems,
-                  double *__restrict__ partials) {
-    constexpr bool PHIP = Store<T, ST>::phi_plane;
-    extern __shared__ __align__(128) unsigned char smem[];
-    uint64_t *bar = fast_bar<T, ST, NW, MR>(smem);
-    if (threadIdx.x == 0) mbar_init(bar, 1);
-    uint32_t phase = 0;
-    int fenced = -1;   // grid whose tensor maps this CTA has acquired in this launch
-    for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
-        const int4 w = items[it];
-        const BatchGrid<T> *G = grids + w.x;
-        const long long step = G->step;
-        if (step >= G->target) continue;   // frozen grid (uniform for the CTA)
-        StepParams<T> p;
-        FastExtra<T> fe;
-        const int2 roles = batch_step_params<T, ST>(u, G, p, fe);
-        const int cur = (int)(step & 1), iPc = roles.x, iPo = roles.y;
-        if (threadIdx.x == 0 && w.x != fenced) {
-            // tensor maps written to global memory by the host: order them for the TMA
-            // unit (once per grid: the descriptors do not change during a launch)
-            fenced = w.x;
-            asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&G->tmX[cur]) : "memory");
-            asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&G->tmPhi[iPo]) : "memory");
-            if constexpr (PHIP)
-                asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&G->tmPhi[iPc]) : "memory");
-        }
-        if (!fast_tile<T, ST, ORDER, FLUX, NW, MR>(p, cf, fe, &G->tmX[cur], &G->tmPhi[iPo], &G->tmPhi[iPc], w.y, w.z,
-                                                  partials + it, smem, bar, phase))
-            return;
-        phase ^= 1u;
-    }
-}
-
-// After a batch step: per-grid FP64 mass (fixed-order sum of its tile partials)
-// and the step counter. One CTA per grid.
-template <typename T>
-__global__ void __launch_bounds__(256)
-batch_advance_kernel(BatchGrid<T> *grids, const double *partials, double *mass, int *status, double dt) {
-    __shared__ double sred[32];
-    BatchGrid<T> *G = grids + blockIdx.x;
-    if (G->step >= G->target) return;   // uniform for the CTA
-    double s = 0.0;
-    for (int i = threadIdx.x; i < G->nitems; i += blockDim.x) s += partials[G->item0 + i];
-    s = block_sum(s, sred);
-    if (threadIdx.x == 0) {
-        mass[blockIdx.x] = s;
-        if (!isfinite(s)) atomicOr(status, 1);
-        G->step = G->step + 1;
-        batch_time_factors(G, dt);
-    }
-}
-
-// The factors of every grid after an upload of the descriptors (one thread per grid).
-template <typename T>
-__global__ void __launch_bounds__(128) batch_factors_kernel(BatchGrid<T> *grids, int n, double dt) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) batch_time_factors(grids + i, dt);
 }
 
 }  // namespace dugks

@@ -185,8 +185,8 @@ inline MarchCoefs<T> make_march_coefs(int order, double h) {
     m.gd = (T)(h / 24.0);
     m.b2 = (T)(q * h / 16.0);
     m.h = (T)h;
-    m.cp = (T)(0.5 - h);
-    m.cm = (T)(-0.5 - h);
+    m.cu = (T)(0.5 + h);
+    m.cd = (T)(0.5 - h);
     m.hk = (T)(h / 24.0);
     return m;
 }
@@ -204,21 +204,38 @@ inline MarchCoefs<T> make_march_coefs(int order, double h) {
 // FP64: the FP64 unit of each scheduler issues a warp instruction in 64 cycles whatever the
 // number of active lanes, so a step costs the rows of the busiest scheduler: the warps it gets
 // times s + 2.5 rows (the rows at a segment's ends leave out what they do not need).
-struct MarchPlan { int cols, width, strips, rows, early; };
-inline MarchPlan march_plan(int variant, int nx, int ny, int precision, int sms) {
+struct MarchPlan { int cols, rows, early; };
+// strips of a grid for lanes of `cols` columns, their width, segments of about `want` rows and
+// their equal length
+inline int march_strips(int cols, int nx) {
+    return cols == 2 ? MarchTile<float2, float>::strips(nx) : MarchTile<float, float>::strips(nx);
+}
+inline int march_width(int cols, int nx) {   // (single columns: spread over the strips)
+    const int n = march_strips(cols, nx);
+    return cols == 2 ? MarchTile<float2, float>::TX : (nx + n - 1) / n;
+}
+inline int march_segments(int want, int ny) { return (ny + want - 1) / want; }
+inline int march_segment_rows(int want, int ny) {
+    const int n = march_segments(want, ny);
+    return (ny + n - 1) / n;
+}
+// for `count` grids of sizes (x, y) stepped together
+inline MarchPlan march_plan(int variant, const int2 *sizes, int count, int precision, int sms) {
     static constexpr int fixed[6] = {16, 8, 0, 32, 0, 64};   // variants 2 and 4: by the rule
-    MarchPlan m{};
+    MarchPlan m{precision == DUGKS_FP64 ? 1 : 2, 16, 0};
     double best = 1e300;
     const int forced = variant >= 0 && variant < 6 ? fixed[variant] : 0;
     const bool f64 = precision == DUGKS_FP64;
     for (int cols = precision == DUGKS_FP16F ? 2 : 1; cols <= (f64 ? 1 : 2); cols++) {
-        int strips = cols == 2 ? MarchTile<float2, float>::strips(nx) : MarchTile<float, float>::strips(nx);
-        const int width = cols == 2 ? MarchTile<float2, float>::TX : (nx + strips - 1) / strips;
-        if (cols == 1) strips = (nx + width - 1) / width;
         const double slots = (cols == 2 ? 8.0 : 12.0) * sms, unit = cols == 2 ? 1.42 : 1.05;
         for (int want = forced ? forced : 1; want <= (forced ? forced : 64); want++) {
-            const int segs = (ny + want - 1) / want, rows = (ny + segs - 1) / segs;   // segments of equal length
-            const double w = (double)strips * segs, W = w / slots, n = w / (4.0 * sms);
+            double w = 0.0;
+            int rows = 1;
+            for (int i = 0; i < count; i++) {
+                w += (double)march_strips(cols, sizes[i].x) * march_segments(want, sizes[i].y);
+                rows = std::max(rows, march_segment_rows(want, sizes[i].y));
+            }
+            const double W = w / slots, n = w / (4.0 * sms);
             double cost;
             if (f64) {
                 cost = (n > 3.0 ? n + 0.5 : std::ceil(n)) * (rows + 2.5);
@@ -232,7 +249,7 @@ inline MarchPlan march_plan(int variant, int nx, int ny, int precision, int sms)
                 // (512^2: 15.5 against 16.5 us). On a chip half full it costs instead, because the
                 // waiting warps fill some SMs and leave others idle (256^2, 860 warps: 10.2 against
                 // 9.1), and in FP64, where a scheduler with two warps takes twice as long.
-                m = MarchPlan{cols, width, strips, rows, !f64 && (W > 0.6 || W < 0.15)};
+                m = MarchPlan{cols, want, !f64 && (W > 0.6 || W < 0.15)};
             }
         }
     }

@@ -4,6 +4,6 @@
 
 namespace dugks {
 template cudaError_t Launch<float,__half>::step_march(const StepParams<float> &, const MarchCoefs<float> &, const FastExtra<float> &, int, int, int, cudaStream_t);
-template cudaError_t Launch<float,__half>::batch_march(const BatchUniform<float> &, const MarchCoefs<float> &, const BatchGrid<float> *, const int4 *, int, int, double *, int, int, cudaStream_t);
-template int Launch<float,__half>::march_ctas_per_sm(int, int);
+template cudaError_t Launch<float,__half>::batch_step(const BatchUniform<float> &, const MarchCoefs<float> &, const BatchGrid<float> *, const int4 *, int, int, int, int, int, int, cudaStream_t);
+template int Launch<float,__half>::batch_ctas_per_sm(int, int, int);
 }  // namespace dugks

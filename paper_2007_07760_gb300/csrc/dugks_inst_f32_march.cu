@@ -4,6 +4,7 @@
 
 namespace dugks {
 template cudaError_t Launch<float,float>::step_march(const StepParams<float> &, const MarchCoefs<float> &, const FastExtra<float> &, int, int, int, cudaStream_t);
-template cudaError_t Launch<float,float>::batch_march(const BatchUniform<float> &, const MarchCoefs<float> &, const BatchGrid<float> *, const int4 *, int, int, double *, int, int, cudaStream_t);
-template int Launch<float,float>::march_ctas_per_sm(int, int);
+template cudaError_t Launch<float,float>::batch_step(const BatchUniform<float> &, const MarchCoefs<float> &, const BatchGrid<float> *, const int4 *, int, int, int, int, int, int, cudaStream_t);
+template int Launch<float,float>::batch_ctas_per_sm(int, int, int);
+template cudaError_t launch_batch_advance<float>(BatchGrid<float> *, int, int, double, cudaStream_t);
 }  // namespace dugks

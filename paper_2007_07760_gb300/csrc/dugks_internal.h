@@ -17,13 +17,11 @@ constexpr int TILE_X = 32;
 constexpr int TILE_Y = 8;
 constexpr int STEP_THREADS = 256;
 
-// Fast-kernel variants (warps per CTA x rows per thread): 0 = 8 x 4 (FP64: 8 x 2),
-// 1 = 16 x 1, 2 = 8 x 2, 3 = 12 x 3, 4 = 8 x 3, 5 = 10 x 4. Fewer rows per thread:
-// fewer registers and more resident warps, more halo overhead; taller tiles (3, 5):
-// less halo per cell, fewer resident CTAs.
+// Variants of the two-stage kernel of orders 2 and 3: rows of a segment of the row march,
+// 0 = 16, 1 = 8, 3 = 32, 5 = 64; 2 and 4 (the defaults) by the rule of march_plan.
 constexpr int FAST_VARIANTS = 6;
 
-// Geometry of a TMA-staged (fast) variant.
+// Geometry of a TMA-staged kernel (orders 4 and 5, and the three-stage scheme).
 struct FastGeom {
     int threads, tile_w, tile_h;   // cells written per CTA
     int box_w, box_h;              // state box (elements, rows)
@@ -38,19 +36,16 @@ struct Launch {
     static cudaError_t phi(const StepParams<T> &p, T *out, cudaStream_t s);
     // phi widened to double on the device (host read-out: one copy, no host conversion)
     static cudaError_t phi64(const StepParams<T> &p, double *out, cudaStream_t s);
-    static FastGeom fast_geom(int variant, int order = 3, int stages = 2);
-    static cudaError_t batch_step(const BatchUniform<T> &u, const FaceCoefs<T> &cf, const BatchGrid<T> *grids,
-                                  const int4 *items, int nitems, double *partials, int order, int flux, int variant,
-                                  int ctas, cudaStream_t s);
-    static int batch_ctas_per_sm(int order, int flux, int variant);
-    // the row march (two-stage, orders 2 and 3, phi a plane of its own): one strip segment
-    // of p.tile_h rows per CTA
+    static FastGeom fast_geom(int order, int stages);
+    // the row march (two-stage, orders 2 and 3): one strip segment of p.tile_h rows per CTA,
+    // `cols` columns a lane
     static cudaError_t step_march(const StepParams<T> &p, const MarchCoefs<T> &cf, const FastExtra<T> &fe, int flux,
                                   int cols, int early, cudaStream_t s);
-    static cudaError_t batch_march(const BatchUniform<T> &u, const MarchCoefs<T> &cf, const BatchGrid<T> *grids,
-                                   const int4 *items, int nitems, int max_rows, double *partials, int flux, int ctas,
-                                   cudaStream_t s);
-    static int march_ctas_per_sm(int flux, int rows);
+    // step `ofs` of a group for the grids of a work list; rows: the longest segment
+    static cudaError_t batch_step(const BatchUniform<T> &u, const MarchCoefs<T> &cf, const BatchGrid<T> *grids,
+                                  const int4 *items, int nitems, int rows, int ofs, int flux, int cols, int ctas,
+                                  cudaStream_t s);
+    static int batch_ctas_per_sm(int flux, int cols, int rows);
     // order 4 (radius-2 stencils) on the TMA-staged path, tile 8 warps x 2 rows: the
     // two-stage step (KIND_T2) or a kernel of the three-stage step (full storage only)
     static cudaError_t step_fast4(const StepParams<T> &p, const FaceCoefs<T, 2> &cf, const FastExtra<T> &fe,
@@ -65,10 +60,7 @@ struct Launch {
 };
 
 template <typename T>
-cudaError_t launch_batch_advance(BatchGrid<T> *grids, int ngrids, const double *partials, double *mass, int *status,
-                                 double dt, cudaStream_t s);
-template <typename T>
-cudaError_t launch_batch_factors(BatchGrid<T> *grids, int ngrids, double dt, cudaStream_t s);
+cudaError_t launch_batch_advance(BatchGrid<T> *grids, int ngrids, int n, double dt, cudaStream_t s);
 
 cudaError_t launch_mass_final(const double *partial, int n, double *out, int *status, cudaStream_t s);
 

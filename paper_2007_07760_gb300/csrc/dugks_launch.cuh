@@ -79,10 +79,6 @@ cudaError_t Launch<T, ST>::mass_partial(const StepParams<T> &p, cudaStream_t s) 
     return cudaGetLastError();
 }
 
-// rows of cells per thread in the fast kernel: 4 (FP32 arithmetic) or 2 (FP64)
-template <typename T>
-constexpr int fast_mr() { return sizeof(T) == 8 ? 2 : 4; }
-
 template <typename T, typename ST, int NW, int MR, int R = 1>
 static FastGeom geom_t() {
     using FT = FastTile<T, ST, NW, MR, R>;
@@ -98,19 +94,9 @@ template <typename T>
 constexpr int o4_mr() { return sizeof(T) == 8 ? 2 : 3; }
 
 template <typename T, typename ST>
-FastGeom Launch<T, ST>::fast_geom(int variant, int order, int stages) {
-    if (order >= 4) {   // one tile shape per scheme for radius-2 stencils (orders 4 and 5)
-        if (stages == 2) return geom_t<T, ST, o4_nw<T>(), o4_mr<T>(), 2>();
-        return geom_t<T, ST, 8, 2, 2>();
-    }
-    switch (variant) {
-    case 1: return geom_t<T, ST, 16, 1>();
-    case 2: return geom_t<T, ST, 8, 2>();
-    case 3: return geom_t<T, ST, 12, 3>();
-    case 4: return geom_t<T, ST, 8, 3>();
-    case 5: return geom_t<T, ST, 10, 4>();
-    default: return geom_t<T, ST, 8, fast_mr<T>()>();
-    }
+FastGeom Launch<T, ST>::fast_geom(int order, int stages) {
+    if (order >= 4 && stages == 2) return geom_t<T, ST, o4_nw<T>(), o4_mr<T>(), 2>();
+    return order >= 4 ? geom_t<T, ST, 8, 2, 2>() : geom_t<T, ST, 8, 2>();
 }
 
 template <typename T, int ORDER, int FLUX, int KIND>
@@ -197,6 +183,12 @@ cudaError_t Launch<T, ST>::step_fast4(const StepParams<T> &p, const FaceCoefs<T,
     return cudaErrorInvalidValue;
 }
 
+// CALL with the lane type of `cols` columns
+#define DUGKS_LANES(CALL)                                                                     \
+    if constexpr (!Store<T, ST>::deviation)                                                   \
+        if (cols == 1) return CALL(T);                                                        \
+    if constexpr (sizeof(T) == 4) return CALL(float2);
+
 template <typename V, typename ST, int FLUX, bool FIELD>
 static cudaError_t launch_march_t(const StepParams<typename Lane<V>::T> &p, const MarchCoefs<typename Lane<V>::T> &cf,
                                   const FastExtra<typename Lane<V>::T> &fe, int early, cudaStream_t s) {
@@ -226,35 +218,74 @@ static cudaError_t launch_march_v(const StepParams<typename Lane<V>::T> &p, cons
 template <typename T, typename ST>
 cudaError_t Launch<T, ST>::step_march(const StepParams<T> &p, const MarchCoefs<T> &cf, const FastExtra<T> &fe, int flux,
                                       int cols, int early, cudaStream_t s) {
-    if constexpr (!Store<T, ST>::deviation)
-        if (cols == 1) return launch_march_v<T, ST>(p, cf, fe, flux, early, s);
-    if constexpr (sizeof(T) == 4) return launch_march_v<float2, ST>(p, cf, fe, flux, early, s);
+#define CALL(V) launch_march_v<V, ST>(p, cf, fe, flux, early, s)
+    DUGKS_LANES(CALL)
+#undef CALL
     return cudaErrorInvalidValue;
 }
 
-template <typename T, typename ST>
-cudaError_t Launch<T, ST>::batch_march(const BatchUniform<T> &u, const MarchCoefs<T> &cf, const BatchGrid<T> *grids,
-                                       const int4 *items, int nitems, int max_rows, double *partials, int flux,
-                                       int ctas, cudaStream_t s) {
-    if (nitems <= 0) return cudaSuccess;
-    const int smem = MarchTile<float2, ST>::smem_bytes(max_rows), n = ctas < nitems ? ctas : nitems;
-    if (flux == 0) batch_march_kernel<float2, ST, 0><<<n, 32, smem, s>>>(u, cf, grids, items, nitems, partials);
-    else batch_march_kernel<float2, ST, 1><<<n, 32, smem, s>>>(u, cf, grids, items, nitems, partials);
-    return cudaGetLastError();
+// a launch that may be scheduled while the kernel ahead of it drains
+template <typename K, typename... A>
+static cudaError_t launch_dependent(K kern, int blocks, int threads, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+template <typename V, typename ST>
+static cudaError_t launch_batch_v(const BatchUniform<typename Lane<V>::T> &u, const MarchCoefs<typename Lane<V>::T> &cf,
+                                  const BatchGrid<typename Lane<V>::T> *grids, const int4 *items, int nitems, int rows,
+                                  int ofs, int flux, int ctas, cudaStream_t s) {
+    const int smem = MarchTile<V, ST>::smem_bytes(rows), n = ctas < nitems ? ctas : nitems;
+    return flux == 0 ? launch_dependent(batch_march_kernel<V, ST, 0>, n, 32, smem, s, u, cf, grids, items, nitems, ofs)
+                     : launch_dependent(batch_march_kernel<V, ST, 1>, n, 32, smem, s, u, cf, grids, items, nitems, ofs);
 }
 
 template <typename T, typename ST>
-int Launch<T, ST>::march_ctas_per_sm(int flux, int rows) {
+cudaError_t Launch<T, ST>::batch_step(const BatchUniform<T> &u, const MarchCoefs<T> &cf, const BatchGrid<T> *grids,
+                                      const int4 *items, int nitems, int rows, int ofs, int flux, int cols, int ctas,
+                                      cudaStream_t s) {
+    if (nitems <= 0) return cudaSuccess;
+#define CALL(V) launch_batch_v<V, ST>(u, cf, grids, items, nitems, rows, ofs, flux, ctas, s)
+    DUGKS_LANES(CALL)
+#undef CALL
+    return cudaErrorInvalidValue;
+}
+
+template <typename V, typename ST>
+static int batch_occupancy(int rows, int flux) {
     int n = 0;
-    const int smem = MarchTile<float2, ST>::smem_bytes(rows);
+    const int smem = MarchTile<V, ST>::smem_bytes(rows);
     const cudaError_t e =
-        flux == 0 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_march_kernel<float2, ST, 0>, 32, smem)
-                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_march_kernel<float2, ST, 1>, 32, smem);
+        flux == 0 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_march_kernel<V, ST, 0>, 32, smem)
+                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_march_kernel<V, ST, 1>, 32, smem);
     if (e != cudaSuccess) {
         cudaGetLastError();
         n = 1;
     }
     return n > 0 ? n : 1;
+}
+
+template <typename T, typename ST>
+int Launch<T, ST>::batch_ctas_per_sm(int flux, int cols, int rows) {
+#define CALL(V) batch_occupancy<V, ST>(rows, flux)
+    DUGKS_LANES(CALL)
+#undef CALL
+    return 1;
+}
+
+template <typename T>
+cudaError_t launch_batch_advance(BatchGrid<T> *grids, int ngrids, int n, double dt, cudaStream_t s) {
+    if (ngrids <= 0) return cudaSuccess;
+    return launch_dependent(batch_advance_kernel<T>, ngrids, 32, 0, s, grids, n, dt);
 }
 
 template <typename T, typename ST>
@@ -268,96 +299,6 @@ template <typename T, typename ST>
 cudaError_t Launch<T, ST>::phi64(const StepParams<T> &p, double *out, cudaStream_t s) {
     dim3 block(128), grid((p.nx + 127) / 128, p.ny);
     phi_kernel<T, ST, double><<<grid, block, 0, s>>>(p, out);
-    return cudaGetLastError();
-}
-
-
-template <typename T, typename ST, int ORDER, int FLUX, int NW, int MR>
-static cudaError_t launch_batch_t(const BatchUniform<T> &u, const FaceCoefs<T> &cf, const BatchGrid<T> *grids,
-                                  const int4 *items, int nitems, double *partials, int ctas, cudaStream_t s) {
-    using FT = FastTile<T, ST, NW, MR>;
-    auto kern = batch_fast_kernel<T, ST, ORDER, FLUX, NW, MR>;
-    // (the shared-memory attribute was set by batch_ctas_per_sm, outside any capture)
-    if (nitems <= 0) return cudaSuccess;
-    kern<<<ctas < nitems ? ctas : nitems, FT::NT, FT::smem_bytes, s>>>(u, cf, grids, items, nitems, partials);
-    return cudaGetLastError();
-}
-
-template <typename T, typename ST, int ORDER, int FLUX, int NW, int MR>
-static int batch_occupancy_t() {
-    using FT = FastTile<T, ST, NW, MR>;
-    auto kern = batch_fast_kernel<T, ST, ORDER, FLUX, NW, MR>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FT::smem_bytes);
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, FT::NT, FT::smem_bytes) != cudaSuccess) {
-        cudaGetLastError();
-        n = 1;
-    }
-    return n > 0 ? n : 1;
-}
-
-#define DUGKS_BATCH_DISPATCH(CALL)                                                            \
-    switch (variant) {                                                                        \
-    case 1: return CALL(16, 1);                                                               \
-    case 2: return CALL(8, 2);                                                                \
-    case 3: return CALL(12, 3);                                                               \
-    case 4: return CALL(8, 3);                                                                \
-    case 5: return CALL(10, 4);                                                               \
-    default: return CALL(8, fast_mr<T>());                                                    \
-    }
-
-template <typename T, typename ST, int ORDER, int FLUX>
-static cudaError_t launch_batch_v(const BatchUniform<T> &u, const FaceCoefs<T> &cf, const BatchGrid<T> *grids,
-                                  const int4 *items, int nitems, double *partials, int variant, int ctas,
-                                  cudaStream_t s) {
-#define CALL(NW, MR) launch_batch_t<T, ST, ORDER, FLUX, NW, MR>(u, cf, grids, items, nitems, partials, ctas, s)
-    DUGKS_BATCH_DISPATCH(CALL)
-#undef CALL
-}
-
-template <typename T, typename ST, int ORDER, int FLUX>
-static int batch_occ_v(int variant) {
-#define CALL(NW, MR) batch_occupancy_t<T, ST, ORDER, FLUX, NW, MR>()
-    DUGKS_BATCH_DISPATCH(CALL)
-#undef CALL
-}
-
-template <typename T, typename ST>
-cudaError_t Launch<T, ST>::batch_step(const BatchUniform<T> &u, const FaceCoefs<T> &cf, const BatchGrid<T> *grids,
-                                      const int4 *items, int nitems, double *partials, int order, int flux,
-                                      int variant, int ctas, cudaStream_t s) {
-    switch (order * 2 + flux) {
-    case 4: return launch_batch_v<T, ST, 2, 0>(u, cf, grids, items, nitems, partials, variant, ctas, s);
-    case 5: return launch_batch_v<T, ST, 2, 1>(u, cf, grids, items, nitems, partials, variant, ctas, s);
-    case 6: return launch_batch_v<T, ST, 3, 0>(u, cf, grids, items, nitems, partials, variant, ctas, s);
-    case 7: return launch_batch_v<T, ST, 3, 1>(u, cf, grids, items, nitems, partials, variant, ctas, s);
-    default: return cudaErrorInvalidValue;
-    }
-}
-
-template <typename T, typename ST>
-int Launch<T, ST>::batch_ctas_per_sm(int order, int flux, int variant) {
-    switch (order * 2 + flux) {
-    case 4: return batch_occ_v<T, ST, 2, 0>(variant);
-    case 5: return batch_occ_v<T, ST, 2, 1>(variant);
-    case 6: return batch_occ_v<T, ST, 3, 0>(variant);
-    case 7: return batch_occ_v<T, ST, 3, 1>(variant);
-    default: return 1;
-    }
-}
-
-template <typename T>
-cudaError_t launch_batch_advance(BatchGrid<T> *grids, int ngrids, const double *partials, double *mass, int *status,
-                                 double dt, cudaStream_t s) {
-    if (ngrids <= 0) return cudaSuccess;
-    batch_advance_kernel<T><<<ngrids, 256, 0, s>>>(grids, partials, mass, status, dt);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_batch_factors(BatchGrid<T> *grids, int ngrids, double dt, cudaStream_t s) {
-    if (ngrids <= 0) return cudaSuccess;
-    batch_factors_kernel<T><<<(ngrids + 127) / 128, 128, 0, s>>>(grids, ngrids, dt);
     return cudaGetLastError();
 }
 

@@ -37,12 +37,12 @@ namespace dugks {
 //   px, pe           row term px (R - L) + pe (L - 2 C + R) of the expansion at (c, 0)
 //   nu, nm, nd       weights of L + 4 C + R of the rows above, at and below at (0, c)
 //   ge, gp, gd, b2   ties: see the row terms G, Q and B in the kernel
-// Central: h and cp = 1/2 - h, cm = -1/2 - h, hk = h / 24.
+// Central: h, cu = 1/2 + h, cd = 1/2 - h, hk = h / 24.
 template <typename T>
 struct MarchCoefs {
     T dx[3][3], dy[3][3];
     T px, pe, nu, nm, nd, ge, gp, gd, b2;
-    T h, cp, cm, hk;
+    T h, cu, cd, hk;
 };
 
 // ---- a lane's columns of one row: a pair (float2, packed arithmetic) or one value -----
@@ -189,19 +189,17 @@ struct MarchTile {
 };
 static_assert(GHOST >= 5, "strips read 3 columns and rows past the grid");
 
-// What a new row j gives: the flux differences Dbar_k of row j - 1 (k = 1 .. 8) without
-// the part of row j's own cells, that part (late: Dbar_k - late_k is complete; upwind: of
-// the south faces, k = 6, 7, 8; central: of the diagonals), the sum of the late parts, and
-// the contributions of row j - 1 to the face moments phi_b of its four faces.
+// What a new row j gives: of row j - 1 the flux differences Dbar_k, without the differences over
+// rows that wait for row j's own cells; those (e) of row j - 2 (upwind: the south faces, k = 6, 7, 8;
+// central: the diagonals) and their sum; and the contributions of row j - 1 to the face moments
+// phi_b of its four faces. Everything is a difference of face values, taken before it is
+// added to anything: it vanishes where the state is uniform and keeps its digits elsewhere.
 template <typename V>
 struct RowOut {
     V D1, D2, D3, D4, D5, D6, D7, D8;
-    V l2, l4, l6, l7, l8, ls;
+    V e2, e4, e6, e7, e8, es;
     V PE, PW, PN, PS;
 };
-
-using PlusOne = std::integral_constant<int, 1>;
-using MinusOne = std::integral_constant<int, -1>;
 
 // What a row j has to give (uniform over the warp): finished values of row j - 1, its flux
 // differences, the middle terms of row j, the first terms of row j + 1. Only the first and
@@ -221,12 +219,12 @@ struct March<V, 0> {
     // pending expansions: "a" of row j - 1 (waits for row j), "b" of row j (has row j - 1)
     struct Diag { V xa, xb, ya, yb; } g2, g4, g6, g8;
     V z1, q1, z5, q5, z3, m3p, z7, m7p, zA, vAp, zB, vBp, zN, gNp, qN1, qN2;
-    V t3p, n2p, n4p;   // north-face values of row j - 2
+    V t3p, n2p, n4p, s6p, s7p, s8p;   // north- and south-face values of row j - 2
 
     __device__ __forceinline__ void clear(V z) {
         g2 = g4 = g6 = g8 = Diag{z, z, z, z};
         z1 = q1 = z5 = q5 = z3 = m3p = z7 = m7p = zA = vAp = zB = vBp = zN = gNp = qN1 = qN2 = z;
-        t3p = n2p = n4p = z;
+        t3p = n2p = n4p = s6p = s7p = s8p = z;
     }
 
     // a diagonal's row in the basis of its weights: C, R + L, R - L, or C, L, R
@@ -273,11 +271,11 @@ struct March<V, 0> {
 
     __device__ __forceinline__ void advance(const MarchCoefs<T> &cf, V F0, V F1, V F2, V F3, V F4, V F5, V F6, V F7,
                                             V F8, RowOut<V> &o, Need n) {
-        V E2{}, E8{}, W4{}, W6{}, N2{}, N4{};
+        V E2{}, E8{}, W4{}, W6{}, N2{}, N4{}, S6{}, S8{};
         diagonal<1, 1>(cf, F2, g2, E2, N2, n);
-        diagonal<1, -1>(cf, F8, g8, E8, o.l8, n);
+        diagonal<1, -1>(cf, F8, g8, E8, S8, n);
         diagonal<-1, 1>(cf, F4, g4, W4, N4, n);
-        diagonal<-1, -1>(cf, F6, g6, W6, o.l6, n);
+        diagonal<-1, -1>(cf, F6, g6, W6, S6, n);
         const Sides<V> i0 = vsides(F0), i1 = vsides(F1), i5 = vsides(F5), i3 = vsides(F3), i7 = vsides(F7);
         // east face of k = 1, west face of k = 5
         const V e1 = vfma(T(-2), F1, i1.s), e5 = vfma(T(-2), F5, i5.s);
@@ -294,7 +292,7 @@ struct March<V, 0> {
         const V T3 = vfma(cf.nu, m3, z3);
         if (n.mid) z3 = vfma(cf.nd, m3p, vfma(cf.nm, m3, F3));
         m3p = m3;
-        o.l7 = vfma(cf.nd, m7, z7);
+        const V T7 = vfma(cf.nd, m7, z7);
         if (n.mid) z7 = vfma(cf.nu, m7p, vfma(cf.nm, m7, F7));
         m7p = m7;
         // k = 0, 3, 7 at the east and west faces (weight 1/2 each): A even and B odd in x
@@ -330,9 +328,16 @@ struct March<V, 0> {
             qN1 = Q;
         }
         if (!n.out) return;
-        o.ls = vadd(o.l7, vadd(o.l6, o.l8));
         o.PN = vadd(vadd(T3, vadd(N2, N4)), vadd(A, B));
-        o.PS = vadd(o.ls, vsub(A, B));
+        o.PS = vadd(vadd(T7, vadd(S6, S8)), vsub(A, B));
+        // xi_y (f_N(c) - f_N(c - N)) for the directions that come from the row above
+        o.e6 = vsub(s6p, S6);
+        o.e7 = vsub(s7p, T7);
+        o.e8 = vsub(s8p, S8);
+        o.es = vadd(o.e7, vadd(o.e6, o.e8));
+        s6p = S6;
+        s7p = T7;
+        s8p = S8;
         if (n.flux) {
             // Dbar_k = xi_x (f_E(c) - f_E(c - E)) + xi_y (f_N(c) - f_N(c - N))
             o.D1 = vless_left(T1);
@@ -340,9 +345,8 @@ struct March<V, 0> {
             o.D2 = vadd(vless_left(E2), vsub(N2, n2p));
             o.D4 = vadd(vless_right(W4), vsub(N4, n4p));
             o.D3 = vsub(T3, t3p);
-            o.D6 = vadd(vless_right(W6), o.l6);
-            o.D7 = o.l7;
-            o.D8 = vadd(vless_left(E8), o.l8);
+            o.D6 = vless_right(W6);
+            o.D8 = vless_left(E8);
         }
         n2p = N2;
         n4p = N4;
@@ -351,63 +355,65 @@ struct March<V, 0> {
 };
 
 // Central faces (Eq. (25)): f_E = (F_c + F_E) / 2 - h [xi_x (F_E - F_c) + xi_y (gy_c + gy_E) / 2] and
-// likewise north. Their differences over a cell are, per direction,
-//   xi_x (R - L) / 2 - h xi_x^2 (L - 2 C + R), the same over rows, and for a diagonal
-//   - h xi_x xi_y / 2 [gy(c + E) - gy(c - E) + gx(c + N) - gx(c - N)],
-// and their sums over k need the gradients of sum_k xi_y F_k and sum_k xi_x F_k only.
+// likewise north: a part of each of the two cells. The face values are formed and then differenced,
+// so that what one cell loses its neighbour gains whatever the coefficients' rounding. Their sums
+// over k need the gradients of sum_k xi_y F_k and sum_k xi_x F_k only.
 template <typename V>
 struct March<V, 1> {
     using T = typename Lane<V>::T;
     struct Diag {
-        V z, c1, m1, m2, zg, d1, gp;   // pending sum and C, m of rows j - 1, j - 2, gx pending, d, 12 gx of row j - 2
+        V c1, m1, m2, zg, d1, nu, fn;   // C, m of row j - 1, m of row j - 2, gx pending, d; of f_N: own part of row j - 2, row j - 3
     } a2, a4, a6, a8;
-    V q1, q5, z3, c3, z7, c7;          // row j - 1 (k = 1, 5); pending sums and C of row j - 1 (k = 3, 7)
+    V q1, q5, z3, f3, z7, f7;       // Dbar of row j - 1 (k = 1, 5); own part of f_N of row j - 1, f_N of row j - 2 (k = 3, 7)
     V M0p, Mxp, Myp, my1, my2, zx, dx1;
 
     __device__ __forceinline__ void clear(V z) {
         a2 = a4 = a6 = a8 = Diag{z, z, z, z, z, z, z};
-        q1 = q5 = z3 = c3 = z7 = c7 = M0p = Mxp = Myp = my1 = my2 = zx = dx1 = z;
+        q1 = q5 = z3 = f3 = z7 = f7 = M0p = Mxp = Myp = my1 = my2 = zx = dx1 = z;
+    }
+
+    // a row of a diagonal (SX, SY): the difference over columns of row j - 1, over rows of row j - 2
+    template <int SX, int SY>
+    __device__ static __forceinline__ void diagonal(const MarchCoefs<T> &cf, Diag &g, V C, V &D, V &e) {
+        const Sides<V> q = vsides(C);
+        const V m = vfma(T(4), C, q.s);
+        const V gy = vmul(T(SY) * cf.hk, vsub(m, g.m2)), gx = vmul(T(SX) * cf.hk, vadd(g.zg, q.d));   // row j - 1
+        // weights 1/2 + h, 1/2 - h of the upwind and the downwind cell
+        const T up = cf.cu, dn = cf.cd;
+        const V fE = vplus_right(vfma(SX > 0 ? up : dn, g.c1, vneg(gy)), vfma(SX > 0 ? dn : up, g.c1, vneg(gy)));
+        const V own = vfma(SY > 0 ? up : dn, g.c1, vneg(gx)), south = vfma(SY > 0 ? dn : up, g.c1, vneg(gx));
+        const V fN = vadd(g.nu, south);   // of row j - 2
+        D = SX > 0 ? vless_left(fE) : vneg(vless_left(fE));
+        e = SY > 0 ? vsub(fN, g.fn) : vsub(g.fn, fN);
+        g.fn = fN;
+        g.nu = own;
+        g.c1 = C;
+        g.m2 = g.m1;
+        g.m1 = m;
+        g.zg = vfma(T(4), q.d, g.d1);
+        g.d1 = q.d;
     }
 
     __device__ __forceinline__ void advance(const MarchCoefs<T> &cf, V F0, V F1, V F2, V F3, V F4, V F5, V F6, V F7,
                                             V F8, RowOut<V> &o, Need) {
-        const T h = cf.h, hk = cf.hk, cp = cf.cp, cm = cf.cm;
-        auto diag = [&](Diag &g, V C, auto sx, auto sy, V &D, V &late) {
-            constexpr int SX = decltype(sx)::value, SY = decltype(sy)::value;
-            const Sides<V> q = vsides(C);
-            const V s = q.s, d = q.d;
-            const V m = vfma(T(4), C, s);
-            const V gy = vsub(m, g.m2);            // 12 gy of row j - 1
-            const V gx = vadd(g.zg, d);            // 12 gx of row j - 1
-            const V dg = vsides(gy).d;
-            const T k = T(SX * SY) * hk;
-            D = vfma(-k, vsub(dg, g.gp), vfma(SY > 0 ? cp : cm, C, g.z));
-            late = vmul(k, gx);
-            g.z = vfma(SY > 0 ? cm : cp, g.c1, vfma(T(0.5 * SX), d, vfma(-h, s, vmul(T(4) * h, C))));
-            g.c1 = C;
-            g.m2 = g.m1;
-            g.m1 = m;
-            g.zg = vfma(T(4), d, g.d1);
-            g.d1 = d;
-            g.gp = gx;
-        };
-        diag(a2, F2, PlusOne{}, PlusOne{}, o.D2, o.l2);
-        diag(a4, F4, MinusOne{}, PlusOne{}, o.D4, o.l4);
-        diag(a6, F6, MinusOne{}, MinusOne{}, o.D6, o.l6);
-        diag(a8, F8, PlusOne{}, MinusOne{}, o.D8, o.l8);
-        o.l7 = V{};
-        o.ls = vadd(vadd(o.l2, o.l4), vadd(o.l6, o.l8));
+        const T h = cf.h, hk = cf.hk, up = cf.cu, dn = cf.cd;
+        diagonal<1, 1>(cf, a2, F2, o.D2, o.e2);
+        diagonal<-1, 1>(cf, a4, F4, o.D4, o.e4);
+        diagonal<-1, -1>(cf, a6, F6, o.D6, o.e6);
+        diagonal<1, -1>(cf, a8, F8, o.D8, o.e8);
+        o.es = vadd(vadd(o.e2, o.e4), vadd(o.e6, o.e8));
         o.D1 = q1;
-        o.D5 = q5;
-        const Sides<V> h1 = vsides(F1), h5 = vsides(F5);
-        q1 = vfma(T(0.5), h1.d, vfma(-h, h1.s, vmul(T(2) * h, F1)));
-        q5 = vfma(T(-0.5), h5.d, vfma(-h, h5.s, vmul(T(2) * h, F5)));
-        o.D3 = vfma(cp, F3, z3);
-        z3 = vfma(cm, c3, vmul(T(2) * h, F3));
-        c3 = F3;
-        o.D7 = vfma(cm, F7, z7);
-        z7 = vfma(cp, c7, vmul(T(2) * h, F7));
-        c7 = F7;
+        o.D5 = vneg(q5);
+        q1 = vless_left(vplus_right(vmul(up, F1), vmul(dn, F1)));
+        q5 = vless_left(vplus_right(vmul(dn, F5), vmul(up, F5)));
+        V f = vfma(dn, F3, z3);   // f_N of row j - 1
+        o.D3 = vsub(f, f3);
+        f3 = f;
+        z3 = vmul(up, F3);
+        f = vfma(up, F7, z7);
+        o.D7 = vsub(f7, f);
+        f7 = f;
+        z7 = vmul(dn, F7);
         const V e = vadd(F2, F8), w = vadd(F4, F6), n = vadd(F2, F4), u = vadd(F6, F8);
         const V M0 = vadd(vadd(F0, vadd(F1, F5)), vadd(vadd(F3, F7), vadd(e, w)));
         const V Mx = vadd(vsub(F1, F5), vsub(e, w)), My = vadd(vsub(F3, F7), vsub(n, u));
@@ -429,8 +435,9 @@ struct March<V, 1> {
 };
 
 // One strip (rows y0 .. y0 + rows - 1) of one grid. FIELD: the velocity is given at cell
-// centres (p.ufield, p.vfield).
-template <typename V, typename ST, int FLUX, bool FIELD>
+// centres (p.ufield, p.vfield). MASS: its sum of phi goes to mass_out; otherwise a value that is
+// not finite raises the status flag.
+template <typename V, typename ST, int FLUX, bool FIELD, bool MASS>
 __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T> &p,
                                             const MarchCoefs<typename Lane<V>::T> &cf,
                                             const FastExtra<typename Lane<V>::T> &fe, int bx, int y0, int rows,
@@ -632,6 +639,7 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
     V v0x{}, v0y{}, v1x{}, v1y{};      // V of rows j - 1, j - 2
     V f0p{}, f1p{}, f2p{};             // north-face moments of row j - 3
     double msum = 0.0;
+    V check{};                         // 0, or NaN once a value was not finite
     uint32_t cslot = 0;
     const uint32_t seed = PHIP ? mix32(p.seed) : 0u;
     // lanes whose columns have images in the ghost border left or right of the grid
@@ -787,16 +795,16 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
             const V B1 = vless_left(x1), B2 = vadd(vless_left(x2), vsub(y1, f1p)), B3 = vsub(y2, f2p);
             const V S13 = vadd(B1, B3);
             // new phi = phi + gamma sum_k L_k (sum_k w_k xi_k = 0, sum_k w_k xi_a xi_b = delta_ab / 3)
-            const V dph = vfma(T(-1.0 / 3.0), S13, vmul(-gmc, vsub(sDp, ro.ls)));
+            const V dph = vfma(T(-1.0 / 3.0), S13, vmul(-gmc, vadd(sDp, ro.es)));
             if constexpr (PHIP) phn = vadd_sr(pc3, dph, (uint32_t)y * (uint32_t)nx + (uint32_t)x, seed);
             else phn = vadd(pc3, dph);
             {
                 // gamma w_k (c2 Phi_k + c3 Psi_k) = w_k (xi_x A1 + xi_y A2 + xi_x^2 B1 + xi_x xi_y B2 + xi_y^2 B3)
                 const T w1 = wq<T>(1), w2 = wq<T>(2);
-                // (the late parts of Dbar)
-                const V p7 = FLUX == 0 ? vfma(gmc, ro.l7, r7) : r7;
-                const V p6 = vfma(gmc, ro.l6, r6), p8 = vfma(gmc, ro.l8, r8);
-                const V p2 = FLUX == 0 ? r2 : vfma(gmc, ro.l2, r2), p4 = FLUX == 0 ? r4 : vfma(gmc, ro.l4, r4);
+                // (the differences over rows that waited)
+                const V p7 = FLUX == 0 ? vfma(-gmc, ro.e7, r7) : r7;
+                const V p6 = vfma(-gmc, ro.e6, r6), p8 = vfma(-gmc, ro.e8, r8);
+                const V p2 = FLUX == 0 ? r2 : vfma(-gmc, ro.e2, r2), p4 = FLUX == 0 ? r4 : vfma(-gmc, ro.e4, r4);
                 o[1] = vfma(-w1, vadd(B1, A1), r1);
                 o[5] = vfma(-w1, vsub(B1, A1), r5);
                 o[3] = vfma(-w1, vadd(B3, A2), r3);
@@ -823,9 +831,9 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
         r4 = vfma(-gmc, ro.D4, b4);
         r5 = vfma(-gmc, ro.D5, b5);
         r6 = vfma(-gmc, ro.D6, b6);
-        r7 = vfma(-gmc, ro.D7, b7);
+        r7 = FLUX == 0 ? b7 : vfma(-gmc, ro.D7, b7);
         r8 = vfma(-gmc, ro.D8, b8);
-        sDp = vadd(vadd(vadd(ro.D1, ro.D2), vadd(ro.D3, ro.D4)), vadd(vadd(ro.D5, ro.D6), vadd(ro.D7, ro.D8)));
+        sDp = vadd(vadd(vadd(ro.D1, ro.D2), vadd(ro.D3, ro.D4)), vadd(vadd(ro.D5, ro.D6), FLUX == 0 ? ro.D8 : vadd(ro.D7, ro.D8)));
         phEp = vplus_right(ro.PE, ro.PW);
         }
         pNp = ro.PN;
@@ -873,8 +881,12 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
         } else if (st1) {
             put1(g);
         }
-        if (st0) msum += (double)LN::first(phn);
-        if (st1) msum += (double)LN::second(phn);
+        if constexpr (MASS) {
+            if (st0) msum += (double)LN::first(phn);
+            if (st1) msum += (double)LN::second(phn);
+        } else {
+            if (st0 || st1) check = vfma(T(0), phn, check);
+        }
         // periodic images in the ghost border
         if ((st0 || st1) && (xedge || y < GHOST || y >= ny - GHOST)) {
 #pragma unroll 1
@@ -889,9 +901,12 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
         }
     }
     cp_wait<0>();
-    if (mass_out != nullptr) {
+    if constexpr (MASS) {
         for (int o = 16; o > 0; o >>= 1) msum += __shfl_down_sync(ALL, msum, o);
         if (lane == 0) *mass_out = msum;
+    } else {
+        const bool bad = (ok0 && !(LN::first(check) == T(0))) || (ok1 && !(LN::second(check) == T(0)));
+        if (__any_sync(ALL, bad) && lane == 0) atomicOr(p.status, 1);
     }
 }
 
@@ -906,31 +921,130 @@ step_march_kernel(const __grid_constant__ StepParams<typename Lane<V>::T> p,
     extern __shared__ __align__(128) unsigned char smem[];
     if (early) pdl_trigger();
     const int y0 = blockIdx.y * p.tile_h;
-    march_strip<V, ST, FLUX, FIELD>(p, cf, fe, blockIdx.x, y0, min(p.tile_h, p.ny - y0),
-                                    p.mass_partial ? p.mass_partial + blockIdx.y * p.tiles_x + blockIdx.x : nullptr,
-                                    smem);
+    march_strip<V, ST, FLUX, FIELD, true>(p, cf, fe, blockIdx.x, y0, min(p.tile_h, p.ny - y0),
+                                          p.mass_partial + blockIdx.y * p.tiles_x + blockIdx.x, smem);
     if (!early) pdl_trigger();
 }
 
-// Many grids: CTAs stride over the work list (grid, strip, first row, rows).
+// ---- many grids per launch ----------------------------------------------------
+// Steps that one replayed graph takes; the reversal factors of that many are kept ready.
+constexpr int GRAPH_STEPS = 8;
+
+// Per-grid descriptor of a batch, in device memory. `step` counts the grid's steps; with the
+// launch's offset in its group it selects the ping-pong state set and the phi plane roles. It is
+// advanced by batch_advance_kernel at the end of the group, so a captured sequence of launches
+// stays valid while grids join and leave (their step counters differ).
+template <typename T>
+struct BatchGrid {
+    void *X[2];              // state sets 0, 1
+    T *phi[3];               // phi planes
+    long long step, target;  // steps taken; the grid is frozen once step == target
+    size_t plane;
+    int nx, ny, pitch, tile_w;
+    int vel_kind, pad_;
+    double vp[3];            // velocity parameters (FP64; rounded per precision in the kernel)
+    T vc[GRAPH_STEPS][3];    // single vortex: cos(pi t / T) at t, t - dt, t + dt/2 of the next steps
+};
+
+// Parameters common to every grid of a batch (same W, M, cfl, order, flux, precision).
+template <typename T>
+struct BatchUniform {
+    T b, h, c1, c2, c3, be1, ga1, tau, theta_c, phiA, phiB, inv_dt, qscale, qinv;
+    double dt;
+    int dtphiu;
+    int *status;
+};
+
+// The parameters of a grid's step `ofs` of the group.
+template <typename T, typename ST>
+__device__ __forceinline__ void batch_step_params(const BatchUniform<T> &u, const BatchGrid<T> *G, int ofs,
+                                                  StepParams<T> &p, FastExtra<T> &fe) {
+    const long long step = G->step + ofs;
+    p.nx = G->nx;
+    p.ny = G->ny;
+    p.pitch = G->pitch;
+    p.plane = G->plane;
+    p.tile_w = G->tile_w;
+    p.status = u.status;
+    p.ufield = p.vfield = nullptr;
+    p.b = u.b;
+    p.c2 = u.c2;
+    p.c3 = u.c3;
+    p.be1 = u.be1;
+    p.ga1 = u.ga1;
+    p.tau = u.tau;
+    p.theta_c = u.theta_c;
+    p.phiA = u.phiA;
+    p.phiB = u.phiB;
+    p.inv_dtD = u.inv_dt;
+    p.useD = (u.dtphiu && step > 0) ? 1 : 0;
+    p.seed = (uint32_t)step;
+    p.vel_kind = G->vel_kind;
+    p.vp0 = (T)G->vp[0];
+    p.vp1 = (T)G->vp[1];
+    p.vp2 = (T)G->vp[2];
+    p.qscale = u.qscale;
+    p.qinv = u.qinv;
+    fe.vc_t = G->vc[ofs][0];
+    fe.vc_told = G->vc[ofs][1];
+    fe.vc_tface = G->vc[ofs][2];
+    const int cur = (int)(step & 1);
+    p.X = G->X[cur];
+    p.out1 = G->X[1 - cur];
+    int iPc = 0, iPo, iOut;
+    if constexpr (Store<T, ST>::phi_plane) {   // roles rotate with period 3 (see the context API)
+        iPc = (3 - (int)(step % 3)) % 3;
+        iPo = (iPc + 1) % 3;
+        iOut = (iPc + 2) % 3;
+        p.phi_cur = G->phi[iPc];
+    } else {
+        iPo = cur;
+        iOut = 1 - cur;
+        p.phi_cur = nullptr;
+    }
+    p.phi_old = G->phi[iPo];
+    p.phi_out = G->phi[iOut];
+}
+
+// Step `ofs` of the group: CTAs stride over the work list (grid, strip, first row, rows).
 template <typename V, typename ST, int FLUX>
-__global__ void __launch_bounds__(32, 8)
+__global__ void __launch_bounds__(32, (sizeof(V) == 4 ? 12 : 8))
 batch_march_kernel(const __grid_constant__ BatchUniform<typename Lane<V>::T> u,
                    const __grid_constant__ MarchCoefs<typename Lane<V>::T> cf,
                    const BatchGrid<typename Lane<V>::T> *__restrict__ grids, const int4 *__restrict__ items, int nitems,
-                   double *__restrict__ partials) {
+                   int ofs) {
     using T = typename Lane<V>::T;
     extern __shared__ __align__(128) unsigned char smem[];
+    pdl_wait();   // the previous step's output, or the advanced descriptors
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const int4 w = items[it];
         const BatchGrid<T> *G = grids + w.x;
-        if (G->step >= G->target) continue;   // frozen grid
+        if (G->step + ofs >= G->target) continue;   // frozen grid
         StepParams<T> p;
         FastExtra<T> fe;
-        batch_step_params<T, ST>(u, G, p, fe);
-        march_strip<V, ST, FLUX, false>(p, cf, fe, w.y, w.z, w.w, partials + it, smem);
+        batch_step_params<T, ST>(u, G, ofs, p, fe);
+        march_strip<V, ST, FLUX, false, false>(p, cf, fe, w.y, w.z, w.w, nullptr, smem);
         __syncwarp();   // the next strip's copies overwrite the ring
     }
+    pdl_trigger();
+}
+
+// After a group of `n` steps (n = 0: after an upload of the descriptors): the step counters, and
+// the reversal factors of the vortex for the next group. FP64 is slow on this chip and its cost
+// does not fall with idle lanes: one lane a factor.
+template <typename T>
+__global__ void __launch_bounds__(32) batch_advance_kernel(BatchGrid<T> *grids, int n, double dt) {
+    pdl_wait();
+    BatchGrid<T> *G = grids + blockIdx.x;
+    const long long step = n > 0 && G->step < G->target ? min(G->step + n, G->target) : G->step;
+    __syncwarp();
+    if (threadIdx.x == 0) G->step = step;
+    if (G->vel_kind == VEL_VORTEX && threadIdx.x < 3 * GRAPH_STEPS) {
+        const int i = threadIdx.x / 3, q = threadIdx.x - 3 * i;
+        const double t = (double)(step + i) * dt;
+        G->vc[i][q] = (T)cospi((q == 0 ? t : q == 1 ? t - dt : t + 0.5 * dt) / G->vp[2]);
+    }
+    pdl_trigger();
 }
 
 }  // namespace dugks
