@@ -46,7 +46,7 @@ struct dugks_ctx {
     int tile_w = TILE_X, tile_h = TILE_Y, tiles_x = 0, ntiles = 0;
     // TMA-staged two-stage path (orders 2, 3)
     bool fast = false;
-    bool march = false;         // fast, as a row march (two-stage, orders 2 and 3)
+    bool march = false;         // fast, as a row march (orders 2 and 3)
     MarchPlan plan{};
     int variant = 0;
     CUtensorMap tmX[2], tmPhi[4];
@@ -144,7 +144,7 @@ bool encode_map(CUtensorMap *m, void *base, size_t es, bool half, const dugks_ct
 }
 
 // whether the fast path of this context is the row march
-bool marches(const dugks_ctx *c) { return c->p.stages == 2 && c->p.order <= 3; }
+bool marches(const dugks_ctx *c) { return (c->p.stages == 2 || c->p.stages == 3) && c->p.order <= 3; }
 
 template <typename T, typename ST>
 bool setup_fast(dugks_ctx *c) {
@@ -156,7 +156,7 @@ bool setup_fast(dugks_ctx *c) {
         c->tile_h = march_segment_rows(c->plan.rows, size.y);
         return true;
     }
-    const FastGeom g = Launch<T, ST>::fast_geom(c->p.order, c->p.stages);
+    const FastGeom g = Launch<T, ST>::fast_geom(c->p.stages);
     const bool half = Store<T, ST>::deviation;
     for (int s = 0; s < 2; s++)
         if (!encode_map(&c->tmX[s], c->X[s], sizeof(ST), half, c, 9, g.box_w, g.box_h)) return false;
@@ -355,8 +355,8 @@ int step_t3(dugks_ctx *c) {
             keep(c->coefs3[0], make_face_coefs_r<T, 2>(4, c->p.flux, dt / 6.0));
             keep(c->coefs3[1], make_face_coefs_r<T, 2>(4, c->p.flux, 5.0 * dt / 12.0));
         } else {
-            keep(c->coefs3[0], make_face_coefs<T>(c->p.order, c->p.flux, dt / 6.0));
-            keep(c->coefs3[1], make_face_coefs<T>(c->p.order, c->p.flux, 5.0 * dt / 12.0));
+            keep(c->coefs3[0], make_march_coefs<T>(c->p.order, dt / 6.0));
+            keep(c->coefs3[1], make_march_coefs<T>(c->p.order, 5.0 * dt / 12.0));
         }
         c->coef3_dt = dt;
     }
@@ -365,9 +365,9 @@ int step_t3(dugks_ctx *c) {
                                      vortex_factors<T>(c, t, t - dt, t + dt / 6.0), c->tmX[0], c->tmPhi[aPo],
                                      c->tmPhi[aPc], c->p.flux, KIND_T3A, c->stream);
     } else if (c->fast) {
-        const FaceCoefs<T> &cf = *reinterpret_cast<const FaceCoefs<T> *>(c->coefs3[0].data());
-        e = Launch<T, T>::step_fast3(A, cf, vortex_factors<T>(c, t, t - dt, t + dt / 6.0), c->tmX[0],
-                                     c->tmPhi[aPo], c->tmPhi[aPc], c->p.order, c->p.flux, KIND_T3A, c->stream);
+        e = Launch<T, T>::step_march3(A, *reinterpret_cast<const MarchCoefs<T> *>(c->coefs3[0].data()),
+                                      vortex_factors<T>(c, t, t - dt, t + dt / 6.0), c->p.flux, KIND_T3A,
+                                      c->plan.cols, c->plan.early, c->stream);
     } else {
         e = Launch<T, T>::step(A, c->p.order, c->p.flux, KIND_T3A, c->stream);
     }
@@ -403,9 +403,9 @@ int step_t3(dugks_ctx *c) {
                                      vortex_factors<T>(c, t + dt / 3.0, t, t + 0.75 * dt), c->tmX[1],
                                      c->tmPhi[bPo], c->tmPhi[bPc], c->p.flux, KIND_T3B, c->stream);
     } else if (c->fast) {
-        const FaceCoefs<T> &cf = *reinterpret_cast<const FaceCoefs<T> *>(c->coefs3[1].data());
-        e = Launch<T, T>::step_fast3(B, cf, vortex_factors<T>(c, t + dt / 3.0, t, t + 0.75 * dt), c->tmX[1],
-                                     c->tmPhi[bPo], c->tmPhi[bPc], c->p.order, c->p.flux, KIND_T3B, c->stream);
+        e = Launch<T, T>::step_march3(B, *reinterpret_cast<const MarchCoefs<T> *>(c->coefs3[1].data()),
+                                      vortex_factors<T>(c, t + dt / 3.0, t, t + 0.75 * dt), c->p.flux, KIND_T3B,
+                                      c->plan.cols, c->plan.early, c->stream);
     } else {
         e = Launch<T, T>::step(B, c->p.order, c->p.flux, KIND_T3B, c->stream);
     }

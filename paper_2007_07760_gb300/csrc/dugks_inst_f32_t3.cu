@@ -1,7 +1,7 @@
-// TMA-staged kernels of the three-stage step; state and arithmetic in float.
+// row-march kernels of the three-stage step (orders 2 and 3); state and arithmetic in float.
 // (One translation unit per precision and kernel family, so they compile in parallel.)
 #include "dugks_launch.cuh"
 
 namespace dugks {
-template cudaError_t Launch<float,float>::step_fast3(const StepParams<float> &, const FaceCoefs<float> &, const FastExtra<float> &, const CUtensorMap &, const CUtensorMap &, const CUtensorMap &, int, int, int, cudaStream_t);
+template cudaError_t Launch<float,float>::step_march3(const StepParams<float> &, const MarchCoefs<float> &, const FastExtra<float> &, int, int, int, int, cudaStream_t);
 }  // namespace dugks

@@ -21,7 +21,7 @@ constexpr int STEP_THREADS = 256;
 // 0 = 16, 1 = 8, 3 = 32, 5 = 64; 2 and 4 (the defaults) by the rule of march_plan.
 constexpr int FAST_VARIANTS = 6;
 
-// Geometry of a TMA-staged kernel (orders 4 and 5, and the three-stage scheme).
+// Geometry of a TMA-staged kernel (orders 4 and 5).
 struct FastGeom {
     int threads, tile_w, tile_h;   // cells written per CTA
     int box_w, box_h;              // state box (elements, rows)
@@ -36,7 +36,7 @@ struct Launch {
     static cudaError_t phi(const StepParams<T> &p, T *out, cudaStream_t s);
     // phi widened to double on the device (host read-out: one copy, no host conversion)
     static cudaError_t phi64(const StepParams<T> &p, double *out, cudaStream_t s);
-    static FastGeom fast_geom(int order, int stages);
+    static FastGeom fast_geom(int stages);
     // the row march (two-stage, orders 2 and 3): one strip segment of p.tile_h rows per CTA,
     // `cols` columns a lane
     static cudaError_t step_march(const StepParams<T> &p, const MarchCoefs<T> &cf, const FastExtra<T> &fe, int flux,
@@ -51,12 +51,10 @@ struct Launch {
     static cudaError_t step_fast4(const StepParams<T> &p, const FaceCoefs<T, 2> &cf, const FastExtra<T> &fe,
                                   const CUtensorMap &tmX, const CUtensorMap &tmPo, const CUtensorMap &tmPc, int flux,
                                   int kind, cudaStream_t s);
-    // one kernel of the three-stage step (kind KIND_T3A or KIND_T3B) on the TMA-staged
-    // path, tile 8 warps x 2 rows (full storage only: ST == T); tmPc maps the plane of
-    // phi of X where phi is a plane of its own (FP32)
-    static cudaError_t step_fast3(const StepParams<T> &p, const FaceCoefs<T> &cf, const FastExtra<T> &fe,
-                                  const CUtensorMap &tmX, const CUtensorMap &tmPo, const CUtensorMap &tmPc, int order,
-                                  int flux, int kind, cudaStream_t s);
+    // one kernel of the three-stage step (kind KIND_T3A or KIND_T3B; full storage only) as a
+    // row march, orders 2 and 3
+    static cudaError_t step_march3(const StepParams<T> &p, const MarchCoefs<T> &cf, const FastExtra<T> &fe, int flux,
+                                   int kind, int cols, int early, cudaStream_t s);
 };
 
 template <typename T>

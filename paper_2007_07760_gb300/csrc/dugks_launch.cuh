@@ -94,51 +94,8 @@ template <typename T>
 constexpr int o4_mr() { return sizeof(T) == 8 ? 2 : 3; }
 
 template <typename T, typename ST>
-FastGeom Launch<T, ST>::fast_geom(int order, int stages) {
-    if (order >= 4 && stages == 2) return geom_t<T, ST, o4_nw<T>(), o4_mr<T>(), 2>();
-    return order >= 4 ? geom_t<T, ST, 8, 2, 2>() : geom_t<T, ST, 8, 2>();
-}
-
-template <typename T, int ORDER, int FLUX, int KIND>
-static cudaError_t launch_fast3_t(const StepParams<T> &p, const FaceCoefs<T> &cf, const FastExtra<T> &fe,
-                                  const CUtensorMap &tmX, const CUtensorMap &tmPo, const CUtensorMap &tmPc,
-                                  cudaStream_t s) {
-    using FT = FastTile<T, T, 8, 2>;
-    constexpr size_t smem = KIND == KIND_T3A ? FT::smem_bytes_t3a : FT::smem_bytes;
-    auto kern = step_fast_kernel<T, T, ORDER, FLUX, 8, 2, KIND>;
-    static std::atomic<uint64_t> configured{0};
-    if (cudaError_t e = smem_attr_once(kern, (int)smem, configured); e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((p.nx + FT::TX - 1) / FT::TX, (p.ny + FT::TY - 1) / FT::TY);
-    cfg.blockDim = dim3(FT::NT);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, p, cf, fe, tmX, tmPo, tmPc);
-}
-
-template <typename T, typename ST>
-cudaError_t Launch<T, ST>::step_fast3(const StepParams<T> &p, const FaceCoefs<T> &cf, const FastExtra<T> &fe,
-                                      const CUtensorMap &tmX, const CUtensorMap &tmPo, const CUtensorMap &tmPc,
-                                      int order, int flux, int kind, cudaStream_t s) {
-#define DUGKS_T3(O, F)                                                                        \
-    return kind == KIND_T3A ? launch_fast3_t<T, O, F, KIND_T3A>(p, cf, fe, tmX, tmPo, tmPc, s) \
-                            : launch_fast3_t<T, O, F, KIND_T3B>(p, cf, fe, tmX, tmPo, tmPc, s)
-    if (kind != KIND_T3A && kind != KIND_T3B) return cudaErrorInvalidValue;
-    if (order == 2) {
-        if (flux == 0) DUGKS_T3(2, 0);
-        DUGKS_T3(2, 1);
-    }
-    if (order == 3) {
-        if (flux == 0) DUGKS_T3(3, 0);
-        DUGKS_T3(3, 1);
-    }
-#undef DUGKS_T3
-    return cudaErrorInvalidValue;
+FastGeom Launch<T, ST>::fast_geom(int stages) {
+    return stages == 2 ? geom_t<T, ST, o4_nw<T>(), o4_mr<T>(), 2>() : geom_t<T, ST, 8, 2, 2>();
 }
 
 template <typename T, typename ST, int FLUX, int KIND>
@@ -189,36 +146,50 @@ cudaError_t Launch<T, ST>::step_fast4(const StepParams<T> &p, const FaceCoefs<T,
         if (cols == 1) return CALL(T);                                                        \
     if constexpr (sizeof(T) == 4) return CALL(float2);
 
-template <typename V, typename ST, int FLUX, bool FIELD>
+template <typename V, typename ST, int FLUX, bool FIELD, int KIND>
 static cudaError_t launch_march_t(const StepParams<typename Lane<V>::T> &p, const MarchCoefs<typename Lane<V>::T> &cf,
                                   const FastExtra<typename Lane<V>::T> &fe, int early, cudaStream_t s) {
+    using MT = MarchTile<V, ST, KIND>;
+    const int smem = MT::smem_bytes(p.tile_h);
+    static_assert(MT::smem_bytes(64) <= 48 * 1024, "fits without the shared-memory attribute");
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(p.tiles_x, (p.ny + p.tile_h - 1) / p.tile_h);
     cfg.blockDim = dim3(32);
-    cfg.dynamicSmemBytes = MarchTile<V, ST>::smem_bytes(p.tile_h);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, step_march_kernel<V, ST, FLUX, FIELD>, p, cf, fe, early);
+    return cudaLaunchKernelEx(&cfg, step_march_kernel<V, ST, FLUX, FIELD, KIND>, p, cf, fe, early);
 }
 
-template <typename V, typename ST>
+template <typename V, typename ST, int KIND>
 static cudaError_t launch_march_v(const StepParams<typename Lane<V>::T> &p, const MarchCoefs<typename Lane<V>::T> &cf,
                                   const FastExtra<typename Lane<V>::T> &fe, int flux, int early, cudaStream_t s) {
     if (p.vel_kind == VEL_FIELD)
-        return flux == 0 ? launch_march_t<V, ST, 0, true>(p, cf, fe, early, s)
-                         : launch_march_t<V, ST, 1, true>(p, cf, fe, early, s);
-    return flux == 0 ? launch_march_t<V, ST, 0, false>(p, cf, fe, early, s)
-                     : launch_march_t<V, ST, 1, false>(p, cf, fe, early, s);
+        return flux == 0 ? launch_march_t<V, ST, 0, true, KIND>(p, cf, fe, early, s)
+                         : launch_march_t<V, ST, 1, true, KIND>(p, cf, fe, early, s);
+    return flux == 0 ? launch_march_t<V, ST, 0, false, KIND>(p, cf, fe, early, s)
+                     : launch_march_t<V, ST, 1, false, KIND>(p, cf, fe, early, s);
 }
 
 template <typename T, typename ST>
 cudaError_t Launch<T, ST>::step_march(const StepParams<T> &p, const MarchCoefs<T> &cf, const FastExtra<T> &fe, int flux,
                                       int cols, int early, cudaStream_t s) {
-#define CALL(V) launch_march_v<V, ST>(p, cf, fe, flux, early, s)
+#define CALL(V) launch_march_v<V, ST, KIND_T2>(p, cf, fe, flux, early, s)
+    DUGKS_LANES(CALL)
+#undef CALL
+    return cudaErrorInvalidValue;
+}
+
+template <typename T, typename ST>
+cudaError_t Launch<T, ST>::step_march3(const StepParams<T> &p, const MarchCoefs<T> &cf, const FastExtra<T> &fe, int flux,
+                                       int kind, int cols, int early, cudaStream_t s) {
+#define CALL(V)                                                              \
+    (kind == KIND_T3A ? launch_march_v<V, ST, KIND_T3A>(p, cf, fe, flux, early, s) \
+                      : launch_march_v<V, ST, KIND_T3B>(p, cf, fe, flux, early, s))
     DUGKS_LANES(CALL)
 #undef CALL
     return cudaErrorInvalidValue;

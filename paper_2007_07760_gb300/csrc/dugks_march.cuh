@@ -1,5 +1,5 @@
-// dugks_march.cuh -- the two-stage DUGKS step for stencils of radius 1 (orders 2
-// and 3) as a row march (sm_103a): FP32 and FP16 storage.
+// dugks_march.cuh -- the DUGKS step for stencils of radius 1 (orders 2 and 3) as a
+// row march (sm_103a): the two-stage step and the two kernels of the three-stage step.
 //
 // Same method as step_kernel (dugks_kernels.cuh; equation numbers are the paper's).
 // One warp, which is one CTA, owns a strip of 60 columns and a segment of rows and
@@ -167,7 +167,7 @@ struct alignas(16) Row4 { T x, y, z, w; };
 // columns of 64, or 28 of 32. A strip of pairs starts at an odd column, x = 60 bx - 3 (lanes
 // 1 to 30 are written, columns 60 bx - 1 to 60 bx + 58): with the ghost border of 5 a pair
 // then lies on an 8-byte boundary of the plane (4 bytes in FP16 storage).
-template <typename V, typename ST>
+template <typename V, typename ST, int KIND = KIND_T2>
 struct MarchTile {
     using T = typename Lane<V>::T;
     static constexpr int N = Lane<V>::N;
@@ -181,8 +181,13 @@ struct MarchTile {
     static constexpr int oP = oPo + 32 * PB;               // phi, one row ahead: columns -1 .. 32 N
     static constexpr int P0 = N;                           // index of column 0 there (aligned pairs)
     // (without phi planes: the state of the columns before and after the strip, 2 x 9 values)
-    static constexpr int slot = (oP + (PHIP ? 32 * N + P0 + N : 18) * (int)sizeof(T) + 15) / 16 * 16;
-    static constexpr int oRow = DEPTH * slot;              // velocity factors of the segment's rows
+    // second kernel of the three-stage scheme: the accumulator's moving directions and the plane
+    // of its phi two rows below (without phi planes: all nine directions)
+    static constexpr int oAcc = (oP + (PHIP ? 32 * N + P0 + N : 18) * (int)sizeof(T) + 15) / 16 * 16;
+    static constexpr int slot = oAcc + (KIND == KIND_T3B ? 9 * 32 * PB : 0);
+    // first kernel of the three-stage scheme: X + be (g - X) of its two outputs, rows j to j - 2
+    static constexpr int oBase = DEPTH * slot;
+    static constexpr int oRow = oBase + (KIND == KIND_T3A ? 3 * 16 * 32 * PB : 0);   // velocity factors of the segment's rows
     static constexpr int rows_extra = 4;                   // rows a segment reads past its own
     static constexpr int strips(int nx) { return (nx + (N == 2 ? 1 : 0) + TX - 1) / TX; }
     static constexpr int smem_bytes(int rows) { return oRow + (rows + rows_extra) * (int)sizeof(Row4<T>); }
@@ -435,16 +440,22 @@ struct March<V, 1> {
 };
 
 // One strip (rows y0 .. y0 + rows - 1) of one grid. FIELD: the velocity is given at cell
-// centres (p.ufield, p.vfield). MASS: its sum of phi goes to mass_out; otherwise a value that is
-// not finite raises the status flag.
-template <typename V, typename ST, int FLUX, bool FIELD, bool MASS>
+// centres (p.ufield, p.vfield). SUM_MASS: its sum of phi goes to mass_out; SUM_CHECK: a value that
+// is not finite raises the status flag. KIND_T3A, KIND_T3B: the two kernels of the three-stage step
+// (Sec. II.B.2),
+//   T3A  out1 = X + be1 (g - X) + ga1 L (tilde f at t'), out2 = X + be2 (g - X) + ga2 L (the accumulator)
+//   T3B  out1 = acc + be1 (g - X) + ga1 L (hat f at t_n + dt)
+// with phi planes, phi of each output is that of its base plus the flux sum (two draws in T3A).
+enum Sum { SUM_NONE, SUM_CHECK, SUM_MASS };
+template <typename V, typename ST, int FLUX, bool FIELD, int KIND, int SUM>
 __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T> &p,
                                             const MarchCoefs<typename Lane<V>::T> &cf,
                                             const FastExtra<typename Lane<V>::T> &fe, int bx, int y0, int rows,
                                             double *mass_out, unsigned char *smem) {
     using T = typename Lane<V>::T;
     using LN = Lane<V>;
-    using MT = MarchTile<V, ST>;
+    using MT = MarchTile<V, ST, KIND>;
+    constexpr bool T3A = KIND == KIND_T3A, T3B = KIND == KIND_T3B;
     constexpr bool DEV = Store<T, ST>::deviation;
     constexpr bool PHIP = MT::PHIP;
     // FP64 arithmetic is the scarce resource there: rows that complete nothing skip it
@@ -470,7 +481,9 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
     Row4<T> *sRow = reinterpret_cast<Row4<T> *>(smem + MT::oRow);
     const bool reversing = p.vel_kind == VEL_VORTEX || p.vel_kind == VEL_DEFORM;
     const T vct = reversing ? fe.vc_t : T(1), vco = reversing ? fe.vc_told : T(1), vcf = reversing ? fe.vc_tface : T(1);
-    const T gc2 = p.ga1 * p.c2, hg3 = T(0.5) * p.ga1 * p.c3;
+    // flux terms carry the output's gamma; with two outputs they are kept without it
+    const T ga = T3A ? T(1) : p.ga1;
+    const T gc2 = ga * p.c2, hg3 = T(0.5) * ga * p.c3;
     const T f3 = T(3) * gc2;               // (face velocities carry 3 gamma c2)
     V cu{}, cv{}, cuE{}, cvE{};            // column factors at the centres and east faces
     if constexpr (!FIELD) {
@@ -539,6 +552,8 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
     const bool halo = wide && (lane == 0 || lane == 31);
     const uint32_t hdst = MT::oP + (PHIP ? lane == 0 ? MT::P0 - 1 : MT::P0 + 32 * N : lane == 0 ? 0 : 9) * (int)sizeof(T);
     const int packets = PHIP ? npk : npk + 1;
+    const T *gA = T3B ? static_cast<const T *>(p.acc) + row0 + col : nullptr;
+    const T *gPa = T3B && PHIP ? p.phi_acc + row0 - 2 * p.pitch + col : nullptr;
     const size_t plane = p.plane;
     int fetched = 0;
     uint32_t fslot = 0;   // byte offset of the slot the next packet goes to
@@ -554,6 +569,16 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
             } else if (halo) {
 #pragma unroll
                 for (int k = 0; k < 9; k++) cp_async<(int)sizeof(T)>(s + hdst + k * (int)sizeof(T), gH + k * plane);
+            }
+            if constexpr (T3B) {
+#pragma unroll
+                for (int k = PHIP ? 1 : 0; k < 9; k++)
+                    cp_async<PB>(s + MT::oAcc + k * 32 * PB + lane * PB, gA + k * plane);
+                if constexpr (PHIP) {
+                    cp_async<PB>(s + MT::oAcc + lane * PB, gPa);
+                    gPa += p.pitch;
+                }
+                gA += p.pitch;
             }
             gX += p.pitch;
             gPo += p.pitch;
@@ -629,7 +654,7 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
         pz = vfma(T(4), pd1, d0);
         pc1 = b;
     }
-    const T gmc = p.ga1 * (T(1) - p.c2);
+    const T gmc = ga * (T(1) - p.c2);
     March<V, FLUX> mx;
     mx.clear(V{});
     // rows in flight: X + be (g - X) of row j - 1; the same less the flux of row j - 2
@@ -640,6 +665,7 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
     V f0p{}, f1p{}, f2p{};             // north-face moments of row j - 3
     double msum = 0.0;
     V check{};                         // 0, or NaN once a value was not finite
+    V pa0{}, pa1{}, pa2{};             // T3B without phi planes: phi of the accumulator, rows j to j - 2
     uint32_t cslot = 0;
     const uint32_t seed = PHIP ? mix32(p.seed) : 0u;
     // lanes whose columns have images in the ghost border left or right of the grid
@@ -725,7 +751,8 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
         V F0, F1, F2, F3, F4, F5, F6, F7, F8;
         V nb1, nb2, nb3, nb4, nb5, nb6, nb7, nb8;
         {
-            auto cell = [&](int k, V g, V &F) -> V {     // returns X + be (g - X)
+            // returns X + be (g - X) (T3B: with the accumulator in the place of X)
+            auto cell = [&](int k, V g, V &F) -> V {
                 const T wk = wq<T>(k);
                 const unsigned char *q = sl + k * 32 * XB + lane * XB;
                 V X, t;
@@ -738,8 +765,17 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
                     t = vfma(wk, g, vneg(X));
                 }
                 F = vfma(p.b, t, X);
-                if (SKIP && (it < 2 || it > npk - 3)) return V{};
-                return vfma(p.be1, t, X);
+                if (k == 0 || (SKIP && (it < 2 || it > npk - 3))) return V{};
+                if constexpr (T3A) {
+                    V *q2 = reinterpret_cast<V *>(smem + MT::oBase + (it % 3) * 16 * 32 * PB) + (2 * k - 2) * 32 + lane;
+                    q2[0] = vfma(p.be1, t, X);
+                    q2[32] = vfma(p.be2, t, X);
+                    return V{};
+                } else if constexpr (T3B) {
+                    return vfma(p.be1, t, *reinterpret_cast<const V *>(sl + MT::oAcc + k * 32 * PB + lane * PB));
+                } else {
+                    return vfma(p.be1, t, X);
+                }
             };
             const V gp = vadd(ph, Px), gm = vsub(ph, Px);
             cell(0, ph, F0);
@@ -751,6 +787,15 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
             nb6 = cell(6, vsub(gm, Py), F6);
             nb7 = cell(7, vsub(ph, Py), F7);
             nb8 = cell(8, vsub(gp, Py), F8);
+            if constexpr (T3B && !PHIP) {
+                pa2 = pa1; pa1 = pa0;
+                if (it >= 2 && it <= npk - 3) {
+                    pa0 = V{};
+#pragma unroll
+                    for (int k = 0; k < 9; k++)
+                        pa0 = vadd(pa0, *reinterpret_cast<const V *>(sl + MT::oAcc + k * 32 * PB + lane * PB));
+                }
+            }
         }
 
         // ---- expansions: row j completes row j - 1 -----------------------------------
@@ -761,8 +806,8 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
 
         // ---- row j - 2 is complete: faces, flux and store ----------------------------
         // (FP32: computed in the first rows too, where nothing is stored: one straight block)
-        V phn{};
-        V o[9];
+        V phn{}, phn2{};
+        V o[9], o2[9];
         const int y = y0 + it - 4;
         if (!SKIP || it >= 3) {
         const V phN = vadd(pNp, ro.PS), phE = phEp;
@@ -796,8 +841,16 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
             const V S13 = vadd(B1, B3);
             // new phi = phi + gamma sum_k L_k (sum_k w_k xi_k = 0, sum_k w_k xi_a xi_b = delta_ab / 3)
             const V dph = vfma(T(-1.0 / 3.0), S13, vmul(-gmc, vadd(sDp, ro.es)));
-            if constexpr (PHIP) phn = vadd_sr(pc3, dph, (uint32_t)y * (uint32_t)nx + (uint32_t)x, seed);
-            else phn = vadd(pc3, dph);
+            V phb = pc3;
+            if constexpr (T3B) phb = PHIP ? *reinterpret_cast<const V *>(sl + MT::oAcc + lane * PB) : pa2;
+            const V dph1 = T3A ? vmul(p.ga1, dph) : dph;
+            if constexpr (PHIP) phn = vadd_sr(phb, dph1, (uint32_t)y * (uint32_t)nx + (uint32_t)x, seed);
+            else phn = vadd(phb, dph1);
+            if constexpr (T3A) {
+                const V dph2 = vmul(p.ga2, dph);
+                if constexpr (PHIP) phn2 = vadd_sr(phb, dph2, (uint32_t)y * (uint32_t)nx + (uint32_t)x, ~seed);
+                else phn2 = vadd(phb, dph2);
+            }
             {
                 // gamma w_k (c2 Phi_k + c3 Psi_k) = w_k (xi_x A1 + xi_y A2 + xi_x^2 B1 + xi_x xi_y B2 + xi_y^2 B3)
                 const T w1 = wq<T>(1), w2 = wq<T>(2);
@@ -814,6 +867,16 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
                 o[6] = vfma(-w2, vsub(sp, ap), p6);
                 o[8] = vfma(-w2, vadd(sm, am), p8);
                 o[4] = vfma(-w2, vsub(sm, am), p4);
+                if constexpr (T3A) {
+                    const V *q2 = reinterpret_cast<const V *>(smem + MT::oBase + ((it + 1) % 3) * 16 * 32 * PB) + lane;
+#pragma unroll
+                    for (int k = 1; k < 9; k++) {
+                        o2[k] = vfma(p.ga2, o[k], q2[(2 * k - 1) * 32]);
+                        o[k] = vfma(p.ga1, o[k], q2[(2 * k - 2) * 32]);
+                    }
+                    o2[0] = vsub(phn2, vadd(vadd(vadd(o2[1], o2[2]), vadd(o2[3], o2[4])),
+                                            vadd(vadd(o2[5], o2[6]), vadd(o2[7], o2[8]))));
+                }
                 // rest component: the new phi is exactly phn (up to this subtraction)
                 o[0] = vsub(phn, vadd(vadd(vadd(o[1], o[2]), vadd(o[3], o[4])), vadd(vadd(o[5], o[6]), vadd(o[7], o[8]))));
             }
@@ -825,6 +888,7 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
         const V pho = PHIP ? phn : pc3;   // (without phi planes: phi of X, the next step's older level)
         // ---- row j - 1: X + be (g - X) - gamma (1 - c2) Dbar ---------------------------
         if (!SKIP || (it >= 3 && it <= npk - 2)) {
+        // (b is 0 where the bases are kept apart: T3A)
         r1 = vfma(-gmc, ro.D1, b1);
         r2 = vfma(-gmc, ro.D2, b2);
         r3 = vfma(-gmc, ro.D3, b3);
@@ -845,66 +909,76 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
         // ---- store row j - 2 -----------------------------------------------------------
         const bool st0 = ok0 && it >= 4, st1 = ok1 && it >= 4;
         using OV = typename std::conditional<DEV, __half2, V>::type;
-        OV ov[9];
+        const size_t g0 = (size_t)(y + GHOST) * p.pitch + (size_t)(x + GHOST);
+        // nine values and (unless Q is null) phi; images: also into the ghost border
+        auto store = [&](const OV (&ov)[9], ST *O, const V ph, T *Q, bool images) {
+            // one column of this lane at element offset g
+            auto put0 = [&](long long g) {
+#pragma unroll
+                for (int k = 0; k < 9; k++) {
+                    if constexpr (N == 2) O[(long long)(k * plane) + g] = ov[k].x;
+                    else O[(long long)(k * plane) + g] = ov[k];
+                }
+                if constexpr (!T3B || PHIP) Q[g] = LN::first(ph);
+            };
+            auto put1 = [&](long long g) {
+                if constexpr (N == 2) {
+#pragma unroll
+                    for (int k = 0; k < 9; k++) O[(long long)(k * plane) + g + 1] = ov[k].y;
+                    if constexpr (!T3B || PHIP) Q[g + 1] = LN::second(ph);
+                }
+            };
+            if (st0 && (N == 1 || st1)) {
+#pragma unroll
+                for (int k = 0; k < 9; k++) *reinterpret_cast<OV *>(O + k * plane + g0) = ov[k];
+                if constexpr (!T3B || PHIP) *reinterpret_cast<V *>(Q + g0) = ph;
+            } else if (st0) {
+                put0(g0);
+            } else if (st1) {
+                put1(g0);
+            }
+            // periodic images in the ghost border
+            if (images && (st0 || st1) && (xedge || y < GHOST || y >= ny - GHOST)) {
+#pragma unroll 1
+                for (int im = 0; im < 9; im++) {
+                    const int ay = im / 3 - 1, ax = im - 3 * (im / 3) - 1;
+                    const int yy = y + ay * ny, xx = x + ax * nx;
+                    if (im == 4 || yy < -GHOST || yy >= ny + GHOST) continue;
+                    const long long gi = (long long)(yy + GHOST) * p.pitch + (xx + GHOST);
+                    if (st0 && xx >= -GHOST && xx < nx + GHOST) put0(gi);
+                    if (st1 && xx + 1 >= -GHOST && xx + 1 < nx + GHOST) put1(gi);
+                }
+            }
+        };
         if constexpr (DEV) {
+            OV ov[9];
 #pragma unroll
             for (int k = 0; k < 9; k++)
                 ov[k] = __float22half2_rn(vmul(p.qscale / wq<T>(k), vfma(-wq<T>(k), phn, o[k])));
+            store(ov, static_cast<ST *>(p.out1), pho, p.phi_out, true);
         } else {
+            store(o, static_cast<ST *>(p.out1), pho, p.phi_out, true);
+            if constexpr (T3A) {   // the accumulator is read per cell only: no images
+                if constexpr (PHIP) {
+                    store(o2, p.out2, phn2, p.phi_out2, false);
+                } else if (st0) {
 #pragma unroll
-            for (int k = 0; k < 9; k++) ov[k] = o[k];
-        }
-        ST *O = static_cast<ST *>(p.out1);
-        // one column of this lane at element offset g
-        auto put0 = [&](long long g) {
-#pragma unroll
-            for (int k = 0; k < 9; k++) {
-                if constexpr (N == 2) O[(long long)(k * plane) + g] = ov[k].x;
-                else O[(long long)(k * plane) + g] = ov[k];
+                    for (int k = 0; k < 9; k++) p.out2[k * plane + g0] = o2[k];
+                }
             }
-            p.phi_out[g] = LN::first(pho);
-        };
-        auto put1 = [&](long long g) {
-            if constexpr (N == 2) {
-#pragma unroll
-                for (int k = 0; k < 9; k++) O[(long long)(k * plane) + g + 1] = ov[k].y;
-                p.phi_out[g + 1] = LN::second(pho);
-            }
-        };
-        const size_t g = (size_t)(y + GHOST) * p.pitch + (size_t)(x + GHOST);
-        if (st0 && (N == 1 || st1)) {
-#pragma unroll
-            for (int k = 0; k < 9; k++) *reinterpret_cast<OV *>(O + k * plane + g) = ov[k];
-            *reinterpret_cast<V *>(p.phi_out + g) = pho;
-        } else if (st0) {
-            put0(g);
-        } else if (st1) {
-            put1(g);
         }
-        if constexpr (MASS) {
+        if constexpr (SUM == SUM_MASS) {
             if (st0) msum += (double)LN::first(phn);
             if (st1) msum += (double)LN::second(phn);
-        } else {
+        } else if constexpr (SUM == SUM_CHECK) {
             if (st0 || st1) check = vfma(T(0), phn, check);
-        }
-        // periodic images in the ghost border
-        if ((st0 || st1) && (xedge || y < GHOST || y >= ny - GHOST)) {
-#pragma unroll 1
-            for (int im = 0; im < 9; im++) {
-                const int ay = im / 3 - 1, ax = im - 3 * (im / 3) - 1;
-                const int yy = y + ay * ny, xx = x + ax * nx;
-                if (im == 4 || yy < -GHOST || yy >= ny + GHOST) continue;
-                const long long gi = (long long)(yy + GHOST) * p.pitch + (xx + GHOST);
-                if (st0 && xx >= -GHOST && xx < nx + GHOST) put0(gi);
-                if (st1 && xx + 1 >= -GHOST && xx + 1 < nx + GHOST) put1(gi);
-            }
         }
     }
     cp_wait<0>();
-    if constexpr (MASS) {
+    if constexpr (SUM == SUM_MASS) {
         for (int o = 16; o > 0; o >>= 1) msum += __shfl_down_sync(ALL, msum, o);
         if (lane == 0) *mass_out = msum;
-    } else {
+    } else if constexpr (SUM == SUM_CHECK) {
         const bool bad = (ok0 && !(LN::first(check) == T(0))) || (ok1 && !(LN::second(check) == T(0)));
         if (__any_sync(ALL, bad) && lane == 0) atomicOr(p.status, 1);
     }
@@ -913,7 +987,7 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
 // One grid: blockIdx.x = strip, blockIdx.y = segment of p.tile_h rows. EARLY: dependents may
 // be scheduled at once (a grid that leaves room for them on the chip: their velocity factors
 // are ready when this grid ends).
-template <typename V, typename ST, int FLUX, bool FIELD>
+template <typename V, typename ST, int FLUX, bool FIELD, int KIND>
 __global__ void __launch_bounds__(32, (sizeof(V) == 4 ? 12 : 8))
 step_march_kernel(const __grid_constant__ StepParams<typename Lane<V>::T> p,
                   const __grid_constant__ MarchCoefs<typename Lane<V>::T> cf,
@@ -921,8 +995,9 @@ step_march_kernel(const __grid_constant__ StepParams<typename Lane<V>::T> p,
     extern __shared__ __align__(128) unsigned char smem[];
     if (early) pdl_trigger();
     const int y0 = blockIdx.y * p.tile_h;
-    march_strip<V, ST, FLUX, FIELD, true>(p, cf, fe, blockIdx.x, y0, min(p.tile_h, p.ny - y0),
-                                          p.mass_partial + blockIdx.y * p.tiles_x + blockIdx.x, smem);
+    march_strip<V, ST, FLUX, FIELD, KIND, KIND == KIND_T3A ? SUM_NONE : SUM_MASS>(
+        p, cf, fe, blockIdx.x, y0, min(p.tile_h, p.ny - y0),
+        KIND == KIND_T3A ? nullptr : p.mass_partial + blockIdx.y * p.tiles_x + blockIdx.x, smem);
     if (!early) pdl_trigger();
 }
 
@@ -1023,7 +1098,7 @@ batch_march_kernel(const __grid_constant__ BatchUniform<typename Lane<V>::T> u,
         StepParams<T> p;
         FastExtra<T> fe;
         batch_step_params<T, ST>(u, G, ofs, p, fe);
-        march_strip<V, ST, FLUX, false, false>(p, cf, fe, w.y, w.z, w.w, nullptr, smem);
+        march_strip<V, ST, FLUX, false, KIND_T2, SUM_CHECK>(p, cf, fe, w.y, w.z, w.w, nullptr, smem);
         __syncwarp();   // the next strip's copies overwrite the ring
     }
     pdl_trigger();
