@@ -162,6 +162,40 @@ __device__ __forceinline__ void sincospi_(double x, double &s, double &c) { sinc
 template <typename T>
 struct alignas(16) Row4 { T x, y, z, w; };
 
+// Every prescribed velocity but the cell field is a product of a column and a row factor, u = cu(x)
+// ru(y), v = cv(x) rv(y) (times the reversal factor). One sine and cosine serve both factors at an
+// abscissa (ordinate) s: vortex sin^2(pi s / L), sin(2 pi s / L); deformation sin, cos(4 pi s / L).
+template <typename T>
+__device__ __forceinline__ void vel_waves(const StepParams<T> &p, T s, T &a, T &b) {
+    T sn, cs;
+    const bool def = p.vel_kind == VEL_DEFORM;
+    sincospi_((def ? T(4) * s : s) / p.vp0, sn, cs);
+    a = def ? sn : sn * sn;
+    b = def ? cs : T(2) * sn * cs;
+}
+template <typename T>
+__device__ __forceinline__ void vel_column(const StepParams<T> &p, T s, T &a, T &b) {
+    if (p.vel_kind == VEL_VORTEX || p.vel_kind == VEL_DEFORM) {
+        vel_waves(p, s, a, b);
+        a *= -p.vp1;
+        b *= p.vel_kind == VEL_DEFORM ? -p.vp1 : p.vp1;
+    } else {
+        a = p.vel_kind == VEL_UNIFORM ? p.vp0 : T(1);
+        b = p.vel_kind == VEL_UNIFORM ? p.vp1 : p.vp2 * (s - p.vp0);
+    }
+}
+template <typename T>
+__device__ __forceinline__ void vel_row(const StepParams<T> &p, T s, T &a, T &b) {
+    if (p.vel_kind == VEL_DEFORM) {
+        vel_waves(p, s, a, b);
+    } else if (p.vel_kind == VEL_VORTEX) {   // u takes sin(2 pi y / L), v sin^2(pi y / L)
+        vel_waves(p, s, b, a);
+    } else {
+        a = p.vel_kind == VEL_UNIFORM ? T(1) : -p.vp2 * (s - p.vp1);
+        b = T(1);
+    }
+}
+
 // Geometry of a warp: 32 lanes x N columns; bar f^+ is valid on all of them, the expansions
 // on all but the outer ones, and the cells but two columns from each edge are written: 60
 // columns of 64, or 28 of 32. A strip of pairs starts at an odd column, x = 60 bx - 3 (lanes
@@ -476,8 +510,7 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
     const bool ok0 = wr && x >= 0 && x < nx, ok1 = N == 2 && wr && x + 1 >= 0 && x + 1 < nx;
     const int npk = rows + MT::rows_extra;
 
-    // ---- velocity: every prescribed kind but the cell field is a product of a column
-    // and a row factor, u = cu(x) ru(y), v = cv(x) rv(y) (times the reversal factor)
+    // ---- velocity factors
     Row4<T> *sRow = reinterpret_cast<Row4<T> *>(smem + MT::oRow);
     const bool reversing = p.vel_kind == VEL_VORTEX || p.vel_kind == VEL_DEFORM;
     const T vct = reversing ? fe.vc_t : T(1), vco = reversing ? fe.vc_told : T(1), vcf = reversing ? fe.vc_tface : T(1);
@@ -487,51 +520,21 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
     const T f3 = T(3) * gc2;               // (face velocities carry 3 gamma c2)
     V cu{}, cv{}, cuE{}, cvE{};            // column factors at the centres and east faces
     if constexpr (!FIELD) {
-        // one sine and cosine serve both factors at an abscissa (ordinate) s:
-        // vortex sin^2(pi s / L), sin(2 pi s / L); deformation sin, cos(4 pi s / L)
-        auto waves = [&](T s, T &a, T &b) {
-            T sn, cs;
-            sincospi_((p.vel_kind == VEL_DEFORM ? T(4) * s : s) / p.vp0, sn, cs);
-            const bool def = p.vel_kind == VEL_DEFORM;
-            a = def ? sn : sn * sn;
-            b = def ? cs : T(2) * sn * cs;
-        };
-        auto col_factor = [&](T s, T &a, T &b) {
-            if (reversing) {
-                waves(s, a, b);
-                a *= -p.vp1;
-                b *= p.vel_kind == VEL_DEFORM ? -p.vp1 : p.vp1;
-            } else {
-                a = p.vel_kind == VEL_UNIFORM ? p.vp0 : T(1);
-                b = p.vel_kind == VEL_UNIFORM ? p.vp1 : p.vp2 * (s - p.vp0);
-            }
-        };
         const T g0 = T(wrap_small(x, nx)), g1 = T(wrap_small(x + 1, nx)), ff = vcf * f3;
         T a0, b0, a1 = T(0), b1 = T(0);
-        col_factor(g0 + T(0.5), a0, b0);
-        if (N == 2) col_factor(g1 + T(0.5), a1, b1);
+        vel_column(p, g0 + T(0.5), a0, b0);
+        if (N == 2) vel_column(p, g1 + T(0.5), a1, b1);
         cu = LN::make(a0, a1);
         cv = LN::make(b0, b1);
-        col_factor(g0 + T(1), a0, b0);
-        if (N == 2) col_factor(g1 + T(1), a1, b1);
+        vel_column(p, g0 + T(1), a0, b0);
+        if (N == 2) vel_column(p, g1 + T(1), a1, b1);
         cuE = LN::make(a0 * ff, a1 * ff);
         cvE = LN::make(b0 * ff, b1 * ff);
         for (int i = lane; i < npk; i += 32) {
             const T g = T(wrap_small(y0 - 2 + i, ny));
             Row4<T> r;
-            if (reversing) {   // (vortex: u takes sin(2 pi y / L), v sin^2(pi y / L))
-                T a, b;
-                waves(g + T(0.5), a, b);
-                r.x = p.vel_kind == VEL_DEFORM ? a : b;
-                r.y = p.vel_kind == VEL_DEFORM ? b : a;
-                waves(g + T(1), a, b);
-                r.z = p.vel_kind == VEL_DEFORM ? a : b;
-                r.w = p.vel_kind == VEL_DEFORM ? b : a;
-            } else {
-                r.x = p.vel_kind == VEL_UNIFORM ? T(1) : -p.vp2 * (g + T(0.5) - p.vp1);
-                r.z = p.vel_kind == VEL_UNIFORM ? T(1) : -p.vp2 * (g + T(1) - p.vp1);
-                r.y = r.w = T(1);
-            }
+            vel_row(p, g + T(0.5), r.x, r.y);
+            vel_row(p, g + T(1), r.z, r.w);
             r.z *= ff;
             r.w *= ff;
             sRow[i] = r;
@@ -672,9 +675,9 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
     const bool xedge = x < GHOST || x + N - 1 >= nx - GHOST;
 
     __syncwarp();
-    constexpr int UNROLL = sizeof(T) == 8 ? 1 : 2;   // (FP64: the arithmetic hides the moves that two rows would save)
-#pragma unroll UNROLL
-    for (int it = 0; it < npk; it++) {
+    // one row of the march; `light`: the first two rows, which only enter the pending sums
+    auto row = [&](int it, auto light) {
+        constexpr bool LIGHT = decltype(light)::value;
         cp_wait<1>();
         __syncwarp();
         fetch();
@@ -765,7 +768,7 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
                     t = vfma(wk, g, vneg(X));
                 }
                 F = vfma(p.b, t, X);
-                if (k == 0 || (SKIP && (it < 2 || it > npk - 3))) return V{};
+                if (k == 0 || LIGHT || (SKIP && it > npk - 3)) return V{};
                 if constexpr (T3A) {
                     V *q2 = reinterpret_cast<V *>(smem + MT::oBase + (it % 3) * 16 * 32 * PB) + (2 * k - 2) * 32 + lane;
                     q2[0] = vfma(p.be1, t, X);
@@ -798,17 +801,19 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
             }
         }
 
+        V phn{}, phn2{}, pho{};
+        V o[9], o2[9];
+        const int y = y0 + it - 4;
         // ---- expansions: row j completes row j - 1 -----------------------------------
         RowOut<V> ro;
         mx.advance(cf, F0, F1, F2, F3, F4, F5, F6, F7, F8, ro,
-                   SKIP ? Need{it >= 2, it >= 3 && it <= npk - 2, it >= 1 && it <= npk - 2, it <= npk - 3}
-                        : Need{true, true, true, true});
+                   LIGHT  ? Need{false, false, !SKIP || it >= 1, true}
+                   : SKIP ? Need{true, it >= 3 && it <= npk - 2, it <= npk - 2, it <= npk - 3}
+                          : Need{true, true, true, true});
+        if constexpr (!LIGHT) {
 
         // ---- row j - 2 is complete: faces, flux and store ----------------------------
-        // (FP32: computed in the first rows too, where nothing is stored: one straight block)
-        V phn{}, phn2{};
-        V o[9], o2[9];
-        const int y = y0 + it - 4;
+        // (FP32: computed in the next two rows too, where nothing is stored: one straight block)
         if (!SKIP || it >= 3) {
         const V phN = vadd(pNp, ro.PS), phE = phEp;
         // face moments: phi_b and (3 gamma c2 phi_b u_b + gamma c3 V_b) at the east and north faces
@@ -885,7 +890,7 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
         f1p = y1;
         f2p = y2;
         }
-        const V pho = PHIP ? phn : pc3;   // (without phi planes: phi of X, the next step's older level)
+        pho = PHIP ? phn : pc3;   // (without phi planes: phi of X, the next step's older level)
         // ---- row j - 1: X + be (g - X) - gamma (1 - c2) Dbar ---------------------------
         if (!SKIP || (it >= 3 && it <= npk - 2)) {
         // (b is 0 where the bases are kept apart: T3A)
@@ -901,10 +906,12 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
         phEp = vplus_right(ro.PE, ro.PW);
         }
         pNp = ro.PN;
+        }
         b1 = nb1; b2 = nb2; b3 = nb3; b4 = nb4; b5 = nb5; b6 = nb6; b7 = nb7; b8 = nb8;
         v1x = v0x; v1y = v0y;
         v0x = Vx; v0y = Vy;
         pc3 = pc2; pc2 = pc1; pc1 = pc0;
+        if constexpr (LIGHT) return;
 
         // ---- store row j - 2 -----------------------------------------------------------
         const bool st0 = ok0 && it >= 4, st1 = ok1 && it >= 4;
@@ -973,7 +980,15 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
         } else if constexpr (SUM == SUM_CHECK) {
             if (st0 || st1) check = vfma(T(0), phn, check);
         }
-    }
+    };
+    // (pairs with central faces: a second loop body costs registers, 4096^2 323 -> 371 us; else it
+    // gives 256^2 9.1 -> 8.4, 1024^2 38.5 -> 37.6, 4096^2 354 -> 350 us)
+    constexpr int LIGHT_ROWS = N == 2 && FLUX == 1 ? 0 : 2;
+#pragma unroll 1
+    for (int it = 0; it < LIGHT_ROWS; it++) row(it, std::true_type{});
+    constexpr int UNROLL = sizeof(T) == 8 ? 1 : 2;   // (FP64: the arithmetic hides the moves that two rows would save)
+#pragma unroll UNROLL
+    for (int it = LIGHT_ROWS; it < npk; it++) row(it, std::false_type{});
     cp_wait<0>();
     if constexpr (SUM == SUM_MASS) {
         for (int o = 16; o > 0; o >>= 1) msum += __shfl_down_sync(ALL, msum, o);
