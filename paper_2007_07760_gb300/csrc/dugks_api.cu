@@ -151,7 +151,7 @@ bool setup_fast(dugks_ctx *c) {
     if (marches(c)) {
         c->march = true;
         const int2 size = make_int2(c->p.nx, c->p.ny);
-        c->plan = march_plan(c->variant, &size, 1, c->p.precision, c->sms);
+        c->plan = march_plan(march_shape(), c->variant, &size, 1, c->p.precision, c->sms);
         c->tile_w = march_width(c->plan.cols, size.x);
         c->tile_h = march_segment_rows(c->plan.rows, size.y);
         return true;
@@ -173,7 +173,12 @@ bool fast_capable(const dugks_ctx *c) {
 }
 
 // strips of the row march start one column before the grid
-int strips(const dugks_ctx *c) { return c->fast && c->march ? march_strips(c->plan.cols, c->p.nx) : (c->p.nx + c->tile_w - 1) / c->tile_w; }
+// (the DVM of orders 2 and 3 has a march of its own)
+bool dvm_marches(const dugks_ctx *c) { return c->p.stages == 1 && c->p.order <= 3; }
+int strips(const dugks_ctx *c) {
+    if (dvm_marches(c)) return dvm_march_strips(c->plan.cols, c->p.nx);
+    return c->fast && c->march ? march_strips(c->plan.cols, c->p.nx) : (c->p.nx + c->tile_w - 1) / c->tile_w;
+}
 
 template <typename T, typename ST>
 int run_init(dugks_ctx *c) {
@@ -436,7 +441,20 @@ int step_dvm(dugks_ctx *c) {
     dv.s = dt >= 0.5 ? 1 : 0;
     dv.d = (T)(dv.s - dt);
     dv.beta = (T)(2.0 * dt / (2.0 * tau + dt));
-    cudaError_t e = launch_dvm<T>(q, dv, c->p.order, dt == 1.0, c->stream);
+    dv.early = c->plan.early;
+    cudaError_t e;
+    if (c->p.order <= 3) {
+        if (c->coef_h != dt) {
+            const MarchCoefs<T> cf = make_dvm_coefs<T>(c->p.order, dv.s - dt);
+            c->coefs.assign(reinterpret_cast<const unsigned char *>(&cf),
+                            reinterpret_cast<const unsigned char *>(&cf) + sizeof cf);
+            c->coef_h = dt;
+        }
+        e = launch_dvm_march<T>(q, dv, *reinterpret_cast<const MarchCoefs<T> *>(c->coefs.data()),
+                                vortex_factors<T>(c, t + dt, t, t), dt == 1.0, c->plan.cols, c->stream);
+    } else {
+        e = launch_dvm<T>(q, dv, c->p.order, dt == 1.0, c->stream);
+    }
     if (e != cudaSuccess) return cuda_fail(c, e, "DVM kernel");
     c->cur = 1 - c->cur;
     if (PHIP) {
@@ -673,6 +691,12 @@ int dugks_create(const dugks_params *p, const double *phi0_host, void *cuda_stre
             c->tile_w = TILE_X;
             c->tile_h = TILE_Y;
         }
+    }
+    if (dvm_marches(c)) {
+        const int2 size = make_int2(p->nx, p->ny);
+        c->plan = march_plan(dvm_shape(), -1, &size, 1, p->precision, c->sms);
+        c->tile_w = dvm_march_width(c->plan.cols);
+        c->tile_h = march_segment_rows(c->plan.rows, p->ny);
     }
     c->tiles_x = strips(c);
     c->ntiles = c->tiles_x * ((p->ny + c->tile_h - 1) / c->tile_h);

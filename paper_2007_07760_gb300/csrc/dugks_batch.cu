@@ -325,7 +325,7 @@ int rebuild_t(dugks_batch *b) {
     std::vector<int2> sizes;
     for (const Slot &s : b->slots)
         if (live(s)) sizes.push_back(make_int2(s.nx, s.ny));
-    b->plan = march_plan(b->variant, sizes.data(), (int)sizes.size(), b->p.precision, b->sms);
+    b->plan = march_plan(march_shape(), b->variant, sizes.data(), (int)sizes.size(), b->p.precision, b->sms);
     int nitems = 0;
     b->rows = 1;
     for (const int2 &q : sizes) {

@@ -219,30 +219,49 @@ inline int march_segment_rows(int want, int ny) {
     const int n = march_segments(want, ny);
     return (ny + n - 1) / n;
 }
+// What the rule needs of a kernel, for single columns and pairs (index: columns - 1): strips of
+// a grid, resident warps an SM, the cost of a row in a full wave (us), and in a partial wave
+// relative to that, base + slope (n - 1) for n warps a scheduler; rows that a segment costs past its
+// own, also in FP64.
+struct MarchShape {
+    int (*strips)(int cols, int nx);
+    double slots[2], unit[2], base[2], slope[2], extra, extra64;
+};
+inline const MarchShape &march_shape() {
+    static const MarchShape s{march_strips, {12, 8}, {1.05, 1.42}, {0.89, 1.0}, {0.3, 0.37}, 5.0, 2.5};
+    return s;
+}
+// the DVM (measured in FP32 at dt = 0.8: 256^2 7.8 us, single columns, 2 rows, against 8.8 for pairs;
+// 512^2 14.2, pairs, 4 rows; 1024^2 27.8, pairs, 12 rows, against 31.1 for single columns)
+inline const MarchShape &dvm_shape() {
+    static const MarchShape s{dvm_march_strips, {16, 12}, {0.85, 1.05}, {1.0, 1.0}, {0.05, 0.14}, 7.0, 6.0};
+    return s;
+}
 // for `count` grids of sizes (x, y) stepped together
-inline MarchPlan march_plan(int variant, const int2 *sizes, int count, int precision, int sms) {
+inline MarchPlan march_plan(const MarchShape &sh, int variant, const int2 *sizes, int count, int precision, int sms) {
     static constexpr int fixed[6] = {16, 8, 0, 32, 0, 64};   // variants 2 and 4: by the rule
     MarchPlan m{precision == DUGKS_FP64 ? 1 : 2, 16, 0};
     double best = 1e300;
     const int forced = variant >= 0 && variant < 6 ? fixed[variant] : 0;
     const bool f64 = precision == DUGKS_FP64;
     for (int cols = precision == DUGKS_FP16F ? 2 : 1; cols <= (f64 ? 1 : 2); cols++) {
-        const double slots = (cols == 2 ? 8.0 : 12.0) * sms, unit = cols == 2 ? 1.42 : 1.05;
+        const int c = cols - 1;
         for (int want = forced ? forced : 1; want <= (forced ? forced : 64); want++) {
             double w = 0.0;
             int rows = 1;
             for (int i = 0; i < count; i++) {
-                w += (double)march_strips(cols, sizes[i].x) * march_segments(want, sizes[i].y);
+                w += (double)sh.strips(cols, sizes[i].x) * march_segments(want, sizes[i].y);
                 rows = std::max(rows, march_segment_rows(want, sizes[i].y));
             }
-            const double W = w / slots, n = w / (4.0 * sms);
+            const double W = w / (sh.slots[c] * sms), n = w / (4.0 * sms);
             double cost;
-            if (f64) {
-                cost = (n > 3.0 ? n + 0.5 : std::ceil(n)) * (rows + 2.5);
-            } else {
-                const double p = std::max(n, 1.0) - 1.0;
-                cost = unit * (rows + 5) * (W > 1.5 ? W + 0.43 : W > 1.0 ? 1.9 : cols == 2 ? 1.0 + 0.37 * p : 0.89 + 0.3 * p);
-            }
+            if (f64)
+                cost = (n > 3.0 ? n + 0.5 : std::ceil(n)) * (rows + sh.extra64);
+            else
+                cost = sh.unit[c] * (rows + sh.extra) *
+                       (W > 1.5   ? W + 0.43
+                        : W > 1.0 ? 1.9
+                                  : sh.base[c] + sh.slope[c] * (std::max(n, 1.0) - 1.0));
             if (cost < best) {
                 best = cost;
                 // Early scheduling of the next kernel hides its launch and velocity factors
@@ -253,6 +272,26 @@ inline MarchPlan march_plan(int variant, const int2 *sizes, int count, int preci
             }
         }
     }
+    return m;
+}
+
+// The expansions of the DVM's streaming (Eq. (12)) at the displacement d xi_k: rows of the
+// stencil of xi = (1, 1) at (d, d) as weights of the row's sum, of R - 2 C + L and of R - L; px, pe as
+// above with c = d; nu, nm: weights of the first and second difference over rows of L + 4 C + R.
+template <typename T>
+inline MarchCoefs<T> make_dvm_coefs(int order, double d) {
+    MarchCoefs<T> m{};
+    const double q = order >= 3 ? 1.0 : 0.0;
+    for (int b = -1; b <= 1; b++) {
+        const double l = taylor_w(order, d, d, -1, b), r = taylor_w(order, d, d, 1, b);
+        m.dx[b + 1][0] = (T)(taylor_w(order, d, d, 0, b) + l + r);
+        m.dx[b + 1][1] = (T)(0.5 * (r + l));
+        m.dx[b + 1][2] = (T)(0.5 * (r - l));
+    }
+    m.px = (T)(d / 12.0);
+    m.pe = (T)(q * d * d / 12.0);
+    m.nu = (T)(d / 12.0);
+    m.nm = (T)(q * d * d / 12.0);
     return m;
 }
 

@@ -31,12 +31,33 @@ cudaError_t launch_dvm_t(const StepParams<T> &p, const DvmExtra<T> &dv, cudaStre
 
 template <typename T, bool LBM>
 cudaError_t launch_dvm_o(const StepParams<T> &p, const DvmExtra<T> &dv, int order, cudaStream_t s) {
-    switch (order) {
-    case 2: return launch_dvm_t<T, 2, LBM>(p, dv, s);
-    case 3: return launch_dvm_t<T, 3, LBM>(p, dv, s);
-    case 4: return launch_dvm_t<T, 4, LBM>(p, dv, s);
-    default: return cudaErrorInvalidValue;
-    }
+    return order == 4 ? launch_dvm_t<T, 4, LBM>(p, dv, s) : cudaErrorInvalidValue;
+}
+
+template <typename V, int MODE>
+cudaError_t launch_dvm_m(const StepParams<typename Lane<V>::T> &p, const DvmExtra<typename Lane<V>::T> &dv,
+                         const MarchCoefs<typename Lane<V>::T> &cf, const FastExtra<typename Lane<V>::T> &fe,
+                         cudaStream_t s) {
+    static_assert(DvmMarch<V>::smem_bytes(64) <= 48 * 1024, "fits without the shared-memory attribute");
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(p.tiles_x, (p.ny + p.tile_h - 1) / p.tile_h);
+    cfg.blockDim = dim3(32);
+    cfg.dynamicSmemBytes = DvmMarch<V>::smem_bytes(p.tile_h);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, dvm_march_kernel<V, MODE>, p, dv, cf, fe);
+}
+
+template <typename V>
+cudaError_t launch_dvm_v(const StepParams<typename Lane<V>::T> &p, const DvmExtra<typename Lane<V>::T> &dv,
+                         const MarchCoefs<typename Lane<V>::T> &cf, const FastExtra<typename Lane<V>::T> &fe, bool lbm,
+                         cudaStream_t s) {
+    return lbm ? launch_dvm_m<V, 2>(p, dv, cf, fe, s)
+               : dv.s ? launch_dvm_m<V, 1>(p, dv, cf, fe, s) : launch_dvm_m<V, 0>(p, dv, cf, fe, s);
 }
 
 }  // namespace
@@ -45,6 +66,18 @@ template <typename T>
 cudaError_t launch_dvm(const StepParams<T> &p, const DvmExtra<T> &dv, int order, bool lbm, cudaStream_t s) {
     return lbm ? launch_dvm_o<T, true>(p, dv, order, s) : launch_dvm_o<T, false>(p, dv, order, s);
 }
+
+template <typename T>
+cudaError_t launch_dvm_march(const StepParams<T> &p, const DvmExtra<T> &dv, const MarchCoefs<T> &cf,
+                             const FastExtra<T> &fe, bool lbm, int cols, cudaStream_t s) {
+    if constexpr (sizeof(T) == 4)
+        if (cols == 2) return launch_dvm_v<float2>(p, dv, cf, fe, lbm, s);
+    return launch_dvm_v<T>(p, dv, cf, fe, lbm, s);
+}
+int dvm_march_strips(int cols, int nx) { return cols == 2 ? DvmMarch<float2>::strips(nx) : DvmMarch<float>::strips(nx); }
+
+template cudaError_t launch_dvm_march<double>(const StepParams<double> &, const DvmExtra<double> &, const MarchCoefs<double> &, const FastExtra<double> &, bool, int, cudaStream_t);
+template cudaError_t launch_dvm_march<float>(const StepParams<float> &, const DvmExtra<float> &, const MarchCoefs<float> &, const FastExtra<float> &, bool, int, cudaStream_t);
 template cudaError_t launch_dvm<double>(const StepParams<double> &, const DvmExtra<double> &, int, bool, cudaStream_t);
 template cudaError_t launch_dvm<float>(const StepParams<float> &, const DvmExtra<float> &, int, bool, cudaStream_t);
 

@@ -68,6 +68,12 @@ template <typename T>
 struct DvmExtra;
 template <typename T>
 cudaError_t launch_dvm(const StepParams<T> &p, const DvmExtra<T> &dv, int order, bool lbm, cudaStream_t s);
+// the same as a row march (orders 2 and 3), `cols` columns a lane, segments of p.tile_h rows
+template <typename T>
+cudaError_t launch_dvm_march(const StepParams<T> &p, const DvmExtra<T> &dv, const MarchCoefs<T> &cf,
+                             const FastExtra<T> &fe, bool lbm, int cols, cudaStream_t s);
+int dvm_march_strips(int cols, int nx);
+constexpr int dvm_march_width(int cols) { return cols == 2 ? 56 : 26; }
 
 // Every device allocation of the library goes through dev_malloc: cudaMalloc
 // behind a host-side test hook (dugks_selftest_fail_allocs) that can make chosen
