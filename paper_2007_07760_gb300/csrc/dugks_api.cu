@@ -57,7 +57,8 @@ struct dugks_ctx {
     int vel_kind = DUGKS_VEL_UNIFORM;
     double vel[4] = {0, 0, 0, 0};
     bool initialized = false;
-    bool mass_valid = false;
+    bool mass_valid = false;    // the mass partials are those of the state
+    bool want_mass = true;      // the step being enqueued writes them (the last of a call)
     int64_t step = 0;
     int sticky = DUGKS_OK;
     std::string err;
@@ -226,6 +227,11 @@ FastExtra<T> vortex_factors(const dugks_ctx *c, double t, double t_old, double t
     return fx;
 }
 
+// Where a step writes its mass partials: nowhere but in the last step of a call, since only the
+// state that the call leaves can be asked for its mass. Their FP64 sums cost FP32 steps 4 to 6 %
+// (1024^2 37.5 -> 36.1 us, 4096^2 351 -> 330); FP64 steps always write them.
+double *step_partials(const dugks_ctx *c) { return c->want_mass || is_fp64(c) ? c->partial : nullptr; }
+
 // One two-stage step, X[cur] -> X[1-cur]. phi as a sum of X (FP64): phi[pr0]
 // holds phi^{n-1}, phi[pr1] receives phi^n. phi as a plane of its own (FP32,
 // FP16F): phi[pr0] = phi^n (of X), phi[pr1] = phi^{n-1}, phi[pr2] receives phi^{n+1}.
@@ -253,7 +259,7 @@ int step_t2(dugks_ctx *c, double *dbg = nullptr) {
     q.inv_dtD = (T)(1.0 / dt);
     q.X = c->X[c->cur];
     q.out1 = c->X[1 - c->cur];
-    q.mass_partial = c->partial;
+    q.mass_partial = step_partials(c);
     int iPc = 0, iPo, iOut;
     if (Store<T, ST>::phi_plane) {
         iPc = c->pr[0]; iPo = c->pr[1]; iOut = c->pr[2];
@@ -402,7 +408,7 @@ int step_t3(dugks_ctx *c) {
         B.phi_acc = static_cast<const T *>(c->phi[3]);
         B.phi_out = static_cast<T *>(c->phi[c->pr[1]]);
     }
-    B.mass_partial = c->partial;
+    B.mass_partial = step_partials(c);
     if (c->fast && c->p.order >= 4) {
         e = Launch<T, T>::step_fast4(B, *reinterpret_cast<const FaceCoefs<T, 2> *>(c->coefs3[1].data()),
                                      vortex_factors<T>(c, t + dt / 3.0, t, t + 0.75 * dt), c->tmX[1],
@@ -434,7 +440,7 @@ int step_dvm(dugks_ctx *c) {
     q.useD = c->p.dtphiu ? 1 : 0;
     q.X = c->X[c->cur];
     q.out1 = c->X[1 - c->cur];
-    q.mass_partial = c->partial;
+    q.mass_partial = step_partials(c);
     q.phi_old = static_cast<const T *>(c->phi[c->pr[0]]);
     q.phi_out = static_cast<T *>(c->phi[PHIP ? c->pr[2] : c->pr[1]]);
     DvmExtra<T> dv;
@@ -481,7 +487,7 @@ int step_once(dugks_ctx *c) {
     }
     if (r == DUGKS_OK) {
         c->step++;
-        c->mass_valid = true;
+        c->mass_valid = step_partials(c) != nullptr;
     }
     return r;
 }
@@ -506,7 +512,8 @@ int enqueue_mass(dugks_ctx *c, double *dev_out) {
         if (e != cudaSuccess) return cuda_fail(c, e, "mass partial kernel");
         c->mass_valid = true;
     }
-    e = launch_mass_final(c->partial, c->ntiles, dev_out, c->dstatus, c->stream);
+    const int early = (c->fast && c->march) || dvm_marches(c) ? c->plan.early : 1;
+    e = launch_mass_final(c->partial, c->ntiles, dev_out, c->dstatus, early, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "mass kernel");
     return DUGKS_OK;
 }
@@ -581,10 +588,14 @@ cudaError_t dev_malloc_pool(void **p, size_t bytes, cudaMemPool_t pool, cudaStre
 // Thread t adds partials t, t + 256, ... in index order with 8 independent loads
 // in flight (one memory latency per 8 partials), then the fixed tree of block_sum.
 // One small CTA: it finds a free slot while the step kernel drains.
-__global__ void __launch_bounds__(256) mass_final_kernel(const double *partial, int n, double *out, int *status) {
+// early: the next kernel may be placed while the step ahead still runs (where that costs the
+// march nothing: MarchPlan::early; FP64 512^2 step and mass: 331 us with, 255 without).
+__global__ void __launch_bounds__(256)
+mass_final_kernel(const double *partial, int n, double *out, int *status, int early) {
     __shared__ double sred[32];
-    pdl_trigger();
+    if (early) pdl_trigger();
     pdl_wait();   // the partials of the step kernel ahead of it
+    if (!early) pdl_trigger();
     constexpr int U = 8;
     double s = 0.0;
     for (int base = threadIdx.x; base < n; base += U * 256) {
@@ -601,7 +612,7 @@ __global__ void __launch_bounds__(256) mass_final_kernel(const double *partial, 
     }
 }
 
-cudaError_t launch_mass_final(const double *partial, int n, double *out, int *status, cudaStream_t s) {
+cudaError_t launch_mass_final(const double *partial, int n, double *out, int *status, int early, cudaStream_t s) {
     // programmatic dependent launch: resident while the step kernel drains, it
     // waits for the partials in the kernel itself
     cudaLaunchConfig_t cfg = {};
@@ -613,7 +624,7 @@ cudaError_t launch_mass_final(const double *partial, int n, double *out, int *st
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, mass_final_kernel, partial, n, out, status);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, mass_final_kernel, partial, n, out, status, early);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
@@ -782,7 +793,10 @@ int dugks_step(dugks_ctx *c, int64_t nsteps) {
     if (c->sticky != DUGKS_OK) return c->sticky;
     cudaSetDevice(c->dev);
     int r = ensure_init(c);
-    for (int64_t s = 0; s < nsteps && r == DUGKS_OK; s++) r = step_once(c);
+    for (int64_t s = 0; s < nsteps && r == DUGKS_OK; s++) {
+        c->want_mass = s + 1 == nsteps;
+        r = step_once(c);
+    }
     return r;
 }
 

@@ -837,7 +837,7 @@ int dugks_batch_mass(dugks_batch *b, int32_t grid_id, double *out) {
     case DUGKS_FP32: { auto q = slot_view<float, float>(b, s); q.mass_partial = part; e = Launch<float, float>::mass_partial(q, b->stream); break; }
     default: { auto q = slot_view<float, __half>(b, s); q.mass_partial = part; e = Launch<float, __half>::mass_partial(q, b->stream); break; }
     }
-    if (e == cudaSuccess) e = launch_mass_final(part, tiles, res, b->d_status, b->stream);
+    if (e == cudaSuccess) e = launch_mass_final(part, tiles, res, b->d_status, 1, b->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(out, res, sizeof(double), cudaMemcpyDeviceToHost, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return bcuda(b, e, "batch mass");

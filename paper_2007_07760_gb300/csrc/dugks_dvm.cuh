@@ -179,7 +179,7 @@ struct DvmMarch {
     static constexpr int smem_bytes(int rows) { return oRow + (rows + 6) * (int)sizeof(Row4<T>); }
 };
 
-template <typename V, int MODE>
+template <typename V, int MODE, bool MASS>
 __device__ __forceinline__ void dvm_strip(const StepParams<typename Lane<V>::T> &p, const DvmExtra<typename Lane<V>::T> &dv,
                                           const MarchCoefs<typename Lane<V>::T> &cf,
                                           const FastExtra<typename Lane<V>::T> &fe, int bx, int y0, int rows,
@@ -434,8 +434,10 @@ __device__ __forceinline__ void dvm_strip(const StepParams<typename Lane<V>::T> 
             put1(g);
             p.phi_out[g + 1] = LN::second(ph);
         }
-        if (ok0) msum += (double)LN::first(ph);
-        if (ok1) msum += (double)LN::second(ph);
+        if constexpr (MASS) {
+            if (ok0) msum += (double)LN::first(ph);
+            if (ok1) msum += (double)LN::second(ph);
+        }
         // periodic images in the ghost border
         if ((ok0 || ok1) && (xedge || y < GHOST || y >= ny - GHOST)) {
 #pragma unroll 1
@@ -450,11 +452,13 @@ __device__ __forceinline__ void dvm_strip(const StepParams<typename Lane<V>::T> 
         }
     }
     cp_wait<0>();
-    for (int o = 16; o > 0; o >>= 1) msum += __shfl_down_sync(ALL, msum, o);
-    if (lane == 0) *mass_out = msum;
+    if constexpr (MASS) {
+        for (int o = 16; o > 0; o >>= 1) msum += __shfl_down_sync(ALL, msum, o);
+        if (lane == 0) *mass_out = msum;
+    }
 }
 
-template <typename V, int MODE>
+template <typename V, int MODE, bool MASS>
 __global__ void __launch_bounds__(32, (sizeof(V) == 4 ? 16 : 8))
 dvm_march_kernel(const __grid_constant__ StepParams<typename Lane<V>::T> p,
                  const __grid_constant__ DvmExtra<typename Lane<V>::T> dv,
@@ -463,8 +467,8 @@ dvm_march_kernel(const __grid_constant__ StepParams<typename Lane<V>::T> p,
     extern __shared__ __align__(128) unsigned char smem[];
     if (dv.early) pdl_trigger();
     const int y0 = blockIdx.y * p.tile_h;
-    dvm_strip<V, MODE>(p, dv, cf, fe, blockIdx.x, y0, min(p.tile_h, p.ny - y0),
-                       p.mass_partial + blockIdx.y * p.tiles_x + blockIdx.x, smem);
+    dvm_strip<V, MODE, MASS>(p, dv, cf, fe, blockIdx.x, y0, min(p.tile_h, p.ny - y0),
+                             MASS ? p.mass_partial + blockIdx.y * p.tiles_x + blockIdx.x : nullptr, smem);
     if (!dv.early) pdl_trigger();
 }
 

@@ -244,7 +244,7 @@ inline MarchPlan march_plan(const MarchShape &sh, int variant, const int2 *sizes
     double best = 1e300;
     const int forced = variant >= 0 && variant < 6 ? fixed[variant] : 0;
     const bool f64 = precision == DUGKS_FP64;
-    for (int cols = precision == DUGKS_FP16F ? 2 : 1; cols <= (f64 ? 1 : 2); cols++) {
+    for (int cols = 1; cols <= (f64 ? 1 : 2); cols++) {
         const int c = cols - 1;
         for (int want = forced ? forced : 1; want <= (forced ? forced : 64); want++) {
             double w = 0.0;

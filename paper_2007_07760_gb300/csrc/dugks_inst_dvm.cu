@@ -49,7 +49,9 @@ cudaError_t launch_dvm_m(const StepParams<typename Lane<V>::T> &p, const DvmExtr
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, dvm_march_kernel<V, MODE>, p, dv, cf, fe);
+    // (the mass partials are written where the caller asks for them)
+    return p.mass_partial != nullptr ? cudaLaunchKernelEx(&cfg, dvm_march_kernel<V, MODE, true>, p, dv, cf, fe)
+                                     : cudaLaunchKernelEx(&cfg, dvm_march_kernel<V, MODE, false>, p, dv, cf, fe);
 }
 
 template <typename V>

@@ -142,12 +142,11 @@ cudaError_t Launch<T, ST>::step_fast4(const StepParams<T> &p, const FaceCoefs<T,
 
 // CALL with the lane type of `cols` columns
 #define DUGKS_LANES(CALL)                                                                     \
-    if constexpr (!Store<T, ST>::deviation)                                                   \
-        if (cols == 1) return CALL(T);                                                        \
+    if (cols == 1) return CALL(T);                                                            \
     if constexpr (sizeof(T) == 4) return CALL(float2);
 
-template <typename V, typename ST, int FLUX, bool FIELD, int KIND>
-static cudaError_t launch_march_t(const StepParams<typename Lane<V>::T> &p, const MarchCoefs<typename Lane<V>::T> &cf,
+template <typename V, typename ST, int FLUX, bool FIELD, int KIND, int SUM>
+static cudaError_t launch_march_s(const StepParams<typename Lane<V>::T> &p, const MarchCoefs<typename Lane<V>::T> &cf,
                                   const FastExtra<typename Lane<V>::T> &fe, int early, cudaStream_t s) {
     using MT = MarchTile<V, ST, KIND>;
     const int smem = MT::smem_bytes(p.tile_h);
@@ -162,7 +161,19 @@ static cudaError_t launch_march_t(const StepParams<typename Lane<V>::T> &p, cons
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, step_march_kernel<V, ST, FLUX, FIELD, KIND>, p, cf, fe, early);
+    return cudaLaunchKernelEx(&cfg, step_march_kernel<V, ST, FLUX, FIELD, KIND, SUM>, p, cf, fe, early);
+}
+
+// (the mass partials are written where the caller asks for them; FP64 steps always do: it is one of
+// about 350 FP64 instructions a row there)
+template <typename V, typename ST, int FLUX, bool FIELD, int KIND>
+static cudaError_t launch_march_t(const StepParams<typename Lane<V>::T> &p, const MarchCoefs<typename Lane<V>::T> &cf,
+                                  const FastExtra<typename Lane<V>::T> &fe, int early, cudaStream_t s) {
+    if constexpr (KIND != KIND_T3A)
+        if (p.mass_partial != nullptr) return launch_march_s<V, ST, FLUX, FIELD, KIND, SUM_MASS>(p, cf, fe, early, s);
+    if constexpr (KIND == KIND_T3A || sizeof(typename Lane<V>::T) == 4)
+        return launch_march_s<V, ST, FLUX, FIELD, KIND, SUM_NONE>(p, cf, fe, early, s);
+    return cudaErrorInvalidValue;
 }
 
 template <typename V, typename ST, int KIND>

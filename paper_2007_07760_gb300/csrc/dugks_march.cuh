@@ -209,7 +209,8 @@ struct MarchTile {
     // phi a plane of its own, or the sum of the state (FP64)
     static constexpr bool PHIP = Store<T, ST>::phi_plane;
     static constexpr int DEPTH = PHIP ? 3 : 4;             // rows in the ring
-    static constexpr int XB = N * (int)sizeof(ST);         // bytes of a lane's columns of the state
+    // bytes of a lane's copy of the state (a single half value comes with its aligned pair)
+    static constexpr int XB = N * (int)sizeof(ST) < 4 ? 4 : N * (int)sizeof(ST);
     static constexpr int PB = N * (int)sizeof(T);          // ... of phi
     static constexpr int oPo = 9 * 32 * XB;                // phi of the older level
     static constexpr int oP = oPo + 32 * PB;               // phi, one row ahead: columns -1 .. 32 N
@@ -475,7 +476,8 @@ struct March<V, 1> {
 
 // One strip (rows y0 .. y0 + rows - 1) of one grid. FIELD: the velocity is given at cell
 // centres (p.ufield, p.vfield). SUM_MASS: its sum of phi goes to mass_out; SUM_CHECK: a value that
-// is not finite raises the status flag. KIND_T3A, KIND_T3B: the two kernels of the three-stage step
+// is not finite raises the status flag. (The sum is in FP64: a scheduler is busy with its conversions
+// and additions for 256 cycles a row of pairs, of about 1200 in all.) KIND_T3A, KIND_T3B: the two kernels of the three-stage step
 // (Sec. II.B.2),
 //   T3A  out1 = X + be1 (g - X) + ga1 L (tilde f at t'), out2 = X + be2 (g - X) + ga2 L (the accumulator)
 //   T3B  out1 = acc + be1 (g - X) + ga1 L (hat f at t_n + dt)
@@ -494,7 +496,6 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
     constexpr bool PHIP = MT::PHIP;
     // FP64 arithmetic is the scarce resource there: rows that complete nothing skip it
     constexpr bool SKIP = sizeof(T) == 8;
-    static_assert(!DEV || LN::N == 2, "half-precision values travel as pairs");
     constexpr int XB = MT::XB, PB = MT::PB, DEPTH = MT::DEPTH, N = LN::N;
     const int lane = threadIdx.x & 31;
     const int nx = p.nx, ny = p.ny;
@@ -546,7 +547,7 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
     // (without phi planes phi of the row above is summed from the next packet)
     const uint32_t ring = smem_u32(smem);
     const size_t row0 = (size_t)(y0 - 2 + GHOST) * p.pitch;
-    const ST *gX = static_cast<const ST *>(p.X) + row0 + col;
+    const ST *gX = static_cast<const ST *>(p.X) + row0 + (DEV && N == 1 ? col & ~1 : col);
     const T *gPo = p.phi_old + row0 + col;
     const T *gP = PHIP ? p.phi_cur + row0 + p.pitch + col : nullptr;
     // lane 0 also fetches the column before the strip, lane 31 the one after it
@@ -760,7 +761,10 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
                 const unsigned char *q = sl + k * 32 * XB + lane * XB;
                 V X, t;
                 if constexpr (DEV) {
-                    X = vfma(p.qinv, __half22float2(*reinterpret_cast<const __half2 *>(q)), ph);
+                    V h;
+                    if constexpr (N == 2) h = __half22float2(*reinterpret_cast<const __half2 *>(q));
+                    else h = __half2float(reinterpret_cast<const __half *>(q)[col & 1]);
+                    X = vfma(p.qinv, h, ph);
                     t = vmul(wk, vsub(g, X));
                     X = vmul(wk, X);
                 } else {
@@ -915,7 +919,7 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
 
         // ---- store row j - 2 -----------------------------------------------------------
         const bool st0 = ok0 && it >= 4, st1 = ok1 && it >= 4;
-        using OV = typename std::conditional<DEV, __half2, V>::type;
+        using OV = typename std::conditional<!DEV, V, typename std::conditional<N == 2, __half2, __half>::type>::type;
         const size_t g0 = (size_t)(y + GHOST) * p.pitch + (size_t)(x + GHOST);
         // nine values and (unless Q is null) phi; images: also into the ghost border
         auto store = [&](const OV (&ov)[9], ST *O, const V ph, T *Q, bool images) {
@@ -960,8 +964,11 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
         if constexpr (DEV) {
             OV ov[9];
 #pragma unroll
-            for (int k = 0; k < 9; k++)
-                ov[k] = __float22half2_rn(vmul(p.qscale / wq<T>(k), vfma(-wq<T>(k), phn, o[k])));
+            for (int k = 0; k < 9; k++) {
+                const V q = vmul(p.qscale / wq<T>(k), vfma(-wq<T>(k), phn, o[k]));
+                if constexpr (N == 2) ov[k] = __float22half2_rn(q);
+                else ov[k] = __float2half_rn(q);
+            }
             store(ov, static_cast<ST *>(p.out1), pho, p.phi_out, true);
         } else {
             store(o, static_cast<ST *>(p.out1), pho, p.phi_out, true);
@@ -1002,7 +1009,7 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
 // One grid: blockIdx.x = strip, blockIdx.y = segment of p.tile_h rows. EARLY: dependents may
 // be scheduled at once (a grid that leaves room for them on the chip: their velocity factors
 // are ready when this grid ends).
-template <typename V, typename ST, int FLUX, bool FIELD, int KIND>
+template <typename V, typename ST, int FLUX, bool FIELD, int KIND, int SUM>
 __global__ void __launch_bounds__(32, (sizeof(V) == 4 ? 12 : 8))
 step_march_kernel(const __grid_constant__ StepParams<typename Lane<V>::T> p,
                   const __grid_constant__ MarchCoefs<typename Lane<V>::T> cf,
@@ -1010,9 +1017,9 @@ step_march_kernel(const __grid_constant__ StepParams<typename Lane<V>::T> p,
     extern __shared__ __align__(128) unsigned char smem[];
     if (early) pdl_trigger();
     const int y0 = blockIdx.y * p.tile_h;
-    march_strip<V, ST, FLUX, FIELD, KIND, KIND == KIND_T3A ? SUM_NONE : SUM_MASS>(
+    march_strip<V, ST, FLUX, FIELD, KIND, SUM>(
         p, cf, fe, blockIdx.x, y0, min(p.tile_h, p.ny - y0),
-        KIND == KIND_T3A ? nullptr : p.mass_partial + blockIdx.y * p.tiles_x + blockIdx.x, smem);
+        SUM == SUM_MASS ? p.mass_partial + blockIdx.y * p.tiles_x + blockIdx.x : nullptr, smem);
     if (!early) pdl_trigger();
 }
 
