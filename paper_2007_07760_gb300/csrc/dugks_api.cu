@@ -595,7 +595,6 @@ mass_final_kernel(const double *partial, int n, double *out, int *status, int ea
     __shared__ double sred[32];
     if (early) pdl_trigger();
     pdl_wait();   // the partials of the step kernel ahead of it
-    if (!early) pdl_trigger();
     constexpr int U = 8;
     double s = 0.0;
     for (int base = threadIdx.x; base < n; base += U * 256) {

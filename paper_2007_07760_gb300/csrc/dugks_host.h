@@ -192,15 +192,14 @@ inline MarchCoefs<T> make_march_coefs(int order, double h) {
 }
 
 // Lane width (columns a lane), segment rows and launch mode of the row march.
-// A segment of s rows reads s + 4, so long segments do less work, and short ones give more
-// warps. The cost below is a fit to the measured steps (FP32, vortex, 64^2 to 4096^2, s from 1
-// to 64, both widths; within 15%): a row takes `unit` microseconds in a full wave of W = 1;
-// several waves overlap but for 0.43 of one; a little over one wave costs nearly two; and
-// a partial wave is bound by the latency of a row, which grows with n, the warps a scheduler.
-// Measured: 64^2 5.3 us (1 column, s = 1) against 7.8 us with pairs; 256^2 9.0 (1, 2) against
-// 11.4; 1024^2 39.0 (2, 16) against 40.8; 4096^2 356 (2, 48) against 392. Segments over
-// 64 rows lose again (4096^2, 241 rows in one wave: 478 us): the rows in flight then lie all over
-// the planes, more pages than the TLB holds.
+// A segment of s rows reads s + 4 (the DVM s + 6), so long segments do less work, and short ones give
+// more warps. The costs below are fits to measured steps (FP32, vortex, 64^2 to 4096^2, s from 1 to 64,
+// both widths; mostly within 5%). In one wave of warps a row takes as long as the most warps on one
+// scheduler make it, in several waves it takes `unit` and part of a wave is lost at the end.
+// Measured: 64^2 5.1 us (1 column, s = 1) against 7.8 us with pairs; 256^2 8.3 (1, 2) against 11.4;
+// 450^2 11.0 (2, 3) against 12.8; 1024^2 36.1 (2, 16) against 39; 4096^2 330 (2, 32) against 383.
+// Segments over 64 rows lose again (4096^2, 241 rows in one wave: 478 us): the rows in flight then
+// lie all over the planes, more pages than the TLB holds.
 // FP64: the FP64 unit of each scheduler issues a warp instruction in 64 cycles whatever the
 // number of active lanes, so a step costs the rows of the busiest scheduler: the warps it gets
 // times s + 2.5 rows (the rows at a segment's ends leave out what they do not need).
@@ -219,22 +218,24 @@ inline int march_segment_rows(int want, int ny) {
     const int n = march_segments(want, ny);
     return (ny + n - 1) / n;
 }
-// What the rule needs of a kernel, for single columns and pairs (index: columns - 1): strips of
-// a grid, resident warps an SM, the cost of a row in a full wave (us), and in a partial wave
-// relative to that, base + slope (n - 1) for n warps a scheduler; rows that a segment costs past its
-// own, also in FP64.
+// What the rule needs of a kernel, for single columns and pairs (index: columns - 1): strips of a
+// grid, resident warps an SM; in one wave, us a launch and a row with 1 to 4 warps on the busiest
+// scheduler; in several, us a row of a full wave; rows that a segment costs past its own in one and
+// in several waves, and in FP64.
 struct MarchShape {
     int (*strips)(int cols, int nx);
-    double slots[2], unit[2], base[2], slope[2], extra, extra64;
+    double slots[2], launch[2], row[2][4], unit[2], extra1, extra2, extra64;
 };
 inline const MarchShape &march_shape() {
-    static const MarchShape s{march_strips, {12, 8}, {1.05, 1.42}, {0.89, 1.0}, {0.3, 0.37}, 5.0, 2.5};
+    static const MarchShape s{march_strips, {12, 8}, {4.9, 5.2}, {{0.92, 1.24, 1.51, 1.51}, {1.45, 1.92, 1.92, 1.92}},
+                              {1.12, 1.36}, 0.0, 3.5, 2.5};
     return s;
 }
 // the DVM (measured in FP32 at dt = 0.8: 256^2 7.8 us, single columns, 2 rows, against 8.8 for pairs;
 // 512^2 14.2, pairs, 4 rows; 1024^2 27.8, pairs, 12 rows, against 31.1 for single columns)
 inline const MarchShape &dvm_shape() {
-    static const MarchShape s{dvm_march_strips, {16, 12}, {0.85, 1.05}, {1.0, 1.0}, {0.05, 0.14}, 7.0, 6.0};
+    static const MarchShape s{dvm_march_strips, {16, 12}, {3.6, 3.6}, {{0.79, 0.89, 0.92, 1.0}, {0.96, 1.05, 1.06, 1.06}},
+                              {0.88, 1.1}, 6.0, 6.0, 6.0};
     return s;
 }
 // for `count` grids of sizes (x, y) stepped together
@@ -254,21 +255,22 @@ inline MarchPlan march_plan(const MarchShape &sh, int variant, const int2 *sizes
                 rows = std::max(rows, march_segment_rows(want, sizes[i].y));
             }
             const double W = w / (sh.slots[c] * sms), n = w / (4.0 * sms);
+            // Early scheduling of the next kernel hides its launch and velocity factors
+            // (512^2: 15.5 against 16.5 us). On a chip half full it costs instead, because the
+            // waiting warps fill some SMs and leave others idle (256^2, 860 warps: 10.2 against
+            // 9.1), and in FP64, where a scheduler with two warps takes twice as long.
+            const bool early = !f64 && (W > 0.6 || W < 0.15);
             double cost;
             if (f64)
                 cost = (n > 3.0 ? n + 0.5 : std::ceil(n)) * (rows + sh.extra64);
+            else if (W <= 1.0)
+                cost = sh.launch[c] + (early ? 0.0 : 0.9) +
+                       (rows + sh.extra1) * sh.row[c][std::min(3, std::max(0, (int)std::ceil(n) - 1))];
             else
-                cost = sh.unit[c] * (rows + sh.extra) *
-                       (W > 1.5   ? W + 0.43
-                        : W > 1.0 ? 1.9
-                                  : sh.base[c] + sh.slope[c] * (std::max(n, 1.0) - 1.0));
+                cost = sh.unit[c] * (rows + sh.extra2) * (W + std::min(0.7, 1.4 / W));
             if (cost < best) {
                 best = cost;
-                // Early scheduling of the next kernel hides its launch and velocity factors
-                // (512^2: 15.5 against 16.5 us). On a chip half full it costs instead, because the
-                // waiting warps fill some SMs and leave others idle (256^2, 860 warps: 10.2 against
-                // 9.1), and in FP64, where a scheduler with two warps takes twice as long.
-                m = MarchPlan{cols, want, !f64 && (W > 0.6 || W < 0.15)};
+                m = MarchPlan{cols, want, early};
             }
         }
     }
