@@ -296,7 +296,7 @@ int step_t2(dugks_ctx *c, double *dbg = nullptr) {
             c->coef_h = h;
         }
         e = Launch<T, ST>::step_march(q, *reinterpret_cast<const MarchCoefs<T> *>(c->coefs.data()),
-                                      vortex_factors<T>(c, t, t - dt, t + h), c->p.flux, c->plan.cols, c->plan.early,
+                                      vortex_factors<T>(c, t, t - dt, t + h), c->p.flux, c->plan.cols, c->plan.mode(),
                                       c->stream);
     } else {
         if (c->p.order == 5) return fail(c, DUGKS_EINVAL, "order 5 needs the TMA-staged kernels");
@@ -378,7 +378,7 @@ int step_t3(dugks_ctx *c) {
     } else if (c->fast) {
         e = Launch<T, T>::step_march3(A, *reinterpret_cast<const MarchCoefs<T> *>(c->coefs3[0].data()),
                                       vortex_factors<T>(c, t, t - dt, t + dt / 6.0), c->p.flux, KIND_T3A,
-                                      c->plan.cols, c->plan.early, c->stream);
+                                      c->plan.cols, c->plan.mode(), c->stream);
     } else {
         e = Launch<T, T>::step(A, c->p.order, c->p.flux, KIND_T3A, c->stream);
     }
@@ -416,7 +416,7 @@ int step_t3(dugks_ctx *c) {
     } else if (c->fast) {
         e = Launch<T, T>::step_march3(B, *reinterpret_cast<const MarchCoefs<T> *>(c->coefs3[1].data()),
                                       vortex_factors<T>(c, t + dt / 3.0, t, t + 0.75 * dt), c->p.flux, KIND_T3B,
-                                      c->plan.cols, c->plan.early, c->stream);
+                                      c->plan.cols, c->plan.mode(), c->stream);
     } else {
         e = Launch<T, T>::step(B, c->p.order, c->p.flux, KIND_T3B, c->stream);
     }
@@ -589,7 +589,7 @@ cudaError_t dev_malloc_pool(void **p, size_t bytes, cudaMemPool_t pool, cudaStre
 // in flight (one memory latency per 8 partials), then the fixed tree of block_sum.
 // One small CTA: it finds a free slot while the step kernel drains.
 // early: the next kernel may be placed while the step ahead still runs (where that costs the
-// march nothing: MarchPlan::early; FP64 512^2 step and mass: 331 us with, 255 without).
+// march nothing: MarchPlan::early; FP64 512^2 step and mass: 331 us with, 258 without).
 __global__ void __launch_bounds__(256)
 mass_final_kernel(const double *partial, int n, double *out, int *status, int early) {
     __shared__ double sred[32];

@@ -197,13 +197,16 @@ inline MarchCoefs<T> make_march_coefs(int order, double h) {
 // both widths; mostly within 5%). In one wave of warps a row takes as long as the most warps on one
 // scheduler make it, in several waves it takes `unit` and part of a wave is lost at the end.
 // Measured: 64^2 5.1 us (1 column, s = 1) against 7.8 us with pairs; 256^2 8.3 (1, 2) against 11.4;
-// 450^2 11.0 (2, 3) against 12.8; 1024^2 36.1 (2, 16) against 39; 4096^2 330 (2, 32) against 383.
+// 450^2 10.8 (2, 3) against 12.8; 1024^2 36.0 (2, 16) against 39; 4096^2 330 (2, 32) against 383.
 // Segments over 64 rows lose again (4096^2, 241 rows in one wave: 478 us): the rows in flight then
 // lie all over the planes, more pages than the TLB holds.
 // FP64: the FP64 unit of each scheduler issues a warp instruction in 64 cycles whatever the
 // number of active lanes, so a step costs the rows of the busiest scheduler: the warps it gets
 // times s + 2.5 rows (the rows at a segment's ends leave out what they do not need).
-struct MarchPlan { int cols, rows, early; };
+struct MarchPlan {
+    int cols, rows, early, one_wave;
+    int mode() const { return (early ? MARCH_EARLY : 0) | (one_wave ? MARCH_ONE_WAVE : 0); }
+};
 // strips of a grid for lanes of `cols` columns, their width, segments of about `want` rows and
 // their equal length
 inline int march_strips(int cols, int nx) {
@@ -227,7 +230,7 @@ struct MarchShape {
     double slots[2], launch[2], row[2][4], unit[2], extra1, extra2, extra64;
 };
 inline const MarchShape &march_shape() {
-    static const MarchShape s{march_strips, {12, 8}, {4.9, 5.2}, {{0.92, 1.24, 1.51, 1.51}, {1.45, 1.92, 1.92, 1.92}},
+    static const MarchShape s{march_strips, {12, 8}, {4.9, 5.7}, {{0.92, 1.24, 1.51, 1.51}, {1.45, 1.92, 1.92, 1.92}},
                               {1.12, 1.36}, 0.0, 3.5, 2.5};
     return s;
 }
@@ -241,7 +244,7 @@ inline const MarchShape &dvm_shape() {
 // for `count` grids of sizes (x, y) stepped together
 inline MarchPlan march_plan(const MarchShape &sh, int variant, const int2 *sizes, int count, int precision, int sms) {
     static constexpr int fixed[6] = {16, 8, 0, 32, 0, 64};   // variants 2 and 4: by the rule
-    MarchPlan m{precision == DUGKS_FP64 ? 1 : 2, 16, 0};
+    MarchPlan m{precision == DUGKS_FP64 ? 1 : 2, 16, 0, 0};
     double best = 1e300;
     const int forced = variant >= 0 && variant < 6 ? fixed[variant] : 0;
     const bool f64 = precision == DUGKS_FP64;
@@ -259,7 +262,9 @@ inline MarchPlan march_plan(const MarchShape &sh, int variant, const int2 *sizes
             // (512^2: 15.5 against 16.5 us). On a chip half full it costs instead, because the
             // waiting warps fill some SMs and leave others idle (256^2, 860 warps: 10.2 against
             // 9.1), and in FP64, where a scheduler with two warps takes twice as long.
-            const bool early = !f64 && (W > 0.6 || W < 0.15);
+            // Single columns: up to two warps a scheduler stay apart (248^2, FP32 7.6 -> 7.2, FP16 storage
+            // 8.3 -> 7.6 us; 260^2, a few more warps: 7.5 with, 8.2 without).
+            const bool early = !f64 && (W > (cols == 1 ? 2.0 / 3.0 : 0.6) || W < 0.15);
             double cost;
             if (f64)
                 cost = (n > 3.0 ? n + 0.5 : std::ceil(n)) * (rows + sh.extra64);
@@ -270,7 +275,7 @@ inline MarchPlan march_plan(const MarchShape &sh, int variant, const int2 *sizes
                 cost = sh.unit[c] * (rows + sh.extra2) * (W + std::min(0.7, 1.4 / W));
             if (cost < best) {
                 best = cost;
-                m = MarchPlan{cols, want, early};
+                m = MarchPlan{cols, want, early, W <= 1.0};
             }
         }
     }

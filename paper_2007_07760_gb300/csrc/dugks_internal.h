@@ -40,7 +40,7 @@ struct Launch {
     // the row march (two-stage, orders 2 and 3): one strip segment of p.tile_h rows per CTA,
     // `cols` columns a lane
     static cudaError_t step_march(const StepParams<T> &p, const MarchCoefs<T> &cf, const FastExtra<T> &fe, int flux,
-                                  int cols, int early, cudaStream_t s);
+                                  int cols, int mode, cudaStream_t s);
     // step `ofs` of a group for the grids of a work list; rows: the longest segment
     static cudaError_t batch_step(const BatchUniform<T> &u, const MarchCoefs<T> &cf, const BatchGrid<T> *grids,
                                   const int4 *items, int nitems, int rows, int ofs, int flux, int cols, int ctas,
@@ -54,7 +54,7 @@ struct Launch {
     // one kernel of the three-stage step (kind KIND_T3A or KIND_T3B; full storage only) as a
     // row march, orders 2 and 3
     static cudaError_t step_march3(const StepParams<T> &p, const MarchCoefs<T> &cf, const FastExtra<T> &fe, int flux,
-                                   int kind, int cols, int early, cudaStream_t s);
+                                   int kind, int cols, int mode, cudaStream_t s);
 };
 
 template <typename T>

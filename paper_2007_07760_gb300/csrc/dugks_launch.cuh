@@ -147,7 +147,7 @@ cudaError_t Launch<T, ST>::step_fast4(const StepParams<T> &p, const FaceCoefs<T,
 
 template <typename V, typename ST, int FLUX, bool FIELD, int KIND, int SUM>
 static cudaError_t launch_march_s(const StepParams<typename Lane<V>::T> &p, const MarchCoefs<typename Lane<V>::T> &cf,
-                                  const FastExtra<typename Lane<V>::T> &fe, int early, cudaStream_t s) {
+                                  const FastExtra<typename Lane<V>::T> &fe, int mode, cudaStream_t s) {
     using MT = MarchTile<V, ST, KIND>;
     const int smem = MT::smem_bytes(p.tile_h);
     static_assert(MT::smem_bytes(64) <= 48 * 1024, "fits without the shared-memory attribute");
@@ -161,35 +161,42 @@ static cudaError_t launch_march_s(const StepParams<typename Lane<V>::T> &p, cons
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, step_march_kernel<V, ST, FLUX, FIELD, KIND, SUM>, p, cf, fe, early);
+    // pairs, upwind: a body of its own for the rows before the first output costs registers that are
+    // spilled. In one wave, where segments are short and a row's latency counts, it gains (450^2, 3 rows:
+    // 10.8 -> 10.3 us, FP16 storage 12.4 -> 11.3; 1024^2, 16 rows: 36.0 -> 34.9); over several it
+    // loses (2048^2: 105.0 -> 105.1, FP16 storage 117.1 -> 123.1)
+    if constexpr (Lane<V>::N == 2 && FLUX == 0)
+        if (mode & MARCH_ONE_WAVE)
+            return cudaLaunchKernelEx(&cfg, step_march_kernel<V, ST, FLUX, FIELD, KIND, SUM, true>, p, cf, fe, mode);
+    return cudaLaunchKernelEx(&cfg, step_march_kernel<V, ST, FLUX, FIELD, KIND, SUM, sizeof(V) == 4>, p, cf, fe, mode);
 }
 
 // (the mass partials are written where the caller asks for them; FP64 steps always do: it is one of
 // about 350 FP64 instructions a row there)
 template <typename V, typename ST, int FLUX, bool FIELD, int KIND>
 static cudaError_t launch_march_t(const StepParams<typename Lane<V>::T> &p, const MarchCoefs<typename Lane<V>::T> &cf,
-                                  const FastExtra<typename Lane<V>::T> &fe, int early, cudaStream_t s) {
+                                  const FastExtra<typename Lane<V>::T> &fe, int mode, cudaStream_t s) {
     if constexpr (KIND != KIND_T3A)
-        if (p.mass_partial != nullptr) return launch_march_s<V, ST, FLUX, FIELD, KIND, SUM_MASS>(p, cf, fe, early, s);
+        if (p.mass_partial != nullptr) return launch_march_s<V, ST, FLUX, FIELD, KIND, SUM_MASS>(p, cf, fe, mode, s);
     if constexpr (KIND == KIND_T3A || sizeof(typename Lane<V>::T) == 4)
-        return launch_march_s<V, ST, FLUX, FIELD, KIND, SUM_NONE>(p, cf, fe, early, s);
+        return launch_march_s<V, ST, FLUX, FIELD, KIND, SUM_NONE>(p, cf, fe, mode, s);
     return cudaErrorInvalidValue;
 }
 
 template <typename V, typename ST, int KIND>
 static cudaError_t launch_march_v(const StepParams<typename Lane<V>::T> &p, const MarchCoefs<typename Lane<V>::T> &cf,
-                                  const FastExtra<typename Lane<V>::T> &fe, int flux, int early, cudaStream_t s) {
+                                  const FastExtra<typename Lane<V>::T> &fe, int flux, int mode, cudaStream_t s) {
     if (p.vel_kind == VEL_FIELD)
-        return flux == 0 ? launch_march_t<V, ST, 0, true, KIND>(p, cf, fe, early, s)
-                         : launch_march_t<V, ST, 1, true, KIND>(p, cf, fe, early, s);
-    return flux == 0 ? launch_march_t<V, ST, 0, false, KIND>(p, cf, fe, early, s)
-                     : launch_march_t<V, ST, 1, false, KIND>(p, cf, fe, early, s);
+        return flux == 0 ? launch_march_t<V, ST, 0, true, KIND>(p, cf, fe, mode, s)
+                         : launch_march_t<V, ST, 1, true, KIND>(p, cf, fe, mode, s);
+    return flux == 0 ? launch_march_t<V, ST, 0, false, KIND>(p, cf, fe, mode, s)
+                     : launch_march_t<V, ST, 1, false, KIND>(p, cf, fe, mode, s);
 }
 
 template <typename T, typename ST>
 cudaError_t Launch<T, ST>::step_march(const StepParams<T> &p, const MarchCoefs<T> &cf, const FastExtra<T> &fe, int flux,
-                                      int cols, int early, cudaStream_t s) {
-#define CALL(V) launch_march_v<V, ST, KIND_T2>(p, cf, fe, flux, early, s)
+                                      int cols, int mode, cudaStream_t s) {
+#define CALL(V) launch_march_v<V, ST, KIND_T2>(p, cf, fe, flux, mode, s)
     DUGKS_LANES(CALL)
 #undef CALL
     return cudaErrorInvalidValue;
@@ -197,10 +204,10 @@ cudaError_t Launch<T, ST>::step_march(const StepParams<T> &p, const MarchCoefs<T
 
 template <typename T, typename ST>
 cudaError_t Launch<T, ST>::step_march3(const StepParams<T> &p, const MarchCoefs<T> &cf, const FastExtra<T> &fe, int flux,
-                                       int kind, int cols, int early, cudaStream_t s) {
+                                       int kind, int cols, int mode, cudaStream_t s) {
 #define CALL(V)                                                              \
-    (kind == KIND_T3A ? launch_march_v<V, ST, KIND_T3A>(p, cf, fe, flux, early, s) \
-                      : launch_march_v<V, ST, KIND_T3B>(p, cf, fe, flux, early, s))
+    (kind == KIND_T3A ? launch_march_v<V, ST, KIND_T3A>(p, cf, fe, flux, mode, s) \
+                      : launch_march_v<V, ST, KIND_T3B>(p, cf, fe, flux, mode, s))
     DUGKS_LANES(CALL)
 #undef CALL
     return cudaErrorInvalidValue;

@@ -483,7 +483,10 @@ struct March<V, 1> {
 //   T3B  out1 = acc + be1 (g - X) + ga1 L (hat f at t_n + dt)
 // with phi planes, phi of each output is that of its base plus the flux sum (two draws in T3A).
 enum Sum { SUM_NONE, SUM_CHECK, SUM_MASS };
-template <typename V, typename ST, int FLUX, bool FIELD, int KIND, int SUM>
+// launch mode: the next kernel may be scheduled at once; the launch fits into one wave of warps
+enum MarchMode { MARCH_EARLY = 1, MARCH_ONE_WAVE = 2 };
+// MID: rows 2 and 3 of a segment, which complete nothing, in a body of their own
+template <typename V, typename ST, int FLUX, bool FIELD, int KIND, int SUM, bool MID = sizeof(V) == 4>
 __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T> &p,
                                             const MarchCoefs<typename Lane<V>::T> &cf,
                                             const FastExtra<typename Lane<V>::T> &fe, int bx, int y0, int rows,
@@ -497,6 +500,8 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
     // FP64 arithmetic is the scarce resource there: rows that complete nothing skip it
     constexpr bool SKIP = sizeof(T) == 8;
     constexpr int XB = MT::XB, PB = MT::PB, DEPTH = MT::DEPTH, N = LN::N;
+    constexpr int LIGHT_ROWS = N == 2 && FLUX == 1 ? 0 : 2;
+    static_assert(!MID || LIGHT_ROWS == 2, "the first four rows have bodies of their own");
     const int lane = threadIdx.x & 31;
     const int nx = p.nx, ny = p.ny;
     // the strip's width and the columns before it. FP64 strips of at most 26 columns leave out
@@ -676,9 +681,11 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
     const bool xedge = x < GHOST || x + N - 1 >= nx - GHOST;
 
     __syncwarp();
-    // one row of the march; `light`: the first two rows, which only enter the pending sums
-    auto row = [&](int it, auto light) {
-        constexpr bool LIGHT = decltype(light)::value;
+    // one row of the march; stage 0: the first two rows, which only enter the pending sums; stage 1:
+    // the next two, which complete no row of the segment; stage 2: the others (and, where MID is false,
+    // rows that the stages before would serve: they store nothing)
+    auto row = [&](int it, auto stage) {
+        constexpr bool LIGHT = decltype(stage)::value == 0, OUT = decltype(stage)::value == 2;
         cp_wait<1>();
         __syncwarp();
         fetch();
@@ -834,7 +841,7 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
         }
         const V y1 = vfma(phN, uN, vmul(hg3, vadd(v1x, v0x)));
         const V y2 = vfma(phN, vN, vmul(hg3, vadd(v1y, v0y)));
-        if (!SKIP || it >= 4) {
+        if (OUT && (MID || !SKIP || it >= 4)) {
             V uE, vE;
             if constexpr (FIELD) {
                 uE = vmul(hf, vplus_right(fu2, fu2));
@@ -915,10 +922,10 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
         v1x = v0x; v1y = v0y;
         v0x = Vx; v0y = Vy;
         pc3 = pc2; pc2 = pc1; pc1 = pc0;
-        if constexpr (LIGHT) return;
+        if constexpr (!OUT) return;
 
         // ---- store row j - 2 -----------------------------------------------------------
-        const bool st0 = ok0 && it >= 4, st1 = ok1 && it >= 4;
+        const bool st0 = ok0 && (MID || it >= 4), st1 = ok1 && (MID || it >= 4);
         using OV = typename std::conditional<!DEV, V, typename std::conditional<N == 2, __half2, __half>::type>::type;
         const size_t g0 = (size_t)(y + GHOST) * p.pitch + (size_t)(x + GHOST);
         // nine values and (unless Q is null) phi; images: also into the ghost border
@@ -989,13 +996,17 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
         }
     };
     // (pairs with central faces: a second loop body costs registers, 4096^2 323 -> 371 us; else it
-    // gives 256^2 9.1 -> 8.4, 1024^2 38.5 -> 37.6, 4096^2 354 -> 350 us)
-    constexpr int LIGHT_ROWS = N == 2 && FLUX == 1 ? 0 : 2;
+    // gives 256^2 9.1 -> 8.4, 1024^2 38.5 -> 37.6, 4096^2 354 -> 350 us. MID, single columns: 64^2
+    // 4.8 -> 3.9, 256^2 7.9 -> 7.6, three-stage 64^2 11.8 -> 9.7 us; FP64 loses: 64^2 47.1 -> 48.8)
 #pragma unroll 1
-    for (int it = 0; it < LIGHT_ROWS; it++) row(it, std::true_type{});
+    for (int it = 0; it < LIGHT_ROWS; it++) row(it, std::integral_constant<int, 0>{});
+    if constexpr (MID) {
+#pragma unroll 1
+        for (int it = 2; it < 4; it++) row(it, std::integral_constant<int, 1>{});
+    }
     constexpr int UNROLL = sizeof(T) == 8 ? 1 : 2;   // (FP64: the arithmetic hides the moves that two rows would save)
 #pragma unroll UNROLL
-    for (int it = LIGHT_ROWS; it < npk; it++) row(it, std::false_type{});
+    for (int it = MID ? 4 : LIGHT_ROWS; it < npk; it++) row(it, std::integral_constant<int, 2>{});
     cp_wait<0>();
     if constexpr (SUM == SUM_MASS) {
         for (int o = 16; o > 0; o >>= 1) msum += __shfl_down_sync(ALL, msum, o);
@@ -1006,21 +1017,21 @@ __device__ __forceinline__ void march_strip(const StepParams<typename Lane<V>::T
     }
 }
 
-// One grid: blockIdx.x = strip, blockIdx.y = segment of p.tile_h rows. EARLY: dependents may
+// One grid: blockIdx.x = strip, blockIdx.y = segment of p.tile_h rows. MARCH_EARLY: dependents may
 // be scheduled at once (a grid that leaves room for them on the chip: their velocity factors
 // are ready when this grid ends).
-template <typename V, typename ST, int FLUX, bool FIELD, int KIND, int SUM>
+template <typename V, typename ST, int FLUX, bool FIELD, int KIND, int SUM, bool MID>
 __global__ void __launch_bounds__(32, (sizeof(V) == 4 ? 12 : 8))
 step_march_kernel(const __grid_constant__ StepParams<typename Lane<V>::T> p,
                   const __grid_constant__ MarchCoefs<typename Lane<V>::T> cf,
-                  const __grid_constant__ FastExtra<typename Lane<V>::T> fe, const int early) {
+                  const __grid_constant__ FastExtra<typename Lane<V>::T> fe, const int mode) {
     extern __shared__ __align__(128) unsigned char smem[];
-    if (early) pdl_trigger();
+    if (mode & MARCH_EARLY) pdl_trigger();
     const int y0 = blockIdx.y * p.tile_h;
-    march_strip<V, ST, FLUX, FIELD, KIND, SUM>(
+    march_strip<V, ST, FLUX, FIELD, KIND, SUM, MID>(
         p, cf, fe, blockIdx.x, y0, min(p.tile_h, p.ny - y0),
         SUM == SUM_MASS ? p.mass_partial + blockIdx.y * p.tiles_x + blockIdx.x : nullptr, smem);
-    if (!early) pdl_trigger();
+    if (!(mode & MARCH_EARLY)) pdl_trigger();
 }
 
 // ---- many grids per launch ----------------------------------------------------
