@@ -148,16 +148,7 @@ bool encode_map(CUtensorMap *m, void *base, size_t es, bool half, const dugks_ct
 bool marches(const dugks_ctx *c) { return (c->p.stages == 2 || c->p.stages == 3) && c->p.order <= 3; }
 
 template <typename T, typename ST>
-bool setup_fast(dugks_ctx *c) {
-    if (marches(c)) {
-        c->march = true;
-        const int2 size = make_int2(c->p.nx, c->p.ny);
-        c->plan = march_plan(march_shape(), c->variant, &size, 1, c->p.precision, c->sms);
-        c->tile_w = march_width(c->plan.cols, size.x);
-        c->tile_h = march_segment_rows(c->plan.rows, size.y);
-        return true;
-    }
-    const FastGeom g = Launch<T, ST>::fast_geom(c->p.stages);
+bool encode_maps(dugks_ctx *c, const FastGeom &g) {
     const bool half = Store<T, ST>::deviation;
     for (int s = 0; s < 2; s++)
         if (!encode_map(&c->tmX[s], c->X[s], sizeof(ST), half, c, 9, g.box_w, g.box_h)) return false;
@@ -166,6 +157,26 @@ bool setup_fast(dugks_ctx *c) {
     c->tile_w = g.tile_w;
     c->tile_h = g.tile_h;
     return true;
+}
+
+template <typename T, typename ST>
+bool setup_fast(dugks_ctx *c) {
+    c->coef_h = -1.0;   // (the march and the tiles lay their coefficients out differently)
+    if (marches(c)) {
+        c->march = true;
+        const int2 size = make_int2(c->p.nx, c->p.ny);
+        c->plan = march_plan(march_shape(), c->variant, &size, 1, c->p.precision, c->sms);
+        c->tile_w = march_width(c->plan.cols, size.x);
+        c->tile_h = march_segment_rows(c->plan.rows, size.y);
+        if constexpr (sizeof(T) == 8) {   // (variants 2 and 4: by the rule)
+            const FastGeom g = Launch<T, ST>::tile_geom();
+            if (c->p.stages == 2 && (c->variant == 2 || c->variant == 4) && encode_fn() != nullptr &&
+                tile64_pays(c->plan, size.x, size.y, g.tile_w, g.tile_h, c->sms))
+                c->march = !encode_maps<T, ST>(c, g);
+        }
+        return true;
+    }
+    return encode_maps<T, ST>(c, Launch<T, ST>::fast_geom(c->p.stages));
 }
 
 // the march needs no tensor maps; the TMA-staged kernels need the driver's encoder
@@ -287,6 +298,21 @@ int step_t2(dugks_ctx *c, double *dbg = nullptr) {
         e = Launch<T, ST>::step_fast4(q, *reinterpret_cast<const FaceCoefs<T, 2> *>(c->coefs.data()),
                                       vortex_factors<T>(c, t, t - dt, t + h), c->tmX[c->cur], c->tmPhi[iPo],
                                       c->tmPhi[iPc], c->p.flux, KIND_T2, c->stream);
+    } else if (c->fast && !c->march) {
+        // orders 2 and 3 in FP64, sizes that suit the tiles
+        if constexpr (sizeof(T) == 8) {
+            if (c->coef_h != h) {
+                const FaceCoefs<T> cf = make_face_coefs<T>(c->p.order, c->p.flux, h);
+                c->coefs.assign(reinterpret_cast<const unsigned char *>(&cf),
+                                reinterpret_cast<const unsigned char *>(&cf) + sizeof cf);
+                c->coef_h = h;
+            }
+            e = Launch<T, ST>::step_tile(q, *reinterpret_cast<const FaceCoefs<T> *>(c->coefs.data()),
+                                         vortex_factors<T>(c, t, t - dt, t + h), c->tmX[c->cur], c->tmPhi[iPo],
+                                         c->tmPhi[iPc], c->p.order, c->p.flux, c->stream);
+        } else {
+            return fail(c, DUGKS_EINVAL, "no tile kernel for this precision");
+        }
     } else if (c->fast) {
         // orders 2 and 3: the row march
         if (c->coef_h != h) {

@@ -205,6 +205,7 @@ inline MarchCoefs<T> make_march_coefs(int order, double h) {
 // times s + 2.5 rows (the rows at a segment's ends leave out what they do not need).
 struct MarchPlan {
     int cols, rows, early, one_wave;
+    double cost;   // of a step, as the rule sees it (FP64: in rows of a warp alone on its scheduler, 12.4 us)
     int mode() const { return (early ? MARCH_EARLY : 0) | (one_wave ? MARCH_ONE_WAVE : 0); }
 };
 // strips of a grid for lanes of `cols` columns, their width, segments of about `want` rows and
@@ -244,7 +245,7 @@ inline const MarchShape &dvm_shape() {
 // for `count` grids of sizes (x, y) stepped together
 inline MarchPlan march_plan(const MarchShape &sh, int variant, const int2 *sizes, int count, int precision, int sms) {
     static constexpr int fixed[6] = {16, 8, 0, 32, 0, 64};   // variants 2 and 4: by the rule
-    MarchPlan m{precision == DUGKS_FP64 ? 1 : 2, 16, 0, 0};
+    MarchPlan m{precision == DUGKS_FP64 ? 1 : 2, 16, 0, 0, 0.0};
     double best = 1e300;
     const int forced = variant >= 0 && variant < 6 ? fixed[variant] : 0;
     const bool f64 = precision == DUGKS_FP64;
@@ -275,11 +276,22 @@ inline MarchPlan march_plan(const MarchShape &sh, int variant, const int2 *sizes
                 cost = sh.unit[c] * (rows + sh.extra2) * (W + std::min(0.7, 1.4 / W));
             if (cost < best) {
                 best = cost;
-                m = MarchPlan{cols, want, early, W <= 1.0};
+                // (FP64 warps on every scheduler of an SM: a row takes a tenth longer)
+                m = MarchPlan{cols, want, early, W <= 1.0, f64 && n > 0.8 && n <= 1.0 ? 1.1 * cost : cost};
             }
         }
     }
     return m;
+}
+
+// Whether the FP64 two-stage step of an nx * ny grid takes the tile kernel (tiles of w * h cells, one
+// CTA an SM) and not the march. Both are bound by the FP64 unit and come in steps: the march by the
+// rows of the busiest scheduler, the tiles in waves of 71 us, 5.75 rows. Measured (vortex, us, tile
+// against march): 192^2 76.7 / 75.9, 198^2 77.0 / 81.0, 246^2 76.6 / 97.3, 252^2 143 / 97, 320^2 146 / 136,
+// 360^2 146.6 / 150.3, 380^2 220 / 163. From three waves on the march was faster at every size.
+inline bool tile64_pays(const MarchPlan &m, int nx, int ny, int w, int h, int sms) {
+    const long long tiles = (long long)((nx + w - 1) / w) * ((ny + h - 1) / h), waves = (tiles + sms - 1) / sms;
+    return waves <= 2 && 5.75 * (double)waves < m.cost;
 }
 
 // The expansions of the DVM's streaming (Eq. (12)) at the displacement d xi_k: rows of the

@@ -37,6 +37,11 @@ struct Launch {
     // phi widened to double on the device (host read-out: one copy, no host conversion)
     static cudaError_t phi64(const StepParams<T> &p, double *out, cudaStream_t s);
     static FastGeom fast_geom(int stages);
+    // the two-stage step of orders 2 and 3 on the TMA-staged path (FP64), tile 8 warps x 2 rows
+    static FastGeom tile_geom();
+    static cudaError_t step_tile(const StepParams<T> &p, const FaceCoefs<T> &cf, const FastExtra<T> &fe,
+                                 const CUtensorMap &tmX, const CUtensorMap &tmPo, const CUtensorMap &tmPc, int order,
+                                 int flux, cudaStream_t s);
     // the row march (two-stage, orders 2 and 3): one strip segment of p.tile_h rows per CTA,
     // `cols` columns a lane
     static cudaError_t step_march(const StepParams<T> &p, const MarchCoefs<T> &cf, const FastExtra<T> &fe, int flux,

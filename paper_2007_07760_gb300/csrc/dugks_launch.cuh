@@ -98,14 +98,15 @@ FastGeom Launch<T, ST>::fast_geom(int stages) {
     return stages == 2 ? geom_t<T, ST, o4_nw<T>(), o4_mr<T>(), 2>() : geom_t<T, ST, 8, 2, 2>();
 }
 
-template <typename T, typename ST, int FLUX, int KIND>
-static cudaError_t launch_fast4_t(const StepParams<T> &p, const FaceCoefs<T, 2> &cf, const FastExtra<T> &fe,
-                                  const CUtensorMap &tmX, const CUtensorMap &tmPo, const CUtensorMap &tmPc,
-                                  cudaStream_t s) {
-    constexpr int NW = KIND == KIND_T2 ? o4_nw<T>() : 8, MR = KIND == KIND_T2 ? o4_mr<T>() : 2;
-    using FT = FastTile<T, ST, NW, MR, 2>;
+// Tiles of radius R: orders 4 and 5 (R = 2, every kind), orders 2 and 3 (R = 1, two-stage)
+template <typename T, typename ST, int ORDER, int FLUX, int KIND>
+static cudaError_t launch_fast_t(const StepParams<T> &p, const FaceCoefs<T, (ORDER == 4 ? 2 : 1)> &cf,
+                                 const FastExtra<T> &fe, const CUtensorMap &tmX, const CUtensorMap &tmPo,
+                                 const CUtensorMap &tmPc, cudaStream_t s) {
+    constexpr int NW = ORDER == 4 && KIND == KIND_T2 ? o4_nw<T>() : 8, MR = ORDER == 4 && KIND == KIND_T2 ? o4_mr<T>() : 2;
+    using FT = FastTile<T, ST, NW, MR, (ORDER == 4 ? 2 : 1)>;
     constexpr size_t smem = KIND == KIND_T3A ? FT::smem_bytes_t3a : FT::smem_bytes;
-    auto kern = step_fast_kernel<T, ST, 4, FLUX, NW, MR, KIND>;
+    auto kern = step_fast_kernel<T, ST, ORDER, FLUX, NW, MR, KIND>;
     static std::atomic<uint64_t> configured{0};
     if (cudaError_t e = smem_attr_once(kern, (int)smem, configured); e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -127,17 +128,31 @@ cudaError_t Launch<T, ST>::step_fast4(const StepParams<T> &p, const FaceCoefs<T,
                                       int flux, int kind, cudaStream_t s) {
     if constexpr (Store<T, ST>::t2)
         if (kind == KIND_T2)
-            return flux == 0 ? launch_fast4_t<T, ST, 0, KIND_T2>(p, cf, fe, tmX, tmPo, tmPc, s)
-                             : launch_fast4_t<T, ST, 1, KIND_T2>(p, cf, fe, tmX, tmPo, tmPc, s);
+            return flux == 0 ? launch_fast_t<T, ST, 4, 0, KIND_T2>(p, cf, fe, tmX, tmPo, tmPc, s)
+                             : launch_fast_t<T, ST, 4, 1, KIND_T2>(p, cf, fe, tmX, tmPo, tmPc, s);
     if constexpr (Store<T, ST>::t3) {
         if (kind == KIND_T3A)
-            return flux == 0 ? launch_fast4_t<T, ST, 0, KIND_T3A>(p, cf, fe, tmX, tmPo, tmPc, s)
-                             : launch_fast4_t<T, ST, 1, KIND_T3A>(p, cf, fe, tmX, tmPo, tmPc, s);
+            return flux == 0 ? launch_fast_t<T, ST, 4, 0, KIND_T3A>(p, cf, fe, tmX, tmPo, tmPc, s)
+                             : launch_fast_t<T, ST, 4, 1, KIND_T3A>(p, cf, fe, tmX, tmPo, tmPc, s);
         if (kind == KIND_T3B)
-            return flux == 0 ? launch_fast4_t<T, ST, 0, KIND_T3B>(p, cf, fe, tmX, tmPo, tmPc, s)
-                             : launch_fast4_t<T, ST, 1, KIND_T3B>(p, cf, fe, tmX, tmPo, tmPc, s);
+            return flux == 0 ? launch_fast_t<T, ST, 4, 0, KIND_T3B>(p, cf, fe, tmX, tmPo, tmPc, s)
+                             : launch_fast_t<T, ST, 4, 1, KIND_T3B>(p, cf, fe, tmX, tmPo, tmPc, s);
     }
     return cudaErrorInvalidValue;
+}
+
+template <typename T, typename ST>
+FastGeom Launch<T, ST>::tile_geom() { return geom_t<T, ST, 8, 2, 1>(); }
+
+template <typename T, typename ST>
+cudaError_t Launch<T, ST>::step_tile(const StepParams<T> &p, const FaceCoefs<T> &cf, const FastExtra<T> &fe,
+                                     const CUtensorMap &tmX, const CUtensorMap &tmPo, const CUtensorMap &tmPc, int order,
+                                     int flux, cudaStream_t s) {
+    if (order == 2)
+        return flux == 0 ? launch_fast_t<T, ST, 2, 0, KIND_T2>(p, cf, fe, tmX, tmPo, tmPc, s)
+                         : launch_fast_t<T, ST, 2, 1, KIND_T2>(p, cf, fe, tmX, tmPo, tmPc, s);
+    return flux == 0 ? launch_fast_t<T, ST, 3, 0, KIND_T2>(p, cf, fe, tmX, tmPo, tmPc, s)
+                     : launch_fast_t<T, ST, 3, 1, KIND_T2>(p, cf, fe, tmX, tmPo, tmPc, s);
 }
 
 // CALL with the lane type of `cols` columns
