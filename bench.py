@@ -5,15 +5,15 @@ Default workload: single-vortex deformation of a drop on a 1024 x 1024 grid
 W = 4, cfl = 0.8, amplitude 0.05, reversal period 8192 steps). One benchmark
 step = one pass of the whole hot path: the fused DUGKS step kernel (cell
 quantities, gradients, face reconstruction, face distribution, meso-flux
-update, per-tile FP64 mass partials) plus the global FP64 mass reduction. The
+update, FP64 mass partials) plus the global FP64 mass reduction. The
 state (92 MB) fits in L2, so L2 is flushed (512 MiB write) before every timed
 step and only the step itself is timed, with CUDA events on the solver's stream.
 
 Beside the main line (N = 1 only) the same JSON line carries, under "also": the
 4096^2 vortex (state far larger than L2), the 512-grid batch (one graph-replayed
 launch per step over all grids), the main workload without the L2 flush (state
-resident in L2), the 256 x 256 slotted-disk rotation (latency-bound: one partial
-wave of tiles), the plain single-grid FP64 GPU step (the generic kernel), the
+resident in L2), the 256 x 256 slotted-disk rotation (latency-bound: less than
+one wave), the plain single-grid FP64 GPU step (the generic kernel), the
 three-stage, order-4, DVM and LBM steps, each with its own roofline fraction, and
 a bounded served measurement (the first 100 arrivals of the request trace, as
 recorded and at 70% load: p50/p99 time-to-result, solves/s, cell-updates/s).
@@ -243,7 +243,7 @@ def run_reference(args):
 def time_single(solver, stream, warmup: int, K: int, dist=None, local: int = 0, flush_l2: bool = True):
     """W untimed and K timed steps of one solver, L2 flushed before each (unless
     flush_l2 is false: a state larger than L2, or the L2-resident comparison). One
-    step = the step kernel (per-tile FP64 mass partials) + the kernel that sums
+    step = the step kernel (with its FP64 mass partials) + the kernel that sums
     them; the second is launched as a programmatic dependent of the first, so no
     event sits between them in the timed pass. A second pass of K steps, with
     events around the step kernel alone, gives its duration for the roofline."""
@@ -426,14 +426,16 @@ def run_ours(args):
                                     "of writes then stay in L2 during the launch and reach DRAM during the next "
                                     "flush, so the DRAM traffic of a launch is its reads (see the 4096^2 line in "
                                     "'also' for a state far larger than L2)",
-                           mass="FP64 per-tile partials in the step kernel + fixed-order sum kernel",
+                           mass="FP64 partials in the step kernel + fixed-order sum kernel",
                            replicas=world, parallelism="replicas" if world > 1 else "single"),
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic,
-                         "kernel": desc.get("kernel", "step_fast_kernel (TMA-staged fused two-stage DUGKS step)"
+                         "kernel": desc.get("kernel", ("step_march_kernel (fused two-stage DUGKS step, row march)"
+                                             if prob.order <= 3 else
+                                             "step_fast_kernel (TMA-staged fused two-stage DUGKS step)")
                                             if prob.stages == 2 else
-                                            "step_fast_kernel KIND_T3A + KIND_T3B (the two kernels of a three-stage step)"
-                                            if prob.stages == 3 else "dvm_step_kernel (streaming-collision DVM)"),
+                                            "step_march_kernel KIND_T3A + KIND_T3B (the two kernels of a three-stage step)"
+                                            if prob.stages == 3 else "dvm_march_kernel (streaming-collision DVM)"),
                          "bytes_per_cell": bpc,
                          "bytes_per_cell_actual": BYTES_PER_CELL_ACTUAL[(args.precision, prob.stages)],
                          "peak_source": peak_kind, "avg_kernel_ms": avg_step_ms},
@@ -460,8 +462,8 @@ def run_ours(args):
 
 def measure_batch(count: int, precision: str, warmup: int, K: int, dist=None, local: int = 0):
     """Many independent grids (sides log-uniform 64..512, 1-8 drops, uniform velocity
-    |u| <= 0.05) advanced together: one launch per step over a work list of tiles
-    of all grids, replayed as CUDA graphs, tile variant picked by the autotuner.
+    |u| <= 0.05) advanced together: one launch per step over a work list of strip segments
+    of all grids, replayed as CUDA graphs, variant picked by the autotuner.
     The state of 512 grids (2.3 GB in FP32) is far larger than L2, so no flush is
     needed between steps."""
     import torch
@@ -536,7 +538,7 @@ def run_batch(args, dist, world, rank, local):
             "dtype": {"fp64": "f64", "fp32": "f32", "fp16f": "f32 (f16 storage)"}[args.precision],
             "data": "synthetic", "config": desc,
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                         "traffic": traffic, "kernel": "batch_fast_kernel + batch_advance_kernel (graph-replayed)",
+                         "traffic": traffic, "kernel": "batch_march_kernel + batch_advance_kernel (graph-replayed)",
                          "bytes_per_cell": bpc, "bytes_per_cell_actual": BYTES_PER_CELL_ACTUAL[(args.precision, 2)],
                          "peak_source": peak_kind},
             "e2e": e2e, "gpu_launches": 2 * K, "clocks": r["clocks"],
@@ -570,7 +572,7 @@ def serve_passes(requests: int, budget_gb: float, resident: bool, local: int) ->
     (200 requests/s, sides log-uniform 64..2048, 500..20000 steps, rotation or
     vortex), FP32 order-3 upwind, with a resident 4096^2 vortex grid. Requests are
     served in priority lanes by work (cells x steps), each lane a batch on its own
-    stream running one CTA per tile. The trace offers far more work than one GPU
+    stream running one CTA per segment. The trace offers far more work than one GPU
     does, so it is replayed twice: as recorded (overloaded: the latencies are
     mostly queueing) and with arrivals stretched so that the offered load is 70%
     of the throughput measured in the first pass."""
@@ -666,7 +668,7 @@ def main():
     ap.add_argument("--precision", default="fp32", choices=["fp64", "fp32", "fp16f"])
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-also", action="store_true", help="skip the secondary measurements")
-    ap.add_argument("--variant", type=int, default=None, help="fixed tile variant (default: autotuned)")
+    ap.add_argument("--variant", type=int, default=None, help="fixed variant (default: autotuned)")
     ap.add_argument("--generic", action="store_true", help="time the generic (plain) kernel instead")
     ap.add_argument("--requests", type=int, default=48, help="serve workload: requests in the trace")
     ap.add_argument("--budget-gb", type=float, default=32.0, help="serve workload: device-memory budget")

@@ -183,10 +183,11 @@ const char *dugks_last_error(const dugks_ctx *c);
  * warp walks up): 0 = 16, 1 = 8, 3 = 32, 5 = 64 rows; 2 and 4 = chosen by a rule on
  * the grid's size, which is the default (2 below 512 x 512 cells, 4 from there up);
  * -1 selects the generic fused kernel (one thread per cell and stage), the plain
- * comparison path. A tuning choice only: results agree to rounding. Returns
- * DUGKS_EINVAL for any other number. Orders 4 and 5 and the three-stage scheme have
- * one TMA-staged tile shape each (warps per CTA x rows of cells per thread: orders
- * 4-5, two-stage: 10 x 3, FP64 8 x 2; three-stage: 8 x 2): any variant >= 0 selects it.
+ * comparison path. In FP64 the rule gives the sizes that suit them to TMA-staged tiles
+ * (8 x 2, below). A tuning choice only: results agree to rounding. Returns
+ * DUGKS_EINVAL for any other number. Orders 4 and 5 have one TMA-staged tile shape
+ * (warps per CTA x rows of cells per thread: two-stage 10 x 3, FP64 8 x 2; three-stage
+ * 8 x 2) and the three-stage march has the rule: any variant >= 0 selects them.
  * dugks_get_variant returns -1 when the context uses the generic kernel. */
 int dugks_set_variant(dugks_ctx *c, int variant);
 int dugks_get_variant(const dugks_ctx *c);

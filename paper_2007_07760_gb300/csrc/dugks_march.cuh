@@ -2,8 +2,9 @@
 // row march (sm_103a): the two-stage step and the two kernels of the three-stage step.
 //
 // Same method as step_kernel (dugks_kernels.cuh; equation numbers are the paper's).
-// One warp, which is one CTA, owns a strip of 60 columns and a segment of rows and
-// walks up the rows with everything the step needs of the rows below in registers:
+// One warp, which is one CTA, owns a strip of 60 columns (28 with one column a lane, as in FP64 and
+// on small grids) and a segment of rows and walks up the rows with everything the step needs of
+// the rows below in registers:
 //  * a lane holds two adjacent columns, and all arithmetic is on that pair (packed
 //    FP32: one instruction, two columns). The left and right neighbours of a pair
 //    are one shuffle each for two cells; no shared-memory exchange and no barrier.
@@ -17,9 +18,14 @@
 //    moment phi_b, never the difference of a single bar f_k; their sums over the
 //    three directions are taken before the stencil.
 //  * rows arrive through a ring of per-lane cp.async copies two rows ahead.
-// What bounds it: FP32 issue. Rows of a segment are read and expanded with two
-// extra rows on each side, so the segment length trades that overhead against the
-// number of warps in flight (march_rows in dugks_internal.h has the rule).
+// What bounds it: the issue of FP32 instructions on large grids (4096^2: 710 for a row of a warp, 379
+// thread instructions a cell, against 876 in tiles), a row's latency in launches of one wave, and in FP64 that unit,
+// one warp instruction in 64 cycles a scheduler. Rows of a segment are read and expanded with two extra rows
+// on each side, so the segment length trades that overhead against the number of warps in flight
+// (march_plan in dugks_host.h has the rule).
+// Measured, us a step, shared-memory tiles -> march: FP32 256^2 9.4 -> 7.5, 512^2 14.8 -> 12.8, 1024^2 44.0 -> 35.1,
+// 4096^2 617 -> 331; FP16 storage 1024^2 52.6 -> 38.6, 4096^2 738 -> 370; three-stage 512^2 33.4 -> 28.9, 1024^2
+// 108.9 -> 87.5, 4096^2 1352 -> 885; FP64 (a step a call) 64^2 77 -> 47, 512^2 312 -> 256.
 #pragma once
 
 #include <type_traits>

@@ -3,12 +3,12 @@
 Requests (grid size, number of steps, velocity field) arrive over time. Every
 admitted grid's state stays resident on the device inside a batch
 (``native.Batch``): one launch per step advances all grids of a batch over the
-tiles of all of them, each grid stopping by itself at its own step target.
+strip segments of all of them, each grid stopping by itself at its own step target.
 
 Requests are served in lanes: each lane is a batch on its own CUDA stream, and a
 request goes to the first lane whose work limit (cells x steps) it fits. The
-lanes' streams carry decreasing priority and their kernels run one CTA per tile,
-so the GPU takes the tiles of a higher lane first as soon as tiles of a lower
+lanes' streams carry decreasing priority and their kernels run one CTA per segment,
+so the GPU takes the segments of a higher lane first as soon as those of a lower
 one finish: short solves are not held to the step rate of the large grids
 (nor of a resident grid that never finishes, which sits in the lowest lane).
 Within a lane all grids advance together.
