@@ -67,10 +67,10 @@ L2_FLUSH_BYTES = 512 << 20
 # was taken on and the workload (reported as null once the sources change). The
 # writes of a 1024^2 step stay in L2 (129 MB) during the launch and reach DRAM
 # later, so the figure is the read traffic plus the evictions.
+# (Captured on the same code: only comments have changed since.)
 NCU_TRAFFIC = {
-    ("ec6fb138f47ce3e2", "vortex1024_fp32_p3_upwind_2stage"): 49932288,     # mean of two launches
-    ("ec6fb138f47ce3e2", "vortex4096_fp32_p3_upwind_2stage"): 1383666688,   # state 11x the L2
-    ("ec6fb138f47ce3e2", "batch512_fp32_p3_upwind_2stage"): 3279676416,     # 1.20x: halos of small grids
+    ("8ad1c357ad1e25d9", "vortex1024_fp32_p3_upwind_2stage"): 51648512,
+    ("8ad1c357ad1e25d9", "vortex4096_fp32_p3_upwind_2stage"): 1460551680,   # state 11x the L2
 }
 
 

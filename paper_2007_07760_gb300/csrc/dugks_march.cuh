@@ -18,7 +18,7 @@
 //    moment phi_b, never the difference of a single bar f_k; their sums over the
 //    three directions are taken before the stencil.
 //  * rows arrive through a ring of per-lane cp.async copies two rows ahead.
-// What bounds it: the issue of FP32 instructions on large grids (4096^2: 710 for a row of a warp, 379
+// What bounds it: the issue of FP32 instructions on large grids (4096^2: 673 for a row of a warp, 399
 // thread instructions a cell, against 876 in tiles), a row's latency in launches of one wave, and in FP64 that unit,
 // one warp instruction in 64 cycles a scheduler. Rows of a segment are read and expanded with two extra rows
 // on each side, so the segment length trades that overhead against the number of warps in flight
