@@ -1121,12 +1121,13 @@ __device__ __forceinline__ void batch_step_params(const BatchUniform<T> &u, cons
 }
 
 // Step `ofs` of the group: CTAs stride over the work list (grid, strip, first row, rows).
+// (The descriptors are read with ordinary loads, not __restrict__: this kernel may be resident while
+// the kernel ahead of it still writes them, and only a load that the wait orders sees the new counters.)
 template <typename V, typename ST, int FLUX>
 __global__ void __launch_bounds__(32, (sizeof(V) == 4 ? 12 : 8))
 batch_march_kernel(const __grid_constant__ BatchUniform<typename Lane<V>::T> u,
                    const __grid_constant__ MarchCoefs<typename Lane<V>::T> cf,
-                   const BatchGrid<typename Lane<V>::T> *__restrict__ grids, const int4 *__restrict__ items, int nitems,
-                   int ofs) {
+                   const BatchGrid<typename Lane<V>::T> *grids, const int4 *items, int nitems, int ofs) {
     using T = typename Lane<V>::T;
     extern __shared__ __align__(128) unsigned char smem[];
     pdl_wait();   // the previous step's output, or the advanced descriptors
