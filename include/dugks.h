@@ -290,7 +290,9 @@ int64_t dugks_batch_step_index(const dugks_batch *b, int32_t grid_id);
 /* Waits and copies phi (ny * nx doubles) of one grid to the host. */
 int dugks_batch_read_phi(dugks_batch *b, int32_t grid_id, double *out_host);
 
-/* Waits and returns one grid's mass (FP64, fixed-order sum over phi of its state). */
+/* Waits and returns one grid's mass (to FP64 precision, fixed-order sum over phi of its state). The first
+ * mass asked of a state is summed alone, the second together with those of all grids, so that a loop over
+ * the grids sums them in a launch or a few. */
 int dugks_batch_mass(dugks_batch *b, int32_t grid_id, double *out);
 
 /* Segment length of the batch kernel (0..5 as for dugks_set_variant; default 4, by the

@@ -6,6 +6,7 @@ namespace dugks {
 template cudaError_t Launch<float,float>::step(const StepParams<float> &, int, int, int, cudaStream_t);
 template cudaError_t Launch<float,float>::init(const StepParams<float> &, const float *, float, int, cudaStream_t);
 template cudaError_t Launch<float,float>::mass_partial(const StepParams<float> &, cudaStream_t);
+template cudaError_t Launch<float,float>::mass(const MassList<float> &, int, int, double *, unsigned *, double *, int *, cudaStream_t);
 template cudaError_t Launch<float,float>::phi(const StepParams<float> &, float *, cudaStream_t);
 template cudaError_t Launch<float,float>::phi64(const StepParams<float> &, double *, cudaStream_t);
 }  // namespace dugks

@@ -33,6 +33,9 @@ struct Launch {
     static cudaError_t step(const StepParams<T> &p, int order, int flux, int kind, cudaStream_t s);
     static cudaError_t init(const StepParams<T> &p, const T *phi0, T frac_dt, int order, cudaStream_t s);
     static cudaError_t mass_partial(const StepParams<T> &p, cudaStream_t s);
+    // masses of `count` grids of at most `tiles` tiles into out[slot]; part: MASS_TILES a grid; counters: 0
+    static cudaError_t mass(const MassList<T> &list, int count, int tiles, double *part, unsigned *counters, double *out,
+                            int *status, cudaStream_t s);
     static cudaError_t phi(const StepParams<T> &p, T *out, cudaStream_t s);
     // phi widened to double on the device (host read-out: one copy, no host conversion)
     static cudaError_t phi64(const StepParams<T> &p, double *out, cudaStream_t s);

@@ -725,6 +725,83 @@ __global__ void __launch_bounds__(256) mass_partial_kernel(const StepParams<T> p
     if (threadIdx.x == 0) p.mass_partial[blockIdx.y * p.tiles_x + blockIdx.x] = s;
 }
 
+// a becomes fl(a + b); returns the error (two-sum)
+__device__ __forceinline__ float two_sum(float &a, float b) {
+    const float t = __fadd_rn(a, b), bb = __fsub_rn(t, a);
+    const float r = __fadd_rn(__fsub_rn(a, __fsub_rn(t, bb)), __fsub_rn(b, bb));
+    a = t;
+    return r;
+}
+
+// The masses of up to MASS_LIST grids in one launch. CTA (t, i) sums tile t of grid i into `part`, the last
+// one of a grid to finish adds its tiles in their order into out[slot], which may be pinned host memory: the
+// caller has only to wait for the stream. count[i] is 0 before and after.
+// A lane sums FP32 cells in FP32: the error of each addition goes to a second word, that word's to
+// a third, so what is lost is below 2^-70 of the sum (an FP64 addition loses 2^-53); with an FP64
+// conversion and addition a cell, 64 cycles of a scheduler's unit each, 4096^2 cells would take 53 us.
+// Bound by the latency of three trips to memory and of the sums' trees, on large grids by the memory. Measured,
+// a call with its wait (two launches over 32 x 8 tiles and a copy before): FP32 64^2 20 -> 15 us, 1024^2 41 -> 18,
+// 2048^2 91 -> 21; all of 64 grids of 64^2 1280 -> 200.
+constexpr int MASS_LIST = 64, MASS_TILES = 576;
+template <typename T>
+struct MassGrid {
+    const void *X;
+    const T *phi;
+    size_t plane;
+    int nx, ny, pitch, tile_w, tile_h, slot;
+};
+template <typename T>
+struct MassList { MassGrid<T> g[MASS_LIST]; };
+
+template <typename T, typename ST>
+__global__ void __launch_bounds__(256)
+mass_kernel(const __grid_constant__ MassList<T> list, double *part, unsigned *count, double *out, int *status) {
+    __shared__ double sred[32];
+    __shared__ bool last;
+    const MassGrid<T> &G = list.g[blockIdx.y];
+    const unsigned across = (G.nx + G.tile_w - 1) / G.tile_w, n = across * ((G.ny + G.tile_h - 1) / G.tile_h);
+    if (blockIdx.x >= n) return;
+    StepParams<T> p;
+    p.X = G.X;
+    p.phi_cur = G.phi;
+    p.plane = G.plane;
+    p.pitch = G.pitch;
+    const int by = blockIdx.x / across, bx = blockIdx.x - by * across, lane = threadIdx.x & 31;
+    const int x1 = min(G.nx, (bx + 1) * G.tile_w), y1 = min(G.ny, (by + 1) * G.tile_h);
+    auto cells = [&](auto add) {
+        for (int gy = by * G.tile_h + (threadIdx.x >> 5); gy < y1; gy += 8)
+#pragma unroll 8
+            for (int gx = bx * G.tile_w + lane; gx < x1; gx += 32) add(cell_phi<T, ST>(p, gidx(p, gx, gy)));
+    };
+    double m = 0.0;
+    if constexpr (sizeof(T) == 8) {
+        cells([&](T v) { m += v; });
+    } else {
+        float s = 0.0f, e = 0.0f, f = 0.0f;
+        cells([&](T v) { f += two_sum(e, two_sum(s, v)); });
+        if (isfinite(s)) m = (double)s + ((double)e + (double)f);
+        else cells([&](T v) { m += (double)v; });   // beyond FP32, or not finite at all
+    }
+    m = block_sum(m, sred);
+    part += (size_t)blockIdx.y * MASS_TILES;
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = m;
+        __threadfence();
+        last = atomicAdd(count + blockIdx.y, 1u) == n - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    m = 0.0;
+    for (unsigned i = threadIdx.x; i < n; i += 256) m += __ldcg(part + i);
+    m = block_sum(m, sred);
+    if (threadIdx.x == 0) {
+        out[G.slot] = m;
+        if (!isfinite(m)) atomicOr(status, 1);
+        count[blockIdx.y] = 0;
+    }
+}
+
 // phi of the state into a dense ny * nx array of T
 template <typename T, typename ST, typename O = T>
 __global__ void phi_kernel(const StepParams<T> p, O *out) {

@@ -79,6 +79,13 @@ cudaError_t Launch<T, ST>::mass_partial(const StepParams<T> &p, cudaStream_t s) 
     return cudaGetLastError();
 }
 
+template <typename T, typename ST>
+cudaError_t Launch<T, ST>::mass(const MassList<T> &list, int count, int tiles, double *part, unsigned *counters,
+                                double *out, int *status, cudaStream_t s) {
+    mass_kernel<T, ST><<<dim3(tiles, count), 256, 0, s>>>(list, part, counters, out, status);
+    return cudaGetLastError();
+}
+
 template <typename T, typename ST, int NW, int MR, int R = 1>
 static FastGeom geom_t() {
     using FT = FastTile<T, ST, NW, MR, R>;
