@@ -65,8 +65,11 @@ struct dugks_batch {
     int nphi = 2;
     int variant = 4;    // segment length: by the rule of march_plan
     MarchPlan plan{};
+    MarchWork work;             // segments of the grids that advance, and their sizes there by slot (0: none)
+    std::vector<int2> counted;
     int rows = 0;       // the longest segment of the work list
     int ctas = 0;
+    int resident = 0, resident_cols = 0, resident_rows = 0;   // CTAs that the GPU holds, for segments of that shape
     int ctas_req = 0;   // 0: resident CTAs (grid-stride); < 0: one CTA per segment; > 0: at most that many
     std::vector<Slot> slots;
     cudaMemPool_t pool = nullptr;   // grid memory, descriptors and the work list
@@ -251,13 +254,17 @@ size_t plane_of(int nx, int ny, int *pitch_out) {
 }
 
 int resident_ctas(dugks_batch *b) {
+    if (b->resident > 0 && b->resident_cols == b->plan.cols && b->resident_rows == b->rows) return b->resident;
     int per = 1;
     switch (b->p.precision) {
     case DUGKS_FP64: per = Launch<double, double>::batch_ctas_per_sm(b->p.flux, b->plan.cols, b->rows); break;
     case DUGKS_FP32: per = Launch<float, float>::batch_ctas_per_sm(b->p.flux, b->plan.cols, b->rows); break;
     default: per = Launch<float, __half>::batch_ctas_per_sm(b->p.flux, b->plan.cols, b->rows); break;
     }
-    return std::max(1, b->sms) * std::max(1, per);
+    b->resident = std::max(1, b->sms) * std::max(1, per);
+    b->resident_cols = b->plan.cols;
+    b->resident_rows = b->rows;
+    return b->resident;
 }
 
 // By default resident CTAs striding over a list that is little longer (32 grids of 64^2 to
@@ -331,9 +338,18 @@ int rebuild_t(dugks_batch *b) {
     }
     auto live = [](const Slot &s) { return s.used && !s.retiring && (s.target < 0 || s.step < s.target); };
     std::vector<int2> sizes;
-    for (const Slot &s : b->slots)
-        if (live(s)) sizes.push_back(make_int2(s.nx, s.ny));
-    b->plan = march_plan(march_shape(), b->variant, sizes.data(), (int)sizes.size(), b->p.precision, b->sms);
+    b->counted.resize(n, make_int2(0, 0));
+    for (int i = 0; i < n; i++) {
+        const Slot &s = b->slots[i];
+        const int2 now = live(s) ? make_int2(s.nx, s.ny) : make_int2(0, 0);
+        int2 &was = b->counted[i];
+        if (now.x) sizes.push_back(now);
+        if (now.x == was.x && now.y == was.y) continue;
+        if (was.x) b->work.count(march_shape(), was, -1);
+        if (now.x) b->work.count(march_shape(), now, 1);
+        was = now;
+    }
+    b->plan = march_plan(march_shape(), b->variant, b->work, sizes.data(), (int)sizes.size(), b->p.precision, b->sms);
     int nitems = 0;
     b->rows = 1;
     for (const int2 &q : sizes) {
