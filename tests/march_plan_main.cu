@@ -1,5 +1,5 @@
-// Host program of test_march_plan.py. Input lines: precision variant sms count x y x y ...; output lines:
-// columns and rows of the plan, from segments that were counted one grid at a time, with others
+// Host program of march_plans.py. Input lines: kernel (0 DUGKS, 1 DVM) precision variant sms count x y x y ...;
+// output lines: columns, rows and mode of the plan, from segments that were counted one grid at a time, with others
 // that came and went, and from a pass over all grids for every plan.
 #include <cstdio>
 
@@ -28,25 +28,28 @@ static MarchPlan by_passes(const MarchShape &sh, int variant, const std::vector<
             for (int c = 0; c < 2; c++)
                 for (int r = 1; r <= MARCH_ROWS; r++)
                     if (c != cols - 1 || r != rows) one.n[c][r] = (int64_t)1 << 50;
-            const MarchPlan p = march_plan(sh, -1, one, nullptr, 0, precision, sms);
+            MarchPlan p = march_plan(sh, -1, one, nullptr, 0, precision, sms);
+            const double n = (double)one.n[cols - 1][rows] / (4.0 * sms);
+            if (precision == DUGKS_FP64 && n > 0.8 && n <= 1.0) p.cost /= 1.1;   // (added once a plan is chosen)
             if (p.cost < best.cost) best = MarchPlan{cols, want, p.early, p.one_wave, p.cost};
         }
     return best;
 }
 
 int main() {
-    int precision, variant, sms, count;
-    while (std::scanf("%d %d %d %d", &precision, &variant, &sms, &count) == 4) {
+    int kernel, precision, variant, sms, count;
+    while (std::scanf("%d %d %d %d %d", &kernel, &precision, &variant, &sms, &count) == 5) {
+        const MarchShape &sh = kernel ? dvm_shape() : march_shape();
         std::vector<int2> sizes(count);
         MarchWork work;
         for (int2 &q : sizes) {
             if (std::scanf("%d %d", &q.x, &q.y) != 2) return 1;
-            work.count(march_shape(), q, 1);
-            work.count(march_shape(), make_int2(q.y + 3, q.x), 1);   // a grid that leaves again
+            work.count(sh, q, 1);
+            work.count(sh, make_int2(q.y + 3, q.x), 1);   // a grid that leaves again
         }
-        for (int2 q : sizes) work.count(march_shape(), make_int2(q.y + 3, q.x), -1);
-        const MarchPlan a = march_plan(march_shape(), variant, work, sizes.data(), count, precision, sms);
-        const MarchPlan b = by_passes(march_shape(), variant, sizes, precision, sms);
+        for (int2 q : sizes) work.count(sh, make_int2(q.y + 3, q.x), -1);
+        const MarchPlan a = march_plan(sh, variant, work, sizes.data(), count, precision, sms);
+        const MarchPlan b = by_passes(sh, variant, sizes, precision, sms);
         std::printf("%d %d %d %d %d %d\n", a.cols, a.rows, a.mode(), b.cols, b.rows, b.mode());
     }
     return 0;
