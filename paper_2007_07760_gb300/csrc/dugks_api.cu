@@ -614,12 +614,13 @@ cudaError_t dev_malloc_pool(void **p, size_t bytes, cudaMemPool_t pool, cudaStre
 // Thread t adds partials t, t + 256, ... in index order with 8 independent loads
 // in flight (one memory latency per 8 partials), then the fixed tree of block_sum.
 // One small CTA: it finds a free slot while the step kernel drains.
-// early: the next kernel may be placed while the step ahead still runs (where that costs the
-// march nothing: MarchPlan::early; FP64 512^2 step and mass: 331 us with, 258 without).
-__global__ void __launch_bounds__(256)
-mass_final_kernel(const double *partial, int n, double *out, int *status, int early) {
+// EARLY: the next kernel may be placed while the step ahead still runs (where that costs the
+// march nothing: MarchPlan::early; FP64 512^2 step and mass: 331 us with, 258 without). Not an argument: loading
+// it first put the next kernel off (order 4, 256^2, step and mass: 15.26 -> 15.37 us, three-stage 200^2 27.10 -> 27.22).
+template <bool EARLY>
+__global__ void __launch_bounds__(256) mass_final_kernel(const double *partial, int n, double *out, int *status) {
     __shared__ double sred[32];
-    if (early) pdl_trigger();
+    if (EARLY) pdl_trigger();
     pdl_wait();   // the partials of the step kernel ahead of it
     constexpr int U = 8;
     double s = 0.0;
@@ -649,7 +650,8 @@ cudaError_t launch_mass_final(const double *partial, int n, double *out, int *st
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, mass_final_kernel, partial, n, out, status, early);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, early ? mass_final_kernel<true> : mass_final_kernel<false>, partial, n, out,
+                                       status);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }

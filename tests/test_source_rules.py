@@ -26,3 +26,10 @@ def test_dependent_kernels_read_with_ordered_loads():
     assert {"step_march_kernel", "batch_march_kernel", "batch_advance_kernel", "dvm_march_kernel", "step_fast_kernel",
             "mass_final_kernel"} <= set(found)
     assert not [k for k, bad in found.items() if bad]
+
+
+def test_mass_sum_triggers_before_it_reads_an_argument():
+    """The next step is placed when the sum's one CTA triggers: 0.11 us later where an argument is loaded first."""
+    params, body = next((p, b) for name, p, b in kernels() if name == "mass_final_kernel")
+    before = body[:body.index("pdl_trigger()")]
+    assert not [w for w in re.findall(r"(\w+)\s*(?:,|$)", params) if re.search(rf"\b{w}\b", before)]
