@@ -165,7 +165,7 @@ bool setup_fast(dugks_ctx *c) {
     if (marches(c)) {
         c->march = true;
         const int2 size = make_int2(c->p.nx, c->p.ny);
-        c->plan = march_plan(march_shape(), c->variant, size, c->p.precision, c->sms);
+        c->plan = march_plan(march_shape(c->p.stages, c->p.flux), c->variant, size, c->p.precision, c->sms);
         c->tile_w = march_width(c->plan.cols, size.x);
         c->tile_h = march_segment_rows(c->plan.rows, size.y);
         if constexpr (sizeof(T) == 8) {   // (variants 2 and 4: by the rule)
@@ -732,7 +732,7 @@ int dugks_create(const dugks_params *p, const double *phi0_host, void *cuda_stre
     }
     if (dvm_marches(c)) {
         const int2 size = make_int2(p->nx, p->ny);
-        c->plan = march_plan(dvm_shape(), -1, size, p->precision, c->sms);
+        c->plan = march_plan(dvm_shape(p->cfl), -1, size, p->precision, c->sms);
         c->tile_w = dvm_march_width(c->plan.cols);
         c->tile_h = march_segment_rows(c->plan.rows, p->ny);
     }

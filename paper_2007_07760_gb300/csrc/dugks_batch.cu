@@ -336,6 +336,7 @@ int rebuild_t(dugks_batch *b) {
         b->d_grids = grids;
         b->grids_cap = cap;
     }
+    const MarchShape &shape = march_shape(2, b->p.flux);
     auto live = [](const Slot &s) { return s.used && !s.retiring && (s.target < 0 || s.step < s.target); };
     std::vector<int2> sizes;
     b->counted.resize(n, make_int2(0, 0));
@@ -345,11 +346,11 @@ int rebuild_t(dugks_batch *b) {
         int2 &was = b->counted[i];
         if (now.x) sizes.push_back(now);
         if (now.x == was.x && now.y == was.y) continue;
-        if (was.x) b->work.count(march_shape(), was, -1);
-        if (now.x) b->work.count(march_shape(), now, 1);
+        if (was.x) b->work.count(shape, was, -1);
+        if (now.x) b->work.count(shape, now, 1);
         was = now;
     }
-    b->plan = march_plan(march_shape(), b->variant, b->work, sizes.data(), (int)sizes.size(), b->p.precision, b->sms);
+    b->plan = march_plan(shape, b->variant, b->work, sizes.data(), (int)sizes.size(), b->p.precision, b->sms);
     int nitems = 0;
     b->rows = 1;
     for (const int2 &q : sizes) {

@@ -193,11 +193,15 @@ inline MarchCoefs<T> make_march_coefs(int order, double h) {
 
 // Lane width (columns a lane), segment rows and launch mode of the row march.
 // A segment of s rows reads s + 4 (the DVM s + 6), so long segments do less work, and short ones give
-// more warps. The costs below are fits to measured steps (FP32, vortex, 64^2 to 4096^2, s from 1 to 64,
-// both widths; mostly within 5%). In one wave of warps a row takes as long as the most warps on one
-// scheduler make it, in several waves it takes `unit` and part of a wave is lost at the end.
-// Measured: 64^2 5.1 us (1 column, s = 1) against 7.8 us with pairs; 256^2 8.3 (1, 2) against 11.4;
-// 450^2 10.8 (2, 3) against 12.8; 1024^2 36.0 (2, 16) against 39; 4096^2 330 (2, 32) against 383.
+// more warps. The costs below are fits to measured steps: FP32 and FP16 storage, 69 sizes from 48^2 to 4096^2
+// and 64 x 256 to 3000 x 300, rows from 1 to 64, both widths, dugks_step(n) and step-and-mass loops. In one wave
+// of warps a row takes longer with every warp that an SM holds, in several waves it takes `unit` and part of
+// a wave is lost at the end. The plan that the costs choose against the best one measured, mean and largest: two-stage
+// upwind 1.008 and 1.07, central 1.006 and 1.07, three-stage 1.006 and 1.10, central 1.002 and 1.04, DVM 1.016
+// and 1.11, below dt = 1/2 1.013 and 1.11, LBM 1.025 and 1.24. (One set of constants for all DUGKS steps
+// and one for all DVM steps had given 1.010 and 1.17, 1.022 and 1.37, 1.031 and 1.36, 1.036 and 1.54, 1.045 and 1.24, 1.043
+// and 1.21, 1.125 and 1.27: central 548^2, 5 rows of pairs 15.4 us, 7 of single columns 14.1; DVM 128^2 7.3 -> 5.0,
+// 256^2 8.6 -> 7.2; LBM 1024^2 23.1 -> 18.8; three-stage 850^2 72.3 -> 63.9.)
 // Segments over 64 rows lose again (4096^2, 241 rows in one wave: 478 us): the rows in flight then
 // lie all over the planes, more pages than the TLB holds.
 // FP64: the FP64 unit of each scheduler issues a warp instruction in 64 cycles whatever the
@@ -222,25 +226,65 @@ inline int march_segment_rows(int want, int ny) {
     const int n = march_segments(want, ny);
     return (ny + n - 1) / n;
 }
-// What the rule needs of a kernel, for single columns and pairs (index: columns - 1): strips of a
-// grid, resident warps an SM; in one wave, us a launch and a row with 1 to 4 warps on the busiest
-// scheduler; in several, us a row of a full wave; rows that a segment costs past its own in one and
-// in several waves, and in FP64.
+// What the rule needs of a kernel with lanes of one width: resident warps an SM; in one wave, us a launch, more where
+// the next kernel is not scheduled early, and a row's us: `row` and `more` for each warp of the fullest SM (counted in
+// steps of `step`), of a segment's rows and `extra1`; in several waves, us a row of a full wave, rows that a segment
+// costs past its own and the largest part of a wave that is lost; the part of a wave from which the next kernel
+// is scheduled early, and the longest segments for which it is. The costs of a three-stage step are those of its two kernels.
+struct MarchLanes {
+    double slots, launch, late, row, more;
+    int step;
+    double extra1, unit, extra2, tail, early;
+    int early_rows;
+};
+// For single columns and pairs; the part of a wave below which the next kernel is scheduled early too, and the rows that a
+// segment costs past its own in FP64.
+// Early scheduling of the next kernel hides its launch and velocity factors (512^2: 15.5 against 16.5 us). On a
+// chip half full it costs instead, because the waiting warps fill some SMs and leave others idle (256^2, 860
+// warps: 10.2 against 9.1), in long segments of pairs in the three-stage scheme (7 rows, 900 x 500 45.1 against 47.7;
+// 9 rows, 768^2 59.3 against 51.1; 12 rows that fill the wave, central 900^2, 70.4 against 66), for the LBM within a wave (512^2, single columns of 6 rows, 11 against
+// 9.4), and in FP64, where a scheduler with two warps takes twice as long.
 struct MarchShape {
     int (*strips)(int cols, int nx);
-    double slots[2], launch[2], row[2][4], unit[2], extra1, extra2, extra64;
+    MarchLanes lanes[2];
+    double few, extra64;
 };
-inline const MarchShape &march_shape() {
-    static const MarchShape s{march_strips, {12, 8}, {4.9, 5.7}, {{0.92, 1.24, 1.51, 1.51}, {1.45, 1.92, 1.92, 1.92}},
-                              {1.12, 1.36}, 0.0, 3.5, 2.5};
-    return s;
+inline const MarchShape &march_shape(int stages, int flux) {
+    static const MarchShape s[4] = {
+        {march_strips,
+         {{12, 4.9, 0.9, 0.62, 0.075, 4, 0, 1.12, 3.5, 0.7, 0.667, 64},
+          {8, 5.7, 0.9, 0.98, 0.1175, 4, 0, 1.36, 3.5, 0.7, 0.52, 64}},
+         0.15, 2.5},
+        {march_strips,
+         {{12, 4.08, 0, 0.81, 0.06, 1, 1.33, 1.02, 4.39, 0.67, 0.667, 64},
+          {8, 0, 0, 1.49, 0.04, 1, 4.55, 1.36, 3.5, 0.7, 0.52, 64}},
+         0.15, 2.5},
+        {march_strips,
+         {{12, 6.2, 0, 1.95, 0.13, 1, 0.57, 4.17, 3.44, 0.47, 0.667, 64},
+          {8, 1.6, 0, 4.09, 0.06, 1, 1.75, 3.03, 6.04, 1.07, 0.52, 7}},
+         0.15, 2.5},
+        {march_strips,
+         {{12, 8.06, 0, 1.57, 0.16, 1, 0.96, 2.73, 3.09, 0.59, 0.667, 64},
+          {8, 0, 0, 3.25, 0.13, 1, 3.97, 3.14, 4.59, 0.64, 0.52, 7}},
+         0.15, 2.5}};
+    return s[(stages == 3 ? 2 : 0) + (flux == 1 ? 1 : 0)];
 }
-// the DVM (measured in FP32 at dt = 0.8: 256^2 7.8 us, single columns, 2 rows, against 8.8 for pairs;
-// 512^2 14.2, pairs, 4 rows; 1024^2 27.8, pairs, 12 rows, against 31.1 for single columns)
-inline const MarchShape &dvm_shape() {
-    static const MarchShape s{dvm_march_strips, {16, 12}, {3.6, 3.6}, {{0.79, 0.89, 0.92, 1.0}, {0.96, 1.05, 1.06, 1.06}},
-                              {0.88, 1.1}, 6.0, 6.0, 6.0};
-    return s;
+// the DVM: displacements below half a cell, from there up, and of one cell (the LBM)
+inline const MarchShape &dvm_shape(double dt) {
+    static const MarchShape s[3] = {
+        {dvm_march_strips,
+         {{16, 0.04, 0.42, 0.86, 0.04, 1, 2.99, 1.42, 4.91, 0.71, 1.0, 64},
+          {12, 0.06, 1.04, 1.05, 0.04, 1, 2.73, 1.13, 2.54, 1.06, 0.667, 64}},
+         0.1, 6.0},
+        {dvm_march_strips,
+         {{16, 0.67, 0.01, 0.79, 0.05, 1, 3.05, 1.31, 4.78, 0.65, 0.76, 64},
+          {12, 0, 0.07, 1.18, 0.06, 1, 3.1, 1.43, 3.05, 0.72, 0.667, 64}},
+         0.1, 6.0},
+        {dvm_march_strips,
+         {{16, 0.06, 0.14, 0.71, 0.03, 1, 4.25, 1.57, 2.75, 0.52, 1.3, 64},
+          {12, 1.14, 0.39, 1.02, 0.07, 1, 1.99, 1.28, 2.44, 0.49, 1.05, 64}},
+         0.15, 6.0}};
+    return s[dt == 1.0 ? 2 : dt >= 0.5 ? 1 : 0];
 }
 // Strip segments that a set of grids gives, for every lane width (index: columns - 1) and segment length.
 // Kept from one plan to the next where grids come and go one at a time.
@@ -272,25 +316,20 @@ inline MarchPlan march_plan(const MarchShape &sh, int variant, const MarchWork &
     for (int i = 0; i < (forced ? count : 0); i++) longest = std::max(longest, march_segment_rows(forced, sizes[i].y));
     for (int cols = 1; cols <= (f64 ? 1 : 2); cols++) {
         const int c = cols - 1;
+        const MarchLanes &q = sh.lanes[c];
         for (int want = forced ? forced : 1; want <= (forced ? forced : MARCH_ROWS); want++) {
             const double w = (double)work.n[c][want];
             const int rows = forced ? longest : want;
-            const double W = w / (sh.slots[c] * sms), n = w / (4.0 * sms);
-            // Early scheduling of the next kernel hides its launch and velocity factors
-            // (512^2: 15.5 against 16.5 us). On a chip half full it costs instead, because the
-            // waiting warps fill some SMs and leave others idle (256^2, 860 warps: 10.2 against
-            // 9.1), and in FP64, where a scheduler with two warps takes twice as long.
-            // Single columns: up to two warps a scheduler stay apart (248^2, FP32 7.6 -> 7.2, FP16 storage
-            // 8.3 -> 7.6 us; 260^2, a few more warps: 7.5 with, 8.2 without).
-            const bool early = !f64 && (W > (cols == 1 ? 2.0 / 3.0 : 0.6) || W < 0.15);
+            const double W = w / (q.slots * sms), n = w / (4.0 * sms);
+            const bool early = !f64 && (rows <= q.early_rows || (W > 0.965 && W <= 1.0)) && (W > q.early || W < sh.few);
             double cost;
             if (f64)
                 cost = (n > 3.0 ? n + 0.5 : std::ceil(n)) * (rows + sh.extra64);
             else if (W <= 1.0)
-                cost = sh.launch[c] + (early ? 0.0 : 0.9) +
-                       (rows + sh.extra1) * sh.row[c][std::min(3, std::max(0, (int)std::ceil(n) - 1))];
+                cost = q.launch + (early && !(rows == 1 && W > 0.9) ? 0.0 : q.late) +   // (no room for the next kernel's warps)
+                       (rows + q.extra1) * (q.row + q.more * q.step * std::ceil(w / (q.step * (double)sms)));
             else
-                cost = sh.unit[c] * (rows + sh.extra2) * (W + std::min(0.7, 1.4 / W));
+                cost = q.unit * (rows + q.extra2) * (W + std::min(q.tail, 1.4 / W));
             if (cost < best) {
                 best = cost;
                 // (FP64 warps on every scheduler of an SM: a row takes a tenth longer)

@@ -1,4 +1,4 @@
-// Host program of march_plans.py. Input lines: kernel (0 DUGKS, 1 DVM) precision variant sms count x y x y ...;
+// Host program of march_plans.py. Input lines: stages flux dt precision variant sms count x y x y ...;
 // output lines: columns, rows and mode of the plan, from segments that were counted one grid at a time, with others
 // that came and went, and from a pass over all grids for every plan.
 #include <cstdio>
@@ -37,9 +37,10 @@ static MarchPlan by_passes(const MarchShape &sh, int variant, const std::vector<
 }
 
 int main() {
-    int kernel, precision, variant, sms, count;
-    while (std::scanf("%d %d %d %d %d", &kernel, &precision, &variant, &sms, &count) == 5) {
-        const MarchShape &sh = kernel ? dvm_shape() : march_shape();
+    int stages, flux, precision, variant, sms, count;
+    double dt;
+    while (std::scanf("%d %d %lf %d %d %d %d", &stages, &flux, &dt, &precision, &variant, &sms, &count) == 7) {
+        const MarchShape &sh = stages == 1 ? dvm_shape(dt) : march_shape(stages, flux);
         std::vector<int2> sizes(count);
         MarchWork work;
         for (int2 &q : sizes) {

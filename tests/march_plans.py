@@ -25,10 +25,10 @@ def run(lines):
     return [[int(v) for v in r.split()] for r in out.splitlines()]
 
 
-def plan(precision, sizes, dvm=False, variant=4, sms=None):
+def plan(precision, sizes, stages=2, flux=0, cfl=0.8, variant=4, sms=None):
     """(columns a lane, rows a segment) for grids of these (nx, ny) stepped together on this device."""
     if sms is None:
         import torch
         sms = torch.cuda.get_device_properties(0).multi_processor_count
     flat = " ".join(f"{x} {y}" for x, y in sizes)
-    return tuple(run([f"{int(dvm)} {PRECISIONS[precision]} {variant} {sms} {len(sizes)} {flat}"])[0][:2])
+    return tuple(run([f"{stages} {flux} {cfl} {PRECISIONS[precision]} {variant} {sms} {len(sizes)} {flat}"])[0][:2])
