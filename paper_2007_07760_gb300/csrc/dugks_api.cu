@@ -485,7 +485,7 @@ int step_dvm(dugks_ctx *c) {
         e = launch_dvm_march<T>(q, dv, *reinterpret_cast<const MarchCoefs<T> *>(c->coefs.data()),
                                 vortex_factors<T>(c, t + dt, t, t), dt == 1.0, c->plan.cols, c->stream);
     } else {
-        e = launch_dvm<T>(q, dv, c->p.order, dt == 1.0, c->stream);
+        e = launch_dvm<T>(q, dv, dt == 1.0, c->stream);
     }
     if (e != cudaSuccess) return cuda_fail(c, e, "DVM kernel");
     c->cur = 1 - c->cur;

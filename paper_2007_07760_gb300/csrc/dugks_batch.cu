@@ -285,8 +285,6 @@ void fill_uniform(dugks_batch *b) {
     const double dt = b->p.cfl, tau = 3.0 * b->p.M, h = 0.5 * dt;
     const double bb = (dt + h) / (2.0 * tau + dt);   // bar f^+ = X + b (g - X)
     u.b = (T)bb;
-    u.h = (T)h;
-    u.c1 = (T)(2.0 * tau / (2.0 * tau + h));
     u.c2 = (T)(h / (2.0 * tau + h));
     u.c3 = (T)(tau * h / (2.0 * tau + h));
     u.be1 = (T)(4.0 / 3.0 * bb);

@@ -37,10 +37,11 @@ struct DvmExtra {
     int early;   // row march: dependents may be scheduled at once
 };
 
-template <typename T, int ORDER, bool LBM>
+// (order 4)
+template <typename T, bool LBM>
 struct DvmTile {
     static constexpr int TX = 32, TY = 8, NT = TX * TY;
-    static constexpr int R = ORDER == 4 ? 2 : 1;          // stencil radius
+    static constexpr int R = 2;                           // stencil radius
     static constexpr int HS = LBM ? R + 1 : 2 * R + 1;    // state halo
     static constexpr int SW = TX + 2 * HS, SH = TY + 2 * HS;
     static constexpr int PW = TX + 2 * R, PH = TY + 2 * R;   // phi(t + dt) region
@@ -52,9 +53,9 @@ struct DvmTile {
     static_assert(RING <= NT, "one ring cell per thread");
 };
 
-template <typename T, int ORDER, bool LBM>
+template <typename T, bool LBM>
 __global__ void __launch_bounds__(256) dvm_step_kernel(const StepParams<T> p, const DvmExtra<T> dv) {
-    using DT = DvmTile<T, ORDER, LBM>;
+    using DT = DvmTile<T, LBM>;
     constexpr int TX = DT::TX, TY = DT::TY, HS = DT::HS, SW = DT::SW, SH = DT::SH, R = DT::R;
     constexpr int PW = DT::PW, PH = DT::PH;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -84,7 +85,7 @@ __global__ void __launch_bounds__(256) dvm_step_kernel(const StepParams<T> p, co
                 fs[k] = F[(y - ey(k) + HS) * SW + (x - ex(k) + HS)];
             } else {
                 const int xn = x - dv.s * ex(k), yn = y - dv.s * ey(k);
-                fs[k] = taylor<T, ORDER>(F + (yn + HS) * SW + (xn + HS), SW, dv.d * T(ex(k)), dv.d * T(ey(k)));
+                fs[k] = taylor<T, 4>(F + (yn + HS) * SW + (xn + HS), SW, dv.d * T(ex(k)), dv.d * T(ey(k)));
             }
             phi += fs[k];   // Eq. (13), the unweighted sum
         }
@@ -116,7 +117,7 @@ __global__ void __launch_bounds__(256) dvm_step_kernel(const StepParams<T> p, co
         const T *P = sP + (ty + R) * PW + (tx + R);
         const T ph = P[0];
         T gxp, gyp;
-        grad_p<T, ORDER>(P, PW, gxp, gyp);
+        grad_p<T, 4>(P, PW, gxp, gyp);
         const T g2 = gxp * gxp + gyp * gyp;
         T nxv = T(0), nyv = T(0);
         if (g2 > T(1e-24)) {

@@ -1,7 +1,7 @@
 // dugks_fast.cuh -- the DUGKS step staged by TMA (sm_103a): the two-stage step of
-// orders 4 and 5 and the two kernels of the three-stage step, orders 2 to 4 (the
-// two-stage step of orders 2 and 3 is the row march, dugks_march.cuh, but for the FP64
-// sizes that tile64_pays of dugks_host.h gives to the tiles).
+// orders 4 and 5 and the two kernels of the three-stage step of order 4. The steps of
+// orders 2 and 3 are the row march (dugks_march.cuh), but for the two-stage step in FP64
+// at the sizes that tile64_pays of dugks_host.h gives to these tiles.
 //
 // Same arithmetic as step_kernel (dugks_kernels.cuh), organised for throughput:
 //  * the tile's 9 distribution planes plus a halo of 1 + 2R cells (stencil radius

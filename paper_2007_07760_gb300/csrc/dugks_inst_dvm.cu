@@ -9,10 +9,10 @@ namespace dugks {
 
 namespace {
 
-template <typename T, int ORDER, bool LBM>
+template <typename T, bool LBM>
 cudaError_t launch_dvm_t(const StepParams<T> &p, const DvmExtra<T> &dv, cudaStream_t s) {
-    using DT = DvmTile<T, ORDER, LBM>;
-    auto kern = dvm_step_kernel<T, ORDER, LBM>;
+    using DT = DvmTile<T, LBM>;
+    auto kern = dvm_step_kernel<T, LBM>;
     // the dynamic shared-memory limit is a per-function, per-device attribute
     static std::atomic<uint64_t> configured{0};
     int dev = 0;
@@ -27,11 +27,6 @@ cudaError_t launch_dvm_t(const StepParams<T> &p, const DvmExtra<T> &dv, cudaStre
     const dim3 grid((p.nx + DT::TX - 1) / DT::TX, (p.ny + DT::TY - 1) / DT::TY);
     kern<<<grid, DT::NT, DT::smem_bytes, s>>>(p, dv);
     return cudaGetLastError();
-}
-
-template <typename T, bool LBM>
-cudaError_t launch_dvm_o(const StepParams<T> &p, const DvmExtra<T> &dv, int order, cudaStream_t s) {
-    return order == 4 ? launch_dvm_t<T, 4, LBM>(p, dv, s) : cudaErrorInvalidValue;
 }
 
 template <typename V, int MODE>
@@ -49,9 +44,10 @@ cudaError_t launch_dvm_m(const StepParams<typename Lane<V>::T> &p, const DvmExtr
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    // (the mass partials are written where the caller asks for them)
-    return p.mass_partial != nullptr ? cudaLaunchKernelEx(&cfg, dvm_march_kernel<V, MODE, true>, p, dv, cf, fe)
-                                     : cudaLaunchKernelEx(&cfg, dvm_march_kernel<V, MODE, false>, p, dv, cf, fe);
+    // (the mass partials are written where the caller asks for them; FP64 steps always do)
+    if constexpr (sizeof(typename Lane<V>::T) == 4)
+        if (p.mass_partial == nullptr) return cudaLaunchKernelEx(&cfg, dvm_march_kernel<V, MODE, false>, p, dv, cf, fe);
+    return cudaLaunchKernelEx(&cfg, dvm_march_kernel<V, MODE, true>, p, dv, cf, fe);
 }
 
 template <typename V>
@@ -65,8 +61,8 @@ cudaError_t launch_dvm_v(const StepParams<typename Lane<V>::T> &p, const DvmExtr
 }  // namespace
 
 template <typename T>
-cudaError_t launch_dvm(const StepParams<T> &p, const DvmExtra<T> &dv, int order, bool lbm, cudaStream_t s) {
-    return lbm ? launch_dvm_o<T, true>(p, dv, order, s) : launch_dvm_o<T, false>(p, dv, order, s);
+cudaError_t launch_dvm(const StepParams<T> &p, const DvmExtra<T> &dv, bool lbm, cudaStream_t s) {
+    return lbm ? launch_dvm_t<T, true>(p, dv, s) : launch_dvm_t<T, false>(p, dv, s);
 }
 
 template <typename T>
@@ -80,7 +76,7 @@ int dvm_march_strips(int cols, int nx) { return cols == 2 ? DvmMarch<float2>::st
 
 template cudaError_t launch_dvm_march<double>(const StepParams<double> &, const DvmExtra<double> &, const MarchCoefs<double> &, const FastExtra<double> &, bool, int, cudaStream_t);
 template cudaError_t launch_dvm_march<float>(const StepParams<float> &, const DvmExtra<float> &, const MarchCoefs<float> &, const FastExtra<float> &, bool, int, cudaStream_t);
-template cudaError_t launch_dvm<double>(const StepParams<double> &, const DvmExtra<double> &, int, bool, cudaStream_t);
-template cudaError_t launch_dvm<float>(const StepParams<float> &, const DvmExtra<float> &, int, bool, cudaStream_t);
+template cudaError_t launch_dvm<double>(const StepParams<double> &, const DvmExtra<double> &, bool, cudaStream_t);
+template cudaError_t launch_dvm<float>(const StepParams<float> &, const DvmExtra<float> &, bool, cudaStream_t);
 
 }  // namespace dugks

@@ -70,12 +70,12 @@ cudaError_t launch_batch_advance(BatchGrid<T> *grids, int ngrids, int n, double 
 
 cudaError_t launch_mass_final(const double *partial, int n, double *out, int *status, int early, cudaStream_t s);
 
-// One step of the streaming-collision DVM (dugks_inst_dvm.cu); lbm: the plain
+// One step of the streaming-collision DVM of order 4 (dugks_inst_dvm.cu); lbm: the plain
 // streaming of dt = 1 (T = double or float, full storage).
 template <typename T>
 struct DvmExtra;
 template <typename T>
-cudaError_t launch_dvm(const StepParams<T> &p, const DvmExtra<T> &dv, int order, bool lbm, cudaStream_t s);
+cudaError_t launch_dvm(const StepParams<T> &p, const DvmExtra<T> &dv, bool lbm, cudaStream_t s);
 // the same as a row march (orders 2 and 3), `cols` columns a lane, segments of p.tile_h rows
 template <typename T>
 cudaError_t launch_dvm_march(const StepParams<T> &p, const DvmExtra<T> &dv, const MarchCoefs<T> &cf,

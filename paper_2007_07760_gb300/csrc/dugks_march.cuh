@@ -1063,7 +1063,7 @@ struct BatchGrid {
 // Parameters common to every grid of a batch (same W, M, cfl, order, flux, precision).
 template <typename T>
 struct BatchUniform {
-    T b, h, c1, c2, c3, be1, ga1, tau, theta_c, phiA, phiB, inv_dt, qscale, qinv;
+    T b, c2, c3, be1, ga1, tau, theta_c, phiA, phiB, inv_dt, qscale, qinv;
     double dt;
     int dtphiu;
     int *status;

@@ -42,3 +42,14 @@ def test_counted_segments_give_the_same_plan(precision):
 def test_plans_measured_best(kw, nx, ny, plans):
     got = march_plans.plan("fp32", [(nx, ny)], sms=152, **kw)
     assert got in plans
+
+
+def test_autotuned_variants_differ():
+    """No two variants that the autotuner times are the same plan at every size."""
+    from paper_2007_07760_gb300 import autotune
+    sizes = [(64, 64), (256, 256), (700, 700), (2048, 2048)]
+    seen = {}
+    for v in autotune.VARIANTS:
+        key = tuple(march_plans.plan("fp32", [s], variant=v, sms=152) for s in sizes)
+        assert key not in seen, (v, seen[key])
+        seen[key] = v

@@ -33,3 +33,14 @@ def test_mass_sum_triggers_before_it_reads_an_argument():
     params, body = next((p, b) for name, p, b in kernels() if name == "mass_final_kernel")
     before = body[:body.index("pdl_trigger()")]
     assert not [w for w in re.findall(r"(\w+)\s*(?:,|$)", params) if re.search(rf"\b{w}\b", before)]
+
+
+def test_batch_constants_are_read():
+    """Every constant that a batch sends with each launch is read by its kernel."""
+    text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "dugks_march.cuh")).read())
+    fields = re.search(r"struct BatchUniform \{(.*?)\};", text, flags=re.S).group(1)
+    names = [w for line in fields.split(";") for w in re.findall(r"\*?(\w+)\s*(?:,|$)", line.strip())]
+    host = open(os.path.join(CSRC, "dugks_batch.cu")).read()
+    assert "be1" in names and "status" in names
+    for n in names:
+        assert re.search(rf"\bu\.{n}\b", text) or re.search(rf"\bu\.{n}\b(?!\s*=)", host), n
