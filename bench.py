@@ -67,10 +67,10 @@ L2_FLUSH_BYTES = 512 << 20
 # was taken on and the workload (reported as null once the sources change). The
 # writes of a 1024^2 step stay in L2 (129 MB) during the launch and reach DRAM
 # later, so the figure is the read traffic plus the evictions.
-# (Captured on the same code: only comments have changed since.)
+# (The launch that also writes the mass partials, as a step and its mass do.)
 NCU_TRAFFIC = {
-    ("8ad1c357ad1e25d9", "vortex1024_fp32_p3_upwind_2stage"): 51648512,
-    ("8ad1c357ad1e25d9", "vortex4096_fp32_p3_upwind_2stage"): 1460551680,   # state 11x the L2
+    ("01411df48670b7ba", "vortex1024_fp32_p3_upwind_2stage"): 51665152,
+    ("01411df48670b7ba", "vortex4096_fp32_p3_upwind_2stage"): 1461232640,   # state 11x the L2
 }
 
 

@@ -164,9 +164,10 @@ __global__ void __launch_bounds__(256) dvm_step_kernel(const StepParams<T> p, co
 // cell c is tilde f'_k of cell c + xi_k: a shuffle over columns, and rows j - 2, j - 1, j for
 // xi_y = -1, 0, 1, so that row j - 2 of tilde f' and of phi(t + dt) is then complete, and row j - 3
 // has its gradient and is written. Without it (MODE 0) row j - 1 is complete; at dt = 1 (MODE 2, the
-// LBM) the rows themselves are shifted. Bound by instruction issue; measured in FP32 at 512^2,
-// order 3, dt = 0.8, a step: 14.2 us against 30 for the tile kernel (every tap read from shared
-// memory, sines and cosines for every cell), at 1024^2 27.8 against 112.
+// LBM) the rows themselves are shifted. Bound by a row's latency in one wave of warps, then by instruction
+// issue; measured in FP32, order 3, dt = 0.8, a step, against the tile kernel that it replaced (every tap read from
+// shared memory, sines and cosines for every cell): 128^2 5.0 us, 14.4 before; 512^2 11.8, 30.1; 1024^2 25.1, 96.3;
+// LBM 1024^2 18.8, 72.8.
 template <typename V>
 struct DvmMarch {
     using T = typename Lane<V>::T;
