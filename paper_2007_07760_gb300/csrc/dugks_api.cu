@@ -20,6 +20,7 @@
 #include "dugks_dvm.cuh"
 #include "dugks_host.h"
 #include "dugks_internal.h"
+#include "dugks_sum.cuh"
 
 using namespace dugks;
 using namespace dugks::host;
@@ -539,7 +540,10 @@ int enqueue_mass(dugks_ctx *c, double *dev_out) {
         c->mass_valid = true;
     }
     const int early = (c->fast && c->march) || dvm_marches(c) ? c->plan.early : 1;
-    e = launch_mass_final(c->partial, c->ntiles, dev_out, c->dstatus, early, c->stream);
+    // (a loop of three-stage steps in pairs takes 2 to 5 % longer after the shorter sum: 512^2 32.5 -> 33.1 us, 575^2
+    // 37.6 -> 38.8)
+    const bool words = !(c->p.stages == 3 && c->march && c->plan.cols == 2);
+    e = launch_mass_final(c->partial, c->ntiles, dev_out, c->dstatus, early, words, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "mass kernel");
     return DUGKS_OK;
 }
@@ -610,24 +614,68 @@ cudaError_t dev_malloc_pool(void **p, size_t bytes, cudaMemPool_t pool, cudaStre
     return cudaMallocFromPoolAsync(p, bytes, pool, s);
 }
 
-// Fixed-order sum of the per-tile partials (deterministic); flags NaN / Inf.
-// Thread t adds partials t, t + 256, ... in index order with 8 independent loads
-// in flight (one memory latency per 8 partials), then the fixed tree of block_sum.
+// Sum of the per-tile partials (deterministic); flags NaN / Inf.
+// Up to 2048 partials, eight a thread, are added as integers (dugks_sum.cuh): the FP64 additions of eight warps
+// and their trees were a fifth of what a step and its mass take longer than the step. The march has several times
+// the partials that tiles had; measured, step and mass: FP32 64^2 6.4 -> 6.2 us, 256^2 10.5 -> 10.1, FP16 storage 312^2 12.8 ->
+// 12.5, 1024^2 39.9 -> 39.5. Few partials (the tiles of small grids of order 4: 256^2 15.7 -> 16.0 us
+// with both ways in one kernel), more of them, and sums past the range of that, in a fixed order in
+// FP64: thread t adds partials t, t + 256, ... with 8 independent loads in flight (one memory latency per
+// 8 partials), then the fixed tree of block_sum.
 // One small CTA: it finds a free slot while the step kernel drains.
 // EARLY: the next kernel may be placed while the step ahead still runs (where that costs the
 // march nothing: MarchPlan::early; FP64 512^2 step and mass: 331 us with, 258 without). Not an argument: loading
 // it first put the next kernel off (order 4, 256^2, step and mass: 15.26 -> 15.37 us, three-stage 200^2 27.10 -> 27.22).
-template <bool EARLY>
+// (A kernel of its own for the former: WORDS.)
+constexpr int SUM_FEW = 128;
+template <bool EARLY, bool WORDS>
 __global__ void __launch_bounds__(256) mass_final_kernel(const double *partial, int n, double *out, int *status) {
     __shared__ double sred[32];
     if (EARLY) pdl_trigger();
     pdl_wait();   // the partials of the step kernel ahead of it
     constexpr int U = 8;
-    double s = 0.0;
-    for (int base = threadIdx.x; base < n; base += U * 256) {
-        double v[U];
+    static_assert(U * 256 == SUM_MAX, "one round of loads");
+    double v[U], s = 0.0;
+    auto load = [&](int base) {
 #pragma unroll
         for (int u = 0; u < U; u++) v[u] = base + u * 256 < n ? partial[base + u * 256] : 0.0;
+    };
+    if constexpr (WORDS) {
+        __shared__ int stop[8];
+        __shared__ __int128 sint[8];
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        load(threadIdx.x);
+        int top = 0;
+#pragma unroll
+        for (int u = 0; u < U; u++) top = max(top, exponent_of(v[u]));
+        top = __reduce_max_sync(0xffffffffu, top);
+        if (lane == 0) stop[warp] = top;
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < 8; w++) top = max(top, stop[w]);
+        if (top >= SUM_LO && top < SUM_HI) {
+            __int128 a = 0;
+#pragma unroll
+            for (int u = 0; u < U; u++) a += aligned(v[u], top);
+            auto tree = [&](int from) {
+                for (int o = from; o > 0; o >>= 1) {
+                    const unsigned long long hi = __shfl_down_sync(0xffffffffu, (unsigned long long)(a >> 64), o);
+                    const unsigned long long lo = __shfl_down_sync(0xffffffffu, (unsigned long long)a, o);
+                    a += (__int128)(((unsigned __int128)hi << 64) | lo);
+                }
+            };
+            tree(16);
+            if (lane == 0) sint[warp] = a;
+            __syncthreads();
+            if (warp > 0) return;
+            a = lane < 8 ? sint[lane] : 0;
+            tree(4);
+            if (lane == 0) *out = unaligned(a, top);
+            return;
+        }
+    }
+    for (int base = threadIdx.x; base < n; base += U * 256) {
+        load(base);
 #pragma unroll
         for (int u = 0; u < U; u++) s += v[u];
     }
@@ -638,7 +686,8 @@ __global__ void __launch_bounds__(256) mass_final_kernel(const double *partial, 
     }
 }
 
-cudaError_t launch_mass_final(const double *partial, int n, double *out, int *status, int early, cudaStream_t s) {
+cudaError_t launch_mass_final(const double *partial, int n, double *out, int *status, int early, bool words,
+                              cudaStream_t s) {
     // programmatic dependent launch: resident while the step kernel drains, it
     // waits for the partials in the kernel itself
     cudaLaunchConfig_t cfg = {};
@@ -650,8 +699,10 @@ cudaError_t launch_mass_final(const double *partial, int n, double *out, int *st
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, early ? mass_final_kernel<true> : mass_final_kernel<false>, partial, n, out,
-                                       status);
+    words = words && n > SUM_FEW && n <= SUM_MAX;
+    auto kern = words ? (early ? mass_final_kernel<true, true> : mass_final_kernel<false, true>)
+                      : (early ? mass_final_kernel<true, false> : mass_final_kernel<false, false>);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, partial, n, out, status);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }

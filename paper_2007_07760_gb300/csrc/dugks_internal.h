@@ -68,7 +68,8 @@ struct Launch {
 template <typename T>
 cudaError_t launch_batch_advance(BatchGrid<T> *grids, int ngrids, int n, double dt, cudaStream_t s);
 
-cudaError_t launch_mass_final(const double *partial, int n, double *out, int *status, int early, cudaStream_t s);
+// words: as integers, where there are as many partials as gain by it
+cudaError_t launch_mass_final(const double *partial, int n, double *out, int *status, int early, bool words, cudaStream_t s);
 
 // One step of the streaming-collision DVM of order 4 (dugks_inst_dvm.cu); lbm: the plain
 // streaming of dt = 1 (T = double or float, full storage).
