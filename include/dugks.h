@@ -148,8 +148,9 @@ int dugks_read_phi_device(dugks_ctx *c, void *dev_out);
  * doubles of device scratch cannot be allocated. */
 int dugks_debug_faces(dugks_ctx *c, double *fbar_E, double *fbar_N, double *f_E, double *f_N);
 
-/* Waits and returns the total mass sum phi over all cells, reduced in FP64 in
- * a fixed order (deterministic). DUGKS_ENONFINITE if it is NaN or Inf. */
+/* Waits and returns the total mass sum phi over all cells, to FP64 precision and
+ * deterministic (partials in FP64 in a fixed order, then their sum, exactly where they
+ * are few enough). DUGKS_ENONFINITE if it is NaN or Inf. */
 int dugks_mass(dugks_ctx *c, double *out);
 
 /* Enqueues the same reduction into dev_out (one double, device); no wait. */
