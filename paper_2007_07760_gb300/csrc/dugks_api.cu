@@ -539,10 +539,12 @@ int enqueue_mass(dugks_ctx *c, double *dev_out) {
         if (e != cudaSuccess) return cuda_fail(c, e, "mass partial kernel");
         c->mass_valid = true;
     }
-    const int early = (c->fast && c->march) || dvm_marches(c) ? c->plan.early : 1;
-    // (a loop of three-stage steps in pairs takes 2 to 5 % longer after the shorter sum: 512^2 32.5 -> 33.1 us, 575^2
-    // 37.6 -> 38.8)
-    const bool words = !(c->p.stages == 3 && c->march && c->plan.cols == 2);
+    const bool march = (c->fast && c->march) || dvm_marches(c);
+    const int early = march ? c->plan.early : 1;
+    // (A loop of three-stage steps in pairs takes 2 to 5 % longer after the shorter sum: 512^2 32.5 -> 33.1 us, 575^2
+    // 37.6 -> 38.8. So do order 4's tiles, whose code has to come back into the instruction caches after every
+    // other kernel, where L2 is flushed between steps: 1024^2 84.2 -> 85.5, central 76.0 -> 78.4.)
+    const bool words = march && !(c->p.stages == 3 && c->plan.cols == 2);
     e = launch_mass_final(c->partial, c->ntiles, dev_out, c->dstatus, early, words, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "mass kernel");
     return DUGKS_OK;
@@ -618,10 +620,9 @@ cudaError_t dev_malloc_pool(void **p, size_t bytes, cudaMemPool_t pool, cudaStre
 // Up to 2048 partials, eight a thread, are added as integers (dugks_sum.cuh): the FP64 additions of eight warps
 // and their trees were a fifth of what a step and its mass take longer than the step. The march has several times
 // the partials that tiles had; measured, step and mass: FP32 64^2 6.4 -> 6.2 us, 256^2 10.5 -> 10.1, FP16 storage 312^2 12.8 ->
-// 12.5, 1024^2 39.9 -> 39.5. Few partials (the tiles of small grids of order 4: 256^2 15.7 -> 16.0 us
-// with both ways in one kernel), more of them, and sums past the range of that, in a fixed order in
-// FP64: thread t adds partials t, t + 256, ... with 8 independent loads in flight (one memory latency per
-// 8 partials), then the fixed tree of block_sum.
+// 12.5, 1024^2 39.9 -> 39.5. Few partials (order 4, 256^2: 15.7 -> 16.0 us with both ways in one kernel), more
+// of them, and sums past the range of that, in a fixed order in FP64: thread t adds partials t, t + 256, ... with 8
+// independent loads in flight (one memory latency per 8 partials), then the fixed tree of block_sum.
 // One small CTA: it finds a free slot while the step kernel drains.
 // EARLY: the next kernel may be placed while the step ahead still runs (where that costs the
 // march nothing: MarchPlan::early; FP64 512^2 step and mass: 331 us with, 258 without). Not an argument: loading
