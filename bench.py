@@ -69,8 +69,8 @@ L2_FLUSH_BYTES = 512 << 20
 # later, so the figure is the read traffic plus the evictions.
 # (The launch that also writes the mass partials, as a step and its mass do.)
 NCU_TRAFFIC = {
-    ("33c4d7bcc4a1c866", "vortex1024_fp32_p3_upwind_2stage"): 52188928,
-    ("33c4d7bcc4a1c866", "vortex4096_fp32_p3_upwind_2stage"): 1461606912,   # state 11x the L2
+    ("afb19a1685ec7efd", "vortex1024_fp32_p3_upwind_2stage"): 51940608,
+    ("afb19a1685ec7efd", "vortex4096_fp32_p3_upwind_2stage"): 1461483520,   # state 11x the L2
 }
 
 
